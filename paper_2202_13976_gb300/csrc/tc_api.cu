@@ -107,11 +107,15 @@ struct tc_graph {
     int32_t hub_cap = 0;
     uint32_t* hub_cnt = nullptr;
     int64_t* hub_start = nullptr;
-    uint32_t* hub_cur = nullptr;
     unsigned long long* hub_cur64 = nullptr;
     int32_t* big_list = nullptr;
-    int32_t* med_list = nullptr;
-    int4* in_rec = nullptr;
+    int32_t* long_list = nullptr;
+    int4* win_task = nullptr;
+    int4* low_task = nullptr;
+    uint2* winrow = nullptr;
+    uint4* winlow = nullptr;
+    uint4* win = nullptr;
+    uint2* in_rec = nullptr;
     int32_t* rowof = nullptr;
     void* plan_tmp = nullptr;
     int32_t src_lo = 0, src_hi = -1;  // ranks of the sources counted (-1: up to n); tc_count_shard
@@ -286,9 +290,14 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
         (st = dalloc(g, &g->small_list[2], nn, &keep)) || (st = dalloc(g, &g->small_list[3], nn, &keep)) ||
         (st = dalloc(g, &g->cta_list, nn, &keep)) ||
         (st = dalloc(g, &g->hub_cnt, hc + 1, &keep)) || (st = dalloc(g, &g->hub_start, hc + 1, &keep)) ||
-        (st = dalloc(g, &g->hub_cur, hc + 1, &keep)) || (st = dalloc(g, &g->hub_cur64, hc + 1, &keep)) ||
+        (st = dalloc(g, &g->hub_cur64, hc + 1, &keep)) ||
         (st = dalloc(g, &g->big_list, hc + 1, &keep)) ||
-        (st = dalloc(g, &g->med_list, hc + 1, &keep)) || (st = dalloc(g, &g->in_rec, (size_t)m, &keep)) ||
+        (st = dalloc(g, &g->long_list, hc + 1, &keep)) ||
+        (st = dalloc(g, &g->win_task, (size_t)hub_task_cap(g->hub_cap, m), &keep)) ||
+        (st = dalloc(g, &g->low_task, (size_t)hub_task_cap(g->hub_cap, m), &keep)) ||
+        (st = dalloc(g, &g->winrow, nn, &keep)) || (st = dalloc(g, &g->winlow, nn, &keep)) ||
+        (st = dalloc(g, &g->win, (size_t)win_vec_cap(n, m), &keep)) ||
+        (st = dalloc(g, &g->in_rec, (size_t)m, &keep)) ||
         (st = dalloc(g, &g->rowof, (size_t)m, &keep)) ||
         (st = dalloc(g, (char**)&g->plan_tmp, scan_tmp_bytes((int64_t)hc + 1), &keep)) ||
         (st = dalloc(g, &g->t_rank, nn, &keep)) ||
@@ -318,9 +327,7 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
     char* tmp = nullptr;
     if ((st = dalloc(g, &B.dmulti, nn, &scratch)) || (st = dalloc(g, &B.keys, nn, &scratch)) ||
         (st = dalloc(g, &B.keys_alt, nn, &scratch)) || (st = dalloc(g, &B.rowcnt, nn + 1, &scratch)) ||
-        (st = dalloc(g, &B.cursor, nn, &scratch)) || (st = dalloc(g, &B.longlist, nn, &scratch)) ||
-        (st = dalloc(g, &B.midlist, nn, &scratch)) || (st = dalloc(g, &B.midlist2, nn, &scratch)) ||
-        (st = dalloc(g, &B.dupin, nn, &scratch)) ||
+        (st = dalloc(g, &B.cursor, nn, &scratch)) || (st = dalloc(g, &B.dupin, nn, &scratch)) ||
         (st = dalloc(g, &B.bcount, (size_t)BUCKET_MAX + 1, &scratch)) ||
         (st = dalloc(g, &B.bcur, (size_t)BUCKET_MAX, &scratch)) ||
         (st = dalloc(g, &B.bstart, (size_t)BUCKET_MAX + 1, &scratch)) ||
@@ -330,6 +337,12 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
         return st;
     }
     B.tmp = tmp;
+    // the input-order pairs and the sorters' row lists share memory with arrays that the
+    // planner writes after the build is done with them
+    B.oriented = reinterpret_cast<int2*>(g->in_rec);
+    B.longlist = g->small_list[0];
+    B.midlist = g->small_list[1];
+    B.midlist2 = g->small_list[2];
     B.rank = g->rank;
     B.rowstart = g->rowstart;
     B.rowlen = g->rowlen;
@@ -386,10 +399,6 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
         const double mean = n > 0 ? 2.0 * (double)m / (double)n : 0.0;
         B.bucket_fill = m > 0 && (double)h.max_deg <= 64.0 * mean;
     }
-    if (m > 0 && (st = dalloc(g, &B.oriented, (size_t)m, &scratch)) != TC_OK) {
-        free_list(g, &scratch);
-        return st;
-    }
     launch_rank(B, deg_bits, g->L);
     if (bev) cudaEventRecord(bev[BP_RANK], g->stream);
     PlanStreams psv{};
@@ -417,10 +426,15 @@ CountBuffers count_buffers(tc_graph* g) {
     C.hub_cap = g->hub_cap;
     C.hub_cnt = g->hub_cnt;
     C.hub_start = g->hub_start;
-    C.hub_cur = g->hub_cur;
     C.hub_cur64 = g->hub_cur64;
     C.big_list = g->big_list;
-    C.med_list = g->med_list;
+    C.long_list = g->long_list;
+    C.win_task = g->win_task;
+    C.low_task = g->low_task;
+    C.winrow = g->winrow;
+    C.winlow = g->winlow;
+    C.win = g->win;
+    C.win_cap = win_vec_cap(g->n, g->m_alloc);
     C.in_rec = g->in_rec;
     C.rowof = g->rowof;
     C.m_cap = g->m_alloc;

@@ -27,16 +27,22 @@ struct DevStats {
     unsigned int cta_count;        // planner: vertices with d+ > 32
     unsigned int cta_next;         // dynamic work counter of the block push kernel
     unsigned int hub_count;        // vertices staged as hubs (ranks n - hub_count .. n-1)
-    unsigned int hub_next;         // dynamic work counter of the hub kernel (big hubs)
+    unsigned int hub_next;         // dynamic work counter of the hub kernel (slices of big hubs)
     unsigned int hub_next2;        // dynamic work counter of the hub kernel (medium hubs)
+    unsigned int hub_next3;        // dynamic work counter of the list kernel (long lists; probe mode)
+    unsigned int hub_next4;        // dynamic work counter of the below-window kernel
     unsigned int hub_candidates;   // vertices whose degree reaches the hub threshold
     unsigned int hub_big;          // hubs processed by whole blocks
     unsigned int mid_count;        // build: rows of 17..256 entries sorted by one warp
     unsigned int mid2_count;       // build: rows of 257..1024 entries sorted by one warp
     unsigned int core_n;           // planner: dense core size (ranks n - core_n .. n-1)
-    unsigned int pad[1];
+    unsigned int hub_tasks;        // window tasks of big hubs (slices of their in-edges)
+    unsigned int hub_med;          // window tasks of the other hubs
+    unsigned int hub_low;          // below-window tasks
+    unsigned int hub_long;         // big hubs with a long list below the window
+    unsigned int win_vecs;         // planner: 16-byte vectors of window entries written
 };
-static_assert(sizeof(DevStats) == 96, "DevStats layout");
+static_assert(sizeof(DevStats) == 120, "DevStats layout");
 
 struct Launch {
     cudaStream_t stream;
@@ -168,6 +174,18 @@ struct Strategy {
 
 // Capacity of the hub kernel's shared-memory bitmap (ranks above the hub).
 constexpr int HUB_BM_BITS = 131072;
+// Window 1 of the hub kernels: the highest min(n, HUB_WIN) ranks, one 32-bit counter
+// each in shared memory.  An entry x of it is kept as four times its index in the
+// window (the counter's byte offset, 16 bits); 4 * HUB_WIN names the slot that no hub
+// marks.  The windows below it have HUB_WIN2 ranks each, an entry kept as its index.
+constexpr int HUB_WIN = 16383;
+constexpr int HUB_WIN2 = 65535;
+static_assert(4 * HUB_WIN <= 0xffff && HUB_WIN2 <= 0xffff, "window offsets fit 16 bits");
+// In-edges of a hub that one block (one warp for the smaller hubs) takes at a time.
+constexpr int HUB_SLICE = 2048;
+// Vectors of window entries: a row's three windows start a vector each.
+inline int64_t win_vec_cap(int32_t n, int64_t m) { return m < m / 8 + 3 * (int64_t)n ? m : m / 8 + 3 * (int64_t)n; }
+inline int64_t hub_task_cap(int64_t hub_cap, int64_t m) { return hub_cap + m / HUB_SLICE + 1; }
 // Largest dense core (tc_core.cu): one core_n x core_n bit matrix.
 constexpr int CORE_MAX = 8192;
 
@@ -184,13 +202,18 @@ struct CountBuffers {
     int32_t hub_cap;         // min(n, HUB_BM_BITS): slots for ranks n - hub_cap .. n-1
     uint32_t* hub_cnt;       // hub_cap + 1
     int64_t* hub_start;      // hub_cap + 1
-    uint32_t* hub_cur;       // hub_cap + 1
     unsigned long long* hub_cur64;  // hub_cap + 1: next free slot of every hub's segment (planner)
-    int32_t* big_list;       // hub_cap: big hubs, highest rank first
-    int32_t* med_list;       // hub_cap: the other hubs, highest rank first
-    int4* in_rec;            // m: in-edge {u, first suffix entry, end of N+(u), 0} (indices into col)
+    int32_t* big_list;       // hub_cap: big hubs, nearly highest rank first
+    int32_t* long_list;      // hub_cap: the big hubs with a long list below the window
+    int4* win_task;          // hub_task_cap: window tasks, big hubs from the front, the others from the back
+    int4* low_task;          // hub_task_cap: tasks below window 1
+    uint2* in_rec;           // m: in-edge {u, entries of N+(u) after the hub}
     int32_t* rowof;          // m: source row of each entry of the non-core rows
     int64_t m_cap;           // entries of col (and of in_rec, rowof)
+    uint2* winrow;           // n: {first vector in win, entries in window 1} of the rows with a hub
+    uint4* winlow;           // n: their place in the windows below (low_len)
+    uint4* win;              // win_vec_cap: window entries of the non-core rows, eight 16-bit offsets each
+    int64_t win_cap;
     void* tmp;               // scan scratch, scan_tmp_bytes(hub_cap + 1)
     // dense core (tc_core.cu): bit rows of core_words words for core indices 0 .. core_cap-1
     int32_t core_cap;        // min(hub_cap, CORE_MAX)

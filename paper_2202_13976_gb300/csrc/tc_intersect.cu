@@ -10,14 +10,14 @@
 // t[v] += c, t[w] += 1 for every w in W.
 //
 // Buckets (each oriented edge belongs to exactly one):
-//  hub    edges into the highest-ranked vertices ("hubs").  One thread block per hub
-//         v stages N+(v) once in shared memory (a bitmap over its rank window with
-//         per-word prefix counts, or the sorted list), then streams the suffix
-//         N+(u)[j+1 ..] of every in-edge (u, v) against it.  This is the on-chip
+//  hub    edges into the highest-ranked vertices ("hubs").  A thread block or a warp
+//         stages N+(v) once in shared memory (marks in a table or a bitmap over a window
+//         of ranks), then streams the suffix N+(u)[j+1 ..] of every in-edge (u, v)
+//         against it, as 16-bit offsets in the window.  This is the on-chip
 //         analogue of the paper's caching of remote adjacency lists ranked by degree
 //         (Sec. IV-B, Observations 1 and 2): the list that most edges need is read
-//         from memory once and reused by all of them.  t[w] increments are summed
-//         per position of N+(v) in shared memory and flushed once per hub.
+//         from memory once and reused by all of them.  t[w] increments of the highest
+//         ranks are summed in shared memory.
 //  small  other edges whose source has 2 <= |N+(u)| <= 32: a group of 8, 16 or 32
 //         lanes stages N+(u); lane j intersects edge j sequentially, by SSI (Alg. 2)
 //         or binary search (Alg. 1), chosen per edge by Eq. 3.
@@ -415,10 +415,125 @@ __global__ void k_row_of(int32_t n, int32_t hub_cap, const int64_t* __restrict__
     }
 }
 
+// Window entries.  The ranks are read in windows from the top: HUB_WIN ranks in window
+// 1, where most suffix entries lie (R-MAT scale 20 / 23: 98% / 91% of what the hub bucket
+// probes), then two windows of HUB_WIN2, which reach below every hub.  Each non-core
+// row's entries from the lowest hub on are kept once more as 16-bit offsets in their
+// window, eight to a 16-byte vector; a row's windows start a vector each, from the
+// first on, and are padded with the offset that no hub marks.  A block takes 256
+// consecutive rows, reserves their vectors with one atomic and writes them a thread
+// per vector.
+constexpr int WIN_THREADS = 256;
+constexpr int WINS = 3;
+
+struct Windows {
+    int32_t first[WINS + 1];  // first rank of window k
+    explicit Windows(int32_t n) {
+        first[0] = n;
+        first[1] = n < HUB_WIN ? 0 : n - HUB_WIN;
+        for (int k = 2; k <= WINS; ++k) first[k] = first[k - 1] < HUB_WIN2 ? 0 : first[k - 1] - HUB_WIN2;
+    }
+};
+static_assert(HUB_WIN + (WINS - 1) * HUB_WIN2 >= HUB_BM_BITS, "the windows reach below every hub");
+
+__device__ __forceinline__ uint32_t vectors_of(uint32_t entries) { return (entries + 7u) >> 3; }
+
+// A row's place in the windows below the first: {first vector of window 2, entries in
+// window 1, entries in window 2 | in window 3 << 16, 0}.
+__device__ __forceinline__ uint32_t low_len(const uint4& r, int k) { return k == 2 ? r.z & 0xffffu : r.z >> 16; }
+
+__global__ void __launch_bounds__(WIN_THREADS) k_win_build(int32_t n, Windows T, const int2* __restrict__ rowinfo,
+                                                           const int32_t* __restrict__ col,
+                                                           uint2* __restrict__ winrow, uint4* __restrict__ winlow,
+                                                           uint4* __restrict__ win, int64_t win_cap, int32_t src_lo,
+                                                           int32_t src_hi, DevStats* stats) {
+    __shared__ uint32_t pref[WIN_THREADS];
+    __shared__ int32_t cut[WINS + 1][WIN_THREADS];  // the row's end, then where its windows 1, 2, ... start in col
+    __shared__ uint32_t wtot[WIN_THREADS / 32];
+    __shared__ uint32_t base_sh;
+    const int32_t c0 = n - (int32_t)stats->core_n;
+    const int32_t R = n - (int32_t)stats->hub_count;
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    if (stats->hub_count == 0) return;
+    for (int64_t t0 = (int64_t)blockIdx.x * WIN_THREADS; t0 < c0; t0 += (int64_t)gridDim.x * WIN_THREADS) {
+        const int64_t u = t0 + threadIdx.x;
+        uint32_t nv = 0, len[WINS + 1] = {};
+        bool hubrow = false;  // a row without a hub has no in-edge records and needs nothing here
+        if (u < c0) {
+            const int2 ri = rowinfo[u];
+            const int32_t end = ri.x + ri.y;
+            hubrow = ri.y > 0 && col[end - 1] >= R;
+            if (hubrow) {
+                int at = ri.y;
+                cut[0][threadIdx.x] = end;
+#pragma unroll
+                for (int k = 1; k <= WINS; ++k) {
+                    const int hi = at;
+                    if (at > 0 && R < T.first[k - 1] && col[ri.x + at - 1] >= R)
+                        at = lower_bound(col + ri.x, 0, at, max(T.first[k], R));
+                    cut[k][threadIdx.x] = ri.x + at;
+                    len[k] = (uint32_t)(hi - at);
+                    nv += vectors_of(len[k]);
+                }
+                // sources outside the shard, and rows of one entry, have no suffix to read
+                if (u < src_lo || u >= src_hi || ri.y < 2) nv = 0;
+            }
+        }
+        const uint32_t inc = warp_inclusive_scan(nv);
+        if (lane == 31) wtot[w] = inc;
+        __syncthreads();
+        uint32_t before = 0, total = 0;
+#pragma unroll
+        for (int k = 0; k < WIN_THREADS / 32; ++k) {
+            before += k < w ? wtot[k] : 0;
+            total += wtot[k];
+        }
+        if (threadIdx.x == 0) base_sh = total ? atomicAdd(&stats->win_vecs, total) : 0u;
+        pref[threadIdx.x] = before + inc - nv;
+        __syncthreads();
+        const uint32_t base = base_sh;
+        if (hubrow) {
+            const uint32_t v0 = base + before + inc - nv;
+            winrow[u] = make_uint2(v0, len[1]);
+            if (R < T.first[1])
+                winlow[u] = make_uint4(v0 + vectors_of(len[1]), len[1], len[2] | len[3] << 16, 0);
+        }
+        for (uint32_t k = threadIdx.x; k < total; k += WIN_THREADS) {
+            int lo = 0;  // the last row whose vectors start at or before k
+#pragma unroll
+            for (int step = WIN_THREADS / 2; step > 0; step >>= 1)
+                if (pref[lo + step] <= k) lo += step;
+            uint32_t rel = k - pref[lo];
+            int win_no = 1;
+            int32_t p1 = cut[0][lo], p0 = cut[1][lo];
+            while (win_no < WINS && rel >= vectors_of(p1 - p0)) {
+                rel -= vectors_of(p1 - p0);
+                p1 = p0;
+                p0 = cut[++win_no][lo];
+            }
+            const int32_t first = win_no == 1 ? T.first[1] : win_no == 2 ? T.first[2] : T.first[3];
+            const uint32_t scale = win_no == 1 ? 4u : 1u, none = win_no == 1 ? 4u * HUB_WIN : (uint32_t)HUB_WIN2;
+            uint32_t o[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int64_t p = (int64_t)p0 + 8 * (int64_t)rel + j;
+                o[j] = p < p1 ? (uint32_t)(col[p] - first) * scale : none;
+            }
+            if ((int64_t)base + k < win_cap)  // always true: win_vec_cap
+                win[base + k] = make_uint4(o[0] | o[1] << 16, o[2] | o[3] << 16, o[4] | o[5] << 16, o[6] | o[7] << 16);
+            else
+                atomicOr(&stats->err, ERR_OVERFLOW);
+        }
+        __syncthreads();  // the shared arrays are reused by the next rows
+    }
+}
+
 // Every oriented entry (u -> v) of a row outside the dense core with v a hub becomes
-// an in-edge record of v: {u, index after v in N+(u), end of N+(u), 0}, one 16-byte
-// store into v's segment.  Blocks take tiles of SCAT_TILE consecutive entries (16
-// bytes per thread and load), so the work is spread evenly whatever the row lengths;
+// an in-edge record of v: {u, entries of N+(u) after v}, one 8-byte store into v's
+// segment (R-MAT scale 23: 0.83 ms; 16-byte records that also named the suffix's place
+// took 1.26 ms, so the hub kernels gather that place by u).  Blocks take tiles of
+// SCAT_TILE consecutive entries (16 bytes per thread and load), so the work is spread
+// evenly whatever the row lengths;
 // entries in the slots deduplication left free are skipped.  The SCAT_TOP highest
 // hubs, whose cursors every tile would contend for, are served per tile: shared-
 // memory counters give each entry its offset, then one global atomic per hub and
@@ -436,7 +551,7 @@ __global__ void __launch_bounds__(SCAT_THREADS) k_hub_scatter(int32_t n, int32_t
                                                               const int32_t* __restrict__ rowof,
                                                               const int64_t* __restrict__ hub_start,
                                                               unsigned long long* __restrict__ cur,
-                                                              int4* __restrict__ in_rec, int32_t src_lo,
+                                                              uint2* __restrict__ in_rec, int32_t src_lo,
                                                               int32_t src_hi, DevStats* stats) {
     __shared__ uint32_t lcnt[SCAT_TOP];
     __shared__ int64_t gbase[SCAT_TOP];
@@ -451,7 +566,7 @@ __global__ void __launch_bounds__(SCAT_THREADS) k_hub_scatter(int32_t n, int32_t
     for (int64_t t0 = (int64_t)blockIdx.x * SCAT_TILE; t0 < mend; t0 += (int64_t)gridDim.x * SCAT_TILE) {
         for (int h = threadIdx.x; h < top; h += SCAT_THREADS) lcnt[h] = 0;
         __syncthreads();
-        int32_t x[SCAT_ITEMS], u[SCAT_ITEMS], end[SCAT_ITEMS];
+        int32_t x[SCAT_ITEMS], u[SCAT_ITEMS], len[SCAT_ITEMS];
         uint32_t loc[SCAT_ITEMS];
 #pragma unroll
         for (int k = 0; k < SCAT_ITEMS / 4; ++k) {
@@ -470,10 +585,10 @@ __global__ void __launch_bounds__(SCAT_THREADS) k_hub_scatter(int32_t n, int32_t
             if (x[e] >= R) {
                 u[e] = rowof[p];
                 const int2 ri = rowinfo[u[e]];
-                end[e] = ri.x + ri.y;
-                if (p >= end[e]) x[e] = -1;  // a slot freed by deduplication
+                len[e] = (int32_t)((int64_t)ri.x + ri.y - p - 1);
+                if (len[e] < 0) x[e] = -1;  // a slot freed by deduplication
                 // a source outside the counted shard keeps its slot with an empty suffix
-                if (u[e] < src_lo || u[e] >= src_hi) end[e] = (int32_t)(p + 1);
+                if (u[e] < src_lo || u[e] >= src_hi) len[e] = 0;
             }
         }
         // the slot reservations of all items first, so that their round trips overlap,
@@ -490,9 +605,8 @@ __global__ void __launch_bounds__(SCAT_THREADS) k_hub_scatter(int32_t n, int32_t
 #pragma unroll
         for (int e = 0; e < SCAT_ITEMS; ++e) {
             if (x[e] < R || x[e] >= T0) continue;
-            const int64_t p = t0 + ((int64_t)(e >> 2) * SCAT_THREADS + threadIdx.x) * 4 + (e & 3);
             if ((int64_t)gslot[e] < total)  // counts and entries disagree only on a bug: never write outside
-                in_rec[gslot[e]] = make_int4(u[e], (int32_t)(p + 1), end[e], 0);
+                in_rec[gslot[e]] = make_uint2((uint32_t)u[e], (uint32_t)len[e]);
             else
                 atomicOr(&stats->err, ERR_OVERFLOW);
         }
@@ -505,10 +619,9 @@ __global__ void __launch_bounds__(SCAT_THREADS) k_hub_scatter(int32_t n, int32_t
 #pragma unroll
         for (int e = 0; e < SCAT_ITEMS; ++e) {
             if (x[e] < T0) continue;
-            const int64_t p = t0 + ((int64_t)(e >> 2) * SCAT_THREADS + threadIdx.x) * 4 + (e & 3);
             const int64_t slot = gbase[x[e] - T0] + loc[e];
             if (slot < total)
-                in_rec[slot] = make_int4(u[e], (int32_t)(p + 1), end[e], 0);
+                in_rec[slot] = make_uint2((uint32_t)u[e], (uint32_t)len[e]);
             else
                 atomicOr(&stats->err, ERR_OVERFLOW);
         }
@@ -533,7 +646,7 @@ __global__ void k_hub_cur_check(int32_t hub_cap, const int64_t* __restrict__ hub
 __global__ void k_hub_scatter_rows(int32_t n, int32_t hub_cap, const int64_t* __restrict__ rowstart,
                                    const int32_t* __restrict__ rowlen, const int32_t* __restrict__ col,
                                    const int64_t* __restrict__ hub_start, unsigned long long* __restrict__ cur,
-                                   int4* __restrict__ in_rec, int32_t src_lo, int32_t src_hi,
+                                   uint2* __restrict__ in_rec, int32_t src_lo, int32_t src_hi,
                                    DevStats* stats) {
     const int32_t R = n - (int32_t)stats->hub_count;
     const int32_t c0 = n - (int32_t)stats->core_n;  // rows of the dense core are counted there
@@ -573,8 +686,7 @@ __global__ void k_hub_scatter_rows(int32_t n, int32_t hub_cap, const int64_t* __
                 if (x[j] >= R) {
                     const int64_t slot = slot0[j] + __popc(peers[j] & lanemask_lt());
                     if (slot < total)  // counts and entries disagree only on a bug: never write outside
-                        in_rec[slot] = make_int4((int32_t)u, (int32_t)(base + p - j + 1),
-                                                 inshard ? (int32_t)(base + du) : (int32_t)(base + p - j + 1), 0);
+                        in_rec[slot] = make_uint2((uint32_t)u, inshard ? (uint32_t)(du - 1 - (p - j)) : 0u);
                     else
                         atomicOr(&stats->err, ERR_OVERFLOW);
                 }
@@ -584,31 +696,72 @@ __global__ void k_hub_scatter_rows(int32_t n, int32_t hub_cap, const int64_t* __
     }
 }
 
-// Hub slot i (0 = highest rank) is big when its in-degree reaches big_in or its list
-// is too long for one warp.
-__global__ void k_hub_flags(int32_t n, const int32_t* __restrict__ rowlen, const uint32_t* __restrict__ indeg,
-                            int32_t hub_cap, int big_in, uint32_t* __restrict__ big, DevStats* stats) {
-    const int64_t K = stats->hub_count;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < K; i += stride) {
-        const int32_t v = n - 1 - (int32_t)i;
-        const uint32_t din = indeg[v - (n - hub_cap)];
-        big[i] = (din >= (uint32_t)big_in || rowlen[v] > HUB_WARP_MAX) && rowlen[v] > 0 && din > 0 ? 1u : 0u;
-    }
+// Work lists of the hubs (hub 0 = highest rank).  A hub is big when its in-degree
+// reaches big_in or its list is too long for one warp.  Its in-edges are cut into
+// slices: a window task is {v, first in-edge, first entry of N+(v) in window 1,
+// in-edges | entries there << TASK_BITS}; a below-window task {v, first in-edge,
+// in-edges, entries of N+(v) below window 1}.  One atomic per list and warp keeps the
+// lists nearly in rank order (blocks start in order), which is all the work queues need.
+constexpr int TASK_BITS = 12;
+static_assert(HUB_SLICE < 1 << TASK_BITS && (int64_t)HUB_WIN << TASK_BITS < INT_MAX, "window task fields");
+
+// First of `mine` slots reserved for this lane in a list (a warp's lanes in order).
+__device__ __forceinline__ unsigned warp_reserve(unsigned mine, unsigned* counter) {
+    const unsigned inc = warp_inclusive_scan(mine);
+    const unsigned tot = __shfl_sync(FULL, inc, 31);
+    unsigned base = 0;
+    if (lane_id() == 0 && tot) base = atomicAdd(counter, tot);
+    return __shfl_sync(FULL, base, 0) + inc - mine;
 }
 
-// Ordered split of the hubs (highest rank first) into the big and medium lists.
-__global__ void k_hub_lists(int32_t n, const uint32_t* __restrict__ big, const uint32_t* __restrict__ pos,
-                            int32_t* __restrict__ big_list, int32_t* __restrict__ med_list, DevStats* stats) {
+__global__ void k_hub_lists(int32_t n, int32_t hub_cap, int32_t T0w, const int2* __restrict__ rowinfo,
+                            const int32_t* __restrict__ col, const uint2* __restrict__ winrow,
+                            const uint32_t* __restrict__ indeg, const int64_t* __restrict__ hub_start, int big_in,
+                            int32_t* __restrict__ big_list, int32_t* __restrict__ long_list,
+                            int4* __restrict__ win_task, int4* __restrict__ low_task, int64_t task_cap,
+                            DevStats* stats) {
     const int64_t K = stats->hub_count;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < K; i += stride) {
+    const int lane = lane_id();
+    // the loop bound is uniform across a warp, as the appends need all 32 lanes
+    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); b < K; b += stride) {
+        const int64_t i = b + lane;
         const int32_t v = n - 1 - (int32_t)i;
-        if (big[i])
-            big_list[pos[i]] = v;
-        else
-            med_list[i - pos[i]] = v;
-        if (i == K - 1) stats->hub_big = pos[i] + big[i];
+        bool big = false;
+        uint32_t din = 0;
+        int dlow = 0, dwin = 0;
+        int2 ri = make_int2(0, 0);
+        int64_t e0 = 0;
+        if (i < K) {
+            din = indeg[v - (n - hub_cap)];
+            ri = rowinfo[v];
+            if (din > 0 && ri.y > 0) {
+                e0 = hub_start[v - (n - hub_cap)];
+                big = din >= (uint32_t)big_in || ri.y > HUB_WARP_MAX;
+                dwin = v >= T0w ? ri.y : (col[ri.x + ri.y - 1] >= T0w ? (int)winrow[v].y : 0);
+                dlow = ri.y - dwin;
+            }
+        }
+        const bool lng = big && dlow > HUB_WARP_MAX;
+        const unsigned pb = warp_append(big, &stats->hub_big);
+        const unsigned pl = warp_append(lng, &stats->hub_long);
+        if (big) big_list[pb] = v;
+        if (lng) long_list[pl] = v;
+        const unsigned ns = (din + HUB_SLICE - 1) / HUB_SLICE;
+        const unsigned tb = warp_reserve(big && dwin > 0 ? ns : 0u, &stats->hub_tasks);
+        const unsigned tm = warp_reserve(!big && dwin > 0 ? ns : 0u, &stats->hub_med);
+        const unsigned tl = warp_reserve(dlow > 0 ? ns : 0u, &stats->hub_low);
+        for (unsigned k = 0; k < ns && dlow + dwin > 0; ++k) {
+            const int64_t slot = big ? (int64_t)tb + k : task_cap - 1 - (int64_t)tm - k;
+            const uint32_t ne = min(din - k * HUB_SLICE, (uint32_t)HUB_SLICE);
+            const int first = (int)(e0 + (int64_t)k * HUB_SLICE);
+            if ((dwin > 0 && (slot < 0 || slot >= task_cap)) || (dlow > 0 && (int64_t)tl + k >= task_cap)) {
+                atomicOr(&stats->err, ERR_OVERFLOW);  // never: hub_task_cap
+                break;
+            }
+            if (dwin > 0) win_task[slot] = make_int4(v, first, ri.x + dlow, (int)(ne | (uint32_t)dwin << TASK_BITS));
+            if (dlow > 0) low_task[tl + k] = make_int4(v, first, (int)ne, dlow);
+        }
     }
 }
 
@@ -1170,11 +1323,19 @@ __global__ void __launch_bounds__(CTA_THREADS) k_tc_cta(int32_t n, const int64_t
 }
 
 // ---- hub bucket ----------------------------------------------------------------
-// Big hubs (in-degree >= the planner's threshold, or lists too long for one warp) are processed
-// by a whole block over a bitmap of N+(v); the remaining hubs by one warp each over
-// a hash set of N+(v) in shared memory.  One persistent kernel drains the big-hub
-// queue first, then every warp takes medium hubs independently.
-
+// Every hub's in-edges stream their suffixes against the hub's staged list N+(v).  The
+// windows of ranks (k_win_build) are counted apart: a suffix's entries in a window come
+// eight to a load as offsets into what is staged of N+(v) there, so a probe is one
+// shared-memory load.
+//   k_tc_hub      window 1, big hubs (in-degree >= the planner's threshold, or lists too
+//                 long for one warp): a block per slice of the in-edges
+//   k_tc_hub_med  window 1, the other hubs: a warp per hub
+//   k_tc_hub_win2 the windows below: a warp per slice
+//   k_tc_hub_low  the same for per-edge support, over a hash set of 32-bit ids
+//   k_tc_hub_list per-edge support of big hubs with a long list below window 1; in probe
+//                 mode all big hubs
+// For R-MAT scale 20 / 23 they take 1.03 / 4.7 ms together; 32-bit ids against one bitmap
+// or hash set per hub took 1.28 / 5.94 ms.
 
 struct BitmapProbe {
     const uint32_t* bm;
@@ -1196,23 +1357,30 @@ struct ListProbe {
     }
 };
 
-// One batch of up to 32 in-edges [k0, min(k0 + 32, e1)) of hub v, processed by one
-// warp.  Suffixes of 32 or more entries are read one in-edge at a time by all lanes
-// (the read stops above max N+(v)); shorter ones are laid end to end and read 32
-// entries at a time.  Matches add to cnt[p] (or t[x] when cnt is null) and to the
+// One batch of up to 32 in-edges [k0, min(k0 + 32, e1)) of hub v, processed by one warp
+// over 32-bit ids (k_tc_hub_list): the whole suffixes (WHOLE), or their entries below
+// window 1.  Suffixes of HUB_LONG or more entries are read by lane groups (the read
+// stops above max N+(v)); shorter ones are laid end to end and read 32 entries at a
+// time.  Matches add to cnt[p] (or t[x] when cnt is null) and to the
 // per-in-edge total, which goes to t[u].  Returns the batch total (all lanes).
-template <bool SUP, class Probe>
-__device__ uint32_t hub_batch(int64_t k0, int64_t e1, const int4* __restrict__ in_rec,
+template <bool SUP, bool WHOLE, class Probe>
+__device__ uint32_t hub_batch(int64_t k0, int64_t e1, const uint2* __restrict__ in_rec,
+                              const int2* __restrict__ rowinfo, const uint2* __restrict__ winrow,
                               const int32_t* __restrict__ col, int32_t maxv, const Probe& probe, uint32_t* cnt,
                               unsigned long long* __restrict__ t, uint32_t* cw, uint32_t* __restrict__ sup_arg,
                               int64_t vbase) {
     uint32_t* const sup = SUP ? sup_arg : nullptr;
     const int lane = lane_id();
     const int64_t k = k0 + lane;
-    const int4 rec = k < e1 ? in_rec[k] : make_int4(0, 0, 0, 0);
-    int32_t uu = rec.x;
-    int32_t b0 = rec.y;
-    int a = rec.z - rec.y;
+    const uint2 rec = k < e1 ? in_rec[k] : make_uint2(0, 0);
+    int32_t uu = (int32_t)rec.x;
+    int32_t b0 = 0;
+    int a = (int)rec.y;
+    if (a > 0) {
+        const int2 ri = rowinfo[uu];
+        b0 = ri.x + ri.y - a;
+        if (!WHOLE) a -= (int)winrow[uu].y;
+    }
     uint32_t total_c = 0;
     const bool islong = a >= HUB_LONG;
     const int nlong = __popc(__ballot_sync(FULL, islong));
@@ -1330,123 +1498,755 @@ __device__ uint32_t hub_batch(int64_t k0, int64_t e1, const int4* __restrict__ i
     return total_c + __reduce_add_sync(FULL, lane < cz ? cu : 0u);
 }
 
-struct HubShared {
-    union {
-        struct {  // big hub, one block
-            union {
-                struct {
-                    uint32_t bm[HUB_BM_WORDS];
-                    uint16_t pre[HUB_BM_WORDS];
-                } b;
-                int32_t list[HUB_CNT_MAX];
-            } s;
-            uint32_t cnt[HUB_CNT_MAX];
-            uint32_t slice[HUB_BM_WORDS / 32];
-        } big;
-        struct {  // medium hubs, one per warp
-            int32_t keys[HUB_WARPS][HUB_HASH_MAX];
-            uint32_t cnt[HUB_WARPS][HUB_HASH_MAX];
-        } med;
-    } u;
-    uint32_t cw[HUB_WARPS][32];
-    unsigned long long vt[HUB_WARPS];
-    int q;
-    unsigned bq;  // next batch of the current big hub
+constexpr int WINK_THREADS = 512;  // three resident blocks per SM: 64 KB of counters each
+constexpr int WINK_WARPS = WINK_THREADS / 32;
+constexpr int WINK_BLOCKS = 3;
+constexpr uint32_t WIN_MARK = 0x80000000u;
+
+// 1 << d for d in [0, 32), 0 for any other d (PTX clamps the shift amount).
+__device__ __forceinline__ unsigned bit_or_none(int d) {
+    unsigned r;
+    asm("shl.b32 %0, 1, %1;" : "=r"(r) : "r"(d));
+    return r;
+}
+
+// Inclusive warp scan whose adds are predicated by the shuffles themselves.
+__device__ __forceinline__ uint32_t warp_scan_u32(uint32_t x) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+        asm("{ .reg .pred p; .reg .u32 y; shfl.sync.up.b32 y|p, %0, %1, 0, 0xffffffff; @p add.u32 %0, %0, y; }"
+            : "+r"(x)
+            : "r"(o));
+    return x;
+}
+
+__device__ __forceinline__ int shared_s32(uint32_t addr) {
+    int v;
+    asm volatile("ld.shared.s32 %0, [%1];" : "=r"(v) : "r"(addr));
+    return v;
+}
+
+// Probes of a lane's eight window offsets: s[j] < 0 iff offset j is an entry of the
+// staged N+(v), whose counter has then been raised; returns how many are.
+struct WinCounters {  // a block's counters, the entries of N+(v) marked in bit 31
+    uint32_t addr;
+    __device__ __forceinline__ uint32_t operator()(const uint32_t (&o)[8], int (&s)[8]) const {
+        uint32_t c = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s[j] = shared_s32(addr + o[j]);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            asm volatile("{ .reg .pred p; setp.lt.s32 p, %1, 0; @p red.shared.add.u32 [%0], 1; }" ::"r"(addr + o[j]),
+                         "r"(s[j])
+                         : "memory");
+            c += (uint32_t)s[j] >> 31;
+        }
+        return c;
+    }
 };
 
+// A block's marks, one bit per warp and rank; matches count in the block's counters of
+// the MED_TOP highest ranks, else directly in t.
+constexpr int MED_TOP = 4096;
+struct WinMarks {
+    uint32_t marks, cnt, first;  // shared addresses; offset of the first rank with a counter
+    int shift;                   // 31 - the warp's bit
+    unsigned long long* t;       // of the window's first rank
+    __device__ __forceinline__ uint32_t operator()(const uint32_t (&o)[8], int (&s)[8]) const {
+        uint32_t c = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            uint32_t m;
+            asm volatile("ld.shared.u16 %0, [%1];" : "=r"(m) : "r"(marks + (o[j] >> 1)));
+            s[j] = (int)(m << shift);
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (s[j] < 0) {
+                if (o[j] >= first)
+                    asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(cnt + (o[j] - first)) : "memory");
+                else
+                    atomicAdd(&t[o[j] >> 2], 1ull);
+                ++c;
+            }
+        return c;
+    }
+};
+
+// The same as a bitmap of one warp with the entries before each word, for counters per
+// entry of N+(v) (per-edge support); the entry's bit is shifted into bit 31 of s[j].
+struct WinBitmap {
+    uint32_t bm, pre, cnt;
+    __device__ __forceinline__ uint32_t operator()(const uint32_t (&o)[8], int (&s)[8]) const {
+        uint32_t c = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            s[j] = (int)__funnelshift_l(0u, (uint32_t)shared_s32(bm + ((o[j] >> 5) & ~3u)), ~(o[j] >> 2));
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (s[j] < 0) {
+                uint32_t before;  // entries before the word, then those below the bit
+                asm volatile("ld.shared.u8 %0, [%1];" : "=r"(before) : "r"(pre + (o[j] >> 7)));
+                const uint32_t pos = before + __popc(s[j]) - 1;
+                asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(cnt + 4 * pos) : "memory");
+                ++c;
+            }
+        return c;
+    }
+};
+
+// One warp's in-edges (up to 32) with something to read, in order: lane i takes the
+// i-th of them.  Their items are laid end to end; at[i] = {base of in-edge i's items
+// less the items before it, their end}.
+struct EdgeItems {
+    int cz, total, excl;  // in-edges; items; first item of this lane's in-edge (-1: none)
+    int seen;             // in-edges that start before the round, less one
+    unsigned upto;        // this lane's bit and those below it
+
+    // items: this lane's in-edge's count; returns the lane whose in-edge this lane takes
+    __device__ __forceinline__ int gather(int items, uint32_t* cw) {
+        const int lane = lane_id();
+        const unsigned nz = __ballot_sync(FULL, items > 0);
+        cz = __popc(nz);
+        if (cz == 0) return 0;
+        if (items > 0) cw[__popc(nz & lanemask_lt())] = (uint32_t)lane;
+        __syncwarp();
+        return lane < cz ? (int)cw[lane] : lane;
+    }
+    // items and base of the in-edge this lane has taken
+    __device__ __forceinline__ void lay(int items, int base, int2* at) {
+        const int lane = lane_id();
+        if (lane >= cz) items = 0;
+        const int incl = (int)warp_scan_u32((uint32_t)items);
+        total = __shfl_sync(FULL, incl, 31);
+        excl = lane < cz ? incl - items : -1;
+        at[lane] = make_int2(base - (incl - items), incl);
+        seen = -1;
+        upto = lane == 31 ? FULL : (2u << lane) - 1u;
+        __syncwarp();
+    }
+    // the in-edge of item r + lane; called for r = 0, 32, 64, ... in turn
+    __device__ __forceinline__ int edge_of(int r) {
+        const unsigned mk = __reduce_or_sync(FULL, bit_or_none(excl - r));
+        const int i = seen + __popc(mk & upto);
+        seen += __popc(mk);
+        return i;
+    }
+};
+
+// One batch of up to 32 in-edges (each lane's record; {0, 0}: none) of the hub whose
+// entries of the window `probe` holds (LOW: window 2 or 3, else window 1).  An item is a vector: a round takes 32 of them, one per lane, each
+// lane probing its eight entries.  The scan over the per-lane matches of two rounds (16
+// bits each) gives, at the last vector of every in-edge, the matches up to it, so an
+// in-edge's count is the difference of two of them.  Returns the batch total (all lanes).
+//
+// What bounds it: shared-memory wavefronts (79% of the peak in k_tc_hub on R-MAT scale
+// 20), the random counter loads (2.9 wavefronts each) and the matches' atomics.  32-bit
+// ids against a bitmap with prefix counts took 1.9 warp instructions per entry, this 0.9.
+// Two rounds per scan: 0.73 instead of 0.75-0.80 ms.  Unconditional atomics, or atomics
+// to a spare slot for the entries that do not match, took 0.83 and 0.77 ms.
+template <bool SUP, bool LOW, class Probe>
+__device__ __forceinline__ uint32_t win_batch(const uint2 rec, int win_no, bool hub_in_window,
+                                              const int2* __restrict__ rowinfo, const uint2* __restrict__ winrow,
+                                              const uint4* __restrict__ winlow,
+                                              const uint4* __restrict__ win, const Probe& probe,
+                                              unsigned long long* __restrict__ t, int2* at, uint32_t* cw,
+                                              uint32_t* __restrict__ sup) {
+    const int lane = lane_id();
+    // the row's entries in the window (len of them, from vector first on), and how many
+    // of them the suffix has
+    uint32_t first = 0, len = 0, suffix = 0;
+    if (rec.y) {
+        if (!LOW) {
+            const uint2 r = winrow[rec.x];
+            first = r.x, len = r.y, suffix = rec.y;
+        } else {
+            const uint4 r = winlow[rec.x];
+            suffix = rec.y - r.y;
+            first = r.x, len = low_len(r, 2);
+            if (win_no == 3) {
+                suffix = suffix > len ? suffix - len : 0u;
+                first += vectors_of(len);
+                len = low_len(r, 3);
+            }
+            if (!suffix) len = 0;
+        }
+    }
+    // a hub in the window: its suffixes begin inside a vector, whose entries before are
+    // not above the hub and meet no mark of it; else the row's whole part of the window
+    const uint32_t off = hub_in_window && suffix ? len - suffix : 0u;
+    const int nv0 = suffix ? (int)vectors_of(len) - (int)(off >> 3) : 0;
+    EdgeItems E;
+    const int src = E.gather(nv0, cw);
+    if (E.cz == 0) return 0;
+    const uint32_t uu = __shfl_sync(FULL, rec.x, src);
+    int32_t b0 = 0, cbase = 0;  // support: col index after v, and of the first vector's first entry
+    if (SUP) {
+        int32_t end = 0;
+        if (rec.y) {
+            const int2 ri = rowinfo[rec.x];
+            end = ri.x + ri.y;
+        }
+        b0 = __shfl_sync(FULL, end - (int32_t)rec.y, src);
+        cbase = __shfl_sync(FULL, end - (int32_t)(len - (off & ~7u)), src);
+    }
+    E.lay(__shfl_sync(FULL, nv0, src), (int)__shfl_sync(FULL, first + (off >> 3), src), at);
+    constexpr uint32_t NONE2 = (LOW ? (uint32_t)HUB_WIN2 : 4u * HUB_WIN) * 0x10001u;
+    uint32_t running = 0;
+    for (int r = 0; r < E.total; r += 64) {
+        const int item = r + lane;
+        int idx[2];
+        int2 e[2];
+        uint4 q[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            idx[h] = 0;
+            e[h] = make_int2(0, 0);
+            q[h] = make_uint4(NONE2, NONE2, NONE2, NONE2);
+            if (h == 0 || r + 32 < E.total) {
+                idx[h] = E.edge_of(r + 32 * h);
+                e[h] = at[idx[h]];
+                if (item + 32 * h < E.total) q[h] = win[(uint32_t)(e[h].x + item + 32 * h)];
+            }
+        }
+        uint32_t c = 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (h == 1 && r + 32 >= E.total) break;
+            const uint32_t o[8] = {q[h].x & 0xffffu, q[h].x >> 16, q[h].y & 0xffffu, q[h].y >> 16,
+                                   q[h].z & 0xffffu, q[h].z >> 16, q[h].w & 0xffffu, q[h].w >> 16};
+            int s[8];
+            const uint32_t ch = probe(o, s);
+            c |= ch << (16 * h);
+            if (SUP) {
+                const int32_t cb = __shfl_sync(FULL, cbase, idx[h]), ex = __shfl_sync(FULL, E.excl, idx[h]);
+                if (ch) {
+                    const int64_t p0 = (int64_t)cb + 8 * (int64_t)(item + 32 * h - ex);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (s[j] < 0) atomicAdd(&sup[p0 + j], 1u);  // edge (u, x)
+                }
+            }
+        }
+        const uint32_t pc = warp_scan_u32(c);
+        const uint32_t tot = __shfl_sync(FULL, pc, 31);
+        if (e[0].y == item + 1) cw[idx[0]] = running + (pc & 0xffffu);  // an in-edge's last vector
+        running += tot & 0xffffu;
+        if (e[1].y == item + 33) cw[idx[1]] = running + (pc >> 16);
+        running += tot >> 16;
+    }
+    __syncwarp();
+    if (lane < E.cz) {
+        const uint32_t c = cw[lane] - (lane ? cw[lane - 1] : 0u);
+        if (c) {
+            if (SUP)
+                atomicAdd(&sup[b0 - 1], c);  // edge (u, v)
+            else
+                atomicAdd(&t[uu], (unsigned long long)c);
+        }
+    }
+    __syncwarp();
+    return running;
+}
+
+// In-edges a warp claims at a time: smaller batches when a slice has fewer than two
+// full ones per warp, so that every warp gets some.
+__device__ __forceinline__ int hub_batch_size(int64_t din, int warps) {
+    return din >= 2 * warps * HUB_BATCH ? HUB_BATCH : max(8, (int)((din + 2 * warps - 1) / (2 * warps)));
+}
+
+struct HubShared {
+    uint32_t cnt[HUB_WIN + 1];  // one counter per window rank and one that no hub marks
+    int2 at[WINK_WARPS][32];
+    uint32_t cw[WINK_WARPS][32];
+    uint32_t vt[WINK_WARPS];
+    unsigned q;
+    unsigned bq;  // next batch of the current task
+};
+
+// Window tasks of the big hubs, one per block: N+(v)'s window entries mark their
+// counters, the slice's suffixes are streamed against the marks, and the marks are
+// taken away again, so a task costs O(|N+(v)|) beside its suffixes.  The counters keep
+// counting t over the block's tasks and are flushed once (with per-edge support, which
+// counts the entries of each N+(v) apart, after every task).  Thread 0 claims the next
+// task while the current one is counted.
 template <bool SUP>
-__global__ void __launch_bounds__(HUB_THREADS) k_tc_hub(int32_t n, int32_t hub_cap, const int64_t* __restrict__ rowstart,
-                                                        const int32_t* __restrict__ rowlen,
-                                                        const int32_t* __restrict__ col,
-                                                        const int64_t* __restrict__ hub_start,
-                                                        const int32_t* __restrict__ big_list,
-                                                        const int32_t* __restrict__ med_list,
-                                                        const int4* __restrict__ in_rec,
-                                                        unsigned long long* __restrict__ t, DevStats* stats,
-                                                        int probe_mode, uint32_t* __restrict__ sup_arg) {
-    uint32_t* const sup = SUP ? sup_arg : nullptr;
+__global__ void __launch_bounds__(WINK_THREADS, WINK_BLOCKS) k_tc_hub(
+    int32_t T0w, const int2* __restrict__ rowinfo, const uint2* __restrict__ winrow, const int32_t* __restrict__ col,
+    const uint4* __restrict__ win, const int4* __restrict__ win_task, const uint2* __restrict__ in_rec,
+    unsigned long long* __restrict__ t, DevStats* stats, uint32_t* __restrict__ sup) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     HubShared& sh = *reinterpret_cast<HubShared*>(smem_raw);
     const int lane = lane_id(), w = threadIdx.x >> 5;
-    const unsigned nbig = stats->hub_big, nmed = stats->hub_count - stats->hub_big;
-    // phase 1: big hubs, one block each
+    const unsigned ntask = stats->hub_tasks;
+    unsigned next = blockIdx.x;
+    if (next >= ntask) return;
+    const WinCounters P{(uint32_t)__cvta_generic_to_shared(sh.cnt)};
+    for (int i = threadIdx.x; i < HUB_WIN + 1; i += WINK_THREADS) sh.cnt[i] = 0;
     for (;;) {
         if (threadIdx.x == 0) {
-            sh.q = (int)atomicAdd(&stats->hub_next, 1u);
+            sh.q = next;
+            sh.bq = 0;
+        }
+        __syncthreads();
+        const unsigned q = sh.q;
+        if (q >= ntask) break;
+        if (threadIdx.x == 0) next = gridDim.x + atomicAdd(&stats->hub_next, 1u);
+        const int4 task = win_task[q];
+        const int32_t v = task.x;
+        const int ne = task.w & ((1 << TASK_BITS) - 1), p1 = task.z + (int)((uint32_t)task.w >> TASK_BITS);
+        const int e1 = task.y + ne;
+        for (int p = task.z + (int)threadIdx.x; p < p1; p += WINK_THREADS) sh.cnt[col[p] - T0w] |= WIN_MARK;
+        __syncthreads();
+        uint32_t vtot = 0;
+        const int bs = hub_batch_size(ne, WINK_WARPS);
+        for (;;) {
+            unsigned k = 0;
+            if (lane == 0) k = atomicAdd(&sh.bq, 1u);
+            k = __shfl_sync(FULL, k, 0) * (unsigned)bs;
+            if (k >= (unsigned)ne) break;
+            const int e = task.y + (int)k + lane;
+            const uint2 rec = lane < bs && e < e1 ? in_rec[e] : make_uint2(0, 0);
+            vtot += win_batch<SUP, false>(rec, 1, v >= T0w, rowinfo, winrow, nullptr, win, P, t, sh.at[w], sh.cw[w], sup);
+        }
+        if (lane == 0) sh.vt[w] = vtot;
+        __syncthreads();
+        for (int p = task.z + (int)threadIdx.x; p < p1; p += WINK_THREADS) {
+            const int x = col[p] - T0w;
+            const uint32_t c = sh.cnt[x] & ~WIN_MARK;
+            sh.cnt[x] = SUP ? 0u : c;
+            if (SUP && c) atomicAdd(&sup[p], c);  // edge (v, x)
+        }
+        if (!SUP && threadIdx.x == 0) {
+            unsigned long long s = 0;
+            for (int k = 0; k < WINK_WARPS; ++k) s += sh.vt[k];
+            if (s) atomicAdd(&t[v], s);
+        }
+    }
+    if (!SUP)
+        for (int i = threadIdx.x; i < HUB_WIN; i += WINK_THREADS)
+            if (sh.cnt[i]) atomicAdd(&t[T0w + i], (unsigned long long)sh.cnt[i]);
+}
+
+template <bool SUP>
+struct MedShared {
+    uint32_t marks[(HUB_WIN + 1) / 2];  // two ranks per word
+    uint32_t cnt[MED_TOP];
+    int2 at[WINK_WARPS][32];
+    uint32_t cw[WINK_WARPS][32];
+};
+template <>
+struct MedShared<true> {
+    struct {
+        uint32_t bm[(HUB_WIN + 1) / 32];
+        uint32_t pre[(HUB_WIN + 1) / 128];  // one byte per word of bm
+        uint32_t cnt[HUB_WARP_MAX];
+    } win[WINK_WARPS];
+    int2 at[WINK_WARPS][32];
+    uint32_t cw[WINK_WARPS][32];
+};
+static_assert(WINK_WARPS == 16, "one mark bit per warp");
+static_assert(HUB_WARP_MAX <= 256, "one-byte prefix counts");
+
+// Window tasks of the other hubs, one per warp (taken from the back of the task list).
+// Each warp owns one bit of the block's marks, so sixteen hubs share one table and a
+// hub costs O(|N+(v)|) beside its suffixes.
+template <bool SUP>
+__global__ void __launch_bounds__(WINK_THREADS, WINK_BLOCKS) k_tc_hub_med(
+    int32_t T0w, int32_t W, const int2* __restrict__ rowinfo, const uint2* __restrict__ winrow,
+    const int32_t* __restrict__ col, const uint4* __restrict__ win, const int4* __restrict__ win_task, int64_t task_cap,
+    const uint2* __restrict__ in_rec, unsigned long long* __restrict__ t, DevStats* stats, uint32_t* __restrict__ sup) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    MedShared<SUP>& sh = *reinterpret_cast<MedShared<SUP>*>(smem_raw);
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    const unsigned nmed = stats->hub_med;
+    if (blockIdx.x * WINK_WARPS >= nmed) return;
+    const int top0 = W > MED_TOP ? W - MED_TOP : 0;  // window index of the first rank with a counter
+    if constexpr (!SUP) {
+        for (int i = threadIdx.x; i < (HUB_WIN + 1) / 2; i += WINK_THREADS) sh.marks[i] = 0;
+        for (int i = threadIdx.x; i < MED_TOP; i += WINK_THREADS) sh.cnt[i] = 0;
+        __syncthreads();
+    }
+    unsigned q = blockIdx.x * WINK_WARPS + w;
+    while (q < nmed) {
+        unsigned nx = 0;
+        if (lane == 0) nx = gridDim.x * WINK_WARPS + atomicAdd(&stats->hub_next2, 1u);
+        const int4 task = win_task[task_cap - 1 - q];
+        const int32_t v = task.x;
+        const int ne = task.w & ((1 << TASK_BITS) - 1), dwin = (int)((uint32_t)task.w >> TASK_BITS);
+        const int e1 = task.y + ne;
+        uint32_t vtot = 0;
+        if constexpr (!SUP) {
+            const WinMarks P{(uint32_t)__cvta_generic_to_shared(sh.marks), (uint32_t)__cvta_generic_to_shared(sh.cnt),
+                             4u * (uint32_t)top0, 31 - w, t + T0w};
+            for (int p = lane; p < dwin; p += 32) {
+                const int x = col[task.z + p] - T0w;
+                atomicOr(&sh.marks[x >> 1], 1u << (w + 16 * (x & 1)));
+            }
+            __syncwarp();
+            uint2 rec = task.y + lane < e1 ? in_rec[task.y + lane] : make_uint2(0, 0);
+            for (int bb = task.y; bb < e1; bb += 32) {
+                const uint2 cur = rec;  // the next batch's records are loaded ahead
+                rec = bb + 32 + lane < e1 ? in_rec[bb + 32 + lane] : make_uint2(0, 0);
+                vtot += win_batch<SUP, false>(cur, 1, v >= T0w, rowinfo, winrow, nullptr, win, P, t, sh.at[w], sh.cw[w], sup);
+            }
+            for (int p = lane; p < dwin; p += 32) {
+                const int x = col[task.z + p] - T0w;
+                atomicAnd(&sh.marks[x >> 1], ~(1u << (w + 16 * (x & 1))));
+            }
+            __syncwarp();
+            if (lane == 0 && vtot) atomicAdd(&t[v], (unsigned long long)vtot);
+        } else {
+            auto& M = sh.win[w];
+            constexpr int WORDS = (HUB_WIN + 1) / 32, PER = WORDS / 32;
+            static_assert(PER == 16, "four bytes a word, four words a lane");
+            if (dwin > HUB_WARP_MAX) {  // the lists never make such a hub medium: do not overrun the counters
+                if (lane == 0) atomicOr(&stats->err, ERR_OVERFLOW);
+                q = __shfl_sync(FULL, nx, 0);
+                continue;
+            }
+            for (int i = lane; i < WORDS; i += 32) M.bm[i] = 0;
+            for (int i = lane; i < dwin; i += 32) M.cnt[i] = 0;
+            __syncwarp();
+            for (int p = lane; p < dwin; p += 32) {
+                const int x = col[task.z + p] - T0w;
+                atomicOr(&M.bm[x >> 5], 1u << (x & 31));
+            }
+            __syncwarp();
+            // lane l counts the entries before words 16 l .. 16 l + 15
+            uint32_t pc[PER], sum = 0;
+#pragma unroll
+            for (int i = 0; i < PER; ++i) {
+                pc[i] = sum;
+                sum += __popc(M.bm[lane * PER + i]);
+            }
+            const uint32_t before = warp_scan_u32(sum) - sum;
+#pragma unroll
+            for (int i = 0; i < PER; i += 4)
+                M.pre[lane * (PER / 4) + i / 4] = ((before + pc[i]) & 0xffu) | ((before + pc[i + 1]) & 0xffu) << 8 |
+                                                  ((before + pc[i + 2]) & 0xffu) << 16 |
+                                                  ((before + pc[i + 3]) & 0xffu) << 24;
+            __syncwarp();
+            const WinBitmap P{(uint32_t)__cvta_generic_to_shared(M.bm), (uint32_t)__cvta_generic_to_shared(M.pre),
+                              (uint32_t)__cvta_generic_to_shared(M.cnt)};
+            for (int bb = task.y; bb < e1; bb += 32) {
+                const uint2 rec = bb + lane < e1 ? in_rec[bb + lane] : make_uint2(0, 0);
+                win_batch<SUP, false>(rec, 1, v >= T0w, rowinfo, winrow, nullptr, win, P, t, sh.at[w], sh.cw[w], sup);
+            }
+            for (int p = lane; p < dwin; p += 32) {
+                const uint32_t c = M.cnt[p];
+                if (c) atomicAdd(&sup[task.z + p], c);  // edge (v, x)
+            }
+            __syncwarp();
+        }
+        q = __shfl_sync(FULL, nx, 0);
+    }
+    if constexpr (!SUP) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < W - top0; i += WINK_THREADS)
+            if (sh.cnt[i]) atomicAdd(&t[T0w + top0 + i], (unsigned long long)sh.cnt[i]);
+    }
+}
+
+// A warp's bitmap of N+(v)'s entries in a window of HUB_WIN2 ranks; matches count
+// directly in t (below window 1 no rank is hot).
+struct WinBits {
+    uint32_t bm;
+    unsigned long long* t;  // of the window's first rank
+    __device__ __forceinline__ uint32_t operator()(const uint32_t (&o)[8], int (&s)[8]) const {
+        uint32_t c = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            s[j] = (int)__funnelshift_l(0u, (uint32_t)shared_s32(bm + ((o[j] >> 3) & ~3u)), ~o[j]);
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (s[j] < 0) {
+                atomicAdd(&t[o[j]], 1ull);
+                ++c;
+            }
+        return c;
+    }
+};
+
+// Below-window tasks: for each window k >= 2 that N+(v) reaches, a warp marks N+(v)'s
+// entries there in a bitmap, streams the in-edges' entries of the window against it and
+// clears the marks.  8 KB of shared memory a warp leave 24 warps per SM; four windows of
+// half the size and 48 warps took longer (R-MAT scale 23: 1.38 instead of 1.18 ms), since
+// hubs then read their in-edges once more per window.
+constexpr int WIN2_THREADS = 256;
+constexpr int WIN2_WARPS = WIN2_THREADS / 32;
+constexpr int WIN2_BLOCKS = 3;
+static_assert(HUB_WIN2 == 0xffff, "the last offset of an 8 KB bitmap is no rank's");
+
+struct Win2Shared {
+    uint32_t bm[WIN2_WARPS][(HUB_WIN2 + 1) / 32];
+    int2 at[WIN2_WARPS][32];
+    uint32_t cw[WIN2_WARPS][32];
+};
+
+__global__ void __launch_bounds__(WIN2_THREADS) k_tc_hub_win2(
+    Windows T, const int2* __restrict__ rowinfo, const uint4* __restrict__ winlow, const int32_t* __restrict__ col,
+    const uint4* __restrict__ win, const int4* __restrict__ low_task, bool probe_mode, int big_in,
+    const uint32_t* __restrict__ indeg, int32_t hub0, const uint2* __restrict__ in_rec,
+    unsigned long long* __restrict__ t, DevStats* stats) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    Win2Shared& sh = *reinterpret_cast<Win2Shared*>(smem_raw);
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    const unsigned nlow = stats->hub_low;
+    if (blockIdx.x * WIN2_WARPS >= nlow) return;
+    uint32_t* const bm = sh.bm[w];
+    const uint32_t bm_addr = (uint32_t)__cvta_generic_to_shared(bm);
+    for (int i = lane; i < (HUB_WIN2 + 1) / 32; i += 32) bm[i] = 0;
+    __syncwarp();
+    unsigned q = blockIdx.x * WIN2_WARPS + w;
+    while (q < nlow) {
+        unsigned nx = 0;
+        if (lane == 0) nx = gridDim.x * WIN2_WARPS + atomicAdd(&stats->hub_next4, 1u);
+        const int4 task = low_task[q];
+        q = __shfl_sync(FULL, nx, 0);
+        const int32_t v = task.x;
+        const int e1 = task.y + task.z;
+        const int2 rv = rowinfo[v];
+        // in probe mode the list kernel counts the big hubs
+        if (probe_mode && (indeg[v - hub0] >= (uint32_t)big_in || rv.y > HUB_WARP_MAX)) continue;
+        uint32_t vtot = 0;
+        int p1 = rv.x + task.w;  // end of N+(v)'s entries not yet taken
+        for (int win_no = 2; win_no <= WINS && p1 > rv.x; ++win_no) {
+            const int32_t first = win_no == 2 ? T.first[2] : T.first[3];
+            int p0 = rv.x;
+            if (v < first) p0 += lower_bound(col + rv.x, 0, p1 - rv.x, first);
+            if (p0 == p1) continue;
+            for (int p = p0 + lane; p < p1; p += 32) {
+                const int x = col[p] - first;
+                atomicOr(&bm[x >> 5], 1u << (x & 31));
+            }
+            __syncwarp();
+            const WinBits P{bm_addr, t + first};
+            uint2 rec = task.y + lane < e1 ? in_rec[task.y + lane] : make_uint2(0, 0);
+            for (int bb = task.y; bb < e1; bb += 32) {
+                const uint2 cur = rec;  // the next batch's records are loaded ahead
+                rec = bb + 32 + lane < e1 ? in_rec[bb + 32 + lane] : make_uint2(0, 0);
+                vtot += win_batch<false, true>(cur, win_no, v >= first, rowinfo, nullptr, winlow, win, P, t, sh.at[w],
+                                               sh.cw[w], nullptr);
+            }
+            for (int p = p0 + lane; p < p1; p += 32) bm[(col[p] - first) >> 5] = 0;
+            __syncwarp();
+            p1 = p0;
+        }
+        if (lane == 0 && vtot) atomicAdd(&t[v], (unsigned long long)vtot);
+    }
+}
+
+// Below-window tasks of the per-edge support, which needs a counter per entry of N+(v):
+// a warp puts the part of N+(v) below window 1 into a hash set and streams the
+// in-edges' 32-bit entries below it end to end, 32 per round, one per lane (two rounds
+// share one scan, as in win_batch).
+constexpr int LOW_THREADS = 256;
+constexpr int LOW_WARPS = LOW_THREADS / 32;
+constexpr int LOW_BLOCKS = 5;
+
+struct LowShared {
+    int32_t keys[LOW_WARPS][HUB_HASH_MAX];
+    uint32_t cnt[LOW_WARPS][HUB_HASH_MAX];
+    int2 at[LOW_WARPS][32];
+    uint32_t cw[LOW_WARPS][32];
+};
+
+__global__ void __launch_bounds__(LOW_THREADS) k_tc_hub_low(
+    const int2* __restrict__ rowinfo, const uint2* __restrict__ winrow, const int32_t* __restrict__ col,
+    const int4* __restrict__ low_task, const uint2* __restrict__ in_rec, DevStats* stats, uint32_t* __restrict__ sup) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    LowShared& sh = *reinterpret_cast<LowShared*>(smem_raw);
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    int32_t* const K = sh.keys[w];
+    uint32_t* const cnt = sh.cnt[w];
+    int2* const at = sh.at[w];
+    uint32_t* const cw = sh.cw[w];
+    const unsigned nlow = stats->hub_low;
+    if (blockIdx.x * LOW_WARPS >= nlow) return;
+    for (int p = lane; p < HUB_HASH_MAX; p += 32) {  // every slot is empty again after each task
+        K[p] = -1;
+        cnt[p] = 0;
+    }
+    __syncwarp();
+    unsigned q = blockIdx.x * LOW_WARPS + w;
+    while (q < nlow) {
+        unsigned nx = 0;
+        if (lane == 0) nx = gridDim.x * LOW_WARPS + atomicAdd(&stats->hub_next4, 1u);
+        nx = __shfl_sync(FULL, nx, 0);
+        const int4 task = low_task[q];
+        q = nx;
+        const int64_t e0 = task.y, e1 = e0 + task.z;
+        const int dlow = task.w;
+        if (dlow > HUB_WARP_MAX) continue;  // the list kernel's
+        const int2 rv = rowinfo[task.x];
+        int lg = 5;
+        while ((1 << lg) < HUB_HASH_LOAD * dlow) ++lg;
+        const unsigned shift = 32u - (unsigned)lg, mask = (1u << lg) - 1u;
+        bool staged = false;  // the set is built when the first entry to probe turns up
+        for (int64_t bb = e0; bb < e1; bb += 32) {
+            const uint2 rec = bb + lane < e1 ? in_rec[bb + lane] : make_uint2(0, 0);
+            int a = (int)rec.y;
+            int32_t b0 = 0;
+            if (a > 0) {
+                a -= (int)winrow[rec.x].y;
+                if (a > 0) {
+                    const int2 ru = rowinfo[rec.x];
+                    b0 = ru.x + ru.y - (int)rec.y;
+                }
+            }
+            EdgeItems E;
+            const int src = E.gather(a, cw);
+            if (E.cz == 0) continue;
+            if (!staged) {
+                for (int p = lane; p < dlow; p += 32) {
+                    const int32_t x = col[rv.x + p];
+                    unsigned h = ((unsigned)x * 0x9e3779b1u) >> shift;
+                    while (atomicCAS(&K[h], -1, x) != -1) h = (h + 1) & mask;  // keys are distinct
+                }
+                staged = true;
+            }
+            b0 = __shfl_sync(FULL, b0, src);
+            E.lay(__shfl_sync(FULL, a, src), b0, at);
+            const HashProbe H{K, shift, mask};
+            uint32_t running = 0;
+            for (int r = 0; r < E.total; r += 64) {
+                const int item = r + lane;
+                int idx[2];
+                int2 e[2];
+                int32_t x[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    idx[h] = 0;
+                    e[h] = make_int2(0, 0);
+                    x[h] = -2;
+                    if (h == 0 || r + 32 < E.total) {
+                        idx[h] = E.edge_of(r + 32 * h);
+                        e[h] = at[idx[h]];
+                        if (item + 32 * h < E.total) x[h] = col[e[h].x + item + 32 * h];
+                    }
+                }
+                uint32_t c = 0;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int slot = x[h] >= 0 ? H(x[h]) : -1;
+                    if (slot >= 0) {
+                        atomicAdd(&cnt[slot], 1u);
+                        atomicAdd(&sup[e[h].x + item + 32 * h], 1u);  // edge (u, x)
+                        c += 1u << (16 * h);
+                    }
+                }
+                const uint32_t pc = warp_scan_u32(c);
+                const uint32_t tot = __shfl_sync(FULL, pc, 31);
+                if (e[0].y == item + 1) cw[idx[0]] = running + (pc & 0xffffu);
+                running += tot & 0xffffu;
+                if (e[1].y == item + 33) cw[idx[1]] = running + (pc >> 16);
+                running += tot >> 16;
+            }
+            __syncwarp();
+            if (lane < E.cz) {
+                const uint32_t c = cw[lane] - (lane ? cw[lane - 1] : 0u);
+                if (c) atomicAdd(&sup[b0 - 1], c);  // edge (u, v)
+            }
+            __syncwarp();
+        }
+        if (staged) {
+            for (int p = lane; p <= (int)mask; p += 32) {
+                const int32_t x = K[p];
+                if (x >= 0) {
+                    const uint32_t c = cnt[p];
+                    if (c) atomicAdd(&sup[rv.x + lower_bound(col + rv.x, 0, dlow, x)], c);  // edge (v, x)
+                    K[p] = -1;
+                    cnt[p] = 0;
+                }
+            }
+            __syncwarp();
+        }
+    }
+}
+
+struct HubListShared {
+    union {
+        struct {
+            uint32_t bm[HUB_BM_WORDS];
+            uint16_t pre[HUB_BM_WORDS];
+        } b;
+        int32_t list[HUB_CNT_MAX];
+    } s;
+    uint32_t cnt[HUB_CNT_MAX];
+    uint32_t slice[HUB_BM_WORDS / 32];
+    uint32_t cw[HUB_WARPS][32];
+    unsigned long long vt[HUB_WARPS];
+    int q;
+    unsigned bq;  // next batch of the current hub
+};
+
+// One block per hub: big hubs whose list below the window is too long for one warp (the
+// suffixes' entries below the window against that part of N+(v), staged as a bitmap
+// with prefix counts); in probe mode every big hub, the whole suffixes against the
+// sorted list N+(v).
+template <bool SUP>
+__global__ void __launch_bounds__(HUB_THREADS) k_tc_hub_list(
+    int32_t n, int32_t hub_cap, const int2* __restrict__ rowinfo, const uint2* __restrict__ winrow,
+    const int32_t* __restrict__ col, const int64_t* __restrict__ hub_start, const int32_t* __restrict__ list,
+    const uint2* __restrict__ in_rec, unsigned long long* __restrict__ t, DevStats* stats, int probe_mode,
+    uint32_t* __restrict__ sup_arg) {
+    uint32_t* const sup = SUP ? sup_arg : nullptr;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    HubListShared& sh = *reinterpret_cast<HubListShared*>(smem_raw);
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    const unsigned nlist = probe_mode ? stats->hub_big : stats->hub_long;
+    for (;;) {
+        if (threadIdx.x == 0) {
+            sh.q = (int)atomicAdd(&stats->hub_next3, 1u);
             sh.bq = 0;
         }
         __syncthreads();
         const int q = sh.q;
-        if ((unsigned)q >= nbig) break;
-        const int32_t v = big_list[q];
+        if ((unsigned)q >= nlist) break;
+        const int32_t v = list[q];
         const int hi = v - (n - hub_cap);
         const int64_t e0 = hub_start[hi], e1 = hub_start[hi + 1];
-        const int dv = rowlen[v];
-        const int64_t base = rowstart[v];
-        const int32_t maxv = col[base + dv - 1];  // big hubs have dv >= 1
+        const int2 ri = rowinfo[v];
+        const int64_t base = ri.x;
+        // a list below the window: rows with a hub have their window entries counted
+        const int dv = probe_mode ? ri.y : ri.y - (int)winrow[v].y;
+        const int32_t maxv = col[base + dv - 1];
         const bool staged = dv <= HUB_CNT_MAX;
         const int W = (maxv - v + 31) >> 5;  // maxv - v < hub_cap <= HUB_BM_BITS
         if (staged)
-            for (int p = threadIdx.x; p < dv; p += HUB_THREADS) sh.u.big.cnt[p] = 0;
+            for (int p = threadIdx.x; p < dv; p += HUB_THREADS) sh.cnt[p] = 0;
         if (!probe_mode) {
-            build_bitmap<HUB_THREADS>(sh.u.big.s.b.bm, sh.u.big.s.b.pre, sh.u.big.slice, col + base, dv, v, W);
+            build_bitmap<HUB_THREADS>(sh.s.b.bm, sh.s.b.pre, sh.slice, col + base, dv, v, W);
         } else {
             if (staged)
-                for (int p = threadIdx.x; p < dv; p += HUB_THREADS) sh.u.big.s.list[p] = col[base + p];
+                for (int p = threadIdx.x; p < dv; p += HUB_THREADS) sh.s.list[p] = col[base + p];
             __syncthreads();
         }
-        uint32_t* cnt = staged ? sh.u.big.cnt : nullptr;
+        uint32_t* cnt = staged ? sh.cnt : nullptr;
         unsigned long long vtot = 0;
-        // batches of bs in-edges, claimed by the warps from a shared counter (the block
-        // waits for its slowest warp); small hubs use smaller batches so that every
-        // warp gets some
-        const int64_t din = e1 - e0;
-        const int bs = din >= 2 * HUB_WARPS * HUB_BATCH ? HUB_BATCH
-                                                        : max(8, (int)((din + 2 * HUB_WARPS - 1) / (2 * HUB_WARPS)));
-        if (!probe_mode) {
-            const BitmapProbe P{sh.u.big.s.b.bm, sh.u.big.s.b.pre, v};
-            for (;;) {
-                unsigned k = 0;
-                if (lane == 0) k = atomicAdd(&sh.bq, 1u);
-                const int64_t bb = e0 + (int64_t)__shfl_sync(FULL, k, 0) * bs;
-                if (bb >= e1) break;
-                vtot += hub_batch<SUP>(bb, min(bb + bs, e1), in_rec, col, maxv, P, cnt, t, sh.cw[w], sup, base);
-            }
-        } else {
-            const ListProbe P{staged ? sh.u.big.s.list : col + base, dv};
-            for (;;) {
-                unsigned k = 0;
-                if (lane == 0) k = atomicAdd(&sh.bq, 1u);
-                const int64_t bb = e0 + (int64_t)__shfl_sync(FULL, k, 0) * bs;
-                if (bb >= e1) break;
-                vtot += hub_batch<SUP>(bb, min(bb + bs, e1), in_rec, col, maxv, P, cnt, t, sh.cw[w], sup, base);
-            }
+        const int bs = hub_batch_size(e1 - e0, HUB_WARPS);
+        const BitmapProbe PB{sh.s.b.bm, sh.s.b.pre, v};
+        const ListProbe PL{staged ? sh.s.list : col + base, dv};
+        for (;;) {
+            unsigned k = 0;
+            if (lane == 0) k = atomicAdd(&sh.bq, 1u);
+            const int64_t bb = e0 + (int64_t)__shfl_sync(FULL, k, 0) * bs;
+            if (bb >= e1) break;
+            const int64_t be = min(bb + bs, e1);
+            if (!probe_mode)
+                vtot += hub_batch<SUP, false>(bb, be, in_rec, rowinfo, winrow, col, maxv, PB, cnt, t, sh.cw[w], sup, base);
+            else
+                vtot += hub_batch<SUP, true>(bb, be, in_rec, rowinfo, winrow, col, maxv, PL, cnt, t, sh.cw[w], sup, base);
         }
         if (lane == 0) sh.vt[w] = vtot;
         __syncthreads();
         if (staged) {
-            if (!probe_mode) {
-                for (int i = threadIdx.x; i < W; i += HUB_THREADS) {
-                    const uint32_t word = sh.u.big.s.b.bm[i];
-                    uint32_t rest = word;
-                    while (rest) {
-                        const int bpos = __ffs(rest) - 1;
-                        rest &= rest - 1;
-                        const int p = sh.u.big.s.b.pre[i] + __popc(word & ((1u << bpos) - 1u));
-                        const uint32_t c = sh.u.big.cnt[p];
-                        if (c) {
-                            atomicAdd(&t[v + 1 + i * 32 + bpos], (unsigned long long)c);
-                            if (sup) atomicAdd(&sup[base + p], c);  // edge (v, x)
-                        }
-                    }
-                }
-            } else {
-                for (int p = threadIdx.x; p < dv; p += HUB_THREADS) {
-                    const uint32_t c = sh.u.big.cnt[p];
-                    if (c) {
-                        atomicAdd(&t[sh.u.big.s.list[p]], (unsigned long long)c);
-                        if (sup) atomicAdd(&sup[base + p], c);  // edge (v, x)
-                    }
+            for (int p = threadIdx.x; p < dv; p += HUB_THREADS) {
+                const uint32_t c = sh.cnt[p];
+                if (c) {
+                    atomicAdd(&t[col[base + p]], (unsigned long long)c);
+                    if (sup) atomicAdd(&sup[base + p], c);  // edge (v, x)
                 }
             }
         }
@@ -1456,60 +2256,6 @@ __global__ void __launch_bounds__(HUB_THREADS) k_tc_hub(int32_t n, int32_t hub_c
             if (s) atomicAdd(&t[v], s);
         }
         __syncthreads();
-    }
-    // phase 2: medium hubs, one warp each (no block barriers from here on), probed
-    // through a hash set of N+(v); every slot is empty again after each hub
-    int32_t* K = sh.u.med.keys[w];
-    uint32_t* cnt = sh.u.med.cnt[w];
-    for (int p = lane; p < HUB_HASH_MAX; p += 32) {
-        K[p] = -1;
-        cnt[p] = 0;
-    }
-    __syncwarp();
-    for (;;) {
-        unsigned q = 0;
-        if (lane == 0) q = atomicAdd(&stats->hub_next2, 1u);
-        q = __shfl_sync(FULL, q, 0);
-        if (q >= nmed) break;
-        const int32_t v = med_list[q];
-        const int hi = v - (n - hub_cap);
-        const int64_t e0 = hub_start[hi], e1 = hub_start[hi + 1];
-        const int dv = rowlen[v];
-        if (dv == 0 || e1 == e0) continue;
-        if (dv > HUB_WARP_MAX) {  // the flags never make such a hub medium: do not overrun the table
-            if (lane == 0) atomicOr(&stats->err, ERR_OVERFLOW);
-            continue;
-        }
-        const int64_t base = rowstart[v];
-        int lg = 5;
-        while ((1 << lg) < HUB_HASH_LOAD * dv) ++lg;
-        const unsigned shift = 32u - (unsigned)lg, mask = (1u << lg) - 1u;
-        for (int p = lane; p < dv; p += 32) {
-            const int32_t x = col[base + p];
-            unsigned h = ((unsigned)x * 0x9e3779b1u) >> shift;
-            while (atomicCAS(&K[h], -1, x) != -1) h = (h + 1) & mask;  // keys are distinct
-        }
-        const int32_t maxv = col[base + dv - 1];
-        __syncwarp();
-        const HashProbe P{K, shift, mask};
-        unsigned long long vtot = 0;
-        for (int64_t bb = e0; bb < e1; bb += 32)
-            vtot += hub_batch<SUP>(bb, e1, in_rec, col, maxv, P, cnt, t, sh.cw[w], sup, base);
-        __syncwarp();
-        for (int p = lane; p <= (int)mask; p += 32) {
-            const int32_t x = K[p];
-            if (x >= 0) {
-                const uint32_t c = cnt[p];
-                if (c) {
-                    atomicAdd(&t[x], (unsigned long long)c);
-                    if (sup) atomicAdd(&sup[base + lower_bound(col + base, 0, dv, x)], c);  // edge (v, x)
-                }
-                K[p] = -1;
-                cnt[p] = 0;
-            }
-        }
-        if (lane == 0 && vtot) atomicAdd(&t[v], vtot);
-        __syncwarp();
     }
 }
 
@@ -1600,6 +2346,10 @@ bool launch_plan(const CountBuffers& C, const Strategy& S, const Launch& L, cons
     }
     if (hubs) {
         if (core_max > 0) launch_core_plan(C, H);
+        const Windows T(C.n);
+        k_win_build<<<grid_for(C.n, WIN_THREADS, H.sms), WIN_THREADS, 0, H.stream>>>(
+            C.n, T, C.rowinfo, C.col, C.winrow, C.winlow, C.win, C.win_cap, C.src_lo, C.src_hi, C.stats);
+        count_launch();
         k_hub_indeg<<<grid_for(C.hub_cap, THREADS, H.sms), THREADS, 0, H.stream>>>(C.n, C.hub_cap, C.deg, C.rowlen,
                                                                                   C.core_cnt, C.hub_cnt, C.stats);
         count_launch();
@@ -1621,14 +2371,10 @@ bool launch_plan(const CountBuffers& C, const Strategy& S, const Launch& L, cons
         k_hub_cur_check<<<grid_for(C.hub_cap, THREADS, H.sms), THREADS, 0, H.stream>>>(C.hub_cap, C.hub_start,
                                                                                       C.hub_cur64, C.stats);
         count_launch();
-        // hub_cur is free again: it holds the big flags, hub_cnt (still the in-degrees
-        // until here) is overwritten by their exclusive scan
-        k_hub_flags<<<grid_for(C.hub_cap, THREADS, H.sms), THREADS, 0, H.stream>>>(
-            C.n, C.rowlen, C.hub_cnt, C.hub_cap, S.hub_big_in > 0 ? S.hub_big_in : 1, C.hub_cur, C.stats);
-        count_launch();
-        scan_u32_to_u32(C.hub_cur, C.hub_cnt, C.hub_cap, C.tmp, H);
-        k_hub_lists<<<grid_for(C.hub_cap, THREADS, H.sms), THREADS, 0, H.stream>>>(C.n, C.hub_cur, C.hub_cnt,
-                                                                                  C.big_list, C.med_list, C.stats);
+        k_hub_lists<<<grid_for(C.hub_cap, THREADS, H.sms), THREADS, 0, H.stream>>>(
+            C.n, C.hub_cap, T.first[1], C.rowinfo, C.col, C.winrow, C.hub_cnt, C.hub_start,
+            S.hub_big_in > 0 ? S.hub_big_in : 1, C.big_list, C.long_list, C.win_task, C.low_task,
+            hub_task_cap(C.hub_cap, C.m_cap), C.stats);
         count_launch();
     }
     if (forked) cudaEventRecord(ps->join, H.stream);
@@ -1647,9 +2393,19 @@ cudaError_t intersect_init_attributes() {
         (e = cudaFuncSetAttribute(k_tc_cta<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CtaShared))) ||
         (e = cudaFuncSetAttribute(k_tc_small_wide<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, wide)) ||
         (e = cudaFuncSetAttribute(k_tc_small_wide<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, wide)) ||
-        (e = cudaFuncSetAttribute(k_tc_hub<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(HubShared))))
+        (e = cudaFuncSetAttribute(k_tc_hub<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(HubShared))) ||
+        (e = cudaFuncSetAttribute(k_tc_hub<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(HubShared))) ||
+        (e = cudaFuncSetAttribute(k_tc_hub_med<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)sizeof(MedShared<false>))) ||
+        (e = cudaFuncSetAttribute(k_tc_hub_med<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)sizeof(MedShared<true>))) ||
+        (e = cudaFuncSetAttribute(k_tc_hub_win2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Win2Shared))) ||
+        (e = cudaFuncSetAttribute(k_tc_hub_low, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LowShared))) ||
+        (e = cudaFuncSetAttribute(k_tc_hub_list<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)sizeof(HubListShared))))
         return e;
-    return cudaFuncSetAttribute(k_tc_hub<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(HubShared));
+    return cudaFuncSetAttribute(k_tc_hub_list<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)sizeof(HubListShared));
 }
 
 template <bool SUP>
@@ -1700,11 +2456,34 @@ void intersect_impl(const CountBuffers& C, const Strategy& S, cudaEvent_t* ev, c
     if (ev) cudaEventRecord(ev[PH_HUB], L.stream);
     if (C.hub_cap > 0) {
         if (S.hub_core > 0) launch_core_count(C, L);
-        cudaMemsetAsync(&C.stats->hub_next, 0, 2 * sizeof(unsigned), L.stream);
-        k_tc_hub<SUP><<<L.sms * HUB_BLOCKS, HUB_THREADS, sizeof(HubShared), L.stream>>>(
-            C.n, C.hub_cap, C.rowstart, C.rowlen, C.col, C.hub_start, C.big_list, C.med_list, C.in_rec, C.t_rank,
-            C.stats, S.strat[TC_BUCKET_HUB] == TC_STRAT_PROBE ? 1 : 0, C.sup);
+        cudaMemsetAsync(&C.stats->hub_next, 0, 4 * sizeof(unsigned), L.stream);
+        const bool probe = S.strat[TC_BUCKET_HUB] == TC_STRAT_PROBE;
+        const Windows T(C.n);
+        const int64_t task_cap = hub_task_cap(C.hub_cap, C.m_cap);
+        if (!probe) {
+            k_tc_hub<SUP><<<L.sms * WINK_BLOCKS, WINK_THREADS, sizeof(HubShared), L.stream>>>(
+                T.first[1], C.rowinfo, C.winrow, C.col, C.win, C.win_task, C.in_rec, C.t_rank, C.stats, C.sup);
+            count_launch();
+        }
+        k_tc_hub_med<SUP><<<L.sms * WINK_BLOCKS, WINK_THREADS, sizeof(MedShared<SUP>), L.stream>>>(
+            T.first[1], C.n - T.first[1], C.rowinfo, C.winrow, C.col, C.win, C.win_task, task_cap, C.in_rec, C.t_rank, C.stats, C.sup);
         count_launch();
+        if (T.first[1] > 0) {  // something lies below window 1
+            if (SUP)
+                k_tc_hub_low<<<L.sms * LOW_BLOCKS, LOW_THREADS, sizeof(LowShared), L.stream>>>(
+                    C.rowinfo, C.winrow, C.col, C.low_task, C.in_rec, C.stats, C.sup);
+            else
+                k_tc_hub_win2<<<L.sms * WIN2_BLOCKS, WIN2_THREADS, sizeof(Win2Shared), L.stream>>>(
+                    T, C.rowinfo, C.winlow, C.col, C.win, C.low_task, probe, S.hub_big_in > 0 ? S.hub_big_in : 1,
+                    C.hub_cnt, C.n - C.hub_cap, C.in_rec, C.t_rank, C.stats);
+            count_launch();
+        }
+        if (probe || (SUP && T.first[1] > 0)) {
+            k_tc_hub_list<SUP><<<L.sms * HUB_BLOCKS, HUB_THREADS, sizeof(HubListShared), L.stream>>>(
+                C.n, C.hub_cap, C.rowinfo, C.winrow, C.col, C.hub_start, probe ? C.big_list : C.long_list, C.in_rec,
+                C.t_rank, C.stats, probe ? 1 : 0, C.sup);
+            count_launch();
+        }
     }
     if (ev) cudaEventRecord(ev[PH_END], L.stream);
 }
