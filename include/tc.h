@@ -159,8 +159,8 @@ tc_status tc_count_vertex_formula(tc_graph* g, uint64_t* t_out, int mem_kind, ui
  * v_out[k] in the caller's ids, support_out[k] (uint32), each edge once, in an order
  * of the library's choosing (row by row in its internal rank order); all three
  * arrays in mem_kind memory.  Runs the oriented count once more with every triangle
- * also added to its three edges (the dense core off, since it counts words of bits
- * without naming triangles); the graph's tuning is restored afterwards.
+ * added to its three edges (the dense core counts its edges' triangles by words of
+ * bits); the graph's tuning is restored afterwards.
  * Synchronises the stream.  Errors: TC_EINVAL (NULL output, bad mem_kind),
  * TC_ENOMEM, TC_ECUDA, TC_EINTERNAL.
  */

@@ -891,14 +891,14 @@ tc_status tc_edge_support(tc_graph* g, int32_t* u_out, int32_t* v_out, uint32_t*
     if (st != TC_OK) return st;
     if (h.err & ERR_BAD_ID) return TC_EINVAL;
     const size_t nn = (size_t)g->n, me = (size_t)h.m_simple;
-    // the oriented count with every triangle also added to its three edges; the dense
-    // core counts words of bits and names no triangle, so it is switched off here
+    // the oriented count with every triangle added to its three edges instead of its
+    // vertices (the dense core counts its edges' triangles by words of bits); the plan is
+    // the count's own
     const Strategy saved = g->strat;
     Strategy S = saved;
     S.strat[TC_BUCKET_SMALL] = TC_STRAT_HASH;
     S.strat[TC_BUCKET_CTA] = TC_STRAT_BITMAP;
     S.strat[TC_BUCKET_HUB] = TC_STRAT_BITMAP;
-    S.hub_core = 0;
     std::vector<void*> tmp;
     uint32_t* sup = nullptr;
     int32_t* id_of = nullptr;
@@ -913,26 +913,18 @@ tc_status tc_edge_support(tc_graph* g, int32_t* u_out, int32_t* v_out, uint32_t*
         free_list(g, &tmp);
         return st;
     }
-    const bool replan = saved.hub_core != 0;
     g->strat = S;
-    if (replan) g->planned = false;
     g->counted = false;
     cudaError_t e = cudaMemsetAsync(sup, 0, sizeof(uint32_t) * (size_t)g->m_alloc, g->stream);
     if (e == cudaSuccess && (st = run_plan(g)) == TC_OK) {
-        e = cudaMemsetAsync(g->t_rank, 0, sizeof(unsigned long long) * nn, g->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(&g->stats->sum_t, 0, sizeof(unsigned long long), g->stream);
-        if (e == cudaSuccess) {
-            CountBuffers C = count_buffers(g);
-            C.sup = sup;
-            launch_intersect(C, g->strat, nullptr, g->L);
-            launch_sum_t(C, g->L);
-            launch_support_out(g->n, g->rank, g->rowlen, g->rowinfo, g->col, sup, id_of, estart, stmp,
-                               dev ? u_out : du, dev ? v_out : dv, dev ? support_out : ds, g->L);
-            e = cudaGetLastError();
-        }
+        CountBuffers C = count_buffers(g);
+        C.sup = sup;
+        launch_intersect(C, g->strat, nullptr, g->L);  // leaves parts of t in t_rank: the next count starts it anew
+        launch_support_out(g->n, g->rank, g->rowlen, g->rowinfo, g->col, sup, id_of, estart, stmp, dev ? u_out : du,
+                           dev ? v_out : dv, dev ? support_out : ds, g->L);
+        e = cudaGetLastError();
     }
     g->strat = saved;
-    if (replan) g->planned = false;  // the next count plans with the dense core again
     g->counted = false;
     if (st != TC_OK) {
         free_list(g, &tmp);

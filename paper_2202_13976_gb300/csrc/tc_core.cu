@@ -138,6 +138,43 @@ __global__ void __launch_bounds__(CORE_THREADS) k_core_count(int32_t n, const in
     }
 }
 
+// Per-edge support of the core's own triangles: the core edge (x -> y) lies in
+// |Z[x] AND Z[y]| of them, a third core vertex on either side of x or y, so each edge is
+// counted whole where it is met and no triangle has to be named.  Laid out as the
+// count above, with the whole row Z[x] in registers.
+__global__ void __launch_bounds__(CORE_THREADS) k_core_support(int32_t n, const int64_t* __restrict__ rowstart,
+                                                               const int32_t* __restrict__ rowlen,
+                                                               const int32_t* __restrict__ col, int words,
+                                                               const uint32_t* __restrict__ z,
+                                                               const int32_t* __restrict__ lo,
+                                                               const int32_t* __restrict__ hi,
+                                                               uint32_t* __restrict__ sup, const DevStats* stats) {
+    const int core_n = (int)stats->core_n;
+    const int32_t c0 = n - core_n;
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    const int first = lane * CORE_LANE_WORDS;
+    for (int64_t i = blockIdx.x; i < core_n; i += gridDim.x) {
+        const int d = rowlen[c0 + i];
+        const int64_t base = rowstart[c0 + i];
+        uint32_t zx[CORE_LANE_WORDS];
+#pragma unroll
+        for (int h = 0; h < CORE_LANE_WORDS; h += 4) {
+            uint4 a = make_uint4(0, 0, 0, 0);
+            if (first + h < words) a = *reinterpret_cast<const uint4*>(z + i * words + first + h);
+            zx[h] = a.x, zx[h + 1] = a.y, zx[h + 2] = a.z, zx[h + 3] = a.w;
+        }
+        const int xlo = lo[i], xhi = hi[i];
+        for (int p = w; p < d; p += CORE_WARPS) {
+            const int j = col[base + p] - c0;
+            const int b0 = max(xlo, lo[j]), b1 = min(xhi, hi[j]);
+            uint32_t s = 0;
+            if (b0 <= b1 && first < words) s = and_popc(z + (int64_t)j * words, zx, first, b0 >> 5, b1 >> 5);
+            s = __reduce_add_sync(FULL, s);
+            if (lane == 0 && s) atomicAdd(&sup[base + p], s);
+        }
+    }
+}
+
 }  // namespace
 
 int core_words_for(int32_t core_cap) {
@@ -160,6 +197,12 @@ void launch_core_plan(const CountBuffers& C, const Launch& L) {
 
 void launch_core_count(const CountBuffers& C, const Launch& L) {
     if (C.core_cap <= 0) return;
+    if (C.sup) {
+        k_core_support<<<C.core_cap, CORE_THREADS, 0, L.stream>>>(C.n, C.rowstart, C.rowlen, C.col, C.core_words,
+                                                                 C.core_z, C.core_lo, C.core_hi, C.sup, C.stats);
+        count_launch();
+        return;
+    }
     k_core_count<<<C.core_cap, CORE_THREADS, 0, L.stream>>>(C.n, C.rowstart, C.rowlen, C.col, C.core_words, C.core_z,
                                                            C.core_lo, C.core_hi, C.core_hiout, C.t_rank, C.src_lo,
                                                            C.src_hi, C.stats);
