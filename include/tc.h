@@ -523,10 +523,9 @@ tc_status tc_request_run(const tc_request* r, void* cuda_stream, tc_result* out)
  * code that forbids allocation after start-up.
  *
  * Computes the same T, t[] and LCC[] as tc_graph_create_from_edges + tc_count +
- * lcc_compute for a small graph, in one kernel launch whose intermediate arrays
- * live in a fixed device array of TC_NOALLOC_SCRATCH_BYTES bytes inside the
- * library.  Every GPU that loads the library holds that array until the process
- * exits.  The call itself allocates nothing and calls no allocating routine.
+ * lcc_compute for a small graph, in kernels whose intermediate arrays live in a
+ * fixed device array of TC_NOALLOC_SCRATCH_BYTES bytes inside the library.  Every
+ * GPU that loads the library holds that array until the process exits.  The call itself allocates nothing and calls no allocating routine.
  *   n, m        0 <= n <= TC_NOALLOC_MAX_N, 0 <= m <= TC_NOALLOC_MAX_M
  *   src, dst    m int32 ids each, DEVICE memory (may be NULL when m == 0)
  *   T_out       host scalar, receives T
@@ -540,7 +539,7 @@ tc_status tc_request_run(const tc_request* r, void* cuda_stream, tc_result* out)
  * also when the runtime loads this library's device code and places the array on
  * the device, so make it at start-up, before the free memory is handed to another
  * allocator.  All calls share the array and it keeps the previous call's contents
- * (the kernel clears what it needs): calls whose work overlaps on the GPU (other
+ * (each call clears what it needs): calls whose work overlaps on the GPU (other
  * streams or host threads) race on it and must be ordered by the caller.
  * Errors: TC_EINVAL for sizes beyond the limits, NULL pointers or an id outside
  * [0, n); TC_ECUDA; TC_EINTERNAL.
