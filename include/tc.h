@@ -438,7 +438,8 @@ tc_status tc_batch_run(int32_t G, const int32_t* n, const int64_t* edge_off, con
                        const int32_t* dst, uint64_t* T_out, uint64_t* t_out, double* lcc_out,
                        const tc_tuning* tuning, void* cuda_stream, int flags);
 
-/* Frees the CUDA graphs and arrays kept by tc_batch_run. */
+/* Frees the CUDA graphs and arrays kept by tc_batch_run, and the streams and events
+   kept from destroyed graphs for the next ones. */
 void tc_release_cached_graphs(void);
 
 /*

@@ -44,6 +44,75 @@ struct DeviceState {
 std::mutex g_dev_mutex;
 DeviceState g_dev[64];
 
+// What a graph needs of the driver beside memory: the second stream and its events, the
+// events of the build and count phases, and the copy stream and events of host input.
+// Sets are handed from a destroyed graph to the next one of the device: creating them
+// took 20 us per graph, and 500 us with eight threads doing so at once.  A stream still
+// holding a former owner's work only orders the next owner's after it; events are
+// recorded anew.  At most SYNC_KEEP sets stay, until tc_release_cached_graphs.
+struct SyncSet {
+    cudaStream_t side = nullptr, copy = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr, landed = nullptr, allocated = nullptr;
+    cudaEvent_t ev[PH_EVENTS] = {};
+    cudaEvent_t bev[BP_EVENTS] = {};
+
+    cudaError_t create() {
+        cudaError_t e = cudaSuccess;
+        for (cudaStream_t* s : {&side, &copy})
+            if (e == cudaSuccess) e = cudaStreamCreateWithFlags(s, cudaStreamNonBlocking);
+        for (cudaEvent_t* x : {&fork, &join, &landed, &allocated})
+            if (e == cudaSuccess) e = cudaEventCreateWithFlags(x, cudaEventDisableTiming);
+        for (cudaEvent_t& x : ev)
+            if (e == cudaSuccess) e = cudaEventCreate(&x);
+        for (cudaEvent_t& x : bev)
+            if (e == cudaSuccess) e = cudaEventCreate(&x);
+        return e;
+    }
+    void destroy() {
+        for (cudaEvent_t x : {fork, join, landed, allocated})
+            if (x) cudaEventDestroy(x);
+        for (cudaEvent_t x : ev)
+            if (x) cudaEventDestroy(x);
+        for (cudaEvent_t x : bev)
+            if (x) cudaEventDestroy(x);
+        for (cudaStream_t x : {side, copy})
+            if (x) cudaStreamDestroy(x);
+        *this = SyncSet{};
+    }
+};
+constexpr size_t SYNC_KEEP = 64;
+std::mutex g_sync_mutex;
+std::vector<SyncSet> g_sync[64];  // per device
+
+cudaError_t take_sync(int dev, SyncSet* out) {
+    {
+        std::lock_guard<std::mutex> lock(g_sync_mutex);
+        if (!g_sync[dev].empty()) {
+            *out = g_sync[dev].back();
+            g_sync[dev].pop_back();
+            return cudaSuccess;
+        }
+    }
+    const cudaError_t e = out->create();
+    if (e != cudaSuccess) out->destroy();
+    return e;
+}
+
+void give_sync(int dev, SyncSet* s) {
+    {
+        std::lock_guard<std::mutex> lock(g_sync_mutex);
+        if (g_sync[dev].size() < SYNC_KEEP) {
+            try {
+                g_sync[dev].push_back(*s);
+                *s = SyncSet{};
+                return;
+            } catch (const std::bad_alloc&) {
+            }
+        }
+    }
+    s->destroy();
+}
+
 tc_status init_device(int dev, DeviceState** out) {
     if (dev < 0 || dev >= 64) return TC_ECUDA;
     std::lock_guard<std::mutex> lock(g_dev_mutex);
@@ -130,19 +199,18 @@ struct tc_graph {
     bool planned = false;
     bool counted = false;
     Strategy strat{};
-    cudaEvent_t ev[PH_EVENTS] = {};
     bool timed = false;
-    cudaEvent_t bev[BP_EVENTS] = {};  // build phases (not while recording a CUDA graph)
     bool build_timed = false;
     // batch of graphs counted as one disjoint union (tc_batch_create)
     int32_t batch_G = -1;
     int32_t* batch_vbase = nullptr;   // device, G + 1
     int* batch_err = nullptr;         // device flag of the relabel and the per-graph reduction
     bool capture = false;             // work is being recorded into a CUDA graph: no events
-    // the planner's second stream (single graphs only): hub lists and dense core
-    cudaStream_t side = nullptr;
-    cudaEvent_t plan_fork = nullptr, plan_join = nullptr;
-    bool plan_forked = false;         // the last plan ran its hub part on `side`
+    // streams and events (not while recording a CUDA graph); the second stream runs the
+    // long rows' sort and the plan's hub part (single graphs only)
+    SyncSet sync;
+    bool has_sync = false;
+    bool plan_forked = false;         // the last plan ran its hub part on the second stream
 };
 
 namespace {
@@ -176,6 +244,34 @@ tc_status dalloc(tc_graph* g, T** p, size_t count, std::vector<void*>* track) {
     *p = static_cast<T*>(q);
     return TC_OK;
 }
+
+// Arrays of one allocation: listed with add, placed by alloc (each on a 256-byte
+// boundary).  A graph's forty arrays took 60 us to allocate and free one by one.
+class Slab {
+  public:
+    template <typename T>
+    Slab& add(T** p, size_t count) {
+        items_.push_back({[](void* at, void* field) { *static_cast<T**>(field) = static_cast<T*>(at); }, p, bytes_});
+        bytes_ += (count * sizeof(T) + 255) & ~(size_t)255;
+        return *this;
+    }
+    tc_status alloc(tc_graph* g, std::vector<void*>* track) {
+        char* base = nullptr;
+        const tc_status st = dalloc(g, &base, bytes_, track);
+        if (st != TC_OK) return st;
+        for (const Item& i : items_) i.set(base + i.offset, i.field);
+        return TC_OK;
+    }
+
+  private:
+    struct Item {
+        void (*set)(void* at, void* field);
+        void* field;
+        size_t offset;
+    };
+    std::vector<Item> items_;
+    size_t bytes_ = 0;
+};
 
 void free_list(tc_graph* g, std::vector<void*>* list) {
     for (void* p : *list) cudaFreeAsync(p, g->stream);
@@ -246,27 +342,22 @@ struct SegInfo {
     int seg_bits, deg_bits, local_bits;
 };
 
-// The graph's second stream and its two events, created at first use; null when
-// they cannot be created (the work then stays on the graph's stream).
-const PlanStreams* side_streams(tc_graph* g, PlanStreams* out) {
-    if (!g->side) {
-        cudaStream_t s = nullptr;
-        cudaEvent_t f = nullptr, j = nullptr;
-        if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess &&
-            cudaEventCreateWithFlags(&f, cudaEventDisableTiming) == cudaSuccess &&
-            cudaEventCreateWithFlags(&j, cudaEventDisableTiming) == cudaSuccess) {
-            g->side = s;
-            g->plan_fork = f;
-            g->plan_join = j;
-        } else {  // one stream then; the failure is not the caller's
-            if (j) cudaEventDestroy(j);
-            if (f) cudaEventDestroy(f);
-            if (s) cudaStreamDestroy(s);
-            cudaGetLastError();
-            return nullptr;
-        }
+// The graph's streams and events, taken at first use.
+tc_status need_sync(tc_graph* g) {
+    if (g->has_sync) return TC_OK;
+    const cudaError_t e = take_sync(g->device, &g->sync);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return cuda_fail("streams and events", e);
     }
-    *out = PlanStreams{g->side, g->plan_fork, g->plan_join};
+    g->has_sync = true;
+    return TC_OK;
+}
+
+// The second stream, for single graphs that are not recorded into a CUDA graph.
+const PlanStreams* side_streams(tc_graph* g, PlanStreams* out) {
+    if (g->capture || g->batch_G >= 0 || !g->has_sync) return nullptr;
+    *out = PlanStreams{g->sync.side, g->sync.fork, g->sync.join};
     return out;
 }
 
@@ -282,28 +373,19 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
     g->core_cap = g->hub_cap < CORE_MAX ? g->hub_cap : CORE_MAX;
     g->core_words = core_words_for(g->core_cap);
     const size_t cc = (size_t)g->core_cap;
-    if ((st = dalloc(g, &g->stats, 1, &keep)) || (st = dalloc(g, &g->rank, nn, &keep)) ||
-        (st = dalloc(g, &g->rowstart, nn + 1, &keep)) || (st = dalloc(g, &g->rowlen, nn, &keep)) ||
-        (st = dalloc(g, &g->rowinfo, nn, &keep)) ||
-        (st = dalloc(g, &g->col, (size_t)m, &keep)) || (st = dalloc(g, &g->deg, nn, &keep)) ||
-        (st = dalloc(g, &g->small_list[0], nn, &keep)) || (st = dalloc(g, &g->small_list[1], nn, &keep)) ||
-        (st = dalloc(g, &g->small_list[2], nn, &keep)) || (st = dalloc(g, &g->small_list[3], nn, &keep)) ||
-        (st = dalloc(g, &g->cta_list, nn, &keep)) ||
-        (st = dalloc(g, &g->hub_cnt, hc + 1, &keep)) || (st = dalloc(g, &g->hub_start, hc + 1, &keep)) ||
-        (st = dalloc(g, &g->hub_cur64, hc + 1, &keep)) ||
-        (st = dalloc(g, &g->big_list, hc + 1, &keep)) ||
-        (st = dalloc(g, &g->long_list, hc + 1, &keep)) ||
-        (st = dalloc(g, &g->win_task, (size_t)hub_task_cap(g->hub_cap, m), &keep)) ||
-        (st = dalloc(g, &g->low_task, (size_t)hub_task_cap(g->hub_cap, m), &keep)) ||
-        (st = dalloc(g, &g->winrow, nn, &keep)) || (st = dalloc(g, &g->winlow, nn, &keep)) ||
-        (st = dalloc(g, &g->win, (size_t)win_vec_cap(n, m), &keep)) ||
-        (st = dalloc(g, &g->in_rec, (size_t)m, &keep)) ||
-        (st = dalloc(g, &g->rowof, (size_t)m, &keep)) ||
-        (st = dalloc(g, (char**)&g->plan_tmp, scan_tmp_bytes((int64_t)hc + 1), &keep)) ||
-        (st = dalloc(g, &g->t_rank, nn, &keep)) ||
-        (st = dalloc(g, &g->core_bits, cc * (size_t)g->core_words + cc, &keep)) ||
-        (st = dalloc(g, &g->core_lohi, 3 * cc, &keep)))
-        return st;
+    if (!g->capture && (st = need_sync(g)) != TC_OK) return st;
+    Slab kept;
+    kept.add(&g->stats, 1).add(&g->rank, nn).add(&g->rowstart, nn + 1).add(&g->rowlen, nn).add(&g->rowinfo, nn);
+    kept.add(&g->col, (size_t)m).add(&g->deg, nn).add(&g->t_rank, nn);
+    for (int32_t*& list : g->small_list) kept.add(&list, nn);
+    kept.add(&g->cta_list, nn);
+    kept.add(&g->hub_cnt, hc + 1).add(&g->hub_start, hc + 1).add(&g->hub_cur64, hc + 1).add(&g->big_list, hc + 1);
+    kept.add(&g->long_list, hc + 1).add(&g->win_task, (size_t)hub_task_cap(g->hub_cap, m));
+    kept.add(&g->low_task, (size_t)hub_task_cap(g->hub_cap, m)).add(&g->winrow, nn).add(&g->winlow, nn);
+    kept.add(&g->win, (size_t)win_vec_cap(n, m)).add(&g->in_rec, (size_t)m).add(&g->rowof, (size_t)m);
+    kept.add((char**)&g->plan_tmp, scan_tmp_bytes((int64_t)hc + 1));
+    kept.add(&g->core_bits, cc * (size_t)g->core_words + cc).add(&g->core_lohi, 3 * cc);
+    if ((st = kept.alloc(g, &keep)) != TC_OK) return st;
     std::vector<void*> scratch;
     BuildBuffers B{};
     B.src = src;
@@ -325,17 +407,14 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
     size_t rt = radix_tmp_bytes((int64_t)nn);
     if (rt > tmp_bytes) tmp_bytes = rt;
     char* tmp = nullptr;
-    if ((st = dalloc(g, &B.dmulti, nn, &scratch)) || (st = dalloc(g, &B.keys, nn, &scratch)) ||
-        (st = dalloc(g, &B.keys_alt, nn, &scratch)) || (st = dalloc(g, &B.rowcnt, nn + 1, &scratch)) ||
-        (st = dalloc(g, &B.cursor, nn, &scratch)) || (st = dalloc(g, &B.dupin, nn, &scratch)) ||
-        (st = dalloc(g, &B.bcount, (size_t)BUCKET_MAX + 1, &scratch)) ||
-        (st = dalloc(g, &B.bcur, (size_t)BUCKET_MAX, &scratch)) ||
-        (st = dalloc(g, &B.bstart, (size_t)BUCKET_MAX + 1, &scratch)) ||
-        (st = dalloc(g, &B.pairs, (size_t)m, &scratch)) ||
-        (st = dalloc(g, &tmp, tmp_bytes, &scratch))) {
-        free_list(g, &scratch);
-        return st;
-    }
+    Slab work;  // the zeroed counters first: one memset
+    work.add(&B.dmulti, nn).add(&B.dupin, nn).add(&B.rowcnt, nn + 1).add(&B.bcount, (size_t)BUCKET_MAX + 1);
+    work.add(&B.bcur, (size_t)BUCKET_MAX);
+    work.add(&B.keys, nn).add(&B.keys_alt, nn).add(&B.bstart, (size_t)BUCKET_MAX + 1).add(&B.pairs, (size_t)m);
+    work.add(&tmp, tmp_bytes);
+    if ((st = work.alloc(g, &scratch)) != TC_OK) return st;
+    const size_t zeroed = (size_t)((char*)B.keys - (char*)B.dmulti);
+    B.seg = reinterpret_cast<uint32_t*>(g->small_list[3]);  // free until the plan
     B.tmp = tmp;
     // the input-order pairs and the sorters' row lists share memory with arrays that the
     // planner writes after the build is done with them
@@ -350,15 +429,10 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
     B.col = g->col;
     B.deg = g->deg;
     B.stats = g->stats;
-    cudaEvent_t* bev = nullptr;
-    if (!g->capture) {
-        if (!g->bev[0])
-            for (int i = 0; i < BP_EVENTS; ++i) TC_CK(cudaEventCreate(&g->bev[i]));
-        bev = g->bev;
-        cudaEventRecord(bev[BP_START], g->stream);
-    }
+    cudaEvent_t* const bev = g->capture ? nullptr : g->sync.bev;
+    if (bev) cudaEventRecord(bev[BP_START], g->stream);
     cudaMemsetAsync(g->stats, 0, sizeof(DevStats), g->stream);
-    cudaMemsetAsync(B.dmulti, 0, sizeof(uint32_t) * nn, g->stream);
+    cudaMemsetAsync(B.dmulti, 0, zeroed, g->stream);
     if (host && m > 0) {
         const int64_t piece = (m + INGEST_PIECES - 1) / INGEST_PIECES;
         cudaError_t e = cudaSuccess;
@@ -402,7 +476,7 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
     launch_rank(B, deg_bits, g->L);
     if (bev) cudaEventRecord(bev[BP_RANK], g->stream);
     PlanStreams psv{};
-    launch_orient(B, g->L, bev, !g->capture && !seg ? side_streams(g, &psv) : nullptr);
+    launch_orient(B, g->L, bev, seg ? nullptr : side_streams(g, &psv));
     if (bev) {
         cudaEventRecord(bev[BP_END], g->stream);
         g->build_timed = true;
@@ -451,38 +525,28 @@ CountBuffers count_buffers(tc_graph* g) {
     C.stats = g->stats;
     C.src_lo = g->src_lo;
     C.src_hi = g->src_hi < 0 ? g->n : g->src_hi;
-    C.hub_ready = g->plan_forked ? g->plan_join : nullptr;
+    C.hub_ready = g->plan_forked ? g->sync.join : nullptr;
     return C;
-}
-
-tc_status ensure_events(tc_graph* g) {
-    if (g->capture) return TC_OK;
-    if (!g->ev[0])
-        for (int i = 0; i < PH_EVENTS; ++i) TC_CK(cudaEventCreate(&g->ev[i]));
-    return TC_OK;
 }
 
 // Orders the main stream after the hub part of the last plan (no-op when it ran on
 // the main stream): before a replan, before the graph's memory is released, and
 // wherever the hub lists are read outside the count.
 void join_plan(tc_graph* g) {
-    if (g->plan_forked) cudaStreamWaitEvent(g->stream, g->plan_join, 0);
+    if (g->plan_forked) cudaStreamWaitEvent(g->stream, g->sync.join, 0);
 }
 
 // Planning (a4): bucket lists and hub in-edge lists; rerun when hub settings change.
 tc_status run_plan(tc_graph* g) {
     if (g->planned) return TC_OK;
-    tc_status st = ensure_events(g);
-    if (st != TC_OK) return st;
     join_plan(g);  // a previous plan's hub part writes the buffers this one rewrites
     const size_t off = offsetof(DevStats, small_count);
     TC_CK(cudaMemsetAsync(reinterpret_cast<char*>(g->stats) + off, 0, sizeof(DevStats) - off, g->stream));
-    if (!g->capture) TC_CK(cudaEventRecord(g->ev[PH_PLAN], g->stream));
+    if (!g->capture) TC_CK(cudaEventRecord(g->sync.ev[PH_PLAN], g->stream));
     // single graphs build their hub lists on a second stream while the push buckets
     // are counted; batches (which may be recorded into a CUDA graph) keep one stream
     PlanStreams psv{};
-    const PlanStreams* ps = !g->capture && g->batch_G < 0 ? side_streams(g, &psv) : nullptr;
-    g->plan_forked = launch_plan(count_buffers(g), g->strat, g->L, ps);
+    g->plan_forked = launch_plan(count_buffers(g), g->strat, g->L, side_streams(g, &psv));
     TC_CK(cudaGetLastError());
     g->planned = true;
     g->counted = false;
@@ -491,17 +555,16 @@ tc_status run_plan(tc_graph* g) {
 
 tc_status run_count(tc_graph* g) {
     if (g->counted) return TC_OK;
-    tc_status st = ensure_events(g);
-    if (st != TC_OK) return st;
+    tc_status st;
     if (g->planned) {
-        if (!g->capture) TC_CK(cudaEventRecord(g->ev[PH_PLAN], g->stream));  // planning already done: empty phase
+        if (!g->capture) TC_CK(cudaEventRecord(g->sync.ev[PH_PLAN], g->stream));  // planning already done: empty phase
     } else if ((st = run_plan(g)) != TC_OK) {
         return st;
     }
     TC_CK(cudaMemsetAsync(g->t_rank, 0, sizeof(unsigned long long) * (size_t)g->n, g->stream));
     TC_CK(cudaMemsetAsync(&g->stats->sum_t, 0, sizeof(unsigned long long), g->stream));
     CountBuffers C = count_buffers(g);
-    launch_intersect(C, g->strat, g->capture ? nullptr : g->ev, g->L);
+    launch_intersect(C, g->strat, g->capture ? nullptr : g->sync.ev, g->L);
     launch_sum_t(C, g->L);
     TC_CK(cudaGetLastError());
     g->counted = true;
@@ -513,13 +576,7 @@ void destroy(tc_graph* g) {
     if (!g) return;
     join_plan(g);
     free_list(g, &g->blocks);
-    for (int i = 0; i < PH_EVENTS; ++i)
-        if (g->ev[i]) cudaEventDestroy(g->ev[i]);
-    for (int i = 0; i < BP_EVENTS; ++i)
-        if (g->bev[i]) cudaEventDestroy(g->bev[i]);
-    if (g->plan_join) cudaEventDestroy(g->plan_join);
-    if (g->plan_fork) cudaEventDestroy(g->plan_fork);
-    if (g->side) cudaStreamDestroy(g->side);
+    if (g->has_sync) give_sync(g->device, &g->sync);
     delete g;
 }
 
@@ -584,24 +641,21 @@ tc_status tc_graph_create_from_edges(int32_t n, int64_t m, const int32_t* src, c
         free_list(g, &tmp);
         return finish_create(g, st, out);
     }
-    // the side stream may only touch ds and dd once their allocation is ordered
-    HostPairs hp{src, dst, nullptr, nullptr};
-    cudaEvent_t allocated = nullptr;
-    cudaError_t e = cudaStreamCreateWithFlags(&hp.side, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&hp.landed, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&allocated, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventRecord(allocated, g->stream);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(hp.side, allocated, 0);
+    if ((st = need_sync(g)) != TC_OK) {
+        free_list(g, &tmp);
+        return finish_create(g, st, out);
+    }
+    // the copy stream may only touch ds and dd once their allocation is ordered
+    const HostPairs hp{src, dst, g->sync.copy, g->sync.landed};
+    cudaError_t e = cudaEventRecord(g->sync.allocated, g->stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(hp.side, g->sync.allocated, 0);
     if (e != cudaSuccess)
         st = cuda_fail("host input stream", e);
     else
         st = build_graph(g, ds, dd, m, true, &hp);
     // the build read its statistics back on g->stream, which waited for every piece:
-    // the copies are complete; the side stream and events can go
+    // the copies are complete
     if (st != TC_OK) cudaStreamSynchronize(hp.side);
-    if (allocated) cudaEventDestroy(allocated);
-    if (hp.landed) cudaEventDestroy(hp.landed);
-    if (hp.side) cudaStreamDestroy(hp.side);
     free_list(g, &tmp);
     return finish_create(g, st, out);
 }
@@ -1162,10 +1216,10 @@ tc_status tc_graph_set_hubs(tc_graph* g, int32_t min_degree, int32_t max_hubs) {
 
 tc_status tc_graph_build_timing(const tc_graph* g, float* ms, int count) {
     if (!g || !ms || count < 0 || !g->build_timed) return TC_EINVAL;
-    TC_CK(cudaEventSynchronize(g->bev[BP_END]));
+    TC_CK(cudaEventSynchronize(g->sync.bev[BP_END]));
     float v[BP_EVENTS] = {};
-    for (int i = 1; i < BP_EVENTS; ++i) TC_CK(cudaEventElapsedTime(&v[i - 1], g->bev[i - 1], g->bev[i]));
-    TC_CK(cudaEventElapsedTime(&v[BP_EVENTS - 1], g->bev[BP_START], g->bev[BP_END]));
+    for (int i = 1; i < BP_EVENTS; ++i) TC_CK(cudaEventElapsedTime(&v[i - 1], g->sync.bev[i - 1], g->sync.bev[i]));
+    TC_CK(cudaEventElapsedTime(&v[BP_EVENTS - 1], g->sync.bev[BP_START], g->sync.bev[BP_END]));
     for (int i = 0; i < count && i < BP_EVENTS; ++i) ms[i] = v[i];
     return TC_OK;
 }
@@ -1173,13 +1227,13 @@ tc_status tc_graph_build_timing(const tc_graph* g, float* ms, int count) {
 tc_status tc_graph_last_timing(const tc_graph* g, float* ms, int count) {
     if (!g || !ms || count < 0) return TC_EINVAL;
     if (!g->timed) return TC_EINVAL;
-    TC_CK(cudaEventSynchronize(g->ev[PH_END]));
+    TC_CK(cudaEventSynchronize(g->sync.ev[PH_END]));
     float v[5] = {0, 0, 0, 0, 0};
-    TC_CK(cudaEventElapsedTime(&v[0], g->ev[PH_PLAN], g->ev[PH_SMALL]));
-    TC_CK(cudaEventElapsedTime(&v[1], g->ev[PH_SMALL], g->ev[PH_CTA]));
-    TC_CK(cudaEventElapsedTime(&v[2], g->ev[PH_CTA], g->ev[PH_HUB]));
-    TC_CK(cudaEventElapsedTime(&v[3], g->ev[PH_HUB], g->ev[PH_END]));
-    TC_CK(cudaEventElapsedTime(&v[4], g->ev[PH_PLAN], g->ev[PH_END]));
+    TC_CK(cudaEventElapsedTime(&v[0], g->sync.ev[PH_PLAN], g->sync.ev[PH_SMALL]));
+    TC_CK(cudaEventElapsedTime(&v[1], g->sync.ev[PH_SMALL], g->sync.ev[PH_CTA]));
+    TC_CK(cudaEventElapsedTime(&v[2], g->sync.ev[PH_CTA], g->sync.ev[PH_HUB]));
+    TC_CK(cudaEventElapsedTime(&v[3], g->sync.ev[PH_HUB], g->sync.ev[PH_END]));
+    TC_CK(cudaEventElapsedTime(&v[4], g->sync.ev[PH_PLAN], g->sync.ev[PH_END]));
     for (int i = 0; i < count && i < 5; ++i) ms[i] = v[i];
     return TC_OK;
 }
@@ -1544,6 +1598,15 @@ struct RunEntry {
 static std::mutex g_run_mutex;
 static std::vector<RunEntry> g_runs;
 
+static void free_run_entry(RunEntry* r) {
+    if (r->exec) cudaGraphExecDestroy(r->exec);
+    if (r->graph) cudaGraphDestroy(r->graph);
+    cudaFree(r->vbase);
+    cudaFree(r->eoff);
+    cudaFree(r->status);
+    *r = RunEntry{};
+}
+
 static uint64_t fnv(uint64_t h, const void* p, size_t bytes) {
     const unsigned char* c = static_cast<const unsigned char*>(p);
     for (size_t i = 0; i < bytes; ++i) h = (h ^ c[i]) * 1099511628211ull;
@@ -1610,41 +1673,76 @@ extern "C" tc_status tc_batch_run(int32_t G, const int32_t* n, const int64_t* ed
         ent.device = dev;
         std::vector<int32_t> vb((size_t)G + 1, 0);
         for (int32_t i = 0; i < G; ++i) vb[i + 1] = vb[i] + n[i];
-        TC_CK(cudaMalloc(&ent.vbase, sizeof(int32_t) * vb.size()));
-        TC_CK(cudaMalloc(&ent.eoff, sizeof(int64_t) * ((size_t)G + 1)));
-        TC_CK(cudaMalloc(&ent.status, sizeof(int)));
-        TC_CK(cudaMemcpy(ent.vbase, vb.data(), sizeof(int32_t) * vb.size(), cudaMemcpyHostToDevice));
-        if (G > 0) TC_CK(cudaMemcpy(ent.eoff, edge_off, sizeof(int64_t) * ((size_t)G + 1), cudaMemcpyHostToDevice));
         tc_graph* g = nullptr;
         if ((st = new_graph((int32_t)n_total, cuda_stream, &g)) != TC_OK) return st;
+        if (graph_mode) {  // arrays that the recorded graph keeps
+            cudaError_t e = cudaMalloc(&ent.vbase, sizeof(int32_t) * vb.size());
+            if (e == cudaSuccess) e = cudaMalloc(&ent.eoff, sizeof(int64_t) * ((size_t)G + 1));
+            if (e == cudaSuccess) e = cudaMalloc(&ent.status, sizeof(int));
+            if (e == cudaSuccess)
+                e = cudaMemcpy(ent.vbase, vb.data(), sizeof(int32_t) * vb.size(), cudaMemcpyHostToDevice);
+            if (e == cudaSuccess && G > 0)
+                e = cudaMemcpy(ent.eoff, edge_off, sizeof(int64_t) * ((size_t)G + 1), cudaMemcpyHostToDevice);
+            if (e != cudaSuccess) {
+                free_run_entry(&ent);
+                destroy(g);
+                return cuda_fail("tc_batch_run arrays", e);
+            }
+        } else {  // of this call: released with the graph object
+            Slab arrays;
+            arrays.add(&ent.vbase, vb.size()).add(&ent.eoff, (size_t)G + 1).add(&ent.status, 1);
+            st = arrays.alloc(g, &g->blocks);
+            // pageable host memory is staged before these calls return
+            cudaError_t e = cudaSuccess;
+            if (st == TC_OK)
+                e = cudaMemcpyAsync(ent.vbase, vb.data(), sizeof(int32_t) * vb.size(), cudaMemcpyHostToDevice, stream);
+            if (st == TC_OK && e == cudaSuccess && G > 0)
+                e = cudaMemcpyAsync(ent.eoff, edge_off, sizeof(int64_t) * ((size_t)G + 1), cudaMemcpyHostToDevice, stream);
+            if (st == TC_OK && e != cudaSuccess) st = cuda_fail("tc_batch_run copy", e);
+            if (st != TC_OK) {
+                destroy(g);
+                return st;
+            }
+        }
         g->m_in = m;
         g->capture = graph_mode;
         tuning_put(g, &tun);
-        if (graph_mode) TC_CK(cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal));
+        cudaError_t e = graph_mode ? cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal) : cudaSuccess;
+        if (e != cudaSuccess) {
+            free_run_entry(&ent);
+            destroy(g);
+            return cuda_fail("cudaStreamBeginCapture", e);
+        }
         const uint64_t k0 = launch_total();
         const SegInfo seg = batch_seg_info(G, n, edge_off, ent.vbase);
         st = batch_pipeline(g, G, ent.vbase, ent.eoff, src, dst, m, T_out, t_out, lcc_out, ent.status, &seg);
-        g->batch_vbase = nullptr;  // owned by the entry
-        destroy(g);
-        ent.kernels = launch_total() - k0;
-        if (graph_mode) {
-            cudaError_t e = cudaStreamEndCapture(stream, &ent.graph);
+        if (!graph_mode) {
+            if (st == TC_OK) {
+                e = cudaMemcpyAsync(&status_h, ent.status, sizeof(int), cudaMemcpyDeviceToHost, stream);
+                if (e != cudaSuccess) st = cuda_fail("tc_batch_run status", e);
+            }
+            destroy(g);
+            e = cudaStreamSynchronize(stream);
             if (st != TC_OK) return st;
-            if (e != cudaSuccess) return cuda_fail("cudaStreamEndCapture", e);
-            TC_CK(cudaGraphInstantiate(&ent.exec, ent.graph, 0));
-            TC_CK(cudaGraphLaunch(ent.exec, stream));
-        } else if (st != TC_OK) {
-            return st;
-        }
-        TC_CK(cudaMemcpyAsync(&status_h, ent.status, sizeof(int), cudaMemcpyDeviceToHost, stream));
-        TC_CK(cudaStreamSynchronize(stream));
-        if (graph_mode) {
+            if (e != cudaSuccess) return cuda_fail("tc_batch_run", e);
+        } else {
+            g->batch_vbase = nullptr;  // owned by the entry
+            destroy(g);
+            ent.kernels = launch_total() - k0;
+            e = cudaStreamEndCapture(stream, &ent.graph);
+            if (st == TC_OK && e != cudaSuccess) st = cuda_fail("cudaStreamEndCapture", e);
+            if (st == TC_OK && (e = cudaGraphInstantiate(&ent.exec, ent.graph, 0)) != cudaSuccess)
+                st = cuda_fail("cudaGraphInstantiate", e);
+            if (st == TC_OK && (e = cudaGraphLaunch(ent.exec, stream)) != cudaSuccess)
+                st = cuda_fail("cudaGraphLaunch", e);
+            if (st != TC_OK) {
+                free_run_entry(&ent);
+                return st;
+            }
+            TC_CK(cudaMemcpyAsync(&status_h, ent.status, sizeof(int), cudaMemcpyDeviceToHost, stream));
+            TC_CK(cudaStreamSynchronize(stream));
             std::lock_guard<std::mutex> lock(g_run_mutex);
             g_runs.push_back(ent);
-        } else {
-            cudaFree(ent.vbase);
-            cudaFree(ent.eoff);
-            cudaFree(ent.status);
         }
     }
     if (status_h & ERR_BAD_ID) {
@@ -1656,16 +1754,24 @@ extern "C" tc_status tc_batch_run(int32_t G, const int32_t* n, const int64_t* ed
 }
 
 extern "C" void tc_release_cached_graphs(void) {
+    {
+        std::lock_guard<std::mutex> lock(g_sync_mutex);
+        int cur = 0;
+        const bool any = cudaGetDevice(&cur) == cudaSuccess;
+        for (int dev = 0; dev < 64 && any; ++dev) {
+            if (g_sync[dev].empty()) continue;
+            cudaSetDevice(dev);
+            for (SyncSet& x : g_sync[dev]) x.destroy();
+            g_sync[dev].clear();
+            cudaSetDevice(cur);
+        }
+    }
     std::lock_guard<std::mutex> lock(g_run_mutex);
     for (auto& r : g_runs) {
         int cur = 0;
         cudaGetDevice(&cur);
         cudaSetDevice(r.device);
-        if (r.exec) cudaGraphExecDestroy(r.exec);
-        if (r.graph) cudaGraphDestroy(r.graph);
-        cudaFree(r.vbase);
-        cudaFree(r.eoff);
-        cudaFree(r.status);
+        free_run_entry(&r);
         cudaSetDevice(cur);
     }
     g_runs.clear();

@@ -805,7 +805,7 @@ __global__ void k_rank_invert_seg(const uint64_t* __restrict__ sorted, const int
 void launch_rank(const BuildBuffers& B, int deg_bits, const Launch& L) {
     if (B.n <= 0) return;
     if (B.seg_vbase && B.seg_count > 0 && B.seg_bits + B.seg_deg_bits + B.local_bits <= 64) {
-        uint32_t* seg = B.cursor;  // free until the row fill
+        uint32_t* seg = B.seg;
         k_seg_of<<<grid_for((int64_t)B.seg_count * 32, THREADS, L.sms), THREADS, 0, L.stream>>>(B.seg_vbase,
                                                                                                B.seg_count, seg);
         count_launch();
@@ -839,13 +839,9 @@ void bucket_shape(int32_t n, int* shift, int* nb) {
 
 void launch_orient(const BuildBuffers& B, const Launch& L, cudaEvent_t* ev, const PlanStreams* ps) {
     if (B.n <= 0) return;
-    cudaMemsetAsync(B.cursor, 0, sizeof(uint32_t) * (size_t)B.n, L.stream);
-    cudaMemsetAsync(B.dupin, 0, sizeof(uint32_t) * (size_t)B.n, L.stream);
     int shift = 0, nb = 0;
     bucket_shape(B.n, &shift, &nb);
     if (B.bucket_fill && nb > 0) {
-        cudaMemsetAsync(B.bcount, 0, sizeof(uint32_t) * (size_t)nb, L.stream);
-        cudaMemsetAsync(B.bcur, 0, sizeof(uint32_t) * (size_t)nb, L.stream);
         if (B.m > 0) {
             k_bucket_count<<<grid_for(B.m, THREADS * PAIR_UNROLL, L.sms, 8), THREADS, sizeof(uint32_t) * nb, L.stream>>>(
                 B.src, B.dst, B.m, B.n, B.rank, shift, nb, B.bcount, B.oriented, B.dir_bits);
@@ -863,7 +859,6 @@ void launch_orient(const BuildBuffers& B, const Launch& L, cudaEvent_t* ev, cons
             B.n, shift, nb, B.bstart, B.pairs, B.rowstart, B.rowcnt, B.col, B.stats);
         count_launch();
     } else {
-        cudaMemsetAsync(B.rowcnt, 0, sizeof(uint32_t) * (size_t)B.n, L.stream);
         if (B.m > 0) {
             k_orient_count<<<grid_for(B.m, THREADS, L.sms), THREADS, 0, L.stream>>>(B.src, B.dst, B.m, B.n, B.rank,
                                                                                   B.rowcnt, B.oriented, B.dir_bits);

@@ -101,11 +101,11 @@ struct BuildBuffers {
     int64_t m;
     int32_t n;
     // scratch
-    uint32_t* dmulti;     // n
+    uint32_t* dmulti;     // n; this, dupin, rowcnt, bcount and bcur start at zero
     uint64_t* keys;       // n
     uint64_t* keys_alt;   // n
     uint32_t* rowcnt;     // n + 1
-    uint32_t* cursor;     // n
+    uint32_t* seg;        // n: graph of every vertex (batches)
     int32_t* longlist;    // n
     int32_t* midlist;     // n: rows of 17..256 entries
     int32_t* midlist2;    // n: rows of 257..1024 entries

@@ -87,6 +87,7 @@ void run_one(cudaMemPool_t pool, int sms, cudaStream_t stream, const tc_request&
     out->status = TC_OK;
     const size_t n = (size_t)r.n;
     Launch L{stream, sms};
+    char* block = nullptr;  // the pairs, the outputs and their checksums
     int32_t *src = nullptr, *dst = nullptr;
     unsigned long long* t = nullptr;
     double* lcc = nullptr;
@@ -97,16 +98,17 @@ void run_one(cudaMemPool_t pool, int sms, cudaStream_t stream, const tc_request&
     int64_t m_simple = 0;
     auto fail = [&](tc_status st) { out->status = st; };
     do {
-        const size_t me = r.m > 0 ? (size_t)r.m : 1;
-        if ((e = cudaMallocFromPoolAsync((void**)&src, 4 * me, pool, stream)) != cudaSuccess ||
-            (e = cudaMallocFromPoolAsync((void**)&dst, 4 * me, pool, stream)) != cudaSuccess ||
-            (e = cudaMallocFromPoolAsync((void**)&t, 8 * (n ? n : 1), pool, stream)) != cudaSuccess ||
-            (e = cudaMallocFromPoolAsync((void**)&lcc, 8 * (n ? n : 1), pool, stream)) != cudaSuccess ||
-            (e = cudaMallocFromPoolAsync((void**)&sums, 16, pool, stream)) != cudaSuccess) {
+        const size_t pairs = (4 * (size_t)r.m + 255) & ~(size_t)255, verts = (8 * n + 255) & ~(size_t)255;
+        if ((e = cudaMallocFromPoolAsync((void**)&block, 2 * pairs + 2 * verts + 16, pool, stream)) != cudaSuccess) {
             cudaGetLastError();
             fail(TC_ENOMEM);
             break;
         }
+        src = reinterpret_cast<int32_t*>(block);
+        dst = reinterpret_cast<int32_t*>(block + pairs);
+        t = reinterpret_cast<unsigned long long*>(block + 2 * pairs);
+        lcc = reinterpret_cast<double*>(block + 2 * pairs + verts);
+        sums = reinterpret_cast<unsigned long long*>(block + 2 * pairs + 2 * verts);
         if ((e = launch_generate(r.kind, r.n, r.m, r.seed, r.stream_id, src, dst, L)) != cudaSuccess) {
             fail(TC_ECUDA);
             break;
@@ -116,26 +118,25 @@ void run_one(cudaMemPool_t pool, int sms, cudaStream_t stream, const tc_request&
             fail(st);
             break;
         }
-        if ((st = tc_count(g, &out->T)) != TC_OK || (st = lcc_compute(g, reinterpret_cast<uint64_t*>(t), lcc, TC_MEM_DEVICE)) != TC_OK ||
-            (st = tc_graph_info(g, &m_simple, nullptr, nullptr)) != TC_OK) {
+        // everything is queued before the first wait, which tc_count makes
+        if ((st = lcc_compute(g, reinterpret_cast<uint64_t*>(t), lcc, TC_MEM_DEVICE)) != TC_OK) {
             fail(st);
             break;
         }
         cudaMemsetAsync(sums, 0, 16, stream);
         k_checksum<<<grid_for(r.n, 256, sms), 256, 0, stream>>>(r.n, t, lcc, sums);
         count_launch();
-        if ((e = cudaMemcpyAsync(h, sums, 16, cudaMemcpyDeviceToHost, stream)) != cudaSuccess ||
-            (e = cudaStreamSynchronize(stream)) != cudaSuccess) {
+        if ((e = cudaMemcpyAsync(h, sums, 16, cudaMemcpyDeviceToHost, stream)) != cudaSuccess) {
             fail(TC_ECUDA);
+            break;
+        }
+        if ((st = tc_count(g, &out->T)) != TC_OK || (st = tc_graph_info(g, &m_simple, nullptr, nullptr)) != TC_OK) {
+            fail(st);
             break;
         }
     } while (false);
     if (g) tc_graph_destroy(g);
-    if (src) cudaFreeAsync(src, stream);
-    if (dst) cudaFreeAsync(dst, stream);
-    if (t) cudaFreeAsync(t, stream);
-    if (lcc) cudaFreeAsync(lcc, stream);
-    if (sums) cudaFreeAsync(sums, stream);
+    if (block) cudaFreeAsync(block, stream);
     cudaStreamSynchronize(stream);
     out->m_simple = m_simple;
     out->t_hash = h[0];
