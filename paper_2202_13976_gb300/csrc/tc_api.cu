@@ -190,14 +190,15 @@ struct tc_graph {
     int32_t src_lo = 0, src_hi = -1;  // ranks of the sources counted (-1: up to n); tc_count_shard
     int32_t core_cap = 0;
     int32_t core_words = 0;
-    uint32_t* core_bits = nullptr;  // adjacency rows, core in-degrees
-    int32_t* core_lohi = nullptr;   // lowest and highest neighbour, highest out-neighbour
+    uint32_t* core_bits = nullptr;  // adjacency rows; core in-degrees, lowest, highest neighbour, highest out-neighbour
 
     unsigned long long* t_rank = nullptr;
     DevStats* stats = nullptr;
     std::vector<void*> blocks;
     bool planned = false;
     bool counted = false;
+    bool plan_zeroed = false;   // the planner's part of the statistics is zero
+    bool count_zeroed = false;  // t and the count's part of the statistics are zero
     Strategy strat{};
     bool timed = false;
     bool build_timed = false;
@@ -375,8 +376,8 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
     const size_t cc = (size_t)g->core_cap;
     if (!g->capture && (st = need_sync(g)) != TC_OK) return st;
     Slab kept;
-    kept.add(&g->stats, 1).add(&g->rank, nn).add(&g->rowstart, nn + 1).add(&g->rowlen, nn).add(&g->rowinfo, nn);
-    kept.add(&g->col, (size_t)m).add(&g->deg, nn).add(&g->t_rank, nn);
+    kept.add(&g->stats, 1).add(&g->t_rank, nn).add(&g->rank, nn).add(&g->rowstart, nn + 1).add(&g->rowlen, nn).add(&g->rowinfo, nn);
+    kept.add(&g->col, (size_t)m).add(&g->deg, nn);
     for (int32_t*& list : g->small_list) kept.add(&list, nn);
     kept.add(&g->cta_list, nn);
     kept.add(&g->hub_cnt, hc + 1).add(&g->hub_start, hc + 1).add(&g->hub_cur64, hc + 1).add(&g->big_list, hc + 1);
@@ -384,7 +385,7 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
     kept.add(&g->low_task, (size_t)hub_task_cap(g->hub_cap, m)).add(&g->winrow, nn).add(&g->winlow, nn);
     kept.add(&g->win, (size_t)win_vec_cap(n, m)).add(&g->in_rec, (size_t)m).add(&g->rowof, (size_t)m);
     kept.add((char**)&g->plan_tmp, scan_tmp_bytes((int64_t)hc + 1));
-    kept.add(&g->core_bits, cc * (size_t)g->core_words + cc).add(&g->core_lohi, 3 * cc);
+    kept.add(&g->core_bits, cc * (size_t)g->core_words + 4 * cc);
     if ((st = kept.alloc(g, &keep)) != TC_OK) return st;
     std::vector<void*> scratch;
     BuildBuffers B{};
@@ -431,8 +432,10 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
     B.stats = g->stats;
     cudaEvent_t* const bev = g->capture ? nullptr : g->sync.bev;
     if (bev) cudaEventRecord(bev[BP_START], g->stream);
-    cudaMemsetAsync(g->stats, 0, sizeof(DevStats), g->stream);
+    // the statistics and t (for the first count), then the build's counters
+    cudaMemsetAsync(g->stats, 0, (size_t)((char*)(g->t_rank + nn) - (char*)g->stats), g->stream);
     cudaMemsetAsync(B.dmulti, 0, zeroed, g->stream);
+    g->count_zeroed = g->plan_zeroed = true;
     if (host && m > 0) {
         const int64_t piece = (m + INGEST_PIECES - 1) / INGEST_PIECES;
         cudaError_t e = cudaSuccess;
@@ -518,9 +521,9 @@ CountBuffers count_buffers(tc_graph* g) {
     const size_t rows = (size_t)g->core_cap * (size_t)g->core_words;
     C.core_z = g->core_bits;
     C.core_cnt = g->core_bits + rows;
-    C.core_lo = g->core_lohi;
-    C.core_hi = g->core_lohi + g->core_cap;
-    C.core_hiout = g->core_lohi + 2 * (size_t)g->core_cap;
+    C.core_lo = reinterpret_cast<int32_t*>(C.core_cnt + g->core_cap);
+    C.core_hi = C.core_lo + g->core_cap;
+    C.core_hiout = C.core_hi + g->core_cap;
     C.t_rank = g->t_rank;
     C.stats = g->stats;
     C.src_lo = g->src_lo;
@@ -540,8 +543,9 @@ void join_plan(tc_graph* g) {
 tc_status run_plan(tc_graph* g) {
     if (g->planned) return TC_OK;
     join_plan(g);  // a previous plan's hub part writes the buffers this one rewrites
-    const size_t off = offsetof(DevStats, small_count);
-    TC_CK(cudaMemsetAsync(reinterpret_cast<char*>(g->stats) + off, 0, sizeof(DevStats) - off, g->stream));
+    const size_t off = offsetof(DevStats, small_count), end = offsetof(DevStats, cta_next);
+    if (!g->plan_zeroed) TC_CK(cudaMemsetAsync(reinterpret_cast<char*>(g->stats) + off, 0, end - off, g->stream));
+    g->plan_zeroed = false;
     if (!g->capture) TC_CK(cudaEventRecord(g->sync.ev[PH_PLAN], g->stream));
     // single graphs build their hub lists on a second stream while the push buckets
     // are counted; batches (which may be recorded into a CUDA graph) keep one stream
@@ -553,6 +557,17 @@ tc_status run_plan(tc_graph* g) {
     return TC_OK;
 }
 
+// t and the count's part of the statistics start at zero, which they are after the build.
+tc_status zero_counts(tc_graph* g) {
+    if (!g->count_zeroed) {
+        const size_t off = offsetof(DevStats, cta_next);
+        TC_CK(cudaMemsetAsync(g->t_rank, 0, sizeof(unsigned long long) * (size_t)g->n, g->stream));
+        TC_CK(cudaMemsetAsync(reinterpret_cast<char*>(g->stats) + off, 0, sizeof(DevStats) - off, g->stream));
+    }
+    g->count_zeroed = false;
+    return TC_OK;
+}
+
 tc_status run_count(tc_graph* g) {
     if (g->counted) return TC_OK;
     tc_status st;
@@ -561,8 +576,7 @@ tc_status run_count(tc_graph* g) {
     } else if ((st = run_plan(g)) != TC_OK) {
         return st;
     }
-    TC_CK(cudaMemsetAsync(g->t_rank, 0, sizeof(unsigned long long) * (size_t)g->n, g->stream));
-    TC_CK(cudaMemsetAsync(&g->stats->sum_t, 0, sizeof(unsigned long long), g->stream));
+    if ((st = zero_counts(g)) != TC_OK) return st;
     CountBuffers C = count_buffers(g);
     launch_intersect(C, g->strat, g->capture ? nullptr : g->sync.ev, g->L);
     launch_sum_t(C, g->L);
@@ -970,7 +984,7 @@ tc_status tc_edge_support(tc_graph* g, int32_t* u_out, int32_t* v_out, uint32_t*
     g->strat = S;
     g->counted = false;
     cudaError_t e = cudaMemsetAsync(sup, 0, sizeof(uint32_t) * (size_t)g->m_alloc, g->stream);
-    if (e == cudaSuccess && (st = run_plan(g)) == TC_OK) {
+    if (e == cudaSuccess && (st = run_plan(g)) == TC_OK && (st = zero_counts(g)) == TC_OK) {
         CountBuffers C = count_buffers(g);
         C.sup = sup;
         launch_intersect(C, g->strat, nullptr, g->L);  // leaves parts of t in t_rank: the next count starts it anew

@@ -47,13 +47,13 @@ __global__ void __launch_bounds__(CORE_THREADS) k_core_build(int32_t n, const in
             const int j = col[base + p] - c0;  // > i: the row lies above x
             atomicOr(&z[i * words + (j >> 5)], 1u << (j & 31));
             atomicOr(&z[(int64_t)j * words + (i >> 5)], 1u << (i & 31));
-            atomicMin(&lo[j], (int32_t)i);
-            atomicMax(&hi[j], (int32_t)i);
+            atomicMax(&lo[j], CORE_MAX - (int32_t)i);
+            atomicMax(&hi[j], (int32_t)i + 1);
             atomicAdd(&cnt[j], 1u);
         }
         if (d > 0 && lane == 0) {  // the row is sorted: its ends bound i's out-neighbours
-            atomicMin(&lo[i], col[base] - c0);
-            atomicMax(&hi[i], col[base + d - 1] - c0);
+            atomicMax(&lo[i], CORE_MAX - (col[base] - c0));
+            atomicMax(&hi[i], col[base + d - 1] - c0 + 1);
         }
         if (lane == 0) hiout[i] = d > 0 ? col[base + d - 1] - c0 : -1;
     }
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(CORE_THREADS) k_core_count(int32_t n, const in
         unsigned long long tx = 0;
         for (int p = w; p < d; p += CORE_WARPS) {
             const int j = col[base + p] - c0;
-            const int b0 = max(xlo, lo[j]), b1 = min(xhi, hi[j]);
+            const int b0 = max(xlo, CORE_MAX - lo[j]), b1 = min(xhi, hi[j] - 1);
             uint32_t s = 0;
             if (b0 <= b1 && first < words) s = and_popc(z + (int64_t)j * words, ox, first, b0 >> 5, b1 >> 5);
             tx += s;
@@ -163,10 +163,10 @@ __global__ void __launch_bounds__(CORE_THREADS) k_core_support(int32_t n, const 
             if (first + h < words) a = *reinterpret_cast<const uint4*>(z + i * words + first + h);
             zx[h] = a.x, zx[h + 1] = a.y, zx[h + 2] = a.z, zx[h + 3] = a.w;
         }
-        const int xlo = lo[i], xhi = hi[i];
+        const int xlo = CORE_MAX - lo[i], xhi = hi[i] - 1;
         for (int p = w; p < d; p += CORE_WARPS) {
             const int j = col[base + p] - c0;
-            const int b0 = max(xlo, lo[j]), b1 = min(xhi, hi[j]);
+            const int b0 = max(xlo, CORE_MAX - lo[j]), b1 = min(xhi, hi[j] - 1);
             uint32_t s = 0;
             if (b0 <= b1 && first < words) s = and_popc(z + (int64_t)j * words, zx, first, b0 >> 5, b1 >> 5);
             s = __reduce_add_sync(FULL, s);
@@ -185,10 +185,7 @@ int core_words_for(int32_t core_cap) {
 void launch_core_plan(const CountBuffers& C, const Launch& L) {
     if (C.core_cap <= 0) return;
     const size_t rows = (size_t)C.core_cap * (size_t)C.core_words;
-    // z and cnt are one zeroed block; lo starts above and hi below every core index
-    cudaMemsetAsync(C.core_z, 0, sizeof(uint32_t) * (rows + (size_t)C.core_cap), L.stream);
-    cudaMemsetAsync(C.core_lo, 0x7f, sizeof(int32_t) * (size_t)C.core_cap, L.stream);
-    cudaMemsetAsync(C.core_hi, 0xff, sizeof(int32_t) * (size_t)C.core_cap, L.stream);
+    cudaMemsetAsync(C.core_z, 0, sizeof(uint32_t) * (rows + 3 * (size_t)C.core_cap), L.stream);  // z, cnt, lo, hi
     k_core_build<<<grid_for((int64_t)C.core_cap * 32, CORE_THREADS, L.sms), CORE_THREADS, 0, L.stream>>>(
         C.n, C.rowstart, C.rowlen, C.col, C.core_words, C.core_z, C.core_lo, C.core_hi, C.core_hiout, C.core_cnt,
         C.stats);

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include "../../include/tc.h"
@@ -19,30 +20,34 @@ enum : int {
 struct DevStats {
     unsigned long long loops;      // self-loops dropped
     unsigned long long m_simple;   // distinct undirected edges
-    unsigned long long sum_t;      // sum over v of t(v)
     unsigned int max_deg;          // largest multigraph degree
     int err;                       // ERR_* flags
     unsigned int long_count;       // build: rows sorted by whole blocks
-    unsigned int small_count[4];   // planner: vertices per small-list class (d+ <= 8, 16, 32, 256)
-    unsigned int cta_count;        // planner: vertices with d+ > 32
-    unsigned int cta_next;         // dynamic work counter of the block push kernel
-    unsigned int hub_count;        // vertices staged as hubs (ranks n - hub_count .. n-1)
-    unsigned int hub_next;         // dynamic work counter of the hub kernel (slices of big hubs)
-    unsigned int hub_next2;        // dynamic work counter of the hub kernel (medium hubs)
-    unsigned int hub_next3;        // dynamic work counter of the list kernel (long lists; probe mode)
-    unsigned int hub_next4;        // dynamic work counter of the below-window kernel
-    unsigned int hub_candidates;   // vertices whose degree reaches the hub threshold
-    unsigned int hub_big;          // hubs processed by whole blocks
     unsigned int mid_count;        // build: rows of 17..256 entries sorted by one warp
     unsigned int mid2_count;       // build: rows of 257..1024 entries sorted by one warp
+    unsigned int pad;
+    // from here on, zero when a plan starts
+    unsigned int small_count[4];   // planner: vertices per small-list class (d+ <= 8, 16, 32, 256)
+    unsigned int cta_count;        // planner: vertices with d+ > 32
+    unsigned int hub_count;        // vertices staged as hubs (ranks n - hub_count .. n-1)
+    unsigned int hub_candidates;   // vertices whose degree reaches the hub threshold
+    unsigned int hub_blocks;       // planner: blocks that have counted their candidates
+    unsigned int hub_big;          // hubs processed by whole blocks
     unsigned int core_n;           // planner: dense core size (ranks n - core_n .. n-1)
     unsigned int hub_tasks;        // window tasks of big hubs (slices of their in-edges)
     unsigned int hub_med;          // window tasks of the other hubs
     unsigned int hub_low;          // below-window tasks
     unsigned int hub_long;         // big hubs with a long list below the window
     unsigned int win_vecs;         // planner: 16-byte vectors of window entries written
+    // from here on, zero when a count starts
+    unsigned int cta_next;         // dynamic work counter of the block push kernel
+    unsigned int hub_next;         // dynamic work counter of the hub kernel (slices of big hubs)
+    unsigned int hub_next2;        // dynamic work counter of the hub kernel (medium hubs)
+    unsigned int hub_next3;        // dynamic work counter of the list kernel (long lists; probe mode)
+    unsigned int hub_next4;        // dynamic work counter of the below-window kernel
+    unsigned long long sum_t;      // sum over v of t(v)
 };
-static_assert(sizeof(DevStats) == 120, "DevStats layout");
+static_assert(sizeof(DevStats) == 128 && offsetof(DevStats, cta_next) % 4 == 0, "DevStats layout");
 
 struct Launch {
     cudaStream_t stream;
@@ -80,9 +85,11 @@ struct PlanStreams {
 
 // ---- primitives (tc_prims.cu) ------------------------------------------------
 // Exclusive scan of `count` uint32 values into int64 (out has count + 1 entries;
-// out[count] = total).  `tmp` needs scan_tmp_bytes(count) bytes.
+// out[count] = total; out2, if not null, receives the `count` values once more).  `tmp`
+// needs scan_tmp_bytes(count) bytes.
 size_t scan_tmp_bytes(int64_t count);
-void scan_u32_to_i64(const uint32_t* in, int64_t* out, int64_t count, void* tmp, const Launch& L);
+void scan_u32_to_i64(const uint32_t* in, int64_t* out, int64_t count, void* tmp, const Launch& L,
+                     int64_t* out2 = nullptr);
 // Exclusive scan of uint32 in place-capable (out may equal in); out[count] = total.
 void scan_u32_to_u32(const uint32_t* in, uint32_t* out, int64_t count, void* tmp, const Launch& L);
 
@@ -218,10 +225,10 @@ struct CountBuffers {
     // dense core (tc_core.cu): bit rows of core_words words for core indices 0 .. core_cap-1
     int32_t core_cap;        // min(hub_cap, CORE_MAX)
     int32_t core_words;      // core_words_for(core_cap)
-    uint32_t* core_z;        // core_cap * core_words: symmetric adjacency rows; followed by core_cnt
+    uint32_t* core_z;        // core_cap * core_words: symmetric adjacency rows; followed by the next three
     uint32_t* core_cnt;      // core_cap: in-degree from the core
-    int32_t* core_lo;        // core_cap: lowest core neighbour
-    int32_t* core_hi;        // core_cap: highest core neighbour (-1: none)
+    int32_t* core_lo;        // core_cap: CORE_MAX less the lowest core neighbour (0: none)
+    int32_t* core_hi;        // core_cap: one more than the highest core neighbour (0: none)
     int32_t* core_hiout;     // core_cap: highest core out-neighbour (-1: none)
     unsigned long long* t_rank;  // n
     DevStats* stats;

@@ -347,21 +347,29 @@ __device__ uint32_t lane_search_rev(const int32_t* Lu, int a0, int du, const int
 
 // ---- planner -----------------------------------------------------------------
 
-__global__ void k_hub_candidates(int32_t n, const int32_t* __restrict__ deg, int min_degree, DevStats* stats) {
+// Hub candidates; the block that counts last sets the hub count and the core's size.
+__global__ void k_hub_count(int32_t n, const int32_t* __restrict__ deg, int min_degree, int32_t hub_cap, int hub_max,
+                            int core_max, DevStats* stats) {
+    __shared__ unsigned sum;
+    if (threadIdx.x == 0) sum = 0;
+    __syncthreads();
     unsigned c = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += stride)
         c += deg[r] >= min_degree ? 1u : 0u;
-    c = warp_sum(c);
-    if (lane_id() == 0 && c) atomicAdd(&stats->hub_candidates, c);
-}
-
-__global__ void k_hub_count(int32_t hub_cap, int hub_max, int core_max, DevStats* stats) {
-    unsigned k = stats->hub_candidates;
-    k = min(k, (unsigned)hub_max);
-    k = min(k, (unsigned)hub_cap);
-    stats->hub_count = k;
-    stats->core_n = min(k, (unsigned)core_max);
+    c = __reduce_add_sync(FULL, c);
+    if (lane_id() == 0 && c) atomicAdd(&sum, c);
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    if (sum) atomicAdd(&stats->hub_candidates, sum);
+    __threadfence();
+    if (atomicAdd(&stats->hub_blocks, 1u) == gridDim.x - 1) {
+        unsigned k = atomicAdd(&stats->hub_candidates, 0u);
+        k = min(k, (unsigned)hub_max);
+        k = min(k, (unsigned)hub_cap);
+        stats->hub_count = k;
+        stats->core_n = min(k, (unsigned)core_max);
+    }
 }
 
 // In-degree d-(v) = deg(v) - d+(v) of every hub slot (0 for slots below the hubs),
@@ -629,15 +637,6 @@ __global__ void __launch_bounds__(SCAT_THREADS) k_hub_scatter(int32_t n, int32_t
     }
 }
 
-// After the scatter every hub's cursor must stand at the start of the next segment:
-// a count and a scatter that disagree are reported instead of trusted.
-__global__ void k_hub_cur_check(int32_t hub_cap, const int64_t* __restrict__ hub_start,
-                                const unsigned long long* __restrict__ cur, DevStats* stats) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < hub_cap; i += stride)
-        if (cur[i] != (unsigned long long)hub_start[i + 1]) atomicOr(&stats->err, ERR_OVERFLOW);
-}
-
 // The same records when hub entries are a small share of the entries (flat degree
 // distributions): a warp takes 32 consecutive rows (one per lane) and walks their
 // hub tails from the end backwards in lockstep, so rows without a hub cost one
@@ -719,7 +718,7 @@ __global__ void k_hub_lists(int32_t n, int32_t hub_cap, int32_t T0w, const int2*
                             const uint32_t* __restrict__ indeg, const int64_t* __restrict__ hub_start, int big_in,
                             int32_t* __restrict__ big_list, int32_t* __restrict__ long_list,
                             int4* __restrict__ win_task, int4* __restrict__ low_task, int64_t task_cap,
-                            DevStats* stats) {
+                            const unsigned long long* __restrict__ cur, DevStats* stats) {
     const int64_t K = stats->hub_count;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int lane = lane_id();
@@ -733,10 +732,14 @@ __global__ void k_hub_lists(int32_t n, int32_t hub_cap, int32_t T0w, const int2*
         int2 ri = make_int2(0, 0);
         int64_t e0 = 0;
         if (i < K) {
-            din = indeg[v - (n - hub_cap)];
+            const int32_t h = v - (n - hub_cap);
+            din = indeg[h];
             ri = rowinfo[v];
+            e0 = hub_start[h];
+            // the scatter must have filled the hub's segment: a count and a scatter that
+            // disagree are reported instead of trusted
+            if (cur[h] != (unsigned long long)e0 + din) atomicOr(&stats->err, ERR_OVERFLOW);
             if (din > 0 && ri.y > 0) {
-                e0 = hub_start[v - (n - hub_cap)];
                 big = din >= (uint32_t)big_in || ri.y > HUB_WARP_MAX;
                 dwin = v >= T0w ? ri.y : (col[ri.x + ri.y - 1] >= T0w ? (int)winrow[v].y : 0);
                 dlow = ri.y - dwin;
@@ -2327,14 +2330,12 @@ bool launch_plan(const CountBuffers& C, const Strategy& S, const Launch& L, cons
     if (C.n <= 0) return false;
     const int hub_max = S.hub_max < 0 ? 0 : S.hub_max;
     const bool hubs = C.hub_cap > 0 && hub_max > 0;
-    if (hubs) {
-        k_hub_candidates<<<grid_for(C.n, THREADS, L.sms), THREADS, 0, L.stream>>>(C.n, C.deg, S.hub_min_degree,
-                                                                                 C.stats);
+    const int core_max = hubs && C.core_cap > 0 && S.hub_core > 0 ? (S.hub_core < C.core_cap ? S.hub_core : C.core_cap) : 0;
+    if (hubs) {  // else the hub count stays zero
+        k_hub_count<<<grid_for(C.n, THREADS, L.sms), THREADS, 0, L.stream>>>(C.n, C.deg, S.hub_min_degree, C.hub_cap,
+                                                                            hub_max, core_max, C.stats);
         count_launch();
     }
-    const int core_max = hubs && C.core_cap > 0 && S.hub_core > 0 ? (S.hub_core < C.core_cap ? S.hub_core : C.core_cap) : 0;
-    k_hub_count<<<1, 1, 0, L.stream>>>(C.hub_cap, hub_max, core_max, C.stats);
-    count_launch();
     // the hub lists and the dense core need only the hub count: with a second stream
     // they are built while the main stream lists and counts the push buckets
     const bool forked = hubs && ps != nullptr;
@@ -2353,10 +2354,8 @@ bool launch_plan(const CountBuffers& C, const Strategy& S, const Launch& L, cons
         k_hub_indeg<<<grid_for(C.hub_cap, THREADS, H.sms), THREADS, 0, H.stream>>>(C.n, C.hub_cap, C.deg, C.rowlen,
                                                                                   C.core_cnt, C.hub_cnt, C.stats);
         count_launch();
-        scan_u32_to_i64(C.hub_cnt, C.hub_start, C.hub_cap, C.tmp, H);
-        // 64-bit cursors starting at every hub's first slot
-        cudaMemcpyAsync(C.hub_cur64, C.hub_start, sizeof(int64_t) * (size_t)C.hub_cap, cudaMemcpyDeviceToDevice,
-                        H.stream);
+        // and 64-bit cursors starting at every hub's first slot
+        scan_u32_to_i64(C.hub_cnt, C.hub_start, C.hub_cap, C.tmp, H, reinterpret_cast<int64_t*>(C.hub_cur64));
         k_row_of<<<grid_for((int64_t)C.n, THREADS, H.sms), THREADS, 0, H.stream>>>(C.n, C.hub_cap, C.rowstart,
                                                                                   C.hub_start, C.rowof, C.stats);
         count_launch();
@@ -2368,13 +2367,10 @@ bool launch_plan(const CountBuffers& C, const Strategy& S, const Launch& L, cons
             C.n, C.hub_cap, C.rowstart, C.rowinfo, C.col, C.rowof, C.hub_start, C.hub_cur64, C.in_rec, C.src_lo,
             C.src_hi, C.stats);
         count_launch();
-        k_hub_cur_check<<<grid_for(C.hub_cap, THREADS, H.sms), THREADS, 0, H.stream>>>(C.hub_cap, C.hub_start,
-                                                                                      C.hub_cur64, C.stats);
-        count_launch();
         k_hub_lists<<<grid_for(C.hub_cap, THREADS, H.sms), THREADS, 0, H.stream>>>(
             C.n, C.hub_cap, T.first[1], C.rowinfo, C.col, C.winrow, C.hub_cnt, C.hub_start,
             S.hub_big_in > 0 ? S.hub_big_in : 1, C.big_list, C.long_list, C.win_task, C.low_task,
-            hub_task_cap(C.hub_cap, C.m_cap), C.stats);
+            hub_task_cap(C.hub_cap, C.m_cap), C.hub_cur64, C.stats);
         count_launch();
     }
     if (forked) cudaEventRecord(ps->join, H.stream);
@@ -2445,7 +2441,6 @@ void intersect_impl(const CountBuffers& C, const Strategy& S, cudaEvent_t* ev, c
         count_launch();
     }
     if (ev) cudaEventRecord(ev[PH_CTA], L.stream);
-    cudaMemsetAsync(&C.stats->cta_next, 0, sizeof(unsigned), L.stream);
     k_tc_cta<SUP><<<L.sms * 4, CTA_THREADS, sizeof(CtaShared), L.stream>>>(C.n, C.rowstart, C.rowlen, C.rowinfo, C.col,
                                                                      C.cta_list,
                                                                      C.t_rank, C.stats, S.strat[TC_BUCKET_CTA],
@@ -2456,7 +2451,6 @@ void intersect_impl(const CountBuffers& C, const Strategy& S, cudaEvent_t* ev, c
     if (ev) cudaEventRecord(ev[PH_HUB], L.stream);
     if (C.hub_cap > 0) {
         if (S.hub_core > 0) launch_core_count(C, L);
-        cudaMemsetAsync(&C.stats->hub_next, 0, 4 * sizeof(unsigned), L.stream);
         const bool probe = S.strat[TC_BUCKET_HUB] == TC_STRAT_PROBE;
         const Windows T(C.n);
         const int64_t task_cap = hub_task_cap(C.hub_cap, C.m_cap);

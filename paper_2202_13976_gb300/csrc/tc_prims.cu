@@ -52,10 +52,10 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_tile_reduce(const In* __restri
     }
 }
 
-// One block: exclusive scan of partials[0..num) in place; partials[num] = total.
+// One block: exclusive scan of partials[0..num) in place.
 template <typename Acc>
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_partials(Acc* partials, int64_t num) {
-    __shared__ Acc carry_sh;
+    __shared__ Acc tot;
     Acc carry = 0;
     for (int64_t base = 0; base < num; base += SCAN_TILE) {
         Acc v[SCAN_ITEMS];
@@ -66,10 +66,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_partials(Acc* partials, i
             v[k] = i < num ? partials[i] : Acc(0);
             s += v[k];
         }
-        Acc tot;
-        Acc ex = block_exclusive_scan(s, &carry_sh);
-        tot = carry_sh;
-        Acc run = carry + ex;
+        Acc run = carry + block_exclusive_scan(s, &tot);
 #pragma unroll
         for (int k = 0; k < SCAN_ITEMS; ++k) {
             int64_t i = base + (int64_t)threadIdx.x * SCAN_ITEMS + k;
@@ -77,15 +74,27 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_partials(Acc* partials, i
             run += v[k];
         }
         carry += tot;
-        __syncthreads();
+        __syncthreads();  // tot is written again by the next tile
     }
-    if (threadIdx.x == 0) partials[num] = carry;
 }
 
-template <typename In, typename Out, typename Acc>
-__global__ void __launch_bounds__(SCAN_THREADS) k_tile_scan(const In* in, Out* out, int64_t count,
-                                                            const Acc* __restrict__ partials,
-                                                            int64_t num_tiles) {
+// Tile `blockIdx.x` of an exclusive scan, written to out and, if not null, to out2.  With
+// up to SCAN_SELF_MAX tiles (SCANNED false) each block sums the partials of the tiles
+// before its own itself, one launch less than scanning them first.  The last block
+// writes the total behind the last value.
+constexpr int64_t SCAN_SELF_MAX = 1024;  // at most 8 KB of cached loads a block
+
+template <bool SCANNED, typename In, typename Out, typename Acc>
+__global__ void __launch_bounds__(SCAN_THREADS) k_tile_scan(const In* in, Out* out, Out* out2, int64_t count,
+                                                            const Acc* __restrict__ partials) {
+    __shared__ Acc tot;
+    Acc before = SCANNED ? partials[blockIdx.x] : Acc(0);
+    if (!SCANNED) {
+        for (int64_t k = threadIdx.x; k < blockIdx.x; k += SCAN_THREADS) before += partials[k];
+        block_exclusive_scan(before, &tot);
+        before = tot;
+        __syncthreads();
+    }
     const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
     Acc v[SCAN_ITEMS];
     Acc s = 0;
@@ -95,25 +104,68 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_tile_scan(const In* in, Out* o
         v[k] = i < count ? (Acc)in[i] : Acc(0);
         s += v[k];
     }
-    __shared__ Acc tot;
-    Acc run = partials[blockIdx.x] + block_exclusive_scan(s, &tot);
+    Acc run = before + block_exclusive_scan(s, &tot);
 #pragma unroll
     for (int k = 0; k < SCAN_ITEMS; ++k) {
         int64_t i = base + (int64_t)threadIdx.x * SCAN_ITEMS + k;
-        if (i < count) out[i] = (Out)run;
+        if (i < count) {
+            out[i] = (Out)run;
+            if (out2) out2[i] = (Out)run;
+        }
         run += v[k];
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) out[count] = (Out)partials[num_tiles];
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[count] = (Out)(before + tot);
 }
 
+// A short scan in one launch by one block, a tile after the other.
 template <typename In, typename Out, typename Acc>
-void scan_impl(const In* in, Out* out, int64_t count, void* tmp, const Launch& L) {
-    int64_t tiles = (count + SCAN_TILE - 1) / SCAN_TILE;
-    if (tiles < 1) tiles = 1;
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_one(const In* in, Out* out, Out* out2, int64_t count) {
+    __shared__ Acc tot;
+    Acc carry = 0;
+    for (int64_t base = 0; base < count; base += SCAN_TILE) {
+        Acc v[SCAN_ITEMS];
+        Acc s = 0;
+#pragma unroll
+        for (int k = 0; k < SCAN_ITEMS; ++k) {
+            int64_t i = base + (int64_t)threadIdx.x * SCAN_ITEMS + k;
+            v[k] = i < count ? (Acc)in[i] : Acc(0);
+            s += v[k];
+        }
+        Acc run = carry + block_exclusive_scan(s, &tot);
+#pragma unroll
+        for (int k = 0; k < SCAN_ITEMS; ++k) {
+            int64_t i = base + (int64_t)threadIdx.x * SCAN_ITEMS + k;
+            if (i < count) {
+                out[i] = (Out)run;
+                if (out2) out2[i] = (Out)run;
+            }
+            run += v[k];
+        }
+        carry += tot;
+        __syncthreads();  // tot is written again by the next tile
+    }
+    if (threadIdx.x == 0) out[count] = (Out)carry;
+}
+// One block passes over a tile in about 1 us, the two kernels cost about 5 us of launch
+// and GPU time together.
+constexpr int64_t SCAN_ONE_MAX = 4 * SCAN_TILE;
+
+template <typename In, typename Out, typename Acc>
+void scan_impl(const In* in, Out* out, Out* out2, int64_t count, void* tmp, const Launch& L) {
+    if (count <= SCAN_ONE_MAX) {
+        k_scan_one<In, Out, Acc><<<1, SCAN_THREADS, 0, L.stream>>>(in, out, out2, count); count_launch();
+        return;
+    }
+    const int64_t tiles = (count + SCAN_TILE - 1) / SCAN_TILE;
     Acc* partials = static_cast<Acc*>(tmp);
     k_tile_reduce<In, Acc><<<(unsigned)tiles, SCAN_THREADS, 0, L.stream>>>(in, count, partials); count_launch();
-    k_scan_partials<Acc><<<1, SCAN_THREADS, 0, L.stream>>>(partials, tiles); count_launch();
-    k_tile_scan<In, Out, Acc><<<(unsigned)tiles, SCAN_THREADS, 0, L.stream>>>(in, out, count, partials, tiles); count_launch();
+    if (tiles <= SCAN_SELF_MAX) {
+        k_tile_scan<false, In, Out, Acc><<<(unsigned)tiles, SCAN_THREADS, 0, L.stream>>>(in, out, out2, count, partials);
+    } else {
+        k_scan_partials<Acc><<<1, SCAN_THREADS, 0, L.stream>>>(partials, tiles); count_launch();
+        k_tile_scan<true, In, Out, Acc><<<(unsigned)tiles, SCAN_THREADS, 0, L.stream>>>(in, out, out2, count, partials);
+    }
+    count_launch();
 }
 
 // ---- radix sort --------------------------------------------------------------
@@ -207,12 +259,12 @@ size_t scan_tmp_bytes(int64_t count) {
     return (size_t)tiles * 8 + 256;
 }
 
-void scan_u32_to_i64(const uint32_t* in, int64_t* out, int64_t count, void* tmp, const Launch& L) {
-    scan_impl<uint32_t, int64_t, long long>(in, out, count, tmp, L);
+void scan_u32_to_i64(const uint32_t* in, int64_t* out, int64_t count, void* tmp, const Launch& L, int64_t* out2) {
+    scan_impl<uint32_t, int64_t, long long>(in, out, out2, count, tmp, L);
 }
 
 void scan_u32_to_u32(const uint32_t* in, uint32_t* out, int64_t count, void* tmp, const Launch& L) {
-    scan_impl<uint32_t, uint32_t, unsigned long long>(in, out, count, tmp, L);
+    scan_impl<uint32_t, uint32_t, unsigned long long>(in, out, (uint32_t*)nullptr, count, tmp, L);
 }
 
 size_t radix_tmp_bytes(int64_t count) {
