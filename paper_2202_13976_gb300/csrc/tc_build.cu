@@ -68,6 +68,7 @@ __global__ void k_expand_csr(const int64_t* __restrict__ offsets, int32_t n, int
 constexpr int PAIR_UNROLL = 8;  // pairs per thread and round in the pair passes
 constexpr int DEG_SLOTS = 4096;
 constexpr int DEG_PROBES = 4;
+constexpr int32_t INGEST_MAX_N = 32768;  // the last block reads this many degrees in about the time of a launch
 
 __device__ __forceinline__ void deg_add(int32_t x, int32_t* hk, uint32_t* hc, uint32_t* __restrict__ dmulti) {
     unsigned h = ((unsigned)x * 0x9e3779b1u) >> (32 - 12);
@@ -84,6 +85,7 @@ __device__ __forceinline__ void deg_add(int32_t x, int32_t* hk, uint32_t* hc, ui
     atomicAdd(&dmulti[x], 1u);
 }
 
+template <bool TAKE_MAX>
 __global__ void __launch_bounds__(THREADS) k_canon_degree(const int32_t* __restrict__ src,
                                                           const int32_t* __restrict__ dst, int64_t m, int32_t n,
                                                           uint32_t* __restrict__ dmulti, DevStats* stats) {
@@ -127,6 +129,19 @@ __global__ void __launch_bounds__(THREADS) k_canon_degree(const int32_t* __restr
     if (lane_id() == 0) {
         if (loops) atomicAdd(&stats->loops, loops);
         if (err) atomicOr(&stats->err, err);
+    }
+    if constexpr (TAKE_MAX) {
+        // the block that finishes last takes the maximum degree (small graphs: saves a launch)
+        __shared__ bool last;
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(&stats->ingest_blocks, 1u) == gridDim.x - 1;
+        __syncthreads();
+        if (!last) return;
+        uint32_t mx = 0;
+        for (int i = threadIdx.x; i < n; i += THREADS) mx = max(mx, __ldcg(&dmulti[i]));
+        mx = __reduce_max_sync(FULL, mx);
+        if (lane_id() == 0 && mx) atomicMax(&stats->max_deg, mx);
     }
 }
 
@@ -839,12 +854,17 @@ void launch_expand_csr(const int64_t* offsets, int32_t n, int32_t* rows, DevStat
     k_expand_csr<<<grid_for((int64_t)n * 32, THREADS, L.sms), THREADS, 0, L.stream>>>(offsets, n, rows, stats); count_launch();
 }
 
-void launch_canon_degree_part(const BuildBuffers& B, int64_t first, int64_t count, const Launch& L) {
+static void launch_ingest(const BuildBuffers& B, int64_t first, int64_t count, bool take_max, const Launch& L) {
     if (count <= 0) return;
     // 32 KB of shared memory per block: four blocks per SM stay resident
-    k_canon_degree<<<grid_for(count, THREADS, L.sms, 4), THREADS, 0, L.stream>>>(B.src + first, B.dst + first, count,
-                                                                               B.n, B.dmulti, B.stats);
+    const auto kernel = take_max ? k_canon_degree<true> : k_canon_degree<false>;
+    kernel<<<grid_for(count, THREADS, L.sms, 4), THREADS, 0, L.stream>>>(B.src + first, B.dst + first, count, B.n,
+                                                                       B.dmulti, B.stats);
     count_launch();
+}
+
+void launch_canon_degree_part(const BuildBuffers& B, int64_t first, int64_t count, const Launch& L) {
+    launch_ingest(B, first, count, false, L);
 }
 
 void launch_max_deg(const BuildBuffers& B, const Launch& L) {
@@ -852,8 +872,9 @@ void launch_max_deg(const BuildBuffers& B, const Launch& L) {
 }
 
 void launch_canon_degree(const BuildBuffers& B, const Launch& L) {
-    launch_canon_degree_part(B, 0, B.m, L);
-    launch_max_deg(B, L);
+    const bool small = B.n <= INGEST_MAX_N && B.m > 0;
+    launch_ingest(B, 0, B.m, small, L);
+    if (!small) launch_max_deg(B, L);
 }
 
 // Batches: the graph of every vertex (one warp per graph), then keys
@@ -976,25 +997,32 @@ void launch_orient(const BuildBuffers& B, const Launch& L, cudaEvent_t* ev, cons
         B.n, B.rowstart, B.rowcnt, B.col, B.rowlen, B.rowinfo, dupin, B.midlist, B.midlist2, B.longlist, B.stats);
     count_launch();
     // the three sorters take disjoint rows: with a second stream the long rows are
-    // sorted there while the main stream sorts the rows of 17..256
+    // sorted there while the main stream sorts the rows of 17..256.  No row is longer
+    // than the largest degree, if it is known: sorters without rows are left out.
+    const bool longer256 = B.row_bound > 256, longer1024 = B.row_bound > WARP_SORT_MAX;
     Launch S = L;
+    if (!longer256) ps = nullptr;
     if (ps) {
         cudaEventRecord(ps->fork, L.stream);
         cudaStreamWaitEvent(ps->side, ps->fork, 0);
         S.stream = ps->side;
     }
-    k_segsort_warp<WARP_SORT_MAX / 32><<<S.sms * 2, SEG_WARPS * 32, 0, S.stream>>>(B.rowstart, B.rowcnt, B.col,
-                                                                                  B.rowlen, B.rowinfo, dupin,
-                                                                                  B.midlist2, &B.stats->mid2_count,
-                                                                                  B.stats);
-    count_launch();
-    k_segsort_block<<<S.sms * 2, 1024, CTA_SORT_MAX * sizeof(int32_t), S.stream>>>(
-        B.rowstart, B.rowcnt, B.col, B.rowlen, B.rowinfo, dupin, B.longlist, B.stats);
-    count_launch();
+    if (longer256) {
+        k_segsort_warp<WARP_SORT_MAX / 32><<<S.sms * 2, SEG_WARPS * 32, 0, S.stream>>>(
+            B.rowstart, B.rowcnt, B.col, B.rowlen, B.rowinfo, dupin, B.midlist2, &B.stats->mid2_count, B.stats);
+        count_launch();
+    }
+    if (longer1024) {
+        k_segsort_block<<<S.sms * 2, 1024, CTA_SORT_MAX * sizeof(int32_t), S.stream>>>(
+            B.rowstart, B.rowcnt, B.col, B.rowlen, B.rowinfo, dupin, B.longlist, B.stats);
+        count_launch();
+    }
     if (ps) cudaEventRecord(ps->join, S.stream);
-    k_segsort_warp<8><<<L.sms * 4, SEG_WARPS * 32, 0, L.stream>>>(B.rowstart, B.rowcnt, B.col, B.rowlen, B.rowinfo,
-                                                                 dupin, B.midlist, &B.stats->mid_count, B.stats);
-    count_launch();
+    if (B.row_bound > 16) {
+        k_segsort_warp<8><<<L.sms * 4, SEG_WARPS * 32, 0, L.stream>>>(B.rowstart, B.rowcnt, B.col, B.rowlen, B.rowinfo,
+                                                                     dupin, B.midlist, &B.stats->mid_count, B.stats);
+        count_launch();
+    }
     if (ps) cudaStreamWaitEvent(L.stream, ps->join, 0);
     if (ev) cudaEventRecord(ev[BP_SORT], L.stream);
     k_degree<<<grid_for(B.n, THREADS, L.sms), THREADS, 0, L.stream>>>(B.n, B.rowlen, B.dmulti, B.rowcnt, B.dupin,

@@ -25,7 +25,7 @@ struct DevStats {
     unsigned int long_count;       // build: rows sorted by whole blocks
     unsigned int mid_count;        // build: rows of 17..256 entries sorted by one warp
     unsigned int mid2_count;       // build: rows of 257..1024 entries sorted by one warp
-    unsigned int pad;
+    unsigned int ingest_blocks;    // build: blocks that have counted their pairs
     // from here on, zero when a plan starts
     unsigned int small_count[4];   // planner: vertices per small-list class (d+ <= 8, 16, 32, 256)
     unsigned int cta_count;        // planner: vertices with d+ > 32
@@ -122,6 +122,7 @@ struct BuildBuffers {
     int64_t* bstart;      // BUCKET_MAX + 1: first pair of each bucket
     int2* pairs;          // m: (source rank, target rank) grouped by bucket
     int2* oriented;       // m: (source rank, target rank) in input order ((-1, -1): no entry)
+    int64_t row_bound;    // no row has more entries, repeats included
     bool bucket_fill;     // rows counted and filled by source buckets (flat degree distributions)
     // directed input (tc_directed_lcc): every entry is (target rank << 2) | direction
     // bit of its pair (1: source rank below target rank, 2: above), so a pair read in
@@ -232,6 +233,7 @@ struct CountBuffers {
     int32_t* core_hiout;     // core_cap: highest core out-neighbour (-1: none)
     unsigned long long* t_rank;  // n
     DevStats* stats;
+    int64_t dplus_bound;     // no N+(u) has more entries
     uint32_t* sup;           // null, or m_cap per-edge supports indexed like col (tc_edge_support)
     int32_t src_lo, src_hi;  // only triangles whose lowest vertex has a rank in [src_lo, src_hi) are counted
     cudaEvent_t hub_ready;   // null, or recorded once the hub lists and the dense core are built (PlanStreams)

@@ -2410,42 +2410,56 @@ void intersect_impl(const CountBuffers& C, const Strategy& S, cudaEvent_t* ev, c
     if (ev) cudaEventRecord(ev[PH_SMALL], L.stream);
     const int ss = S.strat[TC_BUCKET_SMALL];
     const float sf = S.factor[TC_BUCKET_SMALL];
+    const int64_t top = C.dplus_bound;  // classes of longer sources are empty: left out
     if (ss == TC_STRAT_HASH) {
         // sources of at most 16 entries: one edge per lane (Eq. 3 per edge), whose
         // short merges cost less than building and flushing a set per source
         k_tc_small<8, SUP><<<L.sms * SMALL_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
             C.n, C.rowstart, C.rowlen, C.rowinfo, C.col, C.small_list[0], 0, C.t_rank, C.stats, TC_STRAT_AUTO, sf, C.sup);
         count_launch();
-        k_tc_small<16, SUP><<<L.sms * SMALL_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
-            C.n, C.rowstart, C.rowlen, C.rowinfo, C.col, C.small_list[1], 1, C.t_rank, C.stats, TC_STRAT_AUTO, sf, C.sup);
-        count_launch();
-        k_tc_small_hash<32, 64, SUP><<<L.sms * SMALL_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
-            C.n, C.rowinfo, C.col, C.small_list[2], 2, C.t_rank, C.stats, C.sup);
-        count_launch();
-        k_tc_small_hash<32, 2 * SMALL_WIDE_MAX, SUP><<<L.sms * SMALL_WIDE_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
-            C.n, C.rowinfo, C.col, C.small_list[3], 3, C.t_rank, C.stats, C.sup);
-        count_launch();
+        if (top > 8) {
+            k_tc_small<16, SUP><<<L.sms * SMALL_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
+                C.n, C.rowstart, C.rowlen, C.rowinfo, C.col, C.small_list[1], 1, C.t_rank, C.stats, TC_STRAT_AUTO, sf, C.sup);
+            count_launch();
+        }
+        if (top > 16) {
+            k_tc_small_hash<32, 64, SUP><<<L.sms * SMALL_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
+                C.n, C.rowinfo, C.col, C.small_list[2], 2, C.t_rank, C.stats, C.sup);
+            count_launch();
+        }
+        if (top > 32) {
+            k_tc_small_hash<32, 2 * SMALL_WIDE_MAX, SUP><<<L.sms * SMALL_WIDE_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
+                C.n, C.rowinfo, C.col, C.small_list[3], 3, C.t_rank, C.stats, C.sup);
+            count_launch();
+        }
     } else {
         k_tc_small<8, SUP><<<L.sms * SMALL_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
             C.n, C.rowstart, C.rowlen, C.rowinfo, C.col, C.small_list[0], 0, C.t_rank, C.stats, ss, sf, C.sup);
         count_launch();
-        k_tc_small<16, SUP><<<L.sms * SMALL_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
-            C.n, C.rowstart, C.rowlen, C.rowinfo, C.col, C.small_list[1], 1, C.t_rank, C.stats, ss, sf, C.sup);
-        count_launch();
-        k_tc_small<32, SUP><<<L.sms * SMALL_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
-            C.n, C.rowstart, C.rowlen, C.rowinfo, C.col, C.small_list[2], 2, C.t_rank, C.stats, ss, sf, C.sup);
-        count_launch();
-        k_tc_small_wide<SUP><<<L.sms * SMALL_WIDE_BLOCKS, SMALL_WARPS * 32,
-                          2 * SMALL_WIDE_GROUPS * SMALL_WIDE_MAX * sizeof(int32_t), L.stream>>>(
-            C.n, C.rowinfo, C.col, C.small_list[3], C.t_rank, C.stats, ss, sf, C.sup);
-        count_launch();
+        if (top > 8) {
+            k_tc_small<16, SUP><<<L.sms * SMALL_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
+                C.n, C.rowstart, C.rowlen, C.rowinfo, C.col, C.small_list[1], 1, C.t_rank, C.stats, ss, sf, C.sup);
+            count_launch();
+        }
+        if (top > 16) {
+            k_tc_small<32, SUP><<<L.sms * SMALL_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
+                C.n, C.rowstart, C.rowlen, C.rowinfo, C.col, C.small_list[2], 2, C.t_rank, C.stats, ss, sf, C.sup);
+            count_launch();
+        }
+        if (top > 32) {
+            k_tc_small_wide<SUP><<<L.sms * SMALL_WIDE_BLOCKS, SMALL_WARPS * 32,
+                              2 * SMALL_WIDE_GROUPS * SMALL_WIDE_MAX * sizeof(int32_t), L.stream>>>(
+                C.n, C.rowinfo, C.col, C.small_list[3], C.t_rank, C.stats, ss, sf, C.sup);
+            count_launch();
+        }
     }
     if (ev) cudaEventRecord(ev[PH_CTA], L.stream);
-    k_tc_cta<SUP><<<L.sms * 4, CTA_THREADS, sizeof(CtaShared), L.stream>>>(C.n, C.rowstart, C.rowlen, C.rowinfo, C.col,
-                                                                     C.cta_list,
-                                                                     C.t_rank, C.stats, S.strat[TC_BUCKET_CTA],
-                                                                     S.factor[TC_BUCKET_CTA], C.sup);
-    count_launch();
+    if (top > SMALL_WIDE_MAX) {
+        k_tc_cta<SUP><<<L.sms * 4, CTA_THREADS, sizeof(CtaShared), L.stream>>>(
+            C.n, C.rowstart, C.rowlen, C.rowinfo, C.col, C.cta_list, C.t_rank, C.stats, S.strat[TC_BUCKET_CTA],
+            S.factor[TC_BUCKET_CTA], C.sup);
+        count_launch();
+    }
     // the hub lists and the dense core come from the planner's second stream
     if (C.hub_ready) cudaStreamWaitEvent(L.stream, C.hub_ready, 0);
     if (ev) cudaEventRecord(ev[PH_HUB], L.stream);
