@@ -15,46 +15,89 @@ namespace tcg {
 
 namespace {
 
-// One block per graph (grid-stride): union ids; a pair with a local id outside
-// [0, n_g) becomes a self-loop at vbase[g] (dropped later) and raises ERR_BAD_ID.
-__global__ void k_batch_relabel(int32_t G, const int64_t* __restrict__ edge_off, const int32_t* __restrict__ vbase,
-                                const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
-                                int32_t* __restrict__ usrc, int32_t* __restrict__ udst, int* __restrict__ err) {
-    for (int g = blockIdx.x; g < G; g += gridDim.x) {
-        const int64_t e0 = edge_off[g], e1 = edge_off[g + 1];
-        const int32_t b = vbase[g], ng = vbase[g + 1] - b;
-        int bad = 0;
-        for (int64_t k = e0 + threadIdx.x; k < e1; k += blockDim.x) {
-            int32_t u = src[k], v = dst[k];
+// Union ids; a pair with a local id outside [0, n_g) becomes a self-loop at vbase[g]
+// (dropped later) and raises ERR_BAD_ID.  A warp takes RELABEL_PAIRS consecutive pairs
+// whatever graphs they belong to: it finds the first one's graph by a binary search and
+// its lanes step on from there.  One block per graph left the few large graphs to a
+// block each: 2.0 ms for 66 M pairs in 840 graphs, now 0.21.
+constexpr int RELABEL_PAIRS = 256;
+
+__global__ void __launch_bounds__(256) k_batch_relabel(int32_t G, const int64_t* __restrict__ edge_off,
+                                                       const int32_t* __restrict__ vbase,
+                                                       const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
+                                                       int64_t m, int32_t* __restrict__ usrc, int32_t* __restrict__ udst,
+                                                       int* __restrict__ err) {
+    const int lane = lane_id();
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    int bad = 0;
+    for (int64_t p0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * RELABEL_PAIRS; p0 < m;
+         p0 += warps * RELABEL_PAIRS) {
+        int lo = 0, hi = G;  // the last graph whose pairs start at or before p0
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (edge_off[mid] <= p0)
+                lo = mid;
+            else
+                hi = mid;
+        }
+        int g = lo;
+        int64_t end = edge_off[g + 1];
+        int32_t b = vbase[g], ng = vbase[g + 1] - b;
+#pragma unroll
+        for (int k = 0; k < RELABEL_PAIRS / 32; ++k) {
+            const int64_t p = p0 + k * 32 + lane;
+            if (p >= m) break;
+            int32_t u = src[p], v = dst[p];
+            if (p >= end) {
+                do ++g;
+                while (p >= edge_off[g + 1]);  // ends: p < m = edge_off[G]
+                end = edge_off[g + 1];
+                b = vbase[g];
+                ng = vbase[g + 1] - b;
+            }
             if ((uint32_t)u >= (uint32_t)ng || (uint32_t)v >= (uint32_t)ng) {
                 bad = 1;
                 u = 0;
                 v = 0;
             }
-            usrc[k] = b + u;
-            udst[k] = b + v;
+            usrc[p] = b + u;
+            udst[p] = b + v;
         }
-        bad = __syncthreads_or(bad);
-        if (threadIdx.x == 0 && bad) atomicOr(err, ERR_BAD_ID);
     }
+    if (bad) atomicOr(err, ERR_BAD_ID);
 }
 
-// One block per graph (grid-stride): T_g = (sum of t over the graph's vertices) / 3.
-__global__ void k_batch_T(int32_t G, const int32_t* __restrict__ vbase, const int32_t* __restrict__ rank,
-                          const unsigned long long* __restrict__ t_rank, unsigned long long* __restrict__ T_out,
-                          int* __restrict__ err) {
-    __shared__ unsigned long long ws[32];
+// One block per graph (grid-stride): T_g = (sum of t over the graph's vertices) / 3.  Ranks
+// that run graph by graph (rank null) give a graph's counts in one piece.
+constexpr int BATCH_T_THREADS = 1024;
+
+__global__ void __launch_bounds__(BATCH_T_THREADS) k_batch_T(int32_t G, const int32_t* __restrict__ vbase,
+                                                             const int32_t* __restrict__ rank,
+                                                             const unsigned long long* __restrict__ t_rank,
+                                                             unsigned long long* __restrict__ T_out,
+                                                             int* __restrict__ err) {
+    __shared__ unsigned long long ws[BATCH_T_THREADS / 32];
     for (int g = blockIdx.x; g < G; g += gridDim.x) {
         unsigned long long s = 0;
-        for (int32_t v = vbase[g] + threadIdx.x; v < vbase[g + 1]; v += blockDim.x) s += t_rank[rank[v]];
+        const int64_t v1 = vbase[g + 1];
+        for (int64_t v0 = vbase[g] + threadIdx.x; v0 < v1; v0 += 4 * BATCH_T_THREADS) {
+            unsigned long long x[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int64_t v = v0 + k * BATCH_T_THREADS;
+                x[k] = v < v1 ? t_rank[rank ? rank[v] : v] : 0;
+            }
+            s += x[0] + x[1] + x[2] + x[3];
+        }
         s = warp_sum(s);
         if (lane_id() == 0) ws[threadIdx.x >> 5] = s;
         __syncthreads();
-        if (threadIdx.x == 0) {
-            unsigned long long tot = 0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += ws[w];
-            if (tot % 3 != 0) atomicOr(err, ERR_OVERFLOW);
-            T_out[g] = tot / 3;
+        if (threadIdx.x < 32) {
+            const unsigned long long tot = warp_sum(ws[threadIdx.x]);
+            if (threadIdx.x == 0) {
+                if (tot % 3 != 0) atomicOr(err, ERR_OVERFLOW);
+                T_out[g] = tot / 3;
+            }
         }
         __syncthreads();
     }
@@ -76,17 +119,17 @@ void launch_run_status(const DevStats* stats, const int* batch_err, int* status,
 }
 
 void launch_batch_relabel(int32_t G, const int64_t* edge_off, const int32_t* vbase, const int32_t* src,
-                          const int32_t* dst, int32_t* usrc, int32_t* udst, int* err, const Launch& L) {
-    if (G <= 0) return;
-    k_batch_relabel<<<grid_for((int64_t)G * 256, 256, L.sms, 16), 256, 0, L.stream>>>(G, edge_off, vbase, src, dst,
-                                                                                     usrc, udst, err);
+                          const int32_t* dst, int64_t m, int32_t* usrc, int32_t* udst, int* err, const Launch& L) {
+    if (G <= 0 || m <= 0) return;
+    k_batch_relabel<<<grid_for(m, 8 * RELABEL_PAIRS, L.sms, 16), 256, 0, L.stream>>>(G, edge_off, vbase, src, dst, m,
+                                                                                    usrc, udst, err);
     count_launch();
 }
 
 void launch_batch_T(int32_t G, const int32_t* vbase, const int32_t* rank, const unsigned long long* t_rank,
                     unsigned long long* T_out, int* err, const Launch& L) {
     if (G <= 0) return;
-    k_batch_T<<<grid_for((int64_t)G * 256, 256, L.sms, 16), 256, 0, L.stream>>>(G, vbase, rank, t_rank, T_out, err);
+    k_batch_T<<<grid_for(G, 1, L.sms, 16), BATCH_T_THREADS, 0, L.stream>>>(G, vbase, rank, t_rank, T_out, err);
     count_launch();
 }
 

@@ -182,6 +182,8 @@ struct Strategy {
 
 // Capacity of the hub kernel's shared-memory bitmap (ranks above the hub).
 constexpr int HUB_BM_BITS = 131072;
+// Least degree of a hub, unless set.
+constexpr int HUB_MIN_DEGREE = 32;
 // Window 1 of the hub kernels: the highest min(n, HUB_WIN) ranks, one 32-bit counter
 // each in shared memory.  An entry x of it is kept as four times its index in the
 // window (the counter's byte offset, 16 bits); 4 * HUB_WIN names the slot that no hub
@@ -236,6 +238,7 @@ struct CountBuffers {
     int64_t dplus_bound;     // no N+(u) has more entries
     uint32_t* sup;           // null, or m_cap per-edge supports indexed like col (tc_edge_support)
     int32_t src_lo, src_hi;  // only triangles whose lowest vertex has a rank in [src_lo, src_hi) are counted
+    bool no_hubs;            // plan without hubs (batches whose hubs would cover little)
     cudaEvent_t hub_ready;   // null, or recorded once the hub lists and the dense core are built (PlanStreams)
 };
 
@@ -375,8 +378,9 @@ void launch_rc_score(const RemoteCacheBuffers& R, const RcSimShape& S, const Lau
 
 // ---- batch (tc_batch.cu) -------------------------------------------------------
 void launch_batch_relabel(int32_t G, const int64_t* edge_off, const int32_t* vbase, const int32_t* src,
-                          const int32_t* dst, int32_t* usrc, int32_t* udst, int* err, const Launch& L);
+                          const int32_t* dst, int64_t m, int32_t* usrc, int32_t* udst, int* err, const Launch& L);
 void launch_run_status(const DevStats* stats, const int* batch_err, int* status, const Launch& L);
+// T per graph; rank null: the ranks run graph by graph (every graph's t in one piece).
 void launch_batch_T(int32_t G, const int32_t* vbase, const int32_t* rank, const unsigned long long* t_rank,
                     unsigned long long* T_out, int* err, const Launch& L);
 

@@ -2329,7 +2329,7 @@ void launch_plan_stats(const CountBuffers& C, unsigned long long* out, const Lau
 bool launch_plan(const CountBuffers& C, const Strategy& S, const Launch& L, const PlanStreams* ps) {
     if (C.n <= 0) return false;
     const int hub_max = S.hub_max < 0 ? 0 : S.hub_max;
-    const bool hubs = C.hub_cap > 0 && hub_max > 0;
+    const bool hubs = C.hub_cap > 0 && hub_max > 0 && !C.no_hubs;
     const int core_max = hubs && C.core_cap > 0 && S.hub_core > 0 ? (S.hub_core < C.core_cap ? S.hub_core : C.core_cap) : 0;
     if (hubs) {  // else the hub count stays zero
         k_hub_count<<<grid_for(C.n, THREADS, L.sms), THREADS, 0, L.stream>>>(C.n, C.deg, S.hub_min_degree, C.hub_cap,
@@ -2463,7 +2463,7 @@ void intersect_impl(const CountBuffers& C, const Strategy& S, cudaEvent_t* ev, c
     // the hub lists and the dense core come from the planner's second stream
     if (C.hub_ready) cudaStreamWaitEvent(L.stream, C.hub_ready, 0);
     if (ev) cudaEventRecord(ev[PH_HUB], L.stream);
-    if (C.hub_cap > 0) {
+    if (C.hub_cap > 0 && !C.no_hubs) {
         if (S.hub_core > 0) launch_core_count(C, L);
         const bool probe = S.strat[TC_BUCKET_HUB] == TC_STRAT_PROBE;
         const Windows T(C.n);
