@@ -599,10 +599,44 @@ __device__ __forceinline__ void reg_bitonic(int32_t (&v)[N]) {
     }
 }
 
+// Repeats dropped at a target.  A symmetric CSR drops every entry once, most of them at
+// hubs, where one global atomic each would queue on the same address: a block counts
+// them in a small shared-memory table (one slot looked at) and adds the sums at its end.
+constexpr int DUP_SLOTS = 1024;
+
+struct DupTable {
+    int32_t key[DUP_SLOTS];
+    uint32_t cnt[DUP_SLOTS];
+
+    __device__ __forceinline__ void clear() {
+        for (int i = threadIdx.x; i < DUP_SLOTS; i += blockDim.x) {
+            key[i] = -1;
+            cnt[i] = 0;
+        }
+        __syncthreads();
+    }
+    __device__ __forceinline__ void add(int32_t v, uint32_t* __restrict__ dupin) {
+        const unsigned h = ((unsigned)v * 0x9e3779b1u) >> 22;
+        int32_t k = key[h];
+        if (k == -1) k = atomicCAS(&key[h], -1, v);
+        if (k == -1 || k == v)
+            atomicAdd(&cnt[h], 1u);
+        else
+            atomicAdd(&dupin[v], 1u);
+    }
+    __device__ __forceinline__ void flush(uint32_t* __restrict__ dupin) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < DUP_SLOTS; i += blockDim.x)
+            if (cnt[i]) atomicAdd(&dupin[key[i]], cnt[i]);
+    }
+};
+static_assert(DUP_SLOTS == 1 << 10, "hash width");
+
 // Sorts a row of len <= N entries in registers, writes the distinct entries back
 // to its start and counts each dropped repeat at its target; returns how many were kept.
 template <int N>
-__device__ __forceinline__ int sort_row_regs(int32_t* __restrict__ row, int len, uint32_t* __restrict__ dupin) {
+__device__ __forceinline__ int sort_row_regs(int32_t* __restrict__ row, int len, uint32_t* __restrict__ dupin,
+                                             DupTable& dup) {
     int32_t v[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) v[i] = i < len ? row[i] : INT_MAX;
@@ -615,7 +649,7 @@ __device__ __forceinline__ int sort_row_regs(int32_t* __restrict__ row, int len,
             if (v[i] != prev)
                 row[kept++] = v[i];
             else if (dupin)
-                atomicAdd(&dupin[v[i]], 1u);
+                dup.add(v[i], dupin);
         }
         prev = v[i];
     }
@@ -630,6 +664,8 @@ __global__ void __launch_bounds__(256) k_segsort_thread(int32_t n, const int64_t
                                                         uint32_t* __restrict__ dupin, int32_t* __restrict__ midlist,
                                                         int32_t* __restrict__ midlist2, int32_t* __restrict__ longlist,
                                                         DevStats* stats) {
+    __shared__ DupTable dup;
+    dup.clear();
     unsigned long long kept_total = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     // the loop bound is uniform across a warp, as warp_append needs all 32 lanes
@@ -645,12 +681,14 @@ __global__ void __launch_bounds__(256) k_segsort_thread(int32_t n, const int64_t
         if (lng) longlist[pl] = (int32_t)r;
         if (r < n && len <= 16) {
             const int64_t base = rowstart[r];
-            const int kept = len <= 8 ? sort_row_regs<8>(col + base, len, dupin) : sort_row_regs<16>(col + base, len, dupin);
+            const int kept = len <= 8 ? sort_row_regs<8>(col + base, len, dupin, dup)
+                                      : sort_row_regs<16>(col + base, len, dupin, dup);
             rowlen[r] = kept;
             rowinfo[r] = make_int2((int)base, kept);
             kept_total += (unsigned long long)kept;
         }
     }
+    if (dupin) dup.flush(dupin);
     kept_total = warp_sum(kept_total);
     if (lane_id() == 0 && kept_total) atomicAdd(&stats->m_simple, kept_total);
 }
@@ -696,7 +734,7 @@ __device__ __forceinline__ void warp_reg_sort(int32_t (&v)[K], int lane) {
 // number kept (all lanes).
 template <int K>
 __device__ __forceinline__ int warp_sort_row(int32_t* __restrict__ row, int len, uint32_t* __restrict__ dupin,
-                                             int lane) {
+                                             DupTable& dup, int lane) {
     int32_t v[K];
 #pragma unroll
     for (int r = 0; r < K; ++r) {
@@ -716,7 +754,7 @@ __device__ __forceinline__ int warp_sort_row(int32_t* __restrict__ row, int len,
                 keepmask |= 1u << r;
                 ++nk;
             } else if (dupin) {
-                atomicAdd(&dupin[v[r]], 1u);
+                dup.add(v[r], dupin);
             }
         }
         prev = v[r];
@@ -735,12 +773,14 @@ __device__ __forceinline__ int warp_sort_row(int32_t* __restrict__ row, int len,
 // entries, MAXK = 32 those of 257..1024 (separate kernels keep the register budget
 // of the short classes small).
 template <int MAXK>
-__global__ void __launch_bounds__(SEG_WARPS * 32) k_segsort_warp(const int64_t* __restrict__ rowstart,
+__global__ void __launch_bounds__(SEG_WARPS * 32, MAXK <= 8 ? 4 : 1) k_segsort_warp(const int64_t* __restrict__ rowstart,
                                                                  const uint32_t* __restrict__ rowcnt,
                                                                  int32_t* __restrict__ col, int32_t* __restrict__ rowlen,
                                                                  int2* __restrict__ rowinfo, uint32_t* __restrict__ dupin,
                                                                  const int32_t* __restrict__ list,
                                                                  const unsigned* __restrict__ count, DevStats* stats) {
+    __shared__ DupTable dup;
+    dup.clear();
     const int lane = lane_id(), w = threadIdx.x >> 5;
     const unsigned nrows = *count;
     const unsigned warps = gridDim.x * SEG_WARPS;
@@ -753,20 +793,20 @@ __global__ void __launch_bounds__(SEG_WARPS * 32) k_segsort_warp(const int64_t* 
         int kept;
         if (MAXK <= 8) {
             if (len <= 32)
-                kept = warp_sort_row<1>(row, len, dupin, lane);
+                kept = warp_sort_row<1>(row, len, dupin, dup, lane);
             else if (len <= 64)
-                kept = warp_sort_row<2>(row, len, dupin, lane);
+                kept = warp_sort_row<2>(row, len, dupin, dup, lane);
             else if (len <= 128)
-                kept = warp_sort_row<4>(row, len, dupin, lane);
+                kept = warp_sort_row<4>(row, len, dupin, dup, lane);
             else
-                kept = warp_sort_row<8>(row, len, dupin, lane);
+                kept = warp_sort_row<8>(row, len, dupin, dup, lane);
         } else if (MAXK <= 16) {
-            kept = warp_sort_row<16>(row, len, dupin, lane);
+            kept = warp_sort_row<16>(row, len, dupin, dup, lane);
         } else {
             if (len <= 512)
-                kept = warp_sort_row<16>(row, len, dupin, lane);
+                kept = warp_sort_row<16>(row, len, dupin, dup, lane);
             else
-                kept = warp_sort_row<32>(row, len, dupin, lane);
+                kept = warp_sort_row<32>(row, len, dupin, dup, lane);
         }
         if (lane == 0) {
             rowlen[r] = kept;
@@ -775,6 +815,7 @@ __global__ void __launch_bounds__(SEG_WARPS * 32) k_segsort_warp(const int64_t* 
         }
         __syncwarp();
     }
+    if (dupin) dup.flush(dupin);
     if (lane == 0 && kept_total) atomicAdd(&stats->m_simple, kept_total);
 }
 

@@ -117,43 +117,44 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_tile_scan(const In* in, Out* o
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[count] = (Out)(before + tot);
 }
 
-// A short scan in one launch by one block, a tile after the other.
+// A short scan in one launch, by one block: a thread takes consecutive values.
+constexpr int ONE_THREADS = 1024;
+constexpr int64_t SCAN_ONE_MAX = ONE_THREADS * SCAN_ITEMS;
+
 template <typename In, typename Out, typename Acc>
-__global__ void __launch_bounds__(SCAN_THREADS) k_scan_one(const In* in, Out* out, Out* out2, int64_t count) {
-    __shared__ Acc tot;
-    Acc carry = 0;
-    for (int64_t base = 0; base < count; base += SCAN_TILE) {
-        Acc v[SCAN_ITEMS];
-        Acc s = 0;
+__global__ void __launch_bounds__(ONE_THREADS) k_scan_one(const In* in, Out* out, Out* out2, int64_t count) {
+    __shared__ Acc warp_tot[ONE_THREADS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int per = (int)((count + ONE_THREADS - 1) / ONE_THREADS);  // at most SCAN_ITEMS
+    const int64_t base = (int64_t)threadIdx.x * per;
+    Acc v[SCAN_ITEMS];
+    Acc s = 0;
 #pragma unroll
-        for (int k = 0; k < SCAN_ITEMS; ++k) {
-            int64_t i = base + (int64_t)threadIdx.x * SCAN_ITEMS + k;
-            v[k] = i < count ? (Acc)in[i] : Acc(0);
-            s += v[k];
-        }
-        Acc run = carry + block_exclusive_scan(s, &tot);
-#pragma unroll
-        for (int k = 0; k < SCAN_ITEMS; ++k) {
-            int64_t i = base + (int64_t)threadIdx.x * SCAN_ITEMS + k;
-            if (i < count) {
-                out[i] = (Out)run;
-                if (out2) out2[i] = (Out)run;
-            }
-            run += v[k];
-        }
-        carry += tot;
-        __syncthreads();  // tot is written again by the next tile
+    for (int k = 0; k < SCAN_ITEMS; ++k) {
+        v[k] = k < per && base + k < count ? (Acc)in[base + k] : Acc(0);
+        s += v[k];
     }
-    if (threadIdx.x == 0) out[count] = (Out)carry;
+    const Acc inc = warp_inclusive_scan(s);
+    if (lane == 31) warp_tot[warp] = inc;
+    __syncthreads();
+    Acc before = warp_inclusive_scan(lane < warp ? warp_tot[lane] : Acc(0));
+    before = __shfl_sync(FULL, before, 31);  // of the warps before this one
+    Acc run = before + inc - s;
+#pragma unroll
+    for (int k = 0; k < SCAN_ITEMS; ++k) {
+        if (k < per && base + k < count) {
+            out[base + k] = (Out)run;
+            if (out2) out2[base + k] = (Out)run;
+        }
+        run += v[k];
+    }
+    if (threadIdx.x == ONE_THREADS - 1) out[count] = (Out)run;
 }
-// One block passes over a tile in about 1 us, the two kernels cost about 5 us of launch
-// and GPU time together.
-constexpr int64_t SCAN_ONE_MAX = 4 * SCAN_TILE;
 
 template <typename In, typename Out, typename Acc>
 void scan_impl(const In* in, Out* out, Out* out2, int64_t count, void* tmp, const Launch& L) {
     if (count <= SCAN_ONE_MAX) {
-        k_scan_one<In, Out, Acc><<<1, SCAN_THREADS, 0, L.stream>>>(in, out, out2, count); count_launch();
+        k_scan_one<In, Out, Acc><<<1, ONE_THREADS, 0, L.stream>>>(in, out, out2, count); count_launch();
         return;
     }
     const int64_t tiles = (count + SCAN_TILE - 1) / SCAN_TILE;

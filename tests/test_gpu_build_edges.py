@@ -1,0 +1,43 @@
+"""The build's one-block scans and ranks at their largest sizes, and its table of dropped
+repeats, against the oracle (exact)."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import graphgen
+import oracle
+from tests.gpu_util import assert_matches_oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n", [1023, 1024, 1025, 8191, 8192, 8193, 16383, 16384, 16385])
+def test_one_block_sizes(tc, n):
+    s, d = graphgen.er(n, 6 * n, seed=n)
+    hub = np.arange(1, min(n, 1500), dtype=np.int32)  # a degree past every narrow count
+    s, d = np.concatenate([s, np.zeros_like(hub)]), np.concatenate([d, hub])
+    assert_matches_oracle(tc, n, s, d, device_io=True)
+
+
+@pytest.mark.parametrize("n", [(1 << 21) - 1, 1 << 21, (1 << 21) + 1])
+def test_scan_over_a_thousand_tiles(tc, n):
+    s, d = graphgen.er(n, 1 << 20, seed=8)
+    assert_matches_oracle(tc, n, s, d, device_io=True)
+
+
+@pytest.mark.parametrize("n,hubs,per", [(4000, 1, 3), (4000, 1500, 6), (3000, 3, 300)])
+def test_repeats_at_hubs(tc, n, hubs, per):
+    """A symmetric CSR drops each pair once, at hubs more often than a block's table has
+    slots for; one row repeats its entries."""
+    rng = np.random.default_rng(n + hubs)
+    s = np.repeat(np.arange(n), per)
+    d = np.where(rng.random(n * per) < 0.7, rng.integers(0, hubs, n * per), rng.integers(0, n, n * per))
+    s, d = np.concatenate([s, d, np.full(400, 5)]), np.concatenate([d, s, np.full(400, 9)])
+    order = np.lexsort((d, s))
+    s, d = s[order].astype(np.int32), d[order].astype(np.int32)
+    off = np.zeros(n + 1, np.int64)
+    off[1:] = np.cumsum(np.bincount(s, minlength=n))
+    ref = oracle.triangles(n, s, d)
+    for device_io in (False, True):
+        assert_matches_oracle(tc, n, s, d, ref=ref, csr=(off, d), device_io=device_io)
