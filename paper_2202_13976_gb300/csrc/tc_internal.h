@@ -41,13 +41,14 @@ struct DevStats {
     unsigned int win_vecs;         // planner: 16-byte vectors of window entries written
     // from here on, zero when a count starts
     unsigned int cta_next;         // dynamic work counter of the block push kernel
+    unsigned int small_next[2];    // dynamic work counters of the hash kernels
     unsigned int hub_next;         // dynamic work counter of the hub kernel (slices of big hubs)
     unsigned int hub_next2;        // dynamic work counter of the hub kernel (medium hubs)
     unsigned int hub_next3;        // dynamic work counter of the list kernel (long lists; probe mode)
     unsigned int hub_next4;        // dynamic work counter of the below-window kernel
     unsigned long long sum_t;      // sum over v of t(v)
 };
-static_assert(sizeof(DevStats) == 128 && offsetof(DevStats, cta_next) % 4 == 0, "DevStats layout");
+static_assert(sizeof(DevStats) == 136 && offsetof(DevStats, cta_next) % 4 == 0, "DevStats layout");
 
 struct Launch {
     cudaStream_t stream;

@@ -44,6 +44,8 @@ constexpr int THREADS = 256;
 constexpr int SMALL_WARPS = 8;         // warps per block in the small-bucket kernel
 constexpr int SMALL_BLOCKS = 8;        // its resident blocks per SM (the grid is one wave of them)
 constexpr int SMALL_WIDE_MAX = 256;    // longest N+(u) the warp-per-source kernel stages
+constexpr int HASH_LG_SHORT = 8;       // slots of the hash kernel's sets (log2): sources of at most 32 entries,
+constexpr int HASH_LG_WIDE = 9;        // and of at most SMALL_WIDE_MAX
 constexpr int HASH_CUT = 64;           // rows longer than this are cut at max N+(u) by the hash kernel
 constexpr int CTA_THREADS = 256;       // block push kernel
 constexpr int CTA_WARPS = CTA_THREADS / 32;
@@ -981,175 +983,260 @@ struct HashProbe {
     }
 };
 
+// 1 << d for d in [0, 32), 0 for any other d (PTX clamps the shift amount).
+__device__ __forceinline__ unsigned bit_or_none(int d) {
+    unsigned r;
+    asm("shl.b32 %0, 1, %1;" : "=r"(r) : "r"(d));
+    return r;
+}
+
+// Inclusive warp scan whose adds are predicated by the shuffles themselves.
+__device__ __forceinline__ uint32_t warp_scan_u32(uint32_t x) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+        asm("{ .reg .pred p; .reg .u32 y; shfl.sync.up.b32 y|p, %0, %1, 0, 0xffffffff; @p add.u32 %0, %0, y; }"
+            : "+r"(x)
+            : "r"(o));
+    return x;
+}
+
+// One warp's edges (up to 32) with something to read, in order: lane i takes the i-th of
+// them.  Their items are laid end to end; at[i] = {base of edge i's items less the
+// items before it, their end}.
+struct EdgeItems {
+    int cz, total, excl;  // edges; items; first item of this lane's edge (-1: none)
+    int seen;             // edges that start before the round, less one
+    unsigned upto;        // this lane's bit and those below it
+
+    // items: this lane's edge's count; returns the lane whose edge this lane takes
+    __device__ __forceinline__ int gather(int items, uint32_t* cw) {
+        const int lane = lane_id();
+        const unsigned nz = __ballot_sync(FULL, items > 0);
+        cz = __popc(nz);
+        if (cz == 0) return 0;
+        if (items > 0) cw[__popc(nz & lanemask_lt())] = (uint32_t)lane;
+        __syncwarp();
+        return lane < cz ? (int)cw[lane] : lane;
+    }
+    // items and base of the edge this lane has taken
+    __device__ __forceinline__ void lay(int items, int base, int2* at) {
+        const int lane = lane_id();
+        if (lane >= cz) items = 0;
+        const int incl = (int)warp_scan_u32((uint32_t)items);
+        total = __shfl_sync(FULL, incl, 31);
+        excl = lane < cz ? incl - items : -1;
+        at[lane] = make_int2(base - (incl - items), incl);
+        seen = -1;
+        upto = lane == 31 ? FULL : (2u << lane) - 1u;
+        __syncwarp();
+    }
+    // the edge of item r + lane; called for r = 0, 32, 64, ... in turn
+    __device__ __forceinline__ int edge_of(int r) {
+        const unsigned mk = __reduce_or_sync(FULL, bit_or_none(excl - r));
+        const int i = seen + __popc(mk & upto);
+        seen += __popc(mk);
+        return i;
+    }
+};
+
 // ---- small bucket, hash strategy: N+(u) as a hash set, target rows end to end ----
-//
-// A group of G lanes takes one source u at a time.  N+(u) (at most AMAX entries) goes
-// into an open-addressing hash set of SL >= 2 AMAX slots in shared memory.  Its edges
-// (u, v) into non-hubs are taken G at a time; their rows N+(v) are laid end to end and
-// the group reads G entries per round, one per lane, each entry probed once in the
-// set (entries above max N+(u) are skipped).  A hit at x in N+(v) is a triangle: x is
+
+// Open-addressing set whose slots say in bit 31 whether an insertion went past them: a
+// probe of any other key ends at the first unmarked slot, whatever key it holds (at a
+// quarter of the slots taken, one probe in a hundred goes on; without the marks every
+// fourth).  Ranks are below 2^31 - 1, which marks an empty slot.
+constexpr int32_t SET_EMPTY = INT_MAX;
+
+template <int LG>
+struct MarkedSet {
+    int32_t* keys;
+    static __device__ __forceinline__ unsigned slot(int32_t x) { return ((unsigned)x * 0x9e3779b1u) >> (32 - LG); }
+    static __device__ __forceinline__ unsigned after(unsigned h) { return (h + 1) & ((1u << LG) - 1u); }
+    __device__ __forceinline__ unsigned insert(int32_t x) const {  // keys are distinct
+        unsigned h = slot(x);
+        while (atomicCAS(&keys[h], SET_EMPTY, x) != SET_EMPTY) {
+            atomicOr(&keys[h], INT_MIN);
+            h = after(h);
+        }
+        return h;
+    }
+    __device__ __forceinline__ int operator()(int32_t x) const {
+        unsigned h = slot(x);
+        for (;;) {
+            const int32_t k = keys[h];
+            if ((k & INT_MAX) == x) return (int)h;
+            if (k >= 0) return -1;
+            h = after(h);
+        }
+    }
+};
+
+// A warp takes one source u at a time.  N+(u) (at most SL / 2 entries) goes into a set of
+// SL slots in shared memory.  Its edges (u, v) into non-hubs are taken 32 at a time; their
+// rows N+(v) are laid end to end and read 32 entries per round, one per lane, each probed
+// once (entries above max N+(u) are skipped).  A hit at x in N+(v) is a triangle: x is
 // above v, so it lies in the suffix of N+(u) after v, which is W for the edge (u, v).
-// Hits add to the slot's counter (t[x], flushed once per source) and to the edge's
-// counter (t[v]); their sum goes to t[u].  Every lane reads at every round, so the
-// lanes stay busy whatever the lengths of the rows.
-template <int G, int SL, bool SUP>
-__global__ void __launch_bounds__(SMALL_WARPS * 32) k_tc_small_hash(int32_t n, const int2* __restrict__ rowinfo,
-                                                                   const int32_t* __restrict__ col,
-                                                                   const int32_t* __restrict__ list, int cls,
-                                                                   unsigned long long* __restrict__ t,
-                                                                   DevStats* stats, uint32_t* __restrict__ sup_arg) {
+// Hits add to the slot's counter (t[x], flushed once per source); at an edge's last entry
+// the hits up to it are noted, so that differences give each edge's count (t[v]); their
+// sum goes to t[u].
+//
+// Bound by instruction issue (75 to 78 % of the slots; 27 of 32 lanes active).  A batch of
+// 840 graphs, 66 M pairs, sources of 17..32 and 33..256 entries: one edge at a time with
+// whole warps, 2.0 and 3.3 ms; rows end to end, 1.3 and 3.0; with sources claimed one by
+// one (a static stride left the last warps 20 % longer), 1.1 and 2.5.  4, 5, 7 and 8 blocks
+// per SM are 2 to 25 % slower than 6.
+constexpr int HASH_BLOCKS = 6;  // resident blocks per SM: the grid is one wave of them
+template <int LG, bool SUP>
+__global__ void __launch_bounds__(SMALL_WARPS * 32, SUP ? 4 : HASH_BLOCKS)
+    k_tc_small_hash(int32_t n, const int2* __restrict__ rowinfo, const int32_t* __restrict__ col,
+                    const int32_t* __restrict__ list, int cls, unsigned long long* __restrict__ t, DevStats* stats,
+                    uint32_t* __restrict__ sup_arg) {
     uint32_t* const sup = SUP ? sup_arg : nullptr;
-    static_assert(G == 8 || G == 16 || G == 32, "lane groups within a warp");
-    static_assert((SL & (SL - 1)) == 0 && SL >= 2 * G, "power-of-two table");
-    constexpr int GROUPS = SMALL_WARPS * 32 / G;
-    constexpr int LG = SL == 16 ? 4 : SL == 32 ? 5 : SL == 64 ? 6 : SL == 128 ? 7 : SL == 256 ? 8 : 9;
-    static_assert((1 << LG) == SL, "table size");
-    __shared__ int32_t skeys[GROUPS][SL];
-    __shared__ uint32_t shcnt[GROUPS][SL];
-    __shared__ uint32_t secnt[GROUPS][G];
-    __shared__ uint16_t shpos[GROUPS][SL];  // position in N+(u) of each key (support only)
+    constexpr int SL = 1 << LG;
+    __shared__ int32_t skeys[SMALL_WARPS][SL];
+    __shared__ uint32_t shcnt[SMALL_WARPS][SL];
+    __shared__ uint16_t shpos[SMALL_WARPS][SUP ? SL : 1];  // position in N+(u) of each key (support only)
+    __shared__ int2 sat[SMALL_WARPS][32];
+    __shared__ uint32_t scw[SMALL_WARPS][32];
     const int lane = lane_id(), w = threadIdx.x >> 5;
-    const int grp = lane / G, g = lane % G;
-    const int gi = w * (32 / G) + grp;
-    const unsigned gmask = G == 32 ? FULL : (((1u << G) - 1u) << (grp * G));
-    const unsigned below = (1u << g) - 1u;  // group lanes under this one (group-relative bits)
-    int32_t* keys = skeys[gi];
-    uint32_t* hcnt = shcnt[gi];
-    uint32_t* ecnt = secnt[gi];
-    uint16_t* hpos = shpos[gi];
-    for (int i = g; i < SL; i += G) {
-        keys[i] = -1;
+    const MarkedSet<LG> P{skeys[w]};
+    uint32_t* const hcnt = shcnt[w];
+    uint16_t* const hpos = shpos[w];
+    int2* const at = sat[w];
+    uint32_t* const cw = scw[w];
+    for (int i = lane; i < SL; i += 32) {
+        P.keys[i] = SET_EMPTY;
         hcnt[i] = 0;
     }
-    ecnt[g] = 0;
-    __syncwarp(gmask);
+    __syncwarp();
     const unsigned count = stats->small_count[cls];
     const int32_t R = n - (int32_t)stats->hub_count;
-    const unsigned groups = gridDim.x * GROUPS;
-    const HashProbe P{keys, 32u - LG, SL - 1u};
-    auto gballot = [&](bool p) { return (__ballot_sync(gmask, p) >> (grp * G)) & (G == 32 ? FULL : ((1u << G) - 1u)); };
-    for (unsigned q = blockIdx.x * GROUPS + gi; q < count; q += groups) {
-        const int32_t u = list[q];
-        const int2 ru = rowinfo[u];
+    // sources are claimed one ahead, and the next one's row is fetched meanwhile
+    unsigned q = blockIdx.x * SMALL_WARPS + w;
+    int32_t u = q < count ? list[q] : 0;
+    int2 ru = q < count ? rowinfo[u] : make_int2(0, 0);
+    while (q < count) {
+        unsigned qn = 0;
+        if (lane == 0) qn = gridDim.x * SMALL_WARPS + atomicAdd(&stats->small_next[cls - 2], 1u);
+        qn = __shfl_sync(FULL, qn, 0);
+        const int32_t un = qn < count ? list[qn] : 0;
         const int du = ru.y;
         const int64_t base = ru.x;
         int jh = 0;  // entries below the hubs: the rows are sorted, so they come first
-        for (int i0 = 0; i0 < du; i0 += G) {  // every lane of the group takes every round
-            const bool valid = i0 + g < du;
-            const int32_t x = valid ? col[base + i0 + g] : INT_MAX;
+        for (int i0 = 0; i0 < du; i0 += 32) {
+            const bool valid = i0 + lane < du;
+            const int32_t x = valid ? col[base + i0 + lane] : INT_MAX;
             if (valid) {
-                unsigned h = ((unsigned)x * 0x9e3779b1u) >> (32 - LG);
-                while (atomicCAS(&keys[h], -1, x) != -1) h = (h + 1) & (SL - 1);  // keys are distinct
-                if (sup) hpos[h] = (uint16_t)(i0 + g);
+                const unsigned h = P.insert(x);
+                if (sup) hpos[h] = (uint16_t)(i0 + lane);
             }
-            jh += __popc(gballot(x < R));
+            jh += __popc(__ballot_sync(FULL, x < R));
         }
         const int32_t maxu = col[base + du - 1];
+        const int2 run = qn < count ? rowinfo[un] : make_int2(0, 0);
         const int ne = min(jh, du - 1);  // the last entry has an empty suffix
-        __syncwarp(gmask);
+        __syncwarp();
         uint32_t cu = 0;
-        for (int e0 = 0; e0 < ne; e0 += G) {
-            const bool has = e0 + g < ne;
-            const int32_t v0 = has ? col[base + e0 + g] : 0;
+        for (int e0 = 0; e0 < ne; e0 += 32) {
+            const bool has = e0 + lane < ne;
+            const int32_t v0 = has ? col[base + e0 + lane] : 0;
             const int2 r0 = has ? rowinfo[v0] : make_int2(0, 0);
             // only entries up to max N+(u) can match: long rows are cut there; an edge
             // whose cut row is longer than the suffix a of N+(u) after v by more than
             // Eq. 3 allows (factor 8: one lane's dependent search steps cost more than the
-            // group's parallel probes) is left to its own lane, which searches the a keys
+            // warp's parallel probes) is left to its own lane, which searches the a keys
             // in the row (a log b instead of b probes)
-            int b0 = r0.y;
-            if (b0 > HASH_CUT) b0 = lower_bound(col + r0.x, 0, b0, maxu + 1);
-            const int a0 = du - (e0 + g) - 1;
-            const bool live = has && b0 > 0;
-            const bool srch0 = live && a0 > 0 && b0 > a0 && !eq3_prefers_merge(a0, b0, 8.0f);
-            // lanes reordered: the streamed edges first (ce of them), then the searching
-            // ones (cq), then nothing
-            const unsigned sm = gballot(live && !srch0);
-            const unsigned qm = gballot(srch0);
-            const int ce_n = __popc(sm), cq = __popc(qm);
-            if (ce_n + cq == 0) continue;
-            const int src = g < ce_n ? (int)__fns(sm, 0, g + 1) : (g < ce_n + cq ? (int)__fns(qm, 0, g - ce_n + 1) : g);
-            const int32_t v = __shfl_sync(gmask, v0, src, G);
-            const int jv = e0 + src;  // position of v in N+(u)
-            const int rs = __shfl_sync(gmask, r0.x, src, G);
-            int b = __shfl_sync(gmask, b0, src, G);
-            if (g >= ce_n + cq) b = 0;
-            const bool search = g >= ce_n && g < ce_n + cq;
-            const int streamed = g < ce_n ? b : 0;
-            int incl = streamed;
-#pragma unroll
-            for (int o = 1; o < G; o <<= 1) {
-                const int y = __shfl_up_sync(gmask, incl, o, G);
-                if (g >= o) incl += y;
-            }
-            const int total = __shfl_sync(gmask, incl, G - 1, G);
-            const int excl = incl - streamed;
-            for (int r = 0; r < total; r += G) {
-                // the edge of entry r + g: i0 holds entry r, and every later streamed
-                // edge that starts inside the round marks its first entry in mk
-                const int i0 = __popc(gballot(g < ce_n && incl <= r));
-                const unsigned mk = __reduce_or_sync(gmask, (g > i0 && g < ce_n && excl - r < G) ? (1u << (excl - r)) : 0u);
-                const int idx = min(i0 + __popc(mk & (below | (1u << g))), G - 1);
-                const int bs = __shfl_sync(gmask, rs, idx, G);
-                const int bx = __shfl_sync(gmask, excl, idx, G);
-                const int k = r + g;
-                if (k < total) {
-                    const int64_t px = (int64_t)bs + (k - bx);
-                    const int32_t x = col[px];
-                    if (x <= maxu) {
-                        const int h = P(x);
-                        if (h >= 0) {
-                            atomicAdd(&hcnt[h], 1u);
-                            atomicAdd(&ecnt[idx], 1u);
-                            if (sup) atomicAdd(&sup[px], 1u);  // edge (v, x)
-                        }
-                    }
-                }
-            }
+            int b = r0.y;
+            if (b > HASH_CUT) b = lower_bound(col + r0.x, 0, b, maxu + 1);
+            const int a = du - (e0 + lane) - 1;
+            const bool search = b > 0 && a > 0 && b > a && !eq3_prefers_merge(a, b, 8.0f);
             uint32_t cs = 0;  // a searching lane: the suffix keys after v looked up in N+(v)
             if (search) {
-                const int32_t* B = col + rs;
+                const int32_t* B = col + r0.x;
                 int lo = 0;
-                for (int i = jv + 1; i < du && lo < b; ++i) {
+                for (int i = e0 + lane + 1; i < du && lo < b; ++i) {
                     const int32_t y = col[base + i];
                     const int p = lower_bound(B, lo, b, y);
                     lo = p;
                     if (p < b && B[p] == y) {
                         atomicAdd(&hcnt[P(y)], 1u);
-                        if (sup) atomicAdd(&sup[rs + p], 1u);  // edge (v, y)
+                        if (sup) atomicAdd(&sup[r0.x + p], 1u);  // edge (v, y)
                         ++cs;
                     }
                 }
+                if (cs) {
+                    atomicAdd(&t[v0], (unsigned long long)cs);
+                    if (sup) atomicAdd(&sup[base + e0 + lane], cs);  // edge (u, v)
+                }
             }
-            __syncwarp(gmask);
-            const uint32_t ce = ecnt[g] + cs;
-            ecnt[g] = 0;
-            if (ce) {
-                atomicAdd(&t[v], (unsigned long long)ce);
-                if (sup) atomicAdd(&sup[base + jv], ce);  // edge (u, v)
-                cu += ce;
-            }
-            __syncwarp(gmask);
-        }
+            __syncwarp();
+            cu += cs;
+            EdgeItems E;
+            const int src = E.gather(search ? 0 : b, cw);
+            if (E.cz == 0) continue;
+            const int32_t v = __shfl_sync(FULL, v0, src);
+            E.lay(__shfl_sync(FULL, b, src), __shfl_sync(FULL, r0.x, src), at);
+            uint32_t running = 0;
+            for (int r = 0; r < E.total; r += 64) {
+                const int item = r + lane;
+                int idx[2];
+                int2 e[2];
+                int32_t x[2];
 #pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) cu += __shfl_down_sync(gmask, cu, o, G);
-        if (g == 0 && cu) atomicAdd(&t[u], (unsigned long long)cu);
-        for (int i = g; i < SL; i += G) {  // flush the per-entry counts, empty the set
-            const int32_t x = keys[i];
-            if (x >= 0) {
+                for (int h = 0; h < 2; ++h) {
+                    idx[h] = 0;
+                    e[h] = make_int2(0, 0);
+                    x[h] = INT_MAX;
+                    if (h == 0 || r + 32 < E.total) {
+                        idx[h] = E.edge_of(r + 32 * h);
+                        e[h] = at[idx[h]];
+                        if (item + 32 * h < E.total) x[h] = col[e[h].x + item + 32 * h];
+                    }
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int slot = x[h] <= maxu ? P(x[h]) : -1;
+                    if (slot >= 0) {
+                        atomicAdd(&hcnt[slot], 1u);
+                        if (sup) atomicAdd(&sup[e[h].x + item + 32 * h], 1u);  // edge (v, x)
+                    }
+                    const unsigned hits = __ballot_sync(FULL, slot >= 0);
+                    // an edge's last entry
+                    if (e[h].y == item + 32 * h + 1) cw[idx[h]] = running + __popc(hits & E.upto);
+                    running += __popc(hits);
+                }
+            }
+            __syncwarp();
+            if (lane < E.cz) {
+                const uint32_t ce = cw[lane] - (lane ? cw[lane - 1] : 0u);
+                if (ce) {
+                    atomicAdd(&t[v], (unsigned long long)ce);
+                    if (sup) atomicAdd(&sup[base + e0 + src], ce);  // edge (u, v)
+                    cu += ce;
+                }
+            }
+            __syncwarp();
+        }
+        cu = __reduce_add_sync(FULL, cu);
+        if (lane == 0 && cu) atomicAdd(&t[u], (unsigned long long)cu);
+        for (int i = lane; i < SL; i += 32) {  // flush the per-entry counts, empty the set
+            const int32_t x = P.keys[i] & INT_MAX;
+            if (x != SET_EMPTY) {
                 const uint32_t c = hcnt[i];
                 if (c) {
                     atomicAdd(&t[x], (unsigned long long)c);
                     if (sup) atomicAdd(&sup[base + hpos[i]], c);  // edge (u, x)
                 }
-                keys[i] = -1;
+                P.keys[i] = SET_EMPTY;
                 hcnt[i] = 0;
             }
         }
-        __syncwarp(gmask);
+        __syncwarp();
+        q = qn;
+        u = un;
+        ru = run;
     }
 }
-
 
 // Warp per edge: the entries of B = N+(v) (sorted) are probed in a set of the
 // staged N+(u), two per lane per round, stopping above max N+(u); hits add to the
@@ -1506,23 +1593,6 @@ constexpr int WINK_WARPS = WINK_THREADS / 32;
 constexpr int WINK_BLOCKS = 3;
 constexpr uint32_t WIN_MARK = 0x80000000u;
 
-// 1 << d for d in [0, 32), 0 for any other d (PTX clamps the shift amount).
-__device__ __forceinline__ unsigned bit_or_none(int d) {
-    unsigned r;
-    asm("shl.b32 %0, 1, %1;" : "=r"(r) : "r"(d));
-    return r;
-}
-
-// Inclusive warp scan whose adds are predicated by the shuffles themselves.
-__device__ __forceinline__ uint32_t warp_scan_u32(uint32_t x) {
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1)
-        asm("{ .reg .pred p; .reg .u32 y; shfl.sync.up.b32 y|p, %0, %1, 0, 0xffffffff; @p add.u32 %0, %0, y; }"
-            : "+r"(x)
-            : "r"(o));
-    return x;
-}
-
 __device__ __forceinline__ int shared_s32(uint32_t addr) {
     int v;
     asm volatile("ld.shared.s32 %0, [%1];" : "=r"(v) : "r"(addr));
@@ -1595,45 +1665,6 @@ struct WinBitmap {
                 ++c;
             }
         return c;
-    }
-};
-
-// One warp's in-edges (up to 32) with something to read, in order: lane i takes the
-// i-th of them.  Their items are laid end to end; at[i] = {base of in-edge i's items
-// less the items before it, their end}.
-struct EdgeItems {
-    int cz, total, excl;  // in-edges; items; first item of this lane's in-edge (-1: none)
-    int seen;             // in-edges that start before the round, less one
-    unsigned upto;        // this lane's bit and those below it
-
-    // items: this lane's in-edge's count; returns the lane whose in-edge this lane takes
-    __device__ __forceinline__ int gather(int items, uint32_t* cw) {
-        const int lane = lane_id();
-        const unsigned nz = __ballot_sync(FULL, items > 0);
-        cz = __popc(nz);
-        if (cz == 0) return 0;
-        if (items > 0) cw[__popc(nz & lanemask_lt())] = (uint32_t)lane;
-        __syncwarp();
-        return lane < cz ? (int)cw[lane] : lane;
-    }
-    // items and base of the in-edge this lane has taken
-    __device__ __forceinline__ void lay(int items, int base, int2* at) {
-        const int lane = lane_id();
-        if (lane >= cz) items = 0;
-        const int incl = (int)warp_scan_u32((uint32_t)items);
-        total = __shfl_sync(FULL, incl, 31);
-        excl = lane < cz ? incl - items : -1;
-        at[lane] = make_int2(base - (incl - items), incl);
-        seen = -1;
-        upto = lane == 31 ? FULL : (2u << lane) - 1u;
-        __syncwarp();
-    }
-    // the in-edge of item r + lane; called for r = 0, 32, 64, ... in turn
-    __device__ __forceinline__ int edge_of(int r) {
-        const unsigned mk = __reduce_or_sync(FULL, bit_or_none(excl - r));
-        const int i = seen + __popc(mk & upto);
-        seen += __popc(mk);
-        return i;
     }
 };
 
@@ -2423,12 +2454,12 @@ void intersect_impl(const CountBuffers& C, const Strategy& S, cudaEvent_t* ev, c
             count_launch();
         }
         if (top > 16) {
-            k_tc_small_hash<32, 64, SUP><<<L.sms * SMALL_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
+            k_tc_small_hash<HASH_LG_SHORT, SUP><<<L.sms * (SUP ? 4 : HASH_BLOCKS), SMALL_WARPS * 32, 0, L.stream>>>(
                 C.n, C.rowinfo, C.col, C.small_list[2], 2, C.t_rank, C.stats, C.sup);
             count_launch();
         }
         if (top > 32) {
-            k_tc_small_hash<32, 2 * SMALL_WIDE_MAX, SUP><<<L.sms * SMALL_WIDE_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
+            k_tc_small_hash<HASH_LG_WIDE, SUP><<<L.sms * (SUP ? 4 : HASH_BLOCKS), SMALL_WARPS * 32, 0, L.stream>>>(
                 C.n, C.rowinfo, C.col, C.small_list[3], 3, C.t_rank, C.stats, C.sup);
             count_launch();
         }
