@@ -1238,6 +1238,139 @@ __global__ void __launch_bounds__(SMALL_WARPS * 32, SUP ? 4 : HASH_BLOCKS)
     }
 }
 
+// Sources of at most G = 8 or 16 entries, 32 / G of them by a warp: each lane has one entry
+// of one source, inserts it into that source's set of 4 G slots and keeps its slot.  The
+// edges of all of them go end to end as above; a hit adds to the slot's counter and to the
+// edge's, kept with the lane that has the entry, which so flushes t[x] and the edge's
+// support once.
+//
+// Bound by the random sectors of row records and rows: a uniform graph of 2^23 vertices and
+// 64 M pairs, sources of up to 8 and 9..16 entries: a merge per lane, 10 to 12 lanes of 32
+// active, 0.66 and 1.20 ms; this, 0.47 and 0.75 (the second reads 3.8 GB).  A batch of 840
+// graphs, 66 M pairs: 0.43 and 0.90, now 0.48 and 0.76.  6 blocks per SM (37 registers)
+// instead of 8 take 10 to 20 % longer.
+constexpr int SETS_LONG = 32;   // Eq. 3 (factor 8) searches no row of at most so many entries
+constexpr int SETS_BLOCKS = 8;  // resident blocks per SM: the grid is one wave of them
+template <int G, bool SUP>
+__global__ void __launch_bounds__(SMALL_WARPS * 32, SETS_BLOCKS)
+    k_tc_small_sets(int32_t n, const int2* __restrict__ rowinfo, const int32_t* __restrict__ col,
+                    const int32_t* __restrict__ list, int cls, unsigned long long* __restrict__ t, DevStats* stats,
+                    uint32_t* __restrict__ sup_arg) {
+    uint32_t* const sup = SUP ? sup_arg : nullptr;
+    constexpr int GPW = 32 / G, SL = 4 * G;
+    using Set = MarkedSet<G == 8 ? 5 : 6>;
+    static_assert(SL == (G == 8 ? 32 : 64), "slots of a set");
+    __shared__ int32_t skeys[SMALL_WARPS][GPW * SL];
+    __shared__ uint32_t shcnt[SMALL_WARPS][GPW * SL];
+    __shared__ int2 sat[SMALL_WARPS][32];
+    __shared__ uint32_t sce[SMALL_WARPS][32];
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    const int grp = lane / G, gl = lane % G;
+    int32_t* const keys = skeys[w];
+    uint32_t* const hcnt = shcnt[w];
+    int2* const at = sat[w];
+    uint32_t* const ce = sce[w];
+    for (int i = lane; i < GPW * SL; i += 32) {
+        keys[i] = SET_EMPTY;
+        hcnt[i] = 0;
+    }
+    __syncwarp();
+    const Set own{keys + grp * SL};
+    const unsigned count = stats->small_count[cls];
+    const int32_t R = n - (int32_t)stats->hub_count;
+    const unsigned step = gridDim.x * SMALL_WARPS * GPW;
+    unsigned q0 = (blockIdx.x * SMALL_WARPS + w) * GPW;  // the warp's first source
+    int32_t u = q0 + grp < count ? list[q0 + grp] : 0;
+    int2 ru = q0 + grp < count ? rowinfo[u] : make_int2(0, 0);
+    int32_t x = gl < ru.y ? col[ru.x + gl] : INT_MAX;
+    for (; q0 < count; q0 += step) {
+        const unsigned qn = q0 + step + grp;  // the next source and its row are fetched ahead
+        const int32_t un = qn < count ? list[qn] : 0;
+        const int du = ru.y;
+        const bool has = gl < du;
+        const int2 rx = gl < du - 1 && x < R ? rowinfo[x] : make_int2(0, 0);  // the last entry has an empty suffix
+        const int2 run = qn < count ? rowinfo[un] : make_int2(0, 0);
+        unsigned hs = grp * SL;
+        if (has) hs += own.insert(x);
+        __syncwarp();
+        uint32_t cs = 0;
+        int b = rx.y;
+        if (__any_sync(FULL, b > SETS_LONG)) {  // long rows: as in k_tc_small_hash
+            const int32_t maxu = __shfl_sync(FULL, x, grp * G + (du > 0 ? du - 1 : 0));
+            if (b > HASH_CUT) b = lower_bound(col + rx.x, 0, b, maxu + 1);
+            const int a = du - gl - 1;
+            if (b > SETS_LONG && !eq3_prefers_merge(a, b, 8.0f)) {
+                const int32_t* B = col + rx.x;
+                int lo = 0;
+                for (int i = gl + 1; i < du && lo < b; ++i) {
+                    const int32_t y = col[ru.x + i];
+                    const int p = lower_bound(B, lo, b, y);
+                    lo = p;
+                    if (p < b && B[p] == y) {
+                        atomicAdd(&hcnt[grp * SL + own(y)], 1u);
+                        if (sup) atomicAdd(&sup[rx.x + p], 1u);  // edge (v, y)
+                        ++cs;
+                    }
+                }
+                b = 0;
+            }
+        }
+        __syncwarp();
+        const int32_t xn = gl < run.y ? col[run.x + gl] : INT_MAX;
+        EdgeItems E;
+        const int src = E.gather(b, ce);
+        if (E.cz) {
+            E.lay(__shfl_sync(FULL, b, src), __shfl_sync(FULL, rx.x, src), at);
+            if (lane < E.cz) at[lane].y = src;
+            ce[lane] = 0;
+            __syncwarp();
+            for (int r = 0; r < E.total; r += 64) {
+                const int item = r + lane;
+                int2 e[2];
+                int32_t y[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    e[h] = make_int2(0, 0);
+                    y[h] = INT_MAX;
+                    if (h == 0 || r + 32 < E.total) {
+                        e[h] = at[E.edge_of(r + 32 * h)];
+                        if (item + 32 * h < E.total) y[h] = col[e[h].x + item + 32 * h];
+                    }
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int set = (e[h].y & ~(G - 1)) * (SL / G);
+                    const int slot = y[h] != INT_MAX ? Set{keys + set}(y[h]) : -1;
+                    if (slot >= 0) {
+                        atomicAdd(&hcnt[set + slot], 1u);
+                        atomicAdd(&ce[e[h].y], 1u);
+                        if (sup) atomicAdd(&sup[e[h].x + item + 32 * h], 1u);  // edge (v, y)
+                    }
+                }
+            }
+            __syncwarp();
+            cs += ce[lane];
+        }
+        uint32_t cu = cs;
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) cu += __shfl_xor_sync(FULL, cu, o);
+        if (has) {  // flush the entry's counts, empty its slot
+            const uint32_t cx = hcnt[hs] + cs;
+            if (cx) {
+                atomicAdd(&t[x], (unsigned long long)cx);
+                if (sup) atomicAdd(&sup[ru.x + gl], cx);  // edge (u, x): as v of its edge and as w of others
+            }
+            keys[hs] = SET_EMPTY;
+            hcnt[hs] = 0;
+        }
+        if (gl == 0 && cu) atomicAdd(&t[u], (unsigned long long)cu);
+        __syncwarp();
+        u = un;
+        ru = run;
+        x = xn;
+    }
+}
+
 // Warp per edge: the entries of B = N+(v) (sorted) are probed in a set of the
 // staged N+(u), two per lane per round, stopping above max N+(u); hits add to the
 // set's per-slot counter.  Returns the edge's count (all lanes).
@@ -2443,14 +2576,12 @@ void intersect_impl(const CountBuffers& C, const Strategy& S, cudaEvent_t* ev, c
     const float sf = S.factor[TC_BUCKET_SMALL];
     const int64_t top = C.dplus_bound;  // classes of longer sources are empty: left out
     if (ss == TC_STRAT_HASH) {
-        // sources of at most 16 entries: one edge per lane (Eq. 3 per edge), whose
-        // short merges cost less than building and flushing a set per source
-        k_tc_small<8, SUP><<<L.sms * SMALL_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
-            C.n, C.rowstart, C.rowlen, C.rowinfo, C.col, C.small_list[0], 0, C.t_rank, C.stats, TC_STRAT_AUTO, sf, C.sup);
+        k_tc_small_sets<8, SUP><<<L.sms * SETS_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
+            C.n, C.rowinfo, C.col, C.small_list[0], 0, C.t_rank, C.stats, C.sup);
         count_launch();
         if (top > 8) {
-            k_tc_small<16, SUP><<<L.sms * SMALL_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
-                C.n, C.rowstart, C.rowlen, C.rowinfo, C.col, C.small_list[1], 1, C.t_rank, C.stats, TC_STRAT_AUTO, sf, C.sup);
+            k_tc_small_sets<16, SUP><<<L.sms * SETS_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
+                C.n, C.rowinfo, C.col, C.small_list[1], 1, C.t_rank, C.stats, C.sup);
             count_launch();
         }
         if (top > 16) {

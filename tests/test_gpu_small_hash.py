@@ -1,5 +1,5 @@
-"""The hash-set kernels of the small bucket at the edges of their classes (sources of 17..32
-and 33..256 entries below the hubs), against the oracle (exact)."""
+"""The hash-set kernels of the small bucket at the edges of their classes (sources of 2..8,
+9..16, 17..32 and 33..256 entries below the hubs), against the oracle (exact)."""
 from __future__ import annotations
 
 import numpy as np
@@ -29,8 +29,8 @@ def _fringe(k):
     return BASE + 300, np.concatenate([s, fs]).astype(np.int32), np.concatenate([d, fd]).astype(np.int32)
 
 
-GRAPHS = {f"clique {k}": _clique(k) for k in (15, 16, 17, 31, 32, 33, 64, 255, 256, 257)}
-GRAPHS |= {f"fringe {k}": _fringe(k) for k in (17, 32, 33, 256)}
+GRAPHS = {f"clique {k}": _clique(k) for k in (2, 7, 8, 9, 15, 16, 17, 31, 32, 33, 64, 255, 256, 257)}
+GRAPHS |= {f"fringe {k}": _fringe(k) for k in (2, 8, 9, 16, 17, 32, 33, 256)}
 GRAPHS["uniform"] = (20000, *graphgen.er(20000, 500000, seed=3))
 
 
