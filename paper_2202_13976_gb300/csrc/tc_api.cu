@@ -429,9 +429,10 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
     char* tmp = nullptr;
     Slab work;  // the zeroed counters first: one memset
     work.add(&B.dmulti, nn).add(&B.dupin, nn).add(&B.rowcnt, nn + 1).add(&B.bcount, (size_t)BUCKET_MAX + 1);
-    work.add(&B.bcur, (size_t)BUCKET_MAX);
-    work.add(&B.keys, nn).add(&B.keys_alt, nn).add(&B.bstart, (size_t)BUCKET_MAX + 1).add(&B.pairs, (size_t)m);
+    work.add(&B.keys, nn).add(&B.keys_alt, nn).add(&B.bcap, (size_t)BUCKET_MAX);
+    work.add(&B.bstart, (size_t)BUCKET_MAX + 1).add(&B.bfirst, (size_t)BUCKET_MAX + 1);
     work.add(&tmp, tmp_bytes);
+    if (B.bucket_fill) work.add(&B.pairs, 2 * (size_t)m);
     if ((st = work.alloc(g, &scratch)) != TC_OK) return st;
     const size_t zeroed = (size_t)((char*)B.keys - (char*)B.dmulti);
     B.seg = reinterpret_cast<uint32_t*>(g->small_list[3]);  // free until the plan
@@ -501,6 +502,10 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
         // but for graphs whose rows the direct fill keeps in L2
         const double mean = n > 0 ? 2.0 * (double)m / (double)n : 0.0;
         B.bucket_fill = m >= BUCKET_MIN_M && (double)h.max_deg <= 64.0 * mean;
+        if (B.bucket_fill && (st = dalloc(g, &B.pairs, 2 * (size_t)m, &scratch)) != TC_OK) {
+            free_list(g, &scratch);
+            return st;
+        }
     }
     launch_rank(B, deg_bits, g->L);
     if (bev) cudaEventRecord(bev[BP_RANK], g->stream);

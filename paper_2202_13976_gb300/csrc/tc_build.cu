@@ -337,12 +337,10 @@ __global__ void k_orient_scatter(const int2* __restrict__ oriented, int64_t m,
 
 // Row counts and row fill by buckets of consecutive source ranks (2^shift rows each,
 // nb buckets), with no per-pair global atomic:
-//  k_bucket_count  counts the pairs of each bucket (shared-memory histogram, one
-//                  global atomic per bucket and block) and keeps every pair's
-//                  (source rank, target rank), read back in input order;
-//  k_orient_part   takes PART_TILE pairs per block, groups them by bucket in shared
-//                  memory, reserves each bucket's run with one atomic and writes
-//                  (source, target) into the bucket's segment of `pairs`;
+//  k_bucket_caps   sums the degrees of each bucket's rows, which bound its pairs: the
+//                  buckets' segments of `pairs` are laid out without counting the pairs;
+//  k_orient_part   takes PART_TILE pairs per block, sorts them by bucket in shared memory,
+//                  reserves each bucket's run with one atomic and writes the runs out;
 //  k_bucket_fill   takes one bucket per block: counts its rows in shared memory,
 //                  scans them into rowstart and rowcnt, and moves every pair into its
 //                  row through shared-memory cursors.
@@ -350,111 +348,145 @@ __global__ void k_orient_scatter(const int2* __restrict__ oriented, int64_t m,
 // (BUCKET_ROWS_MAX) and nb is at most BUCKET_MAX.  Skewed graphs take the direct
 // count and scatter above: their heavy rows would pile onto a few buckets and onto
 // single shared-memory counters, while in the direct scatter they stay in cache.
+//
+// A uniform graph of 2^23 vertices, 64 M pairs: a pass that counted the buckets and kept
+// the pairs in rank space, then a partition that wrote each pair by itself, 0.56 + 1.06 ms;
+// one pass that writes runs, 0.74.  Then the fill, 0.52; with buckets claimed one by one and
+// four loads in flight, 0.47.
 constexpr int PART_ITEMS = 16;
-constexpr int PART_THREADS = 1024;  // large tiles: one reservation per bucket and 16384 pairs
+constexpr int PART_THREADS = 512;
 constexpr int PART_TILE = PART_THREADS * PART_ITEMS;
 constexpr int FILL_THREADS = 1024;
+constexpr int FILL_UNROLL = 4;
 
-__global__ void __launch_bounds__(THREADS) k_bucket_count(const int32_t* __restrict__ src,
-                                                          const int32_t* __restrict__ dst, int64_t m, int32_t n,
-                                                          const int32_t* __restrict__ rank, int shift, int nb,
-                                                          uint32_t* __restrict__ bcount, int2* __restrict__ oriented,
-                                                          bool dir_bits) {
-    extern __shared__ uint32_t hist[];  // nb
-    for (int b = threadIdx.x; b < nb; b += THREADS) hist[b] = 0;
+__global__ void __launch_bounds__(THREADS) k_bucket_caps(int32_t n, int shift, const uint32_t* __restrict__ dmulti,
+                                                         uint32_t* __restrict__ bcap) {
+    __shared__ uint32_t part[THREADS / 32];
+    const int64_t r0 = (int64_t)blockIdx.x << shift, r1 = min(r0 + ((int64_t)1 << shift), (int64_t)n);
+    uint32_t s = 0;  // at most twice the pairs
+    for (int64_t r = r0 + threadIdx.x; r < r1; r += THREADS) s += dmulti[r];
+    s = __reduce_add_sync(FULL, s);
+    if (lane_id() == 0) part[threadIdx.x >> 5] = s;
     __syncthreads();
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < m; i0 += PAIR_UNROLL * stride) {
-        int32_t u[PAIR_UNROLL], v[PAIR_UNROLL];
-#pragma unroll
-        for (int k = 0; k < PAIR_UNROLL; ++k) {
-            const int64_t i = i0 + k * stride;
-            u[k] = i < m ? src[i] : 0;
-            v[k] = i < m ? dst[i] : 0;
-        }
-#pragma unroll
-        for (int k = 0; k < PAIR_UNROLL; ++k) {
-            const int64_t i = i0 + k * stride;
-            if (i >= m) break;
-            int2 o = make_int2(-1, -1);  // loop or invalid id: no entry
-            if (u[k] != v[k] && (uint32_t)u[k] < (uint32_t)n && (uint32_t)v[k] < (uint32_t)n) {
-                const int32_t a = rank[u[k]], b = rank[v[k]];
-                o = make_int2(min(a, b), max(a, b));
-                if (dir_bits) o.y = (o.y << 2) | (a < b ? 1 : 2);
-                atomicAdd(&hist[o.x >> shift], 1u);
-            }
-            oriented[i] = o;  // the partition pass reads these instead of gathering ranks again
-        }
+    if (threadIdx.x < 32) {
+        s = __reduce_add_sync(FULL, threadIdx.x < THREADS / 32 ? part[threadIdx.x] : 0u);
+        if (threadIdx.x == 0) bcap[blockIdx.x] = s;
     }
-    __syncthreads();
-    for (int b = threadIdx.x; b < nb; b += THREADS)
-        if (hist[b]) atomicAdd(&bcount[b], hist[b]);
 }
 
-__global__ void __launch_bounds__(PART_THREADS) k_orient_part(const int2* __restrict__ oriented, int64_t m,
-                                                         int shift, int nb, const int64_t* __restrict__ bstart,
-                                                         uint32_t* __restrict__ bcur, int2* __restrict__ pairs,
-                                                         DevStats* stats) {
-    extern __shared__ __align__(8) unsigned char part_sh[];
-    int64_t* base = reinterpret_cast<int64_t*>(part_sh);  // nb
-    uint32_t* hist = reinterpret_cast<uint32_t*>(base + nb);  // nb
+// Shared memory: the tile's pairs by bucket, the buckets' counts and then starts in the
+// tile, and where each bucket's run goes in pairs less its start in the tile.  There are
+// less than 2^32 slots in pairs.
+constexpr size_t PART_SHARED_SM = 220 << 10;  // of an SM, for the blocks it holds
+constexpr size_t part_shared(int nb) { return sizeof(int2) * PART_TILE + 2 * sizeof(uint32_t) * (size_t)nb; }
+
+__global__ void __launch_bounds__(PART_THREADS, 1024 / PART_THREADS)
+    k_orient_part(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int64_t m, int32_t n,
+                  const int32_t* __restrict__ rank, int shift, int nb, const int64_t* __restrict__ bstart,
+                  uint32_t* __restrict__ bcur, int2* __restrict__ pairs, bool dir_bits, DevStats* stats) {
+    extern __shared__ __align__(16) unsigned char part_sh[];
+    int2* const tile = reinterpret_cast<int2*>(part_sh);
+    uint32_t* const first = reinterpret_cast<uint32_t*>(tile + PART_TILE);  // nb
+    uint32_t* const out = first + nb;                                      // nb
+    __shared__ uint32_t part[PART_THREADS / 32];
+    __shared__ int bad;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (threadIdx.x == 0) bad = 0;
+    const int per = (nb + PART_THREADS - 1) / PART_THREADS;
+    const int b0 = min((int)threadIdx.x * per, nb), b1 = min(b0 + per, nb);
     for (int64_t t0 = (int64_t)blockIdx.x * PART_TILE; t0 < m; t0 += (int64_t)gridDim.x * PART_TILE) {
-        for (int b = threadIdx.x; b < nb; b += PART_THREADS) hist[b] = 0;
+        for (int b = threadIdx.x; b < nb; b += PART_THREADS) first[b] = 0;
         __syncthreads();
-        int32_t sv[PART_ITEMS], tv[PART_ITEMS];
+        int2 o[PART_ITEMS];
         uint32_t loc[PART_ITEMS];
 #pragma unroll
         for (int k = 0; k < PART_ITEMS; ++k) {
             const int64_t i = t0 + (int64_t)k * PART_THREADS + threadIdx.x;
-            sv[k] = -1;
-            if (i < m) {
-                const int2 o = oriented[i];
-                sv[k] = o.x;
-                tv[k] = o.y;
-                if (o.x >= 0) loc[k] = atomicAdd(&hist[o.x >> shift], 1u);
-            }
+            o[k] = i < m ? make_int2(src[i], dst[i]) : make_int2(0, 0);
+        }
+#pragma unroll
+        for (int k = 0; k < PART_ITEMS; ++k) {  // loop or invalid id: no entry
+            const bool ok = o[k].x != o[k].y && (uint32_t)o[k].x < (uint32_t)n && (uint32_t)o[k].y < (uint32_t)n;
+            o[k].x = ok ? rank[o[k].x] : -1;
+            o[k].y = ok ? rank[o[k].y] : -1;
+        }
+#pragma unroll
+        for (int k = 0; k < PART_ITEMS; ++k) {
+            const int32_t a = min(o[k].x, o[k].y), c = max(o[k].x, o[k].y);
+            o[k].y = dir_bits ? (c << 2) | (o[k].x < o[k].y ? 1 : 2) : c;
+            o[k].x = a;
+            if (a >= 0) loc[k] = atomicAdd(&first[a >> shift], 1u);
         }
         __syncthreads();
-        for (int b = threadIdx.x; b < nb; b += PART_THREADS) {
-            const uint32_t c = hist[b];
-            if (c) base[b] = bstart[b] + atomicAdd(&bcur[b], c);
+        // exclusive scan over the buckets, thread k those of [k per, (k + 1) per); every
+        // bucket's run is reserved
+        uint32_t sum = 0;
+        for (int b = b0; b < b1; ++b) sum += first[b];
+        const uint32_t inc = warp_inclusive_scan(sum);
+        if (lane == 31) part[w] = inc;
+        __syncthreads();
+        uint32_t run = inc - sum, total = 0;
+        for (int k = 0; k < PART_THREADS / 32; ++k) {
+            if (k < w) run += part[k];
+            total += part[k];
+        }
+        for (int b = b0; b < b1; ++b) {
+            const uint32_t c = first[b];
+            if (c) {
+                const int64_t pos = bstart[b] + atomicAdd(&bcur[b], c);
+                if (pos + c > bstart[b + 1]) bad = 1;  // never, unless the input changes between the passes
+                out[b] = (uint32_t)pos - run;
+            }
+            first[b] = run;
+            run += c;
         }
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < PART_ITEMS; ++k)
-            if (sv[k] >= 0) {
-                const int b = sv[k] >> shift;
-                const int64_t pos = base[b] + loc[k];
-                if (pos < bstart[b + 1])  // always true unless the two passes disagree
-                    pairs[pos] = make_int2(sv[k], tv[k]);
-                else
-                    atomicOr(&stats->err, ERR_OVERFLOW);
-            }
+            if (o[k].x >= 0) tile[first[o[k].x >> shift] + loc[k]] = o[k];
+        __syncthreads();
+        if (bad) {
+            if (threadIdx.x == 0) atomicOr(&stats->err, ERR_OVERFLOW);
+            break;
+        }
+        for (uint32_t i = threadIdx.x; i < total; i += PART_THREADS) {
+            const int2 p = tile[i];
+            pairs[out[p.x >> shift] + i] = p;
+        }
         __syncthreads();
     }
 }
 
 __global__ void __launch_bounds__(FILL_THREADS) k_bucket_fill(int32_t n, int shift, int nb,
                                                               const int64_t* __restrict__ bstart,
-                                                              const int2* __restrict__ pairs,
+                                                              uint32_t* bcount, const int64_t* __restrict__ bfirst,
+                                                              const int2* __restrict__ pairs_all,
                                                               int64_t* __restrict__ rowstart,
                                                               uint32_t* __restrict__ rowcnt, int32_t* __restrict__ col,
                                                               DevStats* stats) {
     extern __shared__ uint32_t rc[];  // 2^shift row counters, then row cursors
     __shared__ uint32_t part[FILL_THREADS / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int b = blockIdx.x; b < nb; b += gridDim.x) {
+    const bool whole = !(stats->err & ERR_OVERFLOW);  // else the partition left out pairs: no rows
+    __shared__ int claimed;
+    for (;;) {  // the buckets differ in size: claimed one by one
+        if (threadIdx.x == 0) claimed = (int)atomicAdd(&bcount[BUCKET_MAX], 1u);
+        __syncthreads();
+        const int b = claimed;
+        if (b >= nb) break;
         const int32_t r0 = b << shift;
         const int nr = (int)min((int64_t)1 << shift, (int64_t)n - r0);
-        const int64_t e0 = bstart[b], e1 = bstart[b + 1];
+        const int2* const pairs = pairs_all + bstart[b];
+        const int64_t e0 = bfirst[b], ne = whole ? bcount[b] : 0;
         for (int i = threadIdx.x; i < nr; i += FILL_THREADS) rc[i] = 0;
         __syncthreads();
-        for (int64_t e = e0 + threadIdx.x; e < e1; e += FILL_THREADS) {
-            const int r = pairs[e].x - r0;
-            if ((unsigned)r < (unsigned)nr)
-                atomicAdd(&rc[r], 1u);
-            else
-                atomicOr(&stats->err, ERR_OVERFLOW);
+        for (int64_t e = threadIdx.x; e < ne; e += FILL_UNROLL * FILL_THREADS) {
+            int r[FILL_UNROLL];
+#pragma unroll
+            for (int k = 0; k < FILL_UNROLL; ++k) r[k] = e + k * FILL_THREADS < ne ? pairs[e + k * FILL_THREADS].x - r0 : -1;
+#pragma unroll
+            for (int k = 0; k < FILL_UNROLL; ++k)
+                if ((unsigned)r[k] < (unsigned)nr) atomicAdd(&rc[r[k]], 1u);
         }
         __syncthreads();
         // exclusive scan of rc[0, nr): thread k sums rows [k*per, (k+1)*per)
@@ -480,14 +512,18 @@ __global__ void __launch_bounds__(FILL_THREADS) k_bucket_fill(int32_t n, int shi
             run += c;
         }
         __syncthreads();
-        for (int64_t e = e0 + threadIdx.x; e < e1; e += FILL_THREADS) {
-            const int2 st = pairs[e];
-            const int r = st.x - r0;
-            if ((unsigned)r < (unsigned)nr) col[e0 + atomicAdd(&rc[r], 1u)] = st.y;
+        for (int64_t e = threadIdx.x; e < ne; e += FILL_UNROLL * FILL_THREADS) {
+            int2 st[FILL_UNROLL];
+#pragma unroll
+            for (int k = 0; k < FILL_UNROLL; ++k)
+                st[k] = e + k * FILL_THREADS < ne ? pairs[e + k * FILL_THREADS] : make_int2(-1, 0);
+#pragma unroll
+            for (int k = 0; k < FILL_UNROLL; ++k)
+                if ((unsigned)(st[k].x - r0) < (unsigned)nr) col[e0 + atomicAdd(&rc[st[k].x - r0], 1u)] = st[k].y;
         }
         __syncthreads();
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) rowstart[n] = bstart[nb];
+    if (blockIdx.x == 0 && threadIdx.x == 0) rowstart[n] = bfirst[nb];
 }
 
 // Simple degree in rank space: distinct out-entries + in-entries before
@@ -985,10 +1021,10 @@ void launch_rank(const BuildBuffers& B, int deg_bits, const Launch& L) {
     k_rank_invert<<<grid_for(B.n, THREADS, L.sms), THREADS, 0, L.stream>>>(sorted, B.n, B.rank, B.dmulti); count_launch();
 }
 
-void bucket_shape(int32_t n, int* shift, int* nb) {
+static void bucket_shape(int32_t n, bool batch, int* shift, int* nb) {
     int bits = 0;
     while (bits < 31 && ((int64_t)1 << bits) < (int64_t)n) ++bits;
-    int sh = bits - BUCKET_BITS;
+    int sh = bits - (batch ? BUCKET_BITS_BATCH : BUCKET_BITS);
     if (sh < 0) sh = 0;
     if (((int64_t)1 << sh) > BUCKET_ROWS_MAX) sh = 0;
     while (((int64_t)1 << sh) < BUCKET_ROWS_MAX && (((int64_t)n + ((int64_t)1 << sh) - 1) >> sh) > BUCKET_MAX) ++sh;
@@ -1000,23 +1036,23 @@ void bucket_shape(int32_t n, int* shift, int* nb) {
 void launch_orient(const BuildBuffers& B, const Launch& L, cudaEvent_t* ev, const PlanStreams* ps) {
     if (B.n <= 0) return;
     int shift = 0, nb = 0;
-    bucket_shape(B.n, &shift, &nb);
+    bucket_shape(B.n, B.seg_vbase != nullptr, &shift, &nb);
     if (B.bucket_fill && nb > 0) {
+        k_bucket_caps<<<nb, THREADS, 0, L.stream>>>(B.n, shift, B.dmulti, B.bcap);
+        count_launch();
+        scan_u32_to_i64(B.bcap, B.bstart, nb, B.tmp, L);
         if (B.m > 0) {
-            k_bucket_count<<<grid_for(B.m, THREADS * PAIR_UNROLL, L.sms, 8), THREADS, sizeof(uint32_t) * nb, L.stream>>>(
-                B.src, B.dst, B.m, B.n, B.rank, shift, nb, B.bcount, B.oriented, B.dir_bits);
+            const int per_sm = (int)(PART_SHARED_SM / part_shared(nb));
+            k_orient_part<<<grid_for(B.m, PART_TILE, L.sms, per_sm < 1024 / PART_THREADS ? per_sm : 1024 / PART_THREADS),
+                            PART_THREADS, part_shared(nb), L.stream>>>(B.src, B.dst, B.m, B.n, B.rank, shift, nb, B.bstart,
+                                                                       B.bcount, B.pairs, B.dir_bits, B.stats);
             count_launch();
         }
-        scan_u32_to_i64(B.bcount, B.bstart, nb, B.tmp, L);
+        scan_u32_to_i64(B.bcount, B.bfirst, nb, B.tmp, L);
         if (ev) cudaEventRecord(ev[BP_COUNT], L.stream);
-        if (B.m > 0) {
-            k_orient_part<<<grid_for(B.m, PART_TILE, L.sms, 1), PART_THREADS, (sizeof(int64_t) + sizeof(uint32_t)) * nb,
-                            L.stream>>>(B.oriented, B.m, shift, nb, B.bstart, B.bcur, B.pairs, B.stats);
-            count_launch();
-        }
-        const int fill_blocks = nb < 4 * L.sms ? nb : 4 * L.sms;
+        const int fill_blocks = nb < 2 * L.sms ? nb : 2 * L.sms;
         k_bucket_fill<<<fill_blocks, FILL_THREADS, sizeof(uint32_t) << shift, L.stream>>>(
-            B.n, shift, nb, B.bstart, B.pairs, B.rowstart, B.rowcnt, B.col, B.stats);
+            B.n, shift, nb, B.bstart, B.bcount, B.bfirst, B.pairs, B.rowstart, B.rowcnt, B.col, B.stats);
         count_launch();
     } else {
         if (B.m > 0) {
@@ -1086,11 +1122,7 @@ cudaError_t build_init_attributes() {
     e = cudaFuncSetAttribute(k_bucket_fill, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              BUCKET_ROWS_MAX * (int)sizeof(uint32_t));
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_orient_part, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             BUCKET_MAX * (int)(sizeof(int64_t) + sizeof(uint32_t)));
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_bucket_count, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                BUCKET_MAX * (int)sizeof(uint32_t));
+    return cudaFuncSetAttribute(k_orient_part, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)part_shared(BUCKET_MAX));
 }
 
 }  // namespace tcg

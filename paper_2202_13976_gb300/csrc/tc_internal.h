@@ -109,7 +109,7 @@ struct BuildBuffers {
     int64_t m;
     int32_t n;
     // scratch
-    uint32_t* dmulti;     // n; this, dupin, rowcnt, bcount and bcur start at zero
+    uint32_t* dmulti;     // n; this, dupin, rowcnt and bcount start at zero
     uint64_t* keys;       // n
     uint64_t* keys_alt;   // n
     uint32_t* rowcnt;     // n + 1
@@ -118,10 +118,11 @@ struct BuildBuffers {
     int32_t* midlist;     // n: rows of 17..256 entries
     int32_t* midlist2;    // n: rows of 257..1024 entries
     uint32_t* dupin;      // n: repeated entries dropped at each target
-    uint32_t* bcount;     // BUCKET_MAX + 1: pairs per source bucket
-    uint32_t* bcur;       // BUCKET_MAX: bucket cursors of the partition pass
-    int64_t* bstart;      // BUCKET_MAX + 1: first pair of each bucket
-    int2* pairs;          // m: (source rank, target rank) grouped by bucket
+    uint32_t* bcount;     // BUCKET_MAX + 1: pairs per source bucket; buckets claimed by the fill
+    uint32_t* bcap;       // BUCKET_MAX: degrees of each bucket's rows
+    int64_t* bstart;      // BUCKET_MAX + 1: first slot of each bucket in pairs
+    int64_t* bfirst;      // BUCKET_MAX + 1: first entry of each bucket in col
+    int2* pairs;          // 2 m (bucket fill): (source rank, target rank) grouped by bucket
     int2* oriented;       // m: (source rank, target rank) in input order ((-1, -1): no entry)
     int64_t row_bound;    // no row has more entries, repeats included
     bool bucket_fill;     // rows counted and filled by source buckets (flat degree distributions)
@@ -162,11 +163,15 @@ void launch_max_deg(const BuildBuffers& B, const Launch& L);
 void launch_rank(const BuildBuffers& B, int deg_bits, const Launch& L);
 void launch_orient(const BuildBuffers& B, const Launch& L, cudaEvent_t* ev = nullptr, const PlanStreams* ps = nullptr);
 // Row fill by source buckets: at most BUCKET_MAX buckets of at most BUCKET_ROWS_MAX
-// rows (2^BUCKET_BITS buckets when that fits); nb = 0 selects the direct fill.
+// rows (2^BUCKET_BITS buckets when that fits); nb = 0 selects the direct fill.  With more
+// buckets the fill finds its second pass over a bucket's pairs in L2, but a tile's runs
+// get shorter.  Partition + fill, 11 / 12 bits: 0.74 + 0.47 / 1.36 + 0.36 ms (uniform, 2^23
+// vertices, 64 M pairs).  A tile of a batch has one or two graphs' pairs, in few buckets:
+// 0.52 + 0.82 / 0.58 + 0.70 / (13 bits) 0.75 + 0.52 (840 graphs, 66 M pairs).
 constexpr int BUCKET_BITS = 11;
+constexpr int BUCKET_BITS_BATCH = 12;
 constexpr int BUCKET_MAX = 8192;
 constexpr int BUCKET_ROWS_MAX = 32768;
-void bucket_shape(int32_t n, int* shift, int* nb);
 cudaError_t build_init_attributes();
 
 // ---- plan + intersect + finalize (tc_intersect.cu) ---------------------------

@@ -41,3 +41,20 @@ def test_repeats_at_hubs(tc, n, hubs, per):
     ref = oracle.triangles(n, s, d)
     for device_io in (False, True):
         assert_matches_oracle(tc, n, s, d, ref=ref, csr=(off, d), device_io=device_io)
+
+
+@pytest.mark.parametrize("m", [8191, 8192, 8193, 40000])
+@pytest.mark.parametrize("n", [2, 300, 4097, 70001])
+def test_bucket_fill_over_batches(tc, n, m):
+    """Batches fill their rows by buckets: tiles of 8192 pairs that end anywhere, buckets of
+    one row and more, every pair of a tile in one bucket."""
+    s, d = graphgen.er_replace(n, m, seed=m)
+    one = np.zeros(m, np.int32)
+    sizes = np.array([n, 2, n], np.int32)
+    off = np.array([0, m, 2 * m, 3 * m], np.int64)
+    with tc.Graph.batch(sizes, off, np.concatenate([s, one, d]), np.concatenate([d, one + 1, s])) as g:
+        T = g.batch_count()
+        t, _ = g.lcc()
+    ref = oracle.triangles(n, s, d)
+    assert [int(x) for x in T] == [ref["T"], 0, ref["T"]]
+    np.testing.assert_array_equal(t, np.concatenate([ref["t"], [0, 0], ref["t"]]))
