@@ -317,10 +317,10 @@ tc_status read_stats(const tc_graph* g, DevStats* h) {
     return TC_OK;
 }
 
-// Pairs from which a flat graph's rows are filled by buckets.  Whole calls on uniform
-// graphs, direct fill / buckets: 20 M pairs 2.05 / 2.10 ms, 40 M 4.20 / 4.05 ms;
-// 32,768 pairs 0.23 / 0.26 ms.
-constexpr int64_t BUCKET_MIN_M = (int64_t)1 << 25;
+// Pairs from which rows are filled by buckets.  Whole calls, direct fill / buckets, uniform
+// and R-MAT graphs: 200,000 pairs 0.28 / 0.29 and 0.36 / 0.35 ms; 1 M 0.34 / 0.35 and
+// 0.54 / 0.50; 4 M 0.75 / 0.73 and 0.95 / 0.90; 32 M 2.65 / 2.18 and 5.30 / 5.08.
+constexpr int64_t BUCKET_MIN_M = (int64_t)1 << 20;
 
 int64_t isqrt(int64_t x) {  // floor of the square root
     int64_t r = (int64_t)std::sqrt((double)x);
@@ -498,10 +498,10 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
         deg_bits = bits_for(h.max_deg);
         B.row_bound = h.max_deg;
         if (g->dplus_bound > (int64_t)h.max_deg) g->dplus_bound = h.max_deg;
-        // flat degree distribution (max degree within 64x the mean): rows through buckets,
-        // but for graphs whose rows the direct fill keeps in L2
+        // rows through buckets, even ones for flat degrees (the largest within 64x the mean)
         const double mean = n > 0 ? 2.0 * (double)m / (double)n : 0.0;
-        B.bucket_fill = m >= BUCKET_MIN_M && (double)h.max_deg <= 64.0 * mean;
+        B.skewed = (double)h.max_deg > 64.0 * mean;
+        B.bucket_fill = m >= BUCKET_MIN_M && (!B.skewed || skewed_buckets_fit(n));
         if (B.bucket_fill && (st = dalloc(g, &B.pairs, 2 * (size_t)m, &scratch)) != TC_OK) {
             free_list(g, &scratch);
             return st;

@@ -335,8 +335,8 @@ __global__ void k_orient_scatter(const int2* __restrict__ oriented, int64_t m,
     if (err && lane_id() == 0) atomicOr(&stats->err, err);
 }
 
-// Row counts and row fill by buckets of consecutive source ranks (2^shift rows each,
-// nb buckets), with no per-pair global atomic:
+// Row counts and row fill by nb buckets of consecutive source ranks, with no per-pair
+// global atomic:
 //  k_bucket_caps   sums the degrees of each bucket's rows, which bound its pairs: the
 //                  buckets' segments of `pairs` are laid out without counting the pairs;
 //  k_orient_part   takes PART_TILE pairs per block, sorts them by bucket in shared memory,
@@ -344,10 +344,11 @@ __global__ void k_orient_scatter(const int2* __restrict__ oriented, int64_t m,
 //  k_bucket_fill   takes one bucket per block: counts its rows in shared memory,
 //                  scans them into rowstart and rowcnt, and moves every pair into its
 //                  row through shared-memory cursors.
-// Used for flat degree distributions when a bucket's rows fit in shared memory
-// (BUCKET_ROWS_MAX) and nb is at most BUCKET_MAX.  Skewed graphs take the direct
-// count and scatter above: their heavy rows would pile onto a few buckets and onto
-// single shared-memory counters, while in the direct scatter they stay in cache.
+// Used when a bucket's rows fit in shared memory (BUCKET_ROWS_MAX) and nb is at most
+// BUCKET_MAX; small and the very largest graphs take the direct count and scatter above.
+// Skewed graphs have buckets of unequal rows (even ones would hold most pairs in a few):
+// R-MAT, 64 M pairs, 1.24 + 0.74 ms for the direct count and scatter and 0.07 for its
+// scans, 1.04 + 0.59 for partition and fill; 16 M pairs, 0.48 against 0.32.
 //
 // A uniform graph of 2^23 vertices, 64 M pairs: a pass that counted the buckets and kept
 // the pairs in rank space, then a partition that wrote each pair by itself, 0.56 + 1.06 ms;
@@ -359,10 +360,57 @@ constexpr int PART_TILE = PART_THREADS * PART_ITEMS;
 constexpr int FILL_THREADS = 1024;
 constexpr int FILL_UNROLL = 4;
 
-__global__ void __launch_bounds__(THREADS) k_bucket_caps(int32_t n, int shift, const uint32_t* __restrict__ dmulti,
+// Buckets in rank order.  Even: 2^shift rows each.  Skewed (degrees differ much, and the
+// rows with many entries have high ranks): by q = n - rank, one row each while q is small,
+// then SKEW_PART buckets for every doubling of q up to 2^SKEW_BITS, then SKEW_ROWS rows each.
+template <bool SKEWED>
+struct Buckets;
+
+template <>
+struct Buckets<false> {
+    int32_t n;
+    int shift;
+    __device__ __forceinline__ int of(int32_t r) const { return r >> shift; }
+    __device__ __forceinline__ void rows(int b, int64_t& r0, int64_t& r1) const {
+        r0 = (int64_t)b << shift;
+        r1 = min(r0 + ((int64_t)1 << shift), (int64_t)n);
+    }
+};
+
+template <>
+struct Buckets<true> {
+    int32_t n;
+    int last;  // index(n), the first bucket's
+    static constexpr int EACH = 2 * SKEW_PART;  // below it one row each
+    static constexpr int LINEAR = (SKEW_BITS - SKEW_PART_BITS + 1) << SKEW_PART_BITS;
+    static __host__ __device__ int index(int32_t q) {  // 1, 2, ... as q grows
+        if (q < EACH) return q;
+        if (q >= 1 << SKEW_BITS) return LINEAR + ((q - (1 << SKEW_BITS)) >> SKEW_ROW_BITS);
+#ifdef __CUDA_ARCH__
+        const int k = 31 - SKEW_PART_BITS - __clz(q);
+#else
+        const int k = 31 - SKEW_PART_BITS - __builtin_clz((unsigned)q);
+#endif
+        return (k << SKEW_PART_BITS) + (q >> k);
+    }
+    __device__ __forceinline__ int of(int32_t r) const { return last - index(n - r); }
+    __device__ __forceinline__ void rows(int b, int64_t& r0, int64_t& r1) const {
+        const int id = last - b;
+        const int k = id < EACH ? 0 : id < LINEAR ? (id >> SKEW_PART_BITS) - 1 : SKEW_ROW_BITS;
+        const int64_t q0 = id < EACH     ? id
+                           : id < LINEAR ? (int64_t)((id & (SKEW_PART - 1)) + SKEW_PART) << k
+                                         : ((int64_t)1 << SKEW_BITS) + ((int64_t)(id - LINEAR) << k);
+        r1 = n - q0 + 1;
+        r0 = max(r1 - ((int64_t)1 << k), (int64_t)0);
+    }
+};
+
+template <bool SKEWED>
+__global__ void __launch_bounds__(THREADS) k_bucket_caps(Buckets<SKEWED> buckets, const uint32_t* __restrict__ dmulti,
                                                          uint32_t* __restrict__ bcap) {
     __shared__ uint32_t part[THREADS / 32];
-    const int64_t r0 = (int64_t)blockIdx.x << shift, r1 = min(r0 + ((int64_t)1 << shift), (int64_t)n);
+    int64_t r0, r1;
+    buckets.rows(blockIdx.x, r0, r1);
     uint32_t s = 0;  // at most twice the pairs
     for (int64_t r = r0 + threadIdx.x; r < r1; r += THREADS) s += dmulti[r];
     s = __reduce_add_sync(FULL, s);
@@ -380,9 +428,10 @@ __global__ void __launch_bounds__(THREADS) k_bucket_caps(int32_t n, int shift, c
 constexpr size_t PART_SHARED_SM = 220 << 10;  // of an SM, for the blocks it holds
 constexpr size_t part_shared(int nb) { return sizeof(int2) * PART_TILE + 2 * sizeof(uint32_t) * (size_t)nb; }
 
+template <bool SKEWED>
 __global__ void __launch_bounds__(PART_THREADS, 1024 / PART_THREADS)
     k_orient_part(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int64_t m, int32_t n,
-                  const int32_t* __restrict__ rank, int shift, int nb, const int64_t* __restrict__ bstart,
+                  const int32_t* __restrict__ rank, Buckets<SKEWED> buckets, int nb, const int64_t* __restrict__ bstart,
                   uint32_t* __restrict__ bcur, int2* __restrict__ pairs, bool dir_bits, DevStats* stats) {
     extern __shared__ __align__(16) unsigned char part_sh[];
     int2* const tile = reinterpret_cast<int2*>(part_sh);
@@ -415,7 +464,7 @@ __global__ void __launch_bounds__(PART_THREADS, 1024 / PART_THREADS)
             const int32_t a = min(o[k].x, o[k].y), c = max(o[k].x, o[k].y);
             o[k].y = dir_bits ? (c << 2) | (o[k].x < o[k].y ? 1 : 2) : c;
             o[k].x = a;
-            if (a >= 0) loc[k] = atomicAdd(&first[a >> shift], 1u);
+            if (a >= 0) loc[k] = atomicAdd(&first[buckets.of(a)], 1u);
         }
         __syncthreads();
         // exclusive scan over the buckets, thread k those of [k per, (k + 1) per); every
@@ -443,7 +492,7 @@ __global__ void __launch_bounds__(PART_THREADS, 1024 / PART_THREADS)
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < PART_ITEMS; ++k)
-            if (o[k].x >= 0) tile[first[o[k].x >> shift] + loc[k]] = o[k];
+            if (o[k].x >= 0) tile[first[buckets.of(o[k].x)] + loc[k]] = o[k];
         __syncthreads();
         if (bad) {
             if (threadIdx.x == 0) atomicOr(&stats->err, ERR_OVERFLOW);
@@ -451,20 +500,21 @@ __global__ void __launch_bounds__(PART_THREADS, 1024 / PART_THREADS)
         }
         for (uint32_t i = threadIdx.x; i < total; i += PART_THREADS) {
             const int2 p = tile[i];
-            pairs[out[p.x >> shift] + i] = p;
+            pairs[out[buckets.of(p.x)] + i] = p;
         }
         __syncthreads();
     }
 }
 
-__global__ void __launch_bounds__(FILL_THREADS) k_bucket_fill(int32_t n, int shift, int nb,
+template <bool SKEWED>
+__global__ void __launch_bounds__(FILL_THREADS) k_bucket_fill(int32_t n, Buckets<SKEWED> buckets, int nb,
                                                               const int64_t* __restrict__ bstart,
                                                               uint32_t* bcount, const int64_t* __restrict__ bfirst,
                                                               const int2* __restrict__ pairs_all,
                                                               int64_t* __restrict__ rowstart,
                                                               uint32_t* __restrict__ rowcnt, int32_t* __restrict__ col,
                                                               DevStats* stats) {
-    extern __shared__ uint32_t rc[];  // 2^shift row counters, then row cursors
+    extern __shared__ uint32_t rc[];  // a bucket's row counters, then row cursors
     __shared__ uint32_t part[FILL_THREADS / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const bool whole = !(stats->err & ERR_OVERFLOW);  // else the partition left out pairs: no rows
@@ -472,10 +522,12 @@ __global__ void __launch_bounds__(FILL_THREADS) k_bucket_fill(int32_t n, int shi
     for (;;) {  // the buckets differ in size: claimed one by one
         if (threadIdx.x == 0) claimed = (int)atomicAdd(&bcount[BUCKET_MAX], 1u);
         __syncthreads();
-        const int b = claimed;
-        if (b >= nb) break;
-        const int32_t r0 = b << shift;
-        const int nr = (int)min((int64_t)1 << shift, (int64_t)n - r0);
+        const int b = nb - 1 - claimed;  // the highest ranks first, whose buckets may be the largest
+        if (b < 0) break;
+        int64_t r0_, r1_;
+        buckets.rows(b, r0_, r1_);
+        const int32_t r0 = (int32_t)r0_;
+        const int nr = (int)(r1_ - r0_);
         const int2* const pairs = pairs_all + bstart[b];
         const int64_t e0 = bfirst[b], ne = whole ? bcount[b] : 0;
         for (int i = threadIdx.x; i < nr; i += FILL_THREADS) rc[i] = 0;
@@ -1033,27 +1085,37 @@ static void bucket_shape(int32_t n, bool batch, int* shift, int* nb) {
     *nb = b <= BUCKET_MAX ? (int)b : 0;  // 0: too many rows for the bucket path
 }
 
+template <bool SKEWED>
+static void launch_buckets(const BuildBuffers& B, const Launch& L, cudaEvent_t* ev, Buckets<SKEWED> buckets, int nb,
+                           int max_rows) {
+    k_bucket_caps<SKEWED><<<nb, THREADS, 0, L.stream>>>(buckets, B.dmulti, B.bcap);
+    count_launch();
+    scan_u32_to_i64(B.bcap, B.bstart, nb, B.tmp, L);
+    if (B.m > 0) {
+        const int fit = (int)(PART_SHARED_SM / part_shared(nb)), most = 1024 / PART_THREADS;
+        k_orient_part<SKEWED><<<grid_for(B.m, PART_TILE, L.sms, fit < most ? fit : most), PART_THREADS, part_shared(nb),
+                                L.stream>>>(B.src, B.dst, B.m, B.n, B.rank, buckets, nb, B.bstart, B.bcount, B.pairs,
+                                            B.dir_bits, B.stats);
+        count_launch();
+    }
+    scan_u32_to_i64(B.bcount, B.bfirst, nb, B.tmp, L);
+    if (ev) cudaEventRecord(ev[BP_COUNT], L.stream);
+    k_bucket_fill<SKEWED><<<nb < 2 * L.sms ? nb : 2 * L.sms, FILL_THREADS, sizeof(uint32_t) * (size_t)max_rows, L.stream>>>(
+        B.n, buckets, nb, B.bstart, B.bcount, B.bfirst, B.pairs, B.rowstart, B.rowcnt, B.col, B.stats);
+    count_launch();
+}
+
+bool skewed_buckets_fit(int32_t n) { return n > 0 && Buckets<true>::index(n) <= BUCKET_MAX; }
+
 void launch_orient(const BuildBuffers& B, const Launch& L, cudaEvent_t* ev, const PlanStreams* ps) {
     if (B.n <= 0) return;
     int shift = 0, nb = 0;
     bucket_shape(B.n, B.seg_vbase != nullptr, &shift, &nb);
-    if (B.bucket_fill && nb > 0) {
-        k_bucket_caps<<<nb, THREADS, 0, L.stream>>>(B.n, shift, B.dmulti, B.bcap);
-        count_launch();
-        scan_u32_to_i64(B.bcap, B.bstart, nb, B.tmp, L);
-        if (B.m > 0) {
-            const int per_sm = (int)(PART_SHARED_SM / part_shared(nb));
-            k_orient_part<<<grid_for(B.m, PART_TILE, L.sms, per_sm < 1024 / PART_THREADS ? per_sm : 1024 / PART_THREADS),
-                            PART_THREADS, part_shared(nb), L.stream>>>(B.src, B.dst, B.m, B.n, B.rank, shift, nb, B.bstart,
-                                                                       B.bcount, B.pairs, B.dir_bits, B.stats);
-            count_launch();
-        }
-        scan_u32_to_i64(B.bcount, B.bfirst, nb, B.tmp, L);
-        if (ev) cudaEventRecord(ev[BP_COUNT], L.stream);
-        const int fill_blocks = nb < 2 * L.sms ? nb : 2 * L.sms;
-        k_bucket_fill<<<fill_blocks, FILL_THREADS, sizeof(uint32_t) << shift, L.stream>>>(
-            B.n, shift, nb, B.bstart, B.bcount, B.bfirst, B.pairs, B.rowstart, B.rowcnt, B.col, B.stats);
-        count_launch();
+    if (B.bucket_fill && B.skewed) {
+        const int last = Buckets<true>::index(B.n);
+        launch_buckets(B, L, ev, Buckets<true>{B.n, last}, last, SKEW_ROWS);
+    } else if (B.bucket_fill && nb > 0) {
+        launch_buckets(B, L, ev, Buckets<false>{B.n, shift}, nb, 1 << shift);
     } else {
         if (B.m > 0) {
             k_orient_count<<<grid_for(B.m, THREADS, L.sms), THREADS, 0, L.stream>>>(B.src, B.dst, B.m, B.n, B.rank,
@@ -1119,10 +1181,13 @@ cudaError_t build_init_attributes() {
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_rank_one, cudaFuncAttributeMaxDynamicSharedMemorySize, RANK_HIST_BYTES);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_bucket_fill, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(k_bucket_fill<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              BUCKET_ROWS_MAX * (int)sizeof(uint32_t));
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_orient_part, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)part_shared(BUCKET_MAX));
+    e = cudaFuncSetAttribute(k_orient_part<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)part_shared(BUCKET_MAX));
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_orient_part<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)part_shared(BUCKET_MAX));
 }
 
 }  // namespace tcg

@@ -125,7 +125,8 @@ struct BuildBuffers {
     int2* pairs;          // 2 m (bucket fill): (source rank, target rank) grouped by bucket
     int2* oriented;       // m: (source rank, target rank) in input order ((-1, -1): no entry)
     int64_t row_bound;    // no row has more entries, repeats included
-    bool bucket_fill;     // rows counted and filled by source buckets (flat degree distributions)
+    bool bucket_fill;     // rows counted and filled by source buckets
+    bool skewed;          // buckets for skewed degrees
     // directed input (tc_directed_lcc): every entry is (target rank << 2) | direction
     // bit of its pair (1: source rank below target rank, 2: above), so a pair read in
     // both directions leaves two entries; repeats are dropped as usual, but not
@@ -171,6 +172,15 @@ void launch_orient(const BuildBuffers& B, const Launch& L, cudaEvent_t* ev = nul
 constexpr int BUCKET_BITS = 11;
 constexpr int BUCKET_BITS_BATCH = 12;
 constexpr int BUCKET_MAX = 8192;
+// Skewed buckets (tc_build.cu).  Partition + fill for R-MAT graphs of 64 M and 16 M pairs:
+// 1.04 + 0.59 and 0.21 + 0.10 ms; with 64 instead of 128 buckets for every doubling
+// 0.82 + 0.77 and 0.18 + 0.13.
+constexpr int SKEW_BITS = 20;
+constexpr int SKEW_PART_BITS = 7;
+constexpr int SKEW_ROW_BITS = 13;
+constexpr int SKEW_PART = 1 << SKEW_PART_BITS, SKEW_ROWS = 1 << SKEW_ROW_BITS;
+static_assert(SKEW_BITS - 1 - SKEW_PART_BITS <= SKEW_ROW_BITS, "no bucket of more than SKEW_ROWS rows");
+bool skewed_buckets_fit(int32_t n);
 constexpr int BUCKET_ROWS_MAX = 32768;
 cudaError_t build_init_attributes();
 

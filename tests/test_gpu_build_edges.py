@@ -58,3 +58,16 @@ def test_bucket_fill_over_batches(tc, n, m):
     ref = oracle.triangles(n, s, d)
     assert [int(x) for x in T] == [ref["T"], 0, ref["T"]]
     np.testing.assert_array_equal(t, np.concatenate([ref["t"], [0, 0], ref["t"]]))
+
+
+@pytest.mark.parametrize("n,skewed", [(2000, False), (257, True), (300, True), (4097, True), ((1 << 20) - 1, True),
+                                      (1 << 20, True), ((1 << 20) + 1, True), ((1 << 20) + 8193, True)])
+def test_bucket_fill_of_large_graphs(tc, n, skewed):
+    """Rows filled by buckets, even ones and those for skewed degrees at the edges of their
+    sizes: half of the pairs at one vertex, some of them repeated."""
+    m = 1 << 20
+    s, d = graphgen.er_replace(n, m, seed=n)
+    if skewed:
+        s[::2] = 0
+        s[1:4000:2], d[1:4000:2] = n - 1, n - 2
+    assert_matches_oracle(tc, n, s, d, device_io=True)
