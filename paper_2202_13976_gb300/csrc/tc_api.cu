@@ -432,7 +432,9 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
     work.add(&B.keys, nn).add(&B.keys_alt, nn).add(&B.bcap, (size_t)BUCKET_MAX);
     work.add(&B.bstart, (size_t)BUCKET_MAX + 1).add(&B.bfirst, (size_t)BUCKET_MAX + 1);
     work.add(&tmp, tmp_bytes);
-    if (B.bucket_fill) work.add(&B.pairs, 2 * (size_t)m);
+    // single graphs decide on buckets once the degrees are known; where both kinds fit, which
+    // is not for the very largest n only, the pairs are allocated ahead
+    if (B.bucket_fill || (m >= BUCKET_MIN_M && skewed_buckets_fit(n))) work.add(&B.pairs, 2 * (size_t)m);
     if ((st = work.alloc(g, &scratch)) != TC_OK) return st;
     const size_t zeroed = (size_t)((char*)B.keys - (char*)B.dmulti);
     B.seg = reinterpret_cast<uint32_t*>(g->small_list[3]);  // free until the plan
@@ -502,7 +504,7 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
         const double mean = n > 0 ? 2.0 * (double)m / (double)n : 0.0;
         B.skewed = (double)h.max_deg > 64.0 * mean;
         B.bucket_fill = m >= BUCKET_MIN_M && (!B.skewed || skewed_buckets_fit(n));
-        if (B.bucket_fill && (st = dalloc(g, &B.pairs, 2 * (size_t)m, &scratch)) != TC_OK) {
+        if (B.bucket_fill && !B.pairs && (st = dalloc(g, &B.pairs, 2 * (size_t)m, &scratch)) != TC_OK) {
             free_list(g, &scratch);
             return st;
         }

@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(WIN_THREADS) k_win_build(int32_t n, Windows T,
 // memory counters give each entry its offset, then one global atomic per hub and
 // tile reserves the tile's run; the other hubs take their slot from a global
 // cursor per entry.  Records of one tile stay together, nearly in source order.
-constexpr int SCAT_THREADS = 256;
+constexpr int SCAT_THREADS = 1024;  // 256 take 4 to 8 % longer (more reservations)
 constexpr int SCAT_ITEMS = 8;  // entries per thread and tile (two 16-byte loads)
 constexpr int SCAT_TILE = SCAT_THREADS * SCAT_ITEMS;
 constexpr int SCAT_TOP = 2048;
@@ -564,7 +564,7 @@ __global__ void __launch_bounds__(SCAT_THREADS) k_hub_scatter(int32_t n, int32_t
                                                               uint2* __restrict__ in_rec, int32_t src_lo,
                                                               int32_t src_hi, DevStats* stats) {
     __shared__ uint32_t lcnt[SCAT_TOP];
-    __shared__ int64_t gbase[SCAT_TOP];
+    __shared__ uint32_t gbase[SCAT_TOP];  // slots are below 2^31
     const int32_t R = n - (int32_t)stats->hub_count;
     const int32_t c0 = n - (int32_t)stats->core_n;  // rows of the dense core are counted there
     const int top = min((int)stats->hub_count, SCAT_TOP);
@@ -603,14 +603,14 @@ __global__ void __launch_bounds__(SCAT_THREADS) k_hub_scatter(int32_t n, int32_t
         }
         // the slot reservations of all items first, so that their round trips overlap,
         // then the records of the hubs below the top ones
-        unsigned long long gslot[SCAT_ITEMS];
+        uint32_t gslot[SCAT_ITEMS];
 #pragma unroll
         for (int e = 0; e < SCAT_ITEMS; ++e) {
             gslot[e] = 0;
             if (x[e] >= T0)
                 loc[e] = atomicAdd(&lcnt[x[e] - T0], 1u);
             else if (x[e] >= R)
-                gslot[e] = atomicAdd(&cur[x[e] - H0], 1ull);
+                gslot[e] = (uint32_t)atomicAdd(&cur[x[e] - H0], 1ull);
         }
 #pragma unroll
         for (int e = 0; e < SCAT_ITEMS; ++e) {
@@ -623,13 +623,13 @@ __global__ void __launch_bounds__(SCAT_THREADS) k_hub_scatter(int32_t n, int32_t
         __syncthreads();
         for (int h = threadIdx.x; h < top; h += SCAT_THREADS) {
             const uint32_t c = lcnt[h];
-            if (c) gbase[h] = (int64_t)atomicAdd(&cur[T0 + h - H0], (unsigned long long)c);
+            if (c) gbase[h] = (uint32_t)atomicAdd(&cur[T0 + h - H0], (unsigned long long)c);
         }
         __syncthreads();
 #pragma unroll
         for (int e = 0; e < SCAT_ITEMS; ++e) {
             if (x[e] < T0) continue;
-            const int64_t slot = gbase[x[e] - T0] + loc[e];
+            const uint32_t slot = gbase[x[e] - T0] + loc[e];
             if (slot < total)
                 in_rec[slot] = make_uint2((uint32_t)u[e], (uint32_t)len[e]);
             else
