@@ -69,12 +69,26 @@ __global__ void k_expand_csr(const int64_t* __restrict__ offsets, int32_t n, int
 // blocks add to different graphs' counts (a batch of 840 graphs, 66 M pairs: 1.08 ms with
 // the pairs strided over the grid, 0.54 so).
 constexpr int PAIR_UNROLL = 8;  // pairs per thread and round in the pair passes
-constexpr int DEG_SLOTS = 4096;
 constexpr int DEG_PROBES = 4;
+// Threads of a block and slots of its table (log2), for few pairs and for many: one block
+// and table per SM hold more of the frequent vertices and flush less.  4 x 4096 / 1 x 16384
+// slots per SM: R-MAT graphs of 1 M, 16 M and 64 M pairs 26 / 16, 227 / 150 and 970 / 790
+// us; a uniform graph of 64 M pairs, whose increments go to L2 one by one, 0.62 ms either
+// way.  Clearing and flushing 16384 slots costs a few us, too much for small graphs.
+struct DegSmall {
+    static constexpr int THREADS_ = 256, LG = 12;
+};
+struct DegLarge {
+    static constexpr int THREADS_ = 1024, LG = 14;
+};
+constexpr int64_t DEG_LARGE_M = (int64_t)1 << 20;
+template <class D>
+constexpr size_t deg_shared() { return (sizeof(int32_t) + sizeof(uint32_t)) << D::LG; }
 constexpr int32_t INGEST_MAX_N = 32768;  // the last block reads this many degrees in about the time of a launch
 
+template <int LG>
 __device__ __forceinline__ void deg_add(int32_t x, int32_t* hk, uint32_t* hc, uint32_t* __restrict__ dmulti) {
-    unsigned h = ((unsigned)x * 0x9e3779b1u) >> (32 - 12);
+    unsigned h = ((unsigned)x * 0x9e3779b1u) >> (32 - LG);
 #pragma unroll
     for (int k = 0; k < DEG_PROBES; ++k) {
         int32_t cur = hk[h];
@@ -83,50 +97,50 @@ __device__ __forceinline__ void deg_add(int32_t x, int32_t* hk, uint32_t* hc, ui
             atomicAdd(&hc[h], 1u);
             return;
         }
-        h = (h + 1) & (DEG_SLOTS - 1);
+        h = (h + 1) & ((1u << LG) - 1u);
     }
     atomicAdd(&dmulti[x], 1u);
 }
 
-template <bool TAKE_MAX>
-__global__ void __launch_bounds__(THREADS) k_canon_degree(const int32_t* __restrict__ src,
-                                                          const int32_t* __restrict__ dst, int64_t m, int32_t n,
-                                                          uint32_t* __restrict__ dmulti, DevStats* stats) {
-    static_assert(DEG_SLOTS == 1 << 12, "hash width");
-    __shared__ int32_t hk[DEG_SLOTS];
-    __shared__ uint32_t hc[DEG_SLOTS];
-    for (int i = threadIdx.x; i < DEG_SLOTS; i += blockDim.x) {
+template <class D, bool TAKE_MAX>
+__global__ void __launch_bounds__(D::THREADS_) k_canon_degree(const int32_t* __restrict__ src,
+                                                             const int32_t* __restrict__ dst, int64_t m, int32_t n,
+                                                             uint32_t* __restrict__ dmulti, DevStats* stats) {
+    constexpr int T = D::THREADS_, SLOTS = 1 << D::LG;
+    extern __shared__ int32_t hk[];
+    uint32_t* const hc = reinterpret_cast<uint32_t*>(hk + SLOTS);
+    for (int i = threadIdx.x; i < SLOTS; i += T) {
         hk[i] = -1;
         hc[i] = 0;
     }
     __syncthreads();
     unsigned long long loops = 0;
     int err = 0;
-    const int64_t per = ((m + gridDim.x - 1) / gridDim.x + THREADS - 1) / THREADS * THREADS;
+    const int64_t per = ((m + gridDim.x - 1) / gridDim.x + T - 1) / T * T;
     const int64_t end = min(m, (blockIdx.x + 1) * per);
-    for (int64_t i0 = blockIdx.x * per + threadIdx.x; i0 < end; i0 += PAIR_UNROLL * THREADS) {
+    for (int64_t i0 = blockIdx.x * per + threadIdx.x; i0 < end; i0 += PAIR_UNROLL * T) {
         int32_t a[PAIR_UNROLL], c[PAIR_UNROLL];
 #pragma unroll
         for (int k = 0; k < PAIR_UNROLL; ++k) {
-            const int64_t i = i0 + k * THREADS;
+            const int64_t i = i0 + k * T;
             a[k] = i < end ? src[i] : 0;
             c[k] = i < end ? dst[i] : 0;
         }
 #pragma unroll
         for (int k = 0; k < PAIR_UNROLL; ++k) {
-            if (i0 + k * THREADS >= end) break;
+            if (i0 + k * T >= end) break;
             if ((uint32_t)a[k] >= (uint32_t)n || (uint32_t)c[k] >= (uint32_t)n) {
                 err = ERR_BAD_ID;
             } else if (a[k] == c[k]) {
                 ++loops;
             } else {
-                deg_add(a[k], hk, hc, dmulti);
-                deg_add(c[k], hk, hc, dmulti);
+                deg_add<D::LG>(a[k], hk, hc, dmulti);
+                deg_add<D::LG>(c[k], hk, hc, dmulti);
             }
         }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < DEG_SLOTS; i += blockDim.x)
+    for (int i = threadIdx.x; i < SLOTS; i += T)
         if (hc[i]) atomicAdd(&dmulti[hk[i]], hc[i]);
     loops = warp_sum(loops);
     err = __reduce_or_sync(FULL, err);
@@ -143,7 +157,7 @@ __global__ void __launch_bounds__(THREADS) k_canon_degree(const int32_t* __restr
         __syncthreads();
         if (!last) return;
         uint32_t mx = 0;
-        for (int i = threadIdx.x; i < n; i += THREADS) mx = max(mx, __ldcg(&dmulti[i]));
+        for (int i = threadIdx.x; i < n; i += T) mx = max(mx, __ldcg(&dmulti[i]));
         mx = __reduce_max_sync(FULL, mx);
         if (lane_id() == 0 && mx) atomicMax(&stats->max_deg, mx);
     }
@@ -987,13 +1001,21 @@ void launch_expand_csr(const int64_t* offsets, int32_t n, int32_t* rows, DevStat
     k_expand_csr<<<grid_for((int64_t)n * 32, THREADS, L.sms), THREADS, 0, L.stream>>>(offsets, n, rows, stats); count_launch();
 }
 
+template <class D>
+static void launch_ingest_as(const BuildBuffers& B, int64_t first, int64_t count, bool take_max, const Launch& L) {
+    const auto kernel = take_max ? k_canon_degree<D, true> : k_canon_degree<D, false>;
+    kernel<<<grid_for(count, D::THREADS_, L.sms, 1024 / D::THREADS_), D::THREADS_, deg_shared<D>(), L.stream>>>(
+        B.src + first, B.dst + first, count, B.n, B.dmulti, B.stats);
+    count_launch();
+}
+
 static void launch_ingest(const BuildBuffers& B, int64_t first, int64_t count, bool take_max, const Launch& L) {
     if (count <= 0) return;
-    // 32 KB of shared memory per block: four blocks per SM stay resident
-    const auto kernel = take_max ? k_canon_degree<true> : k_canon_degree<false>;
-    kernel<<<grid_for(count, THREADS, L.sms, 4), THREADS, 0, L.stream>>>(B.src + first, B.dst + first, count, B.n,
-                                                                       B.dmulti, B.stats);
-    count_launch();
+    // a batch's blocks should not span many graphs
+    if (count >= DEG_LARGE_M && !B.seg_vbase)
+        launch_ingest_as<DegLarge>(B, first, count, take_max, L);
+    else
+        launch_ingest_as<DegSmall>(B, first, count, take_max, L);
 }
 
 void launch_canon_degree_part(const BuildBuffers& B, int64_t first, int64_t count, const Launch& L) {
@@ -1183,6 +1205,12 @@ cudaError_t build_init_attributes() {
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_bucket_fill<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              BUCKET_ROWS_MAX * (int)sizeof(uint32_t));
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_canon_degree<DegLarge, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)deg_shared<DegLarge>());
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_canon_degree<DegLarge, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)deg_shared<DegLarge>());
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_orient_part<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)part_shared(BUCKET_MAX));
     if (e != cudaSuccess) return e;
