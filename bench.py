@@ -365,10 +365,10 @@ def run_ours(args, rank, world, local):
     # dominant intersection kernel and its roofline (algorithmic bytes per oriented
     # edge: 4 (d+u + d+v) adjacency bytes + 8 edge bytes + 16 offset bytes)
     phase = {k: statistics.mean(t[k] for t in timings) for k in timings[0]}
-    # each bucket phase, timed by events around its launches: small = the lane-per-edge
-    # kernels for sources of at most 16 entries and the hash kernels for longer ones
-    # (the default strategy), hub = the dense-core count followed by the hub kernel
-    small_name = ("k_tc_small<8>+k_tc_small<16>+k_tc_small_hash<32,64>+k_tc_small_hash<32,512>"
+    # each bucket phase, timed by events around its launches: small = the hash kernels of
+    # its four classes (the default strategy), hub = the dense-core count followed by the
+    # hub kernels
+    small_name = ("k_tc_small_sets<8>+k_tc_small_sets<16>+k_tc_small_hash<8>+k_tc_small_hash<9>"
                   if not args.strategy or "small:" not in args.strategy
                   else "k_tc_small<8>+k_tc_small<16>+k_tc_small<32>+k_tc_small_wide")
     kernels = {small_name: ("small_ms", "small"), "k_tc_cta": ("cta_ms", "cta"),

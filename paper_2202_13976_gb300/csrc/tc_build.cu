@@ -72,8 +72,8 @@ constexpr int PAIR_UNROLL = 8;  // pairs per thread and round in the pair passes
 constexpr int DEG_PROBES = 4;
 // Threads of a block and slots of its table (log2), for few pairs and for many: one block
 // and table per SM hold more of the frequent vertices and flush less.  4 x 4096 / 1 x 16384
-// slots per SM: R-MAT graphs of 1 M, 16 M and 64 M pairs 26 / 16, 227 / 150 and 970 / 790
-// us; a uniform graph of 64 M pairs, whose increments go to L2 one by one, 0.62 ms either
+// slots per SM: R-MAT graphs of 1 M, 17 M and 67 M pairs 26 / 16, 227 / 150 and 970 / 790
+// us; a uniform graph of 60 M pairs, whose increments go to L2 one by one, 0.62 ms either
 // way.  Clearing and flushing 16384 slots costs a few us, too much for small graphs.
 struct DegSmall {
     static constexpr int THREADS_ = 256, LG = 12;
@@ -361,10 +361,10 @@ __global__ void k_orient_scatter(const int2* __restrict__ oriented, int64_t m,
 // Used when a bucket's rows fit in shared memory (BUCKET_ROWS_MAX) and nb is at most
 // BUCKET_MAX; small and the very largest graphs take the direct count and scatter above.
 // Skewed graphs have buckets of unequal rows (even ones would hold most pairs in a few):
-// R-MAT, 64 M pairs, 1.24 + 0.74 ms for the direct count and scatter and 0.07 for its
-// scans, 1.04 + 0.59 for partition and fill; 16 M pairs, 0.48 against 0.32.
+// R-MAT, 67 M pairs, 1.24 + 0.74 ms for the direct count and scatter and 0.07 for its
+// scans, 1.04 + 0.59 for partition and fill; 17 M pairs, 0.48 against 0.32.
 //
-// A uniform graph of 2^23 vertices, 64 M pairs: a pass that counted the buckets and kept
+// A uniform graph of 2^23 vertices, 60 M pairs: a pass that counted the buckets and kept
 // the pairs in rank space, then a partition that wrote each pair by itself, 0.56 + 1.06 ms;
 // one pass that writes runs, 0.74.  Then the fill, 0.52; with buckets claimed one by one and
 // four loads in flight, 0.47.
@@ -790,7 +790,7 @@ __global__ void __launch_bounds__(256, 4) k_segsort_thread(int32_t n, const int6
         if (lng) longlist[pl] = (int32_t)r;
         // 32 short rows lie end to end: read and written by the warp through shared memory
         // (one row per lane from global memory: 333 us for a uniform graph of 2^23 vertices and
-        // 64 M pairs, 245 so)
+        // 60 M pairs, 245 so)
         const int64_t base = r < n && len <= 16 ? rowstart[r] : 0;
         const int64_t first = __shfl_sync(FULL, base, 0);
         const int off = (int)(base - first), span = __shfl_sync(FULL, off + len, 31);

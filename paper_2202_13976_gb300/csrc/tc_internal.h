@@ -167,12 +167,12 @@ void launch_orient(const BuildBuffers& B, const Launch& L, cudaEvent_t* ev = nul
 // rows (2^BUCKET_BITS buckets when that fits); nb = 0 selects the direct fill.  With more
 // buckets the fill finds its second pass over a bucket's pairs in L2, but a tile's runs
 // get shorter.  Partition + fill, 11 / 12 bits: 0.74 + 0.47 / 1.36 + 0.36 ms (uniform, 2^23
-// vertices, 64 M pairs).  A tile of a batch has one or two graphs' pairs, in few buckets:
+// vertices, 60 M pairs).  A tile of a batch has one or two graphs' pairs, in few buckets:
 // 0.52 + 0.82 / 0.58 + 0.70 / (13 bits) 0.75 + 0.52 (840 graphs, 66 M pairs).
 constexpr int BUCKET_BITS = 11;
 constexpr int BUCKET_BITS_BATCH = 12;
 constexpr int BUCKET_MAX = 8192;
-// Skewed buckets (tc_build.cu).  Partition + fill for R-MAT graphs of 64 M and 16 M pairs:
+// Skewed buckets (tc_build.cu).  Partition + fill for R-MAT graphs of 67 M and 17 M pairs:
 // 1.04 + 0.59 and 0.21 + 0.10 ms; with 64 instead of 128 buckets for every doubling
 // 0.82 + 0.77 and 0.18 + 0.13.
 constexpr int SKEW_BITS = 20;
@@ -185,8 +185,8 @@ constexpr int BUCKET_ROWS_MAX = 32768;
 cudaError_t build_init_attributes();
 
 // ---- plan + intersect + finalize (tc_intersect.cu) ---------------------------
-// Buckets (include/tc.h): small lists (push, lane per edge), large lists (push,
-// block per source vertex), hubs (pull, block per staged hub list).
+// Buckets (include/tc.h): small lists (push, hash sets or a lane per edge), large lists
+// (push, block per source vertex), hubs (pull, staged hub lists).
 struct Strategy {
     int strat[TC_NUM_BUCKETS];
     float factor[TC_NUM_BUCKETS];

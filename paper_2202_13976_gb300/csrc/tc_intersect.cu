@@ -18,10 +18,12 @@
 //         (Sec. IV-B, Observations 1 and 2): the list that most edges need is read
 //         from memory once and reused by all of them.  t[w] increments of the highest
 //         ranks are summed in shared memory.
-//  small  other edges whose source has 2 <= |N+(u)| <= 32: a group of 8, 16 or 32
-//         lanes stages N+(u); lane j intersects edge j sequentially, by SSI (Alg. 2)
-//         or binary search (Alg. 1), chosen per edge by Eq. 3.
-//  block  other edges whose source has |N+(u)| > 32: one thread block stages N+(u),
+//  small  other edges whose source has 2 <= |N+(u)| <= 256.  HASH (the default): N+(u)
+//         becomes a hash set in shared memory, which the rows N+(v) of its edges, laid end
+//         to end, are probed in.  Else a group of 8, 16 or 32 lanes stages N+(u) and lane j
+//         intersects edge j sequentially, by SSI (Alg. 2) or binary search (Alg. 1), or
+//         chosen per edge by Eq. 3.
+//  block  other edges whose source has |N+(u)| > 256: one thread block stages N+(u),
 //         one warp per edge, methods:
 //           MERGE   merge path: the merge of A (suffix) and B = N+(v) is cut into 32
 //                   equal diagonal ranges, one per lane, each running Alg. 2
@@ -1245,7 +1247,7 @@ __global__ void __launch_bounds__(SMALL_WARPS * 32, SUP ? 4 : HASH_BLOCKS)
 // support once.
 //
 // Bound by the random sectors of row records and rows: a uniform graph of 2^23 vertices and
-// 64 M pairs, sources of up to 8 and 9..16 entries: a merge per lane, 10 to 12 lanes of 32
+// 60 M pairs, sources of up to 8 and 9..16 entries: a merge per lane, 10 to 12 lanes of 32
 // active, 0.66 and 1.20 ms; this, 0.47 and 0.75 (the second reads 3.8 GB).  A batch of 840
 // graphs, 66 M pairs: 0.43 and 0.90, now 0.48 and 0.76.  6 blocks per SM (37 registers)
 // instead of 8 take 10 to 20 % longer.
