@@ -401,19 +401,21 @@ __device__ __forceinline__ bool scatter_by_tiles(const int64_t* __restrict__ hub
     return 4 * hub_start[hub_cap] >= rowstart[c0];
 }
 
-// Source row of every entry of the non-core rows (whole row capacity, so that the
+// Source row of every entry of the counted non-core rows (whole row capacity, so that the
 // slots left free by deduplication also name a valid row).  A lane writes its own
 // row when it holds at most 32 entries; longer rows are written by the whole warp.
 __global__ void k_row_of(int32_t n, int32_t hub_cap, const int64_t* __restrict__ rowstart,
-                         const int64_t* __restrict__ hub_start, int32_t* __restrict__ rowof, const DevStats* stats) {
+                         const int64_t* __restrict__ hub_start, int32_t* __restrict__ rowof, int32_t src_lo,
+                         int32_t src_hi, const DevStats* stats) {
     const int32_t c0 = n - (int32_t)stats->core_n;
     if (!scatter_by_tiles(hub_start, hub_cap, rowstart, c0)) return;
     const int lane = lane_id();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int32_t end = min(src_hi, c0);
     // the loop bound is uniform across a warp, as the ballot needs all 32 lanes
-    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); b < c0; b += stride) {
+    for (int64_t b = src_lo + (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); b < end; b += stride) {
         const int64_t u = b + lane;
-        const int64_t a0 = u < c0 ? rowstart[u] : 0, a1 = u < c0 ? rowstart[u + 1] : 0;
+        const int64_t a0 = u < end ? rowstart[u] : 0, a1 = u < end ? rowstart[u + 1] : 0;
         const bool longrow = a1 - a0 > 32;
         if (!longrow)
             for (int64_t p = a0; p < a1; ++p) rowof[p] = (int32_t)u;
@@ -573,9 +575,10 @@ __global__ void __launch_bounds__(SCAT_THREADS) k_hub_scatter(int32_t n, int32_t
     const int32_t T0 = n - top;  // top hubs: ranks T0 .. n-1 (all hubs)
     const int32_t H0 = n - hub_cap;  // rank of hub slot 0
     if (!scatter_by_tiles(hub_start, hub_cap, rowstart, c0)) return;
-    const int64_t mend = rowstart[c0];
+    // the entries of the counted rows
+    const int64_t mbeg = rowstart[min(src_lo, c0)], mend = rowstart[min(src_hi, c0)];
     const int64_t total = hub_start[hub_cap];
-    for (int64_t t0 = (int64_t)blockIdx.x * SCAT_TILE; t0 < mend; t0 += (int64_t)gridDim.x * SCAT_TILE) {
+    for (int64_t t0 = (mbeg & ~(int64_t)3) + (int64_t)blockIdx.x * SCAT_TILE; t0 < mend; t0 += (int64_t)gridDim.x * SCAT_TILE) {
         for (int h = threadIdx.x; h < top; h += SCAT_THREADS) lcnt[h] = 0;
         __syncthreads();
         int32_t x[SCAT_ITEMS], u[SCAT_ITEMS], len[SCAT_ITEMS];
@@ -594,13 +597,12 @@ __global__ void __launch_bounds__(SCAT_THREADS) k_hub_scatter(int32_t n, int32_t
 #pragma unroll
         for (int e = 0; e < SCAT_ITEMS; ++e) {
             const int64_t p = t0 + ((int64_t)(e >> 2) * SCAT_THREADS + threadIdx.x) * 4 + (e & 3);
+            if (p < mbeg) x[e] = -1;
             if (x[e] >= R) {
                 u[e] = rowof[p];
                 const int2 ri = rowinfo[u[e]];
                 len[e] = (int32_t)((int64_t)ri.x + ri.y - p - 1);
                 if (len[e] < 0) x[e] = -1;  // a slot freed by deduplication
-                // a source outside the counted shard keeps its slot with an empty suffix
-                if (u[e] < src_lo || u[e] >= src_hi) len[e] = 0;
             }
         }
         // the slot reservations of all items first, so that their round trips overlap,
@@ -657,11 +659,12 @@ __global__ void k_hub_scatter_rows(int32_t n, int32_t hub_cap, const int64_t* __
     const int64_t total = hub_start[hub_cap];
     const int lane = lane_id();
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t w0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; w0 < c0; w0 += warps * 32) {
+    const int32_t end = min(src_hi, c0);  // of the counted rows
+    for (int64_t w0 = src_lo + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; w0 < end;
+         w0 += warps * 32) {
         const int64_t u = w0 + lane;
-        const int du = u < c0 ? rowlen[u] : 0;
+        const int du = u < end ? rowlen[u] : 0;
         const int64_t base = u < n ? rowstart[u] : 0;
-        const bool inshard = u >= src_lo && u < src_hi;  // else its records get empty suffixes
         int p = du - 1;
         // SCAT_STEPS steps at a time: their loads, then their slot reservations, are
         // independent and in flight together.  Walking backwards, the hub entries of a
@@ -689,7 +692,7 @@ __global__ void k_hub_scatter_rows(int32_t n, int32_t hub_cap, const int64_t* __
                 if (x[j] >= R) {
                     const int64_t slot = slot0[j] + __popc(peers[j] & lanemask_lt());
                     if (slot < total)  // counts and entries disagree only on a bug: never write outside
-                        in_rec[slot] = make_uint2((uint32_t)u, inshard ? (uint32_t)(du - 1 - (p - j)) : 0u);
+                        in_rec[slot] = make_uint2((uint32_t)u, (uint32_t)(du - 1 - (p - j)));
                     else
                         atomicOr(&stats->err, ERR_OVERFLOW);
                 }
@@ -722,7 +725,7 @@ __global__ void k_hub_lists(int32_t n, int32_t hub_cap, int32_t T0w, const int2*
                             const uint32_t* __restrict__ indeg, const int64_t* __restrict__ hub_start, int big_in,
                             int32_t* __restrict__ big_list, int32_t* __restrict__ long_list,
                             int4* __restrict__ win_task, int4* __restrict__ low_task, int64_t task_cap,
-                            const unsigned long long* __restrict__ cur, DevStats* stats) {
+                            const unsigned long long* __restrict__ cur, bool shard, DevStats* stats) {
     const int64_t K = stats->hub_count;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int lane = lane_id();
@@ -741,13 +744,15 @@ __global__ void k_hub_lists(int32_t n, int32_t hub_cap, int32_t T0w, const int2*
             ri = rowinfo[v];
             e0 = hub_start[h];
             // the scatter must have filled the hub's segment: a count and a scatter that
-            // disagree are reported instead of trusted
-            if (cur[h] != (unsigned long long)e0 + din) atomicOr(&stats->err, ERR_OVERFLOW);
+            // disagree are reported instead of trusted.  A shard's sources fill its front.
+            const unsigned long long filled = cur[h] - (unsigned long long)e0;
+            if (shard ? filled > din : filled != din) atomicOr(&stats->err, ERR_OVERFLOW);
             if (din > 0 && ri.y > 0) {
                 big = din >= (uint32_t)big_in || ri.y > HUB_WARP_MAX;
                 dwin = v >= T0w ? ri.y : (col[ri.x + ri.y - 1] >= T0w ? (int)winrow[v].y : 0);
                 dlow = ri.y - dwin;
             }
+            if (shard) din = (uint32_t)min(filled, (unsigned long long)din);
         }
         const bool lng = big && dlow > HUB_WARP_MAX;
         const unsigned pb = warp_append(big, &stats->hub_big);
@@ -2522,8 +2527,14 @@ bool launch_plan(const CountBuffers& C, const Strategy& S, const Launch& L, cons
         count_launch();
         // and 64-bit cursors starting at every hub's first slot
         scan_u32_to_i64(C.hub_cnt, C.hub_start, C.hub_cap, C.tmp, H, reinterpret_cast<int64_t*>(C.hub_cur64));
+        // Of a shard's plan only its sources' records are written, at the front of each hub's
+        // segment; the list kernel of probe mode reads whole segments.
+        const bool shard = C.src_lo > 0 || C.src_hi < C.n;
+        if (shard && S.strat[TC_BUCKET_HUB] == TC_STRAT_PROBE)
+            cudaMemsetAsync(C.in_rec, 0, sizeof(uint2) * (size_t)C.m_cap, H.stream);
         k_row_of<<<grid_for((int64_t)C.n, THREADS, H.sms), THREADS, 0, H.stream>>>(C.n, C.hub_cap, C.rowstart,
-                                                                                  C.hub_start, C.rowof, C.stats);
+                                                                                  C.hub_start, C.rowof, C.src_lo,
+                                                                                  C.src_hi, C.stats);
         count_launch();
         k_hub_scatter_rows<<<grid_for(C.n, THREADS, H.sms), THREADS, 0, H.stream>>>(
             C.n, C.hub_cap, C.rowstart, C.rowlen, C.col, C.hub_start, C.hub_cur64, C.in_rec, C.src_lo, C.src_hi,
@@ -2536,7 +2547,7 @@ bool launch_plan(const CountBuffers& C, const Strategy& S, const Launch& L, cons
         k_hub_lists<<<grid_for(C.hub_cap, THREADS, H.sms), THREADS, 0, H.stream>>>(
             C.n, C.hub_cap, T.first[1], C.rowinfo, C.col, C.winrow, C.hub_cnt, C.hub_start,
             S.hub_big_in > 0 ? S.hub_big_in : 1, C.big_list, C.long_list, C.win_task, C.low_task,
-            hub_task_cap(C.hub_cap, C.m_cap), C.hub_cur64, C.stats);
+            hub_task_cap(C.hub_cap, C.m_cap), C.hub_cur64, shard, C.stats);
         count_launch();
     }
     if (forked) cudaEventRecord(ps->join, H.stream);
