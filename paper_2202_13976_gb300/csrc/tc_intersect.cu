@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(WIN_THREADS) k_win_build(int32_t n, Windows T,
         const int64_t u = t0 + threadIdx.x;
         uint32_t nv = 0, len[WINS + 1] = {};
         bool hubrow = false;  // a row without a hub has no in-edge records and needs nothing here
-        if (u < c0) {
+        if (u < c0 && ((u >= src_lo && u < src_hi) || u >= R)) {  // a shard: its sources and the hubs
             const int2 ri = rowinfo[u];
             const int32_t end = ri.x + ri.y;
             hubrow = ri.y > 0 && col[end - 1] >= R;
