@@ -896,9 +896,11 @@ __device__ __forceinline__ int warp_sort_row(int32_t* __restrict__ row, int len,
 
 // One warp per listed row, sorted in registers: MAXK = 8 takes the rows of 17..256
 // entries, MAXK = 32 those of 257..1024 (separate kernels keep the register budget
-// of the short classes small).
+// of the short classes small).  The long class waits on its shuffles with 8 warps per SM at
+// 255 registers; two blocks at 128, with spills, take 161 instead of 188 us on R-MAT scale
+// 20 beside the short class (three or four slow that one down by more).
 template <int MAXK>
-__global__ void __launch_bounds__(SEG_WARPS * 32, MAXK <= 8 ? 4 : 1) k_segsort_warp(const int64_t* __restrict__ rowstart,
+__global__ void __launch_bounds__(SEG_WARPS * 32, MAXK <= 8 ? 4 : 2) k_segsort_warp(const int64_t* __restrict__ rowstart,
                                                                  const uint32_t* __restrict__ rowcnt,
                                                                  int32_t* __restrict__ col, int32_t* __restrict__ rowlen,
                                                                  int2* __restrict__ rowinfo, uint32_t* __restrict__ dupin,
