@@ -97,6 +97,10 @@ tc_status tc_count(tc_graph* g, uint64_t* T_out);
  * the outputs live; with TC_MEM_DEVICE the results are written by kernels on the
  * graph's stream, with TC_MEM_HOST they are copied back and the stream is
  * synchronised.  Degree-0/1 vertices report t = 0 and LCC = +0.0.
+ * Errors: TC_EINVAL (NULL graph, bad mem_kind), TC_ENOMEM, TC_ECUDA, TC_EINTERNAL (a
+ * consistency check of the build or the count failed; with TC_MEM_DEVICE the call does
+ * not wait, and the next one that reads the graph back reports it: tc_count,
+ * tc_graph_info, tc_graph_size with m_oriented).
  */
 tc_status lcc_compute(tc_graph* g, uint64_t* t_out, double* lcc_out, int mem_kind);
 
@@ -132,7 +136,8 @@ tc_status tc_count_shard(tc_graph* g, int32_t shard, int32_t nshards, uint64_t* 
  * The arithmetic is the same as lcc_compute's: LCC(v) = 2 t(v) / (d(v) (d(v) - 1)),
  * one correctly rounded division, and +0.0 for d(v) < 2 or t(v) = 0.
  * t and lcc_out both live where mem_kind says.
- * Errors: TC_EINVAL (NULL, bad mem_kind), TC_ENOMEM, TC_ECUDA.
+ * Errors: TC_EINVAL (NULL, bad mem_kind), TC_ENOMEM, TC_ECUDA, TC_EINTERNAL (as
+ * lcc_compute).
  */
 tc_status tc_lcc_from_counts(tc_graph* g, const uint64_t* t, double* lcc_out, int mem_kind);
 
@@ -148,7 +153,7 @@ tc_status tc_lcc_from_counts(tc_graph* g, const uint64_t* t, double* lcc_out, in
  * ablation: same results, far more work on skewed graphs.  t_out[n] (uint64) in the
  * caller's ids, in mem_kind memory; the stream is synchronised.  *T_out (may be
  * NULL) receives sum t / 3.  Errors: TC_EINVAL (NULL t_out, bad mem_kind), TC_ENOMEM,
- * TC_ECUDA, TC_EINTERNAL (sum t is not a multiple of 3).
+ * TC_ECUDA, TC_EINTERNAL (a consistency check failed).
  */
 tc_status tc_count_vertex_formula(tc_graph* g, uint64_t* t_out, int mem_kind, uint64_t* T_out);
 
@@ -187,7 +192,7 @@ tc_status tc_edge_support(tc_graph* g, int32_t* u_out, int32_t* v_out, uint32_t*
  *   part_stats        host tc_remote_part[parts] or NULL
  * The graph's stream is synchronised.  Errors: TC_EINVAL (NULL graph, parts < 1 or >
  * n, ncap < 0, NULL or decreasing capacities, a graph built from bad ids), TC_ENOMEM,
- * TC_ECUDA.
+ * TC_ECUDA, TC_EINTERNAL.
  */
 enum { TC_CACHE_ADJ_LRU = 0, TC_CACHE_ADJ_SCORE = 1, TC_CACHE_OFF_LRU = 2, TC_CACHE_OFF_SCORE = 3,
        TC_CACHE_KINDS = 4 };
@@ -225,7 +230,8 @@ tc_status tc_remote_cache(tc_graph* g, int32_t parts, int32_t ncap, const uint64
  * tc_count is, with two direction bits per edge; scratch comes from the library's
  * device pool and is released before the call returns.  Errors: TC_EINVAL (an id
  * outside [0, n), n < 0, m out of range, NULL src/dst with m > 0, bad mem_kind or
- * flags; the outputs are then left untouched), TC_ENOMEM, TC_ECUDA.
+ * flags; the outputs are then left untouched), TC_ENOMEM, TC_ECUDA, TC_EINTERNAL (a
+ * consistency check of the build failed; likewise).
  */
 enum { TC_DIRECTED_TIMED = 1 };
 
@@ -249,13 +255,14 @@ tc_status tc_directed_lcc(int32_t n, int64_t m, const int32_t* src, const int32_
  * Input accounting (Sec. II-A: the input is read as a simple graph, so self-loops
  * and repeated pairs leave it): number of distinct undirected edges |E|, self-loops
  * dropped and repeated pairs dropped.  Any pointer may be NULL.  Synchronises the
- * stream.  Errors: TC_EINVAL for a NULL graph; TC_ECUDA.
+ * stream.  Errors: TC_EINVAL for a NULL graph; TC_ECUDA; TC_EINTERNAL (a consistency
+ * check of the build or the count failed).
  */
 tc_status tc_graph_info(const tc_graph* g, int64_t* m_simple, int64_t* loops_dropped,
                         int64_t* dups_dropped);
 
 /* Number of vertices |V| and of oriented edges (Sec. II-C orients every edge of E
- * once, so this is |E|).  Errors: TC_EINVAL for a NULL graph; TC_ECUDA. */
+ * once, so this is |E|).  Errors: as tc_graph_info. */
 tc_status tc_graph_size(const tc_graph* g, int32_t* n, int64_t* m_oriented);
 
 /* Release the graph's device memory (back to the library's device pool).  NULL is

@@ -198,6 +198,7 @@ struct tc_graph {
     std::vector<void*> blocks;
     bool planned = false;
     bool counted = false;
+    mutable bool verified = false;  // the statistics have been read since the last build, plan or count, without a flag
     bool plan_zeroed = false;   // the planner's part of the statistics is zero
     bool count_zeroed = false;  // t and the count's part of the statistics are zero
     Strategy strat{};
@@ -315,6 +316,27 @@ tc_status read_stats(const tc_graph* g, DevStats* h) {
     TC_CK(cudaMemcpyAsync(h, g->stats, sizeof(DevStats), cudaMemcpyDeviceToHost, g->stream));
     TC_CK(cudaStreamSynchronize(g->stream));
     return TC_OK;
+}
+
+// The statistics of a built graph.  A guard of the build, the plan or the count that has
+// fired (rows that could not be filled are empty) fails every call that answers from the
+// graph.
+tc_status read_result_stats(const tc_graph* g, DevStats* h) {
+    const tc_status st = read_stats(g, h);
+    if (st != TC_OK) return st;
+    if (h->err & ERR_OVERFLOW) {
+        snprintf(g_last_error, sizeof(g_last_error), "internal count mismatch (overflow guard)");
+        return TC_EINTERNAL;
+    }
+    g->verified = true;
+    return TC_OK;
+}
+
+// The same check for calls that wait for the stream but need no statistics.
+tc_status verify(const tc_graph* g) {
+    if (g->verified) return TC_OK;
+    DevStats h;
+    return read_result_stats(g, &h);
 }
 
 // Pairs from which rows are filled by buckets.  Whole calls, direct fill / buckets, uniform
@@ -596,6 +618,7 @@ tc_status run_plan(tc_graph* g) {
     TC_CK(cudaGetLastError());
     g->planned = true;
     g->counted = false;
+    g->verified = false;
     return TC_OK;
 }
 
@@ -624,6 +647,7 @@ tc_status run_count(tc_graph* g) {
     launch_sum_t(C, g->L);
     TC_CK(cudaGetLastError());
     g->counted = true;
+    g->verified = false;
     g->timed = !g->capture;
     return TC_OK;
 }
@@ -665,7 +689,7 @@ tc_status build_undirected_rows(int32_t n, int64_t m, const int32_t* src, const 
     }
     if (st != TC_OK) return st;
     DevStats h;
-    if ((st = read_stats(*g, &h)) != TC_OK) return st;
+    if ((st = read_result_stats(*g, &h)) != TC_OK) return st;
     out->m_simple = (int64_t)h.m_simple;
     out->loops = (int64_t)h.loops;
     out->rank = (*g)->rank;
@@ -787,11 +811,7 @@ tc_status tc_count(tc_graph* g, uint64_t* T_out) {
     tc_status st = run_count(g);
     if (st != TC_OK) return st;
     DevStats h;
-    if ((st = read_stats(g, &h)) != TC_OK) return st;
-    if (h.err & ERR_OVERFLOW) {
-        snprintf(g_last_error, sizeof(g_last_error), "internal count mismatch (overflow guard)");
-        return TC_EINTERNAL;
-    }
+    if ((st = read_result_stats(g, &h)) != TC_OK) return st;
     if (h.sum_t % 3 != 0) {
         snprintf(g_last_error, sizeof(g_last_error), "sum of t is not a multiple of 3");
         return TC_EINTERNAL;
@@ -827,7 +847,7 @@ tc_status lcc_compute(tc_graph* g, uint64_t* t_out, double* lcc_out, int mem_kin
     free_list(g, &tmp);
     if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
     if (e != cudaSuccess) return cuda_fail("lcc_compute copy", e);
-    return TC_OK;
+    return verify(g);
 }
 
 // Counts one shard, then restores the whole source range on every path out (the
@@ -873,8 +893,8 @@ tc_status tc_count_shard(tc_graph* g, int32_t shard, int32_t nshards, uint64_t* 
     tc_status st = run_count(g);
     if (st != TC_OK) return st;
     DevStats h;
-    if ((st = read_stats(g, &h)) != TC_OK) return st;
-    if ((h.err & ERR_OVERFLOW) || h.sum_t % 3 != 0) {
+    if ((st = read_result_stats(g, &h)) != TC_OK) return st;
+    if (h.sum_t % 3 != 0) {
         snprintf(g_last_error, sizeof(g_last_error), "internal count mismatch in a shard");
         return TC_EINTERNAL;
     }
@@ -924,7 +944,7 @@ tc_status tc_lcc_from_counts(tc_graph* g, const uint64_t* t, double* lcc_out, in
     if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
     free_list(g, &tmp);
     if (e != cudaSuccess) return cuda_fail("lcc_from_counts", e);
-    return TC_OK;
+    return verify(g);
 }
 
 // Scratch of the symmetric rows (tc_vertex.cu) for g; pool memory tracked in tmp.
@@ -960,7 +980,7 @@ static tc_status symmetric_buffers(tc_graph* g, const DevStats& h, VertexFormula
 tc_status tc_count_vertex_formula(tc_graph* g, uint64_t* t_out, int mem_kind, uint64_t* T_out) {
     if (!g || !t_out || (mem_kind != TC_MEM_HOST && mem_kind != TC_MEM_DEVICE)) return TC_EINVAL;
     DevStats h;
-    tc_status st = read_stats(g, &h);
+    tc_status st = read_result_stats(g, &h);
     if (st != TC_OK) return st;
     if (h.err & ERR_BAD_ID) return TC_EINVAL;
     const size_t nn = (size_t)g->n;
@@ -997,7 +1017,7 @@ tc_status tc_edge_support(tc_graph* g, int32_t* u_out, int32_t* v_out, uint32_t*
     if (!g || !u_out || !v_out || !support_out || (mem_kind != TC_MEM_HOST && mem_kind != TC_MEM_DEVICE))
         return TC_EINVAL;
     DevStats h;
-    tc_status st = read_stats(g, &h);
+    tc_status st = read_result_stats(g, &h);
     if (st != TC_OK) return st;
     if (h.err & ERR_BAD_ID) return TC_EINVAL;
     const size_t nn = (size_t)g->n, me = (size_t)h.m_simple;
@@ -1049,11 +1069,7 @@ tc_status tc_edge_support(tc_graph* g, int32_t* u_out, int32_t* v_out, uint32_t*
     free_list(g, &tmp);
     if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
     if (e != cudaSuccess) return cuda_fail("tc_edge_support", e);
-    if (read_stats(g, &h) == TC_OK && (h.err & ERR_OVERFLOW)) {
-        snprintf(g_last_error, sizeof(g_last_error), "internal count mismatch (overflow guard)");
-        return TC_EINTERNAL;
-    }
-    return TC_OK;
+    return read_result_stats(g, &h);
 }
 
 tc_status tc_remote_cache(tc_graph* g, int32_t parts, int32_t ncap, const uint64_t* capacity_bytes, uint64_t* hits,
@@ -1064,7 +1080,7 @@ tc_status tc_remote_cache(tc_graph* g, int32_t parts, int32_t ncap, const uint64
     for (int32_t c = 1; c < ncap; ++c)
         if (capacity_bytes[c] < capacity_bytes[c - 1]) return TC_EINVAL;
     DevStats h;
-    tc_status st = read_stats(g, &h);
+    tc_status st = read_result_stats(g, &h);
     if (st != TC_OK) return st;
     if (h.err & ERR_BAD_ID) return TC_EINVAL;
     const size_t cells = (size_t)TC_CACHE_KINDS * (size_t)parts * (size_t)ncap;
@@ -1211,7 +1227,7 @@ tc_status tc_remote_cache(tc_graph* g, int32_t parts, int32_t ncap, const uint64
 tc_status tc_graph_info(const tc_graph* g, int64_t* m_simple, int64_t* loops_dropped, int64_t* dups_dropped) {
     if (!g) return TC_EINVAL;
     DevStats h;
-    tc_status st = read_stats(g, &h);
+    tc_status st = read_result_stats(g, &h);
     if (st != TC_OK) return st;
     if (m_simple) *m_simple = (int64_t)h.m_simple;
     if (loops_dropped) *loops_dropped = (int64_t)h.loops;
@@ -1224,7 +1240,7 @@ tc_status tc_graph_size(const tc_graph* g, int32_t* n, int64_t* m_oriented) {
     if (n) *n = g->n;
     if (m_oriented) {
         DevStats h;
-        tc_status st = read_stats(g, &h);
+        tc_status st = read_result_stats(g, &h);
         if (st != TC_OK) return st;
         *m_oriented = (int64_t)h.m_simple;
     }
@@ -1444,7 +1460,7 @@ static tc_status batch_check(tc_graph* g) {
         snprintf(g_last_error, sizeof(g_last_error), "vertex id outside [0, n_g) in a batch graph");
         return TC_EINVAL;
     }
-    if ((err & ERR_OVERFLOW) || h.sum_t % 3 != 0) return TC_EINTERNAL;
+    if (((err | h.err) & ERR_OVERFLOW) || h.sum_t % 3 != 0) return TC_EINTERNAL;
     return TC_OK;
 }
 

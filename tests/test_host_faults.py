@@ -1,0 +1,124 @@
+"""The host code of the library (tc_api.cu) against a fake CUDA runtime: what it answers when
+the device code raises a flag or a call of the runtime fails."""
+from __future__ import annotations
+
+import ctypes
+
+import numpy as np
+import pytest
+
+from tests import fake_cuda
+
+OK, EINVAL, ENOMEM, ECUDA, ETIMEOUT, EBUSY, EINTERNAL = range(7)
+HOST, DEVICE = 0, 1
+OVERFLOW = 4  # ERR_OVERFLOW: a guard of the build or of the plan has fired
+
+
+@pytest.fixture(scope="session")
+def fake_lib(tmp_path_factory):
+    return fake_cuda.load(str(tmp_path_factory.mktemp("fake_cuda")))
+
+
+@pytest.fixture
+def fake(fake_lib):
+    fake_lib.fake_reset()
+    yield fake_lib
+    fake_lib.fake_reset()
+
+
+def _ptr(a):
+    return a.ctypes.data if a is not None else None
+
+
+def _pairs(m):
+    return np.zeros(m, np.int32), np.ones(m, np.int32)
+
+
+def _graph(fake, n=50, m=60, kind=DEVICE, stream=None):
+    s, d = _pairs(m)
+    g = ctypes.c_void_p()
+    st = fake.tc_graph_create_from_edges(n, m, _ptr(s), _ptr(d), kind, stream, ctypes.byref(g))
+    assert st == OK
+    return g
+
+
+def _batch(fake):
+    n, off = np.array([30, 20], np.int32), np.array([0, 25, 60], np.int64)
+    s, d = _pairs(60)
+    g = ctypes.c_void_p()
+    assert fake.tc_batch_create(2, _ptr(n), _ptr(off), _ptr(s), _ptr(d), DEVICE, None, ctypes.byref(g)) == OK
+    return g
+
+
+def _calls(fake, g, kind):
+    """The calls that read a graph's results or statistics back, by name."""
+    T, t, lcc = ctypes.c_uint64(), np.zeros(50, np.uint64), np.zeros(50)
+    m = ctypes.c_int64()
+    e = [np.zeros(60, np.int32) for _ in range(3)]
+    cap = np.array([16], np.uint64)
+    return {
+        "tc_count": lambda: fake.tc_count(g, ctypes.byref(T)),
+        "lcc_compute": lambda: fake.lcc_compute(g, ctypes.c_void_p(_ptr(t)), ctypes.c_void_p(_ptr(lcc)), HOST),
+        "tc_count_shard": lambda: fake.tc_count_shard(g, 0, 2, None, HOST, ctypes.byref(T)),
+        "tc_lcc_from_counts": lambda: fake.tc_lcc_from_counts(g, ctypes.c_void_p(_ptr(t)),
+                                                              ctypes.c_void_p(_ptr(lcc)), HOST),
+        "tc_count_vertex_formula": lambda: fake.tc_count_vertex_formula(g, ctypes.c_void_p(_ptr(t)), kind,
+                                                                        ctypes.byref(T)),
+        "tc_edge_support": lambda: fake.tc_edge_support(g, *(ctypes.c_void_p(_ptr(a)) for a in e), kind),
+        "tc_remote_cache": lambda: fake.tc_remote_cache(g, 2, 1, ctypes.c_void_p(_ptr(cap)), None, None, None),
+        "tc_graph_info": lambda: fake.tc_graph_info(g, ctypes.byref(m), None, None),
+        "tc_graph_size": lambda: fake.tc_graph_size(g, None, ctypes.byref(m)),
+    }
+
+
+CALLS = ["tc_count", "lcc_compute", "tc_count_shard", "tc_lcc_from_counts", "tc_count_vertex_formula",
+         "tc_edge_support", "tc_remote_cache", "tc_graph_info", "tc_graph_size"]
+
+
+@pytest.mark.parametrize("call", CALLS)
+@pytest.mark.parametrize("flag", [0, OVERFLOW])
+def test_a_guard_of_the_build_is_reported(fake, call, flag):
+    """Rows that the partition could not fill are empty: every call that reads the graph back
+    says so instead of answering from them."""
+    fake.fake_flags(flag, 0)
+    g = _graph(fake)
+    try:
+        f = _calls(fake, g, DEVICE)[call]
+        for _ in range(2):
+            assert f() == (EINTERNAL if flag else OK)
+    finally:
+        fake.tc_graph_destroy(g)
+
+
+@pytest.mark.parametrize("flag", [0, OVERFLOW])
+@pytest.mark.parametrize("during_build", [0, 1])
+def test_a_guard_in_a_batch_is_reported(fake, flag, during_build):
+    fake.fake_flags(flag if during_build else 0, 0 if during_build else flag)
+    g = _batch(fake)
+    try:
+        T = np.zeros(2, np.uint64)
+        for kind in (HOST, DEVICE):
+            assert fake.tc_batch_count(g, ctypes.c_void_p(_ptr(T)), kind) == (EINTERNAL if flag else OK)
+    finally:
+        fake.tc_graph_destroy(g)
+
+
+@pytest.mark.parametrize("flag", [0, OVERFLOW])
+@pytest.mark.parametrize("dir_bits", [0, 1])
+def test_a_guard_reaches_the_directed_count(fake, flag, dir_bits):
+    fake.fake_flags(flag, 0)
+    s, d = _pairs(60)
+    assert fake.fake_undirected_rows(50, 60, _ptr(s), _ptr(d), dir_bits) == (EINTERNAL if flag else OK)
+
+
+@pytest.mark.parametrize("call", ["tc_count", "lcc_compute"])
+def test_a_guard_of_the_count_is_reported(fake, call):
+    fake.fake_flags(0, OVERFLOW)
+    g = _graph(fake)
+    try:
+        f = _calls(fake, g, DEVICE)[call]
+        assert f() == EINTERNAL and f() == EINTERNAL
+        T = ctypes.c_uint64()
+        assert fake.tc_count(g, ctypes.byref(T)) == EINTERNAL
+    finally:
+        fake.tc_graph_destroy(g)
