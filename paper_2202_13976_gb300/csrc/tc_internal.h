@@ -39,6 +39,8 @@ struct DevStats {
     unsigned int hub_low;          // below-window tasks
     unsigned int hub_long;         // big hubs with a long list below the window
     unsigned int win_vecs;         // planner: 16-byte vectors of window entries written
+    unsigned int samples;          // planner: hub probes sampled
+    unsigned int sample_hits;      // planner: those of them that hit
     // from here on, zero when a count starts
     unsigned int cta_next;         // dynamic work counter of the block push kernel
     unsigned int small_next[2];    // dynamic work counters of the hash kernels
@@ -48,7 +50,7 @@ struct DevStats {
     unsigned int hub_next4;        // dynamic work counter of the below-window kernel
     unsigned long long sum_t;      // sum over v of t(v)
 };
-static_assert(sizeof(DevStats) == 136 && offsetof(DevStats, cta_next) % 4 == 0, "DevStats layout");
+static_assert(sizeof(DevStats) == 144 && offsetof(DevStats, cta_next) % 4 == 0, "DevStats layout");
 
 struct Launch {
     cudaStream_t stream;
@@ -201,9 +203,10 @@ constexpr int HUB_BM_BITS = 131072;
 // Least degree of a hub, unless set.
 constexpr int HUB_MIN_DEGREE = 32;
 // Window 1 of the hub kernels: the highest min(n, HUB_WIN) ranks, one 32-bit counter
-// each in shared memory.  An entry x of it is kept as four times its index in the
-// window (the counter's byte offset, 16 bits); 4 * HUB_WIN names the slot that no hub
-// marks.  The windows below it have HUB_WIN2 ranks each, an entry kept as its index.
+// each in shared memory.  An entry x of it is kept as four times its place among them
+// (win_place of its index in the window: the counter's byte offset, 16 bits); the place of
+// index HUB_WIN, which no rank has, is the slot that no hub marks.  The windows below it
+// have HUB_WIN2 ranks each, an entry kept as its index.
 constexpr int HUB_WIN = 16383;
 constexpr int HUB_WIN2 = 65535;
 static_assert(4 * HUB_WIN <= 0xffff && HUB_WIN2 <= 0xffff, "window offsets fit 16 bits");

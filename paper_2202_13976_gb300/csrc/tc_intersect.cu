@@ -34,6 +34,7 @@
 //           AUTO    Eq. 3 per edge: merge if |B|/|A| <= f (log2|B| - 1) (|A| <= |B|),
 //                   else the keys of the shorter list are searched in the longer
 #include <climits>
+#include <type_traits>
 
 #include "tc_device.cuh"
 #include "tc_internal.h"
@@ -452,6 +453,18 @@ static_assert(HUB_WIN + (WINS - 1) * HUB_WIN2 >= HUB_BM_BITS, "the windows reach
 
 __device__ __forceinline__ uint32_t vectors_of(uint32_t entries) { return (entries + 7u) >> 3; }
 
+// The place of window 1's rank i among its counters.  Neighbouring ranks' suffixes hold runs
+// of consecutive ranks in graphs whose ids have locality; the lanes of a probe are then
+// eight ranks apart, in four banks if the places were the ranks themselves.  Its own inverse.
+__host__ __device__ __forceinline__ constexpr uint32_t win_place(uint32_t i) { return i ^ ((i >> 5) & 7u); }
+constexpr uint32_t WIN_NONE = 4 * win_place(HUB_WIN);  // the offset that no hub marks
+constexpr bool win_places_ok() {
+    for (uint32_t i = 0; i <= HUB_WIN; ++i)
+        if (win_place(i) > HUB_WIN || win_place(win_place(i)) != i || win_place(i) >> 3 != i >> 3) return false;
+    return true;
+}
+static_assert((HUB_WIN & 7) == 7 && win_places_ok(), "a permutation of each group of eight");
+
 // A row's place in the windows below the first: {first vector of window 2, entries in
 // window 1, entries in window 2 | in window 3 << 16, 0}.
 __device__ __forceinline__ uint32_t low_len(const uint4& r, int k) { return k == 2 ? r.z & 0xffffu : r.z >> 16; }
@@ -526,12 +539,16 @@ __global__ void __launch_bounds__(WIN_THREADS) k_win_build(int32_t n, Windows T,
                 p0 = cut[++win_no][lo];
             }
             const int32_t first = win_no == 1 ? T.first[1] : win_no == 2 ? T.first[2] : T.first[3];
-            const uint32_t scale = win_no == 1 ? 4u : 1u, none = win_no == 1 ? 4u * HUB_WIN : (uint32_t)HUB_WIN2;
+            const uint32_t none = win_no == 1 ? WIN_NONE : (uint32_t)HUB_WIN2;
             uint32_t o[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const int64_t p = (int64_t)p0 + 8 * (int64_t)rel + j;
-                o[j] = p < p1 ? (uint32_t)(col[p] - first) * scale : none;
+                o[j] = none;
+                if (p < p1) {
+                    const uint32_t i = (uint32_t)(col[p] - first);
+                    o[j] = win_no == 1 ? 4u * win_place(i) : i;
+                }
             }
             if ((int64_t)base + k < win_cap)  // always true: win_vec_cap
                 win[base + k] = make_uint4(o[0] | o[1] << 16, o[2] | o[3] << 16, o[4] | o[5] << 16, o[6] | o[7] << 16);
@@ -784,8 +801,41 @@ __global__ void k_hub_lists(int32_t n, int32_t hub_cap, int32_t T0w, const int2*
 constexpr int PLAN_ITEMS = 4;
 constexpr int PLAN_LISTS = 5;  // d+ classes <= 8, <= 16, <= 32, <= SMALL_WIDE_MAX, larger
 
-__global__ void __launch_bounds__(THREADS) k_plan(int32_t n, const int64_t* __restrict__ rowstart,
-                                                  const int32_t* __restrict__ rowlen, const int32_t* __restrict__ col,
+// How often the probes of the hub kernels hit, from rows spread over the ranks: is the entry
+// in the middle of a row's upper half in the list of the one in the row's middle, a hub?
+// Where more than half are, the graph is one of communities (hub_dense).  R-MAT graphs of
+// 2^12 .. 2^23 vertices have 0.23 .. 0.03, uniform ones next to none, geometric ones 0.7,
+// disjoint cliques 1.  The first blocks of k_plan do this beside the others' work.
+constexpr int SAMPLE_BLOCKS_MAX = 64;
+constexpr int sample_blocks(int32_t n) {
+    return n >= SAMPLE_BLOCKS_MAX * 1024 ? SAMPLE_BLOCKS_MAX : (n + 1023) / 1024;
+}
+__device__ __forceinline__ void sample_hubs(int32_t n, int32_t R, int blocks, const int2* __restrict__ rowinfo,
+                                            const int32_t* __restrict__ col, DevStats* stats) {
+    const int64_t i = (int64_t)blockIdx.x * THREADS + threadIdx.x, all = (int64_t)blocks * THREADS;
+    const int2 ru = rowinfo[i * n / all];
+    bool sampled = false, hit = false;
+    if (ru.y >= 2) {
+        const int mid = (ru.y - 1) / 2;  // before the last entry
+        const int32_t v = col[ru.x + mid], x = col[ru.x + mid + (ru.y - mid) / 2];
+        sampled = v >= R;
+        if (sampled) {
+            const int2 rv = rowinfo[v];
+            const int p = lower_bound(col + rv.x, 0, rv.y, x);
+            hit = p < rv.y && col[rv.x + p] == x;
+        }
+    }
+    const unsigned sm = __ballot_sync(FULL, sampled), hm = __ballot_sync(FULL, hit);
+    if (lane_id() == 0 && sm) {
+        atomicAdd(&stats->samples, (unsigned)__popc(sm));
+        if (hm) atomicAdd(&stats->sample_hits, (unsigned)__popc(hm));
+    }
+}
+__device__ __forceinline__ bool hub_dense(const DevStats* stats) { return 2 * stats->sample_hits > stats->samples; }
+
+__global__ void __launch_bounds__(THREADS) k_plan(int32_t n, int samplers, const int64_t* __restrict__ rowstart,
+                                                  const int32_t* __restrict__ rowlen,
+                                                  const int2* __restrict__ rowinfo, const int32_t* __restrict__ col,
                                                   int32_t* __restrict__ l8, int32_t* __restrict__ l16,
                                                   int32_t* __restrict__ l32, int32_t* __restrict__ l256,
                                                   int32_t* __restrict__ lcta, int32_t src_lo, int32_t src_hi,
@@ -797,8 +847,12 @@ __global__ void __launch_bounds__(THREADS) k_plan(int32_t n, const int64_t* __re
     unsigned* counters[PLAN_LISTS] = {&stats->small_count[0], &stats->small_count[1], &stats->small_count[2],
                                       &stats->small_count[3], &stats->cta_count};
     int32_t* lists[PLAN_LISTS] = {l8, l16, l32, l256, lcta};
+    if ((int)blockIdx.x < samplers) {
+        if (R < n) sample_hubs(n, R, samplers, rowinfo, col, stats);
+        return;
+    }
     const int64_t tile = (int64_t)THREADS * PLAN_ITEMS;
-    for (int64_t t0 = (int64_t)blockIdx.x * tile; t0 < n; t0 += (int64_t)gridDim.x * tile) {
+    for (int64_t t0 = (int64_t)(blockIdx.x - samplers) * tile; t0 < n; t0 += (int64_t)(gridDim.x - samplers) * tile) {
         if (threadIdx.x < PLAN_LISTS) bcount[threadIdx.x] = 0;
         __syncthreads();
         int cls[PLAN_ITEMS];
@@ -1759,8 +1813,7 @@ struct WinCounters {  // a block's counters, the entries of N+(v) marked in bit 
 };
 
 // A block's marks, one bit per warp and rank; matches count in the block's counters of
-// the MED_TOP highest ranks, else directly in t.
-constexpr int MED_TOP = 4096;
+// the highest ranks (MED_TOP), else directly in t.
 struct WinMarks {
     uint32_t marks, cnt, first;  // shared addresses; offset of the first rank with a counter
     int shift;                   // 31 - the warp's bit
@@ -1779,7 +1832,7 @@ struct WinMarks {
                 if (o[j] >= first)
                     asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(cnt + (o[j] - first)) : "memory");
                 else
-                    atomicAdd(&t[o[j] >> 2], 1ull);
+                    atomicAdd(&t[win_place(o[j] >> 2)], 1ull);
                 ++c;
             }
         return c;
@@ -1791,15 +1844,17 @@ struct WinMarks {
 struct WinBitmap {
     uint32_t bm, pre, cnt;
     __device__ __forceinline__ uint32_t operator()(const uint32_t (&o)[8], int (&s)[8]) const {
-        uint32_t c = 0;
+        uint32_t c = 0, i[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-            s[j] = (int)__funnelshift_l(0u, (uint32_t)shared_s32(bm + ((o[j] >> 5) & ~3u)), ~(o[j] >> 2));
+        for (int j = 0; j < 8; ++j) {
+            i[j] = win_place(o[j] >> 2);
+            s[j] = (int)__funnelshift_l(0u, (uint32_t)shared_s32(bm + ((i[j] >> 3) & ~3u)), ~i[j]);
+        }
 #pragma unroll
         for (int j = 0; j < 8; ++j)
             if (s[j] < 0) {
                 uint32_t before;  // entries before the word, then those below the bit
-                asm volatile("ld.shared.u8 %0, [%1];" : "=r"(before) : "r"(pre + (o[j] >> 7)));
+                asm volatile("ld.shared.u8 %0, [%1];" : "=r"(before) : "r"(pre + (i[j] >> 5)));
                 const uint32_t pos = before + __popc(s[j]) - 1;
                 asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(cnt + 4 * pos) : "memory");
                 ++c;
@@ -1865,7 +1920,7 @@ __device__ __forceinline__ uint32_t win_batch(const uint2 rec, int win_no, bool 
         cbase = __shfl_sync(FULL, end - (int32_t)(len - (off & ~7u)), src);
     }
     E.lay(__shfl_sync(FULL, nv0, src), (int)__shfl_sync(FULL, first + (off >> 3), src), at);
-    constexpr uint32_t NONE2 = (LOW ? (uint32_t)HUB_WIN2 : 4u * HUB_WIN) * 0x10001u;
+    constexpr uint32_t NONE2 = (LOW ? (uint32_t)HUB_WIN2 : WIN_NONE) * 0x10001u;
     uint32_t running = 0;
     for (int r = 0; r < E.total; r += 64) {
         const int item = r + lane;
@@ -1970,7 +2025,8 @@ __global__ void __launch_bounds__(WINK_THREADS, WINK_BLOCKS) k_tc_hub(
         const int32_t v = task.x;
         const int ne = task.w & ((1 << TASK_BITS) - 1), p1 = task.z + (int)((uint32_t)task.w >> TASK_BITS);
         const int e1 = task.y + ne;
-        for (int p = task.z + (int)threadIdx.x; p < p1; p += WINK_THREADS) sh.cnt[col[p] - T0w] |= WIN_MARK;
+        for (int p = task.z + (int)threadIdx.x; p < p1; p += WINK_THREADS)
+            sh.cnt[win_place((uint32_t)(col[p] - T0w))] |= WIN_MARK;
         __syncthreads();
         uint32_t vtot = 0;
         const int bs = hub_batch_size(ne, WINK_WARPS);
@@ -1986,7 +2042,7 @@ __global__ void __launch_bounds__(WINK_THREADS, WINK_BLOCKS) k_tc_hub(
         if (lane == 0) sh.vt[w] = vtot;
         __syncthreads();
         for (int p = task.z + (int)threadIdx.x; p < p1; p += WINK_THREADS) {
-            const int x = col[p] - T0w;
+            const uint32_t x = win_place((uint32_t)(col[p] - T0w));
             const uint32_t c = sh.cnt[x] & ~WIN_MARK;
             sh.cnt[x] = SUP ? 0u : c;
             if (SUP && c) atomicAdd(&sup[p], c);  // edge (v, x)
@@ -1999,18 +2055,24 @@ __global__ void __launch_bounds__(WINK_THREADS, WINK_BLOCKS) k_tc_hub(
     }
     if (!SUP)
         for (int i = threadIdx.x; i < HUB_WIN; i += WINK_THREADS)
-            if (sh.cnt[i]) atomicAdd(&t[T0w + i], (unsigned long long)sh.cnt[i]);
+            if (const uint32_t c = sh.cnt[win_place((uint32_t)i)]) atomicAdd(&t[T0w + i], (unsigned long long)c);
 }
 
-template <bool SUP>
+// Ranks with a counter in k_tc_hub_med: the MED_TOP highest, or so (their places are
+// permuted in groups of eight).  With 8 KB more a block the kernel has less L1 cache, and
+// R-MAT scale 23 takes 358 instead of 319 us.  In a graph without other ranks (ALL) each has
+// one: disjoint cliques of 200, 16,000 vertices, 480 -> 77 us.
+constexpr int MED_TOP = 4096;
+constexpr int MED_TOP0 = (HUB_WIN - MED_TOP) & ~7;  // the first of them in the window
+template <bool SUP, bool ALL>
 struct MedShared {
     uint32_t marks[(HUB_WIN + 1) / 2];  // two ranks per word
-    uint32_t cnt[MED_TOP];
+    uint32_t cnt[HUB_WIN + 1 - (ALL ? 0 : MED_TOP0)];
     int2 at[WINK_WARPS][32];
     uint32_t cw[WINK_WARPS][32];
 };
-template <>
-struct MedShared<true> {
+template <bool ALL>
+struct MedShared<true, ALL> {
     struct {
         uint32_t bm[(HUB_WIN + 1) / 32];
         uint32_t pre[(HUB_WIN + 1) / 128];  // one byte per word of bm
@@ -2025,20 +2087,23 @@ static_assert(HUB_WARP_MAX <= 256, "one-byte prefix counts");
 // Window tasks of the other hubs, one per warp (taken from the back of the task list).
 // Each warp owns one bit of the block's marks, so sixteen hubs share one table and a
 // hub costs O(|N+(v)|) beside its suffixes.
-template <bool SUP>
+template <bool SUP, bool ALL>
 __global__ void __launch_bounds__(WINK_THREADS, WINK_BLOCKS) k_tc_hub_med(
     int32_t T0w, int32_t W, const int2* __restrict__ rowinfo, const uint2* __restrict__ winrow,
     const int32_t* __restrict__ col, const uint4* __restrict__ win, const int4* __restrict__ win_task, int64_t task_cap,
     const uint2* __restrict__ in_rec, unsigned long long* __restrict__ t, DevStats* stats, uint32_t* __restrict__ sup) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    MedShared<SUP>& sh = *reinterpret_cast<MedShared<SUP>*>(smem_raw);
+    MedShared<SUP, ALL>& sh = *reinterpret_cast<MedShared<SUP, ALL>*>(smem_raw);
     const int lane = lane_id(), w = threadIdx.x >> 5;
     const unsigned nmed = stats->hub_med;
     if (blockIdx.x * WINK_WARPS >= nmed) return;
-    const int top0 = W > MED_TOP ? W - MED_TOP : 0;  // window index of the first rank with a counter
+    // in a graph of communities with ranks below window 1 k_tc_hub_win2 takes these tasks
+    if (!SUP && !ALL && hub_dense(stats)) return;
+    constexpr int top0 = ALL ? 0 : MED_TOP0;
+    const int top = ALL ? (W + 7) & ~7 : HUB_WIN + 1 - MED_TOP0;  // counters in use
     if constexpr (!SUP) {
         for (int i = threadIdx.x; i < (HUB_WIN + 1) / 2; i += WINK_THREADS) sh.marks[i] = 0;
-        for (int i = threadIdx.x; i < MED_TOP; i += WINK_THREADS) sh.cnt[i] = 0;
+        for (int i = threadIdx.x; i < top; i += WINK_THREADS) sh.cnt[i] = 0;
         __syncthreads();
     }
     unsigned q = blockIdx.x * WINK_WARPS + w;
@@ -2052,9 +2117,9 @@ __global__ void __launch_bounds__(WINK_THREADS, WINK_BLOCKS) k_tc_hub_med(
         uint32_t vtot = 0;
         if constexpr (!SUP) {
             const WinMarks P{(uint32_t)__cvta_generic_to_shared(sh.marks), (uint32_t)__cvta_generic_to_shared(sh.cnt),
-                             4u * (uint32_t)top0, 31 - w, t + T0w};
+                             4u * top0, 31 - w, t + T0w};
             for (int p = lane; p < dwin; p += 32) {
-                const int x = col[task.z + p] - T0w;
+                const uint32_t x = win_place((uint32_t)(col[task.z + p] - T0w));
                 atomicOr(&sh.marks[x >> 1], 1u << (w + 16 * (x & 1)));
             }
             __syncwarp();
@@ -2065,7 +2130,7 @@ __global__ void __launch_bounds__(WINK_THREADS, WINK_BLOCKS) k_tc_hub_med(
                 vtot += win_batch<SUP, false>(cur, 1, v >= T0w, rowinfo, winrow, nullptr, win, P, t, sh.at[w], sh.cw[w], sup);
             }
             for (int p = lane; p < dwin; p += 32) {
-                const int x = col[task.z + p] - T0w;
+                const uint32_t x = win_place((uint32_t)(col[task.z + p] - T0w));
                 atomicAnd(&sh.marks[x >> 1], ~(1u << (w + 16 * (x & 1))));
             }
             __syncwarp();
@@ -2117,8 +2182,8 @@ __global__ void __launch_bounds__(WINK_THREADS, WINK_BLOCKS) k_tc_hub_med(
     }
     if constexpr (!SUP) {
         __syncthreads();
-        for (int i = threadIdx.x; i < W - top0; i += WINK_THREADS)
-            if (sh.cnt[i]) atomicAdd(&t[T0w + top0 + i], (unsigned long long)sh.cnt[i]);
+        for (int i = threadIdx.x; i < top; i += WINK_THREADS)
+            if (sh.cnt[i]) atomicAdd(&t[T0w + (int)win_place((uint32_t)(top0 + i))], (unsigned long long)sh.cnt[i]);
     }
 }
 
@@ -2142,15 +2207,86 @@ struct WinBits {
     }
 };
 
+// A warp's set of N+(v)'s entries in a window, with a counter each, for graphs in which most
+// probes hit: a slot is (offset << 16) | matches, at most HUB_SLICE of them.
+constexpr uint32_t SLOT_EMPTY = 0xffff0000u;  // no rank's offset
+constexpr int WIN_SET_LG = 11;
+constexpr int WIN_SET_MAX = 1024;             // entries: half of the slots
+static_assert(HUB_SLICE <= 0xffff && HUB_WIN2 == 0xffff && 4 * HUB_WIN < 0xffff, "slot fields");
+struct WinSet {
+    uint32_t tab;  // shared address
+    static __device__ __forceinline__ uint32_t home(uint32_t o) { return (o * 0x9e3779b1u) >> (32 - WIN_SET_LG); }
+    static __device__ __forceinline__ uint32_t after(uint32_t h) { return (h + 1) & ((1u << WIN_SET_LG) - 1u); }
+    __device__ __forceinline__ uint32_t operator()(const uint32_t (&o)[8], int (&s)[8]) const {
+        uint32_t c = 0, w[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) w[j] = (uint32_t)shared_s32(tab + 4 * home(o[j]));
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            uint32_t h = home(o[j]);
+            while (w[j] != SLOT_EMPTY && w[j] >> 16 != o[j]) {  // ends: half of the slots are empty
+                h = after(h);
+                w[j] = (uint32_t)shared_s32(tab + 4 * h);
+            }
+            s[j] = w[j] != SLOT_EMPTY ? -1 : 0;
+            if (s[j] < 0) {
+                asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(tab + 4 * h) : "memory");
+                ++c;
+            }
+        }
+        return c;
+    }
+    template <bool LOW>
+    static __device__ __forceinline__ uint32_t offset(uint32_t i) { return LOW ? i : 4u * win_place(i); }
+    // The entries p0 .. p1 - 1 of col, in window 1 or (LOW) below it.
+    template <bool LOW>
+    static __device__ __forceinline__ void insert(uint32_t* slots, const int32_t* __restrict__ col, int32_t first, int p0,
+                                                  int p1) {
+        for (int p = p0 + lane_id(); p < p1; p += 32) {
+            const uint32_t o = offset<LOW>((uint32_t)(col[p] - first));
+            uint32_t h = home(o);
+            while (atomicCAS(&slots[h], SLOT_EMPTY, o << 16) != SLOT_EMPTY) h = after(h);  // entries are distinct
+        }
+        __syncwarp();
+    }
+    template <bool LOW>
+    static __device__ __forceinline__ void flush(uint32_t* slots, const int32_t* __restrict__ col, int32_t first, int p0,
+                                                 int p1, unsigned long long* __restrict__ t) {
+        for (int p = p0 + lane_id(); p < p1; p += 32) {
+            const uint32_t o = offset<LOW>((uint32_t)(col[p] - first));
+            uint32_t h = home(o);
+            while (slots[h] >> 16 != o) h = after(h);
+            const uint32_t c = slots[h] & 0xffffu;
+            if (c) atomicAdd(&t[col[p]], (unsigned long long)c);
+        }
+        __syncwarp();
+        // Emptied from every entry's home slot on: whoever empties a slot goes on to the
+        // next, so each run of taken slots is emptied to its end.
+        for (int p = p0 + lane_id(); p < p1; p += 32)
+            for (uint32_t h = home(offset<LOW>((uint32_t)(col[p] - first))); slots[h] != SLOT_EMPTY; h = after(h))
+                slots[h] = SLOT_EMPTY;
+        __syncwarp();
+    }
+};
+
 // Below-window tasks: for each window k >= 2 that N+(v) reaches, a warp marks N+(v)'s
 // entries there in a bitmap, streams the in-edges' entries of the window against it and
 // clears the marks.  8 KB of shared memory a warp leave 24 warps per SM; four windows of
 // half the size and 48 warps took longer (R-MAT scale 23: 1.38 instead of 1.18 ms), since
 // hubs then read their in-edges once more per window.
+//
+// Matches against the bitmap add to t in global memory, one atomic each.  Below window 1 of
+// an R-MAT graph they are few, but in a graph of communities (hub_dense) most probes match
+// and the atomics bind, 150 G/s.  There the lists go into sets in the bitmaps' memory
+// instead, and the medium hubs' window tasks are counted the same way (k_tc_hub_med leaves
+// them).  Whole calls, one atomic per match / sets: disjoint cliques of 100 (100,000
+// vertices) 1.75 / 0.92 ms, of 800 (32,000) 27.2 / 4.5; a ring lattice of 128 neighbours
+// on either side (65,536) 4.50 / 1.5; R-MAT scale 20 and 23 within 0.3 %.
 constexpr int WIN2_THREADS = 256;
 constexpr int WIN2_WARPS = WIN2_THREADS / 32;
 constexpr int WIN2_BLOCKS = 3;
 static_assert(HUB_WIN2 == 0xffff, "the last offset of an 8 KB bitmap is no rank's");
+static_assert((HUB_WIN2 + 1) / 32 == 1 << WIN_SET_LG && 2 * WIN_SET_MAX == 1 << WIN_SET_LG, "slots of a set");
 
 struct Win2Shared {
     uint32_t bm[WIN2_WARPS][(HUB_WIN2 + 1) / 32];
@@ -2159,20 +2295,52 @@ struct Win2Shared {
 };
 
 __global__ void __launch_bounds__(WIN2_THREADS) k_tc_hub_win2(
-    Windows T, const int2* __restrict__ rowinfo, const uint4* __restrict__ winlow, const int32_t* __restrict__ col,
-    const uint4* __restrict__ win, const int4* __restrict__ low_task, bool probe_mode, int big_in,
-    const uint32_t* __restrict__ indeg, int32_t hub0, const uint2* __restrict__ in_rec,
-    unsigned long long* __restrict__ t, DevStats* stats) {
+    Windows T, const int2* __restrict__ rowinfo, const uint2* __restrict__ winrow, const uint4* __restrict__ winlow,
+    const int32_t* __restrict__ col, const uint4* __restrict__ win, const int4* __restrict__ win_task, int64_t task_cap,
+    const int4* __restrict__ low_task, bool probe_mode, int big_in, const uint32_t* __restrict__ indeg, int32_t hub0,
+    const uint2* __restrict__ in_rec, unsigned long long* __restrict__ t, DevStats* stats) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Win2Shared& sh = *reinterpret_cast<Win2Shared*>(smem_raw);
     const int lane = lane_id(), w = threadIdx.x >> 5;
-    const unsigned nlow = stats->hub_low;
-    if (blockIdx.x * WIN2_WARPS >= nlow) return;
+    const bool dense = hub_dense(stats);
+    const unsigned nlow = stats->hub_low, nmed = dense ? stats->hub_med : 0;
+    if (blockIdx.x * WIN2_WARPS >= max(nlow, nmed)) return;
     uint32_t* const bm = sh.bm[w];
     const uint32_t bm_addr = (uint32_t)__cvta_generic_to_shared(bm);
-    for (int i = lane; i < (HUB_WIN2 + 1) / 32; i += 32) bm[i] = 0;
-    __syncwarp();
+    const auto clear = [&](uint32_t word) {
+        for (int i = lane; i < (HUB_WIN2 + 1) / 32; i += 32) bm[i] = word;
+        __syncwarp();
+    };
+    clear(dense ? SLOT_EMPTY : 0u);  // empty sets or bitmaps
+    // a task's in-edges in one window; the next batch's records are loaded ahead
+    const auto stream = [&](auto low, const int4& task, int e1, int win_no, bool hub_in_window, const auto& probe) {
+        uint32_t hits = 0;
+        uint2 rec = task.y + lane < e1 ? in_rec[task.y + lane] : make_uint2(0, 0);
+        for (int bb = task.y; bb < e1; bb += 32) {
+            const uint2 cur = rec;
+            rec = bb + 32 + lane < e1 ? in_rec[bb + 32 + lane] : make_uint2(0, 0);
+            hits += win_batch<false, decltype(low)::value>(cur, win_no, hub_in_window, rowinfo, winrow, winlow, win, probe,
+                                                           t, sh.at[w], sh.cw[w], nullptr);
+        }
+        return hits;
+    };
     unsigned q = blockIdx.x * WIN2_WARPS + w;
+    while (q < nmed) {
+        unsigned nx = 0;
+        if (lane == 0) nx = gridDim.x * WIN2_WARPS + atomicAdd(&stats->hub_next2, 1u);
+        const int4 task = win_task[task_cap - 1 - q];
+        q = __shfl_sync(FULL, nx, 0);
+        const int ne = task.w & ((1 << TASK_BITS) - 1), p1 = task.z + (int)((uint32_t)task.w >> TASK_BITS);
+        if (p1 - task.z > WIN_SET_MAX) {  // the lists never make such a hub medium: do not overrun the set
+            if (lane == 0) atomicOr(&stats->err, ERR_OVERFLOW);
+            continue;
+        }
+        WinSet::insert<false>(bm, col, T.first[1], task.z, p1);
+        const uint32_t hits = stream(std::false_type{}, task, task.y + ne, 1, task.x >= T.first[1], WinSet{bm_addr});
+        WinSet::flush<false>(bm, col, T.first[1], task.z, p1, t);
+        if (lane == 0 && hits) atomicAdd(&t[task.x], (unsigned long long)hits);
+    }
+    q = blockIdx.x * WIN2_WARPS + w;
     while (q < nlow) {
         unsigned nx = 0;
         if (lane == 0) nx = gridDim.x * WIN2_WARPS + atomicAdd(&stats->hub_next4, 1u);
@@ -2190,21 +2358,23 @@ __global__ void __launch_bounds__(WIN2_THREADS) k_tc_hub_win2(
             int p0 = rv.x;
             if (v < first) p0 += lower_bound(col + rv.x, 0, p1 - rv.x, first);
             if (p0 == p1) continue;
+            if (dense && p1 - p0 <= WIN_SET_MAX) {
+                WinSet::insert<true>(bm, col, first, p0, p1);
+                vtot += stream(std::true_type{}, task, e1, win_no, v >= first, WinSet{bm_addr});
+                WinSet::flush<true>(bm, col, first, p0, p1, t);
+                p1 = p0;
+                continue;
+            }
+            if (dense) clear(0u);
             for (int p = p0 + lane; p < p1; p += 32) {
                 const int x = col[p] - first;
                 atomicOr(&bm[x >> 5], 1u << (x & 31));
             }
             __syncwarp();
-            const WinBits P{bm_addr, t + first};
-            uint2 rec = task.y + lane < e1 ? in_rec[task.y + lane] : make_uint2(0, 0);
-            for (int bb = task.y; bb < e1; bb += 32) {
-                const uint2 cur = rec;  // the next batch's records are loaded ahead
-                rec = bb + 32 + lane < e1 ? in_rec[bb + 32 + lane] : make_uint2(0, 0);
-                vtot += win_batch<false, true>(cur, win_no, v >= first, rowinfo, nullptr, winlow, win, P, t, sh.at[w],
-                                               sh.cw[w], nullptr);
-            }
+            vtot += stream(std::true_type{}, task, e1, win_no, v >= first, WinBits{bm_addr, t + first});
             for (int p = p0 + lane; p < p1; p += 32) bm[(col[p] - first) >> 5] = 0;
             __syncwarp();
+            if (dense) clear(SLOT_EMPTY);
             p1 = p0;
         }
         if (lane == 0 && vtot) atomicAdd(&t[v], (unsigned long long)vtot);
@@ -2551,7 +2721,8 @@ bool launch_plan(const CountBuffers& C, const Strategy& S, const Launch& L, cons
         count_launch();
     }
     if (forked) cudaEventRecord(ps->join, H.stream);
-    k_plan<<<grid_for(C.n, THREADS * PLAN_ITEMS, L.sms), THREADS, 0, L.stream>>>(C.n, C.rowstart, C.rowlen, C.col,
+    const int samplers = hubs ? sample_blocks(C.n) : 0;
+    k_plan<<<samplers + grid_for(C.n, THREADS * PLAN_ITEMS, L.sms), THREADS, 0, L.stream>>>(C.n, samplers, C.rowstart, C.rowlen, C.rowinfo, C.col,
                                                                    C.small_list[0], C.small_list[1],
                                                                    C.small_list[2], C.small_list[3], C.cta_list,
                                                                    C.src_lo, C.src_hi, C.stats);
@@ -2568,10 +2739,12 @@ cudaError_t intersect_init_attributes() {
         (e = cudaFuncSetAttribute(k_tc_small_wide<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, wide)) ||
         (e = cudaFuncSetAttribute(k_tc_hub<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(HubShared))) ||
         (e = cudaFuncSetAttribute(k_tc_hub<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(HubShared))) ||
-        (e = cudaFuncSetAttribute(k_tc_hub_med<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)sizeof(MedShared<false>))) ||
-        (e = cudaFuncSetAttribute(k_tc_hub_med<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)sizeof(MedShared<true>))) ||
+        (e = cudaFuncSetAttribute(k_tc_hub_med<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)sizeof(MedShared<false, false>))) ||
+        (e = cudaFuncSetAttribute(k_tc_hub_med<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)sizeof(MedShared<false, true>))) ||
+        (e = cudaFuncSetAttribute(k_tc_hub_med<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)sizeof(MedShared<true, false>))) ||
         (e = cudaFuncSetAttribute(k_tc_hub_win2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Win2Shared))) ||
         (e = cudaFuncSetAttribute(k_tc_hub_low, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LowShared))) ||
         (e = cudaFuncSetAttribute(k_tc_hub_list<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2648,7 +2821,9 @@ void intersect_impl(const CountBuffers& C, const Strategy& S, cudaEvent_t* ev, c
                 T.first[1], C.rowinfo, C.winrow, C.col, C.win, C.win_task, C.in_rec, C.t_rank, C.stats, C.sup);
             count_launch();
         }
-        k_tc_hub_med<SUP><<<L.sms * WINK_BLOCKS, WINK_THREADS, sizeof(MedShared<SUP>), L.stream>>>(
+        const bool all = !SUP && T.first[1] == 0;
+        const auto med = all ? k_tc_hub_med<SUP, !SUP> : k_tc_hub_med<SUP, false>;
+        med<<<L.sms * WINK_BLOCKS, WINK_THREADS, all ? sizeof(MedShared<SUP, !SUP>) : sizeof(MedShared<SUP, false>), L.stream>>>(
             T.first[1], C.n - T.first[1], C.rowinfo, C.winrow, C.col, C.win, C.win_task, task_cap, C.in_rec, C.t_rank, C.stats, C.sup);
         count_launch();
         if (T.first[1] > 0) {  // something lies below window 1
@@ -2657,7 +2832,7 @@ void intersect_impl(const CountBuffers& C, const Strategy& S, cudaEvent_t* ev, c
                     C.rowinfo, C.winrow, C.col, C.low_task, C.in_rec, C.stats, C.sup);
             else
                 k_tc_hub_win2<<<L.sms * WIN2_BLOCKS, WIN2_THREADS, sizeof(Win2Shared), L.stream>>>(
-                    T, C.rowinfo, C.winlow, C.col, C.win, C.low_task, probe, S.hub_big_in > 0 ? S.hub_big_in : 1,
+                    T, C.rowinfo, C.winrow, C.winlow, C.col, C.win, C.win_task, task_cap, C.low_task, probe, S.hub_big_in > 0 ? S.hub_big_in : 1,
                     C.hub_cnt, C.n - C.hub_cap, C.in_rec, C.t_rank, C.stats);
             count_launch();
         }
