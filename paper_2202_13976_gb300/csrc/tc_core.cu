@@ -182,6 +182,8 @@ constexpr int COUNT_BLOCKS = 7;
 // Bound by instruction issue: R-MAT scale 20 / 23 0.207 / 0.257 ms, a 600,011-pair graph
 // 39 us.  One row at a time, eight popcounts a lane and one atomic per entry took 0.31 /
 // 0.39 ms and 54 us; two rows in flight 0.209 / 0.262 ms, blocks of 256 0.231 / 0.285 ms.
+// Rows whose range nowhere overlaps x's are passed over, four at a time: the support of a
+// complete bipartite graph of 3,000 + 3,000 vertices took 0.79 ms, 0.35 so.
 template <bool SUP>
 __global__ void __launch_bounds__(COUNT_THREADS, COUNT_BLOCKS) k_core_count(
     int32_t n, const int64_t* __restrict__ rowstart, const int32_t* __restrict__ rowlen, const int32_t* __restrict__ col,
@@ -219,9 +221,10 @@ __global__ void __launch_bounds__(COUNT_THREADS, COUNT_BLOCKS) k_core_count(
             }
             const int w0 = b0 >> 5, w1 = b0 <= b1 ? min(b1 >> 5, used - 1) : -1;
             uint32_t sum = 0;  // lane k < CORE_CHUNK: the bits shared with entry p0 + k
+            const unsigned live = __ballot_sync(FULL, w1 >= 0);
 #pragma unroll
             for (int g = 0; g < CORE_CHUNK; g += CORE_AHEAD) {
-                if (p0 + g >= d) break;
+                if (!(live >> g & ((1u << CORE_AHEAD) - 1u))) continue;  // ranges that nowhere overlap
                 uint32_t v[CORE_AHEAD][CORE_LANE_WORDS];
 #pragma unroll
                 for (int k = 0; k < CORE_AHEAD; ++k)

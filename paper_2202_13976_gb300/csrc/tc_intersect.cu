@@ -728,6 +728,13 @@ __global__ void k_hub_scatter_rows(int32_t n, int32_t hub_cap, const int64_t* __
 constexpr int TASK_BITS = 12;
 static_assert(HUB_SLICE < 1 << TASK_BITS && (int64_t)HUB_WIN << TASK_BITS < INT_MAX, "window task fields");
 
+// Per-edge support: the part below window 1 of a big hub's list is taken by a block from so
+// many entries on (a long one has to be: HUB_WARP_MAX).  Block + warp kernel, from 0 / 64 /
+// 256 entries on: G(60,000) of 16.8 M pairs 1.34 + 0.03, 1.19 + 1.05, 0.37 + 3.58 ms; R-MAT
+// scale 20 54 + 127, 3 + 151, 3 + 150 us.
+constexpr int HUB_LIST_MIN = 64;
+static_assert(HUB_LIST_MIN <= HUB_WARP_MAX, "what a warp stages");
+
 // First of `mine` slots reserved for this lane in a list (a warp's lanes in order).
 __device__ __forceinline__ unsigned warp_reserve(unsigned mine, unsigned* counter) {
     const unsigned inc = warp_inclusive_scan(mine);
@@ -771,7 +778,7 @@ __global__ void k_hub_lists(int32_t n, int32_t hub_cap, int32_t T0w, const int2*
             }
             if (shard) din = (uint32_t)min(filled, (unsigned long long)din);
         }
-        const bool lng = big && dlow > HUB_WARP_MAX;
+        const bool lng = big && dlow > HUB_LIST_MIN;
         const unsigned pb = warp_append(big, &stats->hub_big);
         const unsigned pl = warp_append(lng, &stats->hub_long);
         if (big) big_list[pb] = v;
@@ -1948,12 +1955,22 @@ __device__ __forceinline__ uint32_t win_batch(const uint2 rec, int win_no, bool 
             const uint32_t ch = probe(o, s);
             c |= ch << (16 * h);
             if (SUP) {
+                // edges (u, x): eight lanes take a vector's eight entries, which lie in one or
+                // two sectors (k_tc_hub for 150 shuffled cliques of 300: each lane its own
+                // entries one by one 1.61 ms, so 0.78)
                 const int32_t cb = __shfl_sync(FULL, cbase, idx[h]), ex = __shfl_sync(FULL, E.excl, idx[h]);
-                if (ch) {
-                    const int64_t p0 = (int64_t)cb + 8 * (int64_t)(item + 32 * h - ex);
+                const int32_t p0 = cb + 8 * (item + 32 * h - ex);
+                uint32_t m = 0;
 #pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        if (s[j] < 0) atomicAdd(&sup[p0 + j], 1u);  // edge (u, x)
+                for (int j = 0; j < 8; ++j) m |= (uint32_t)(s[j] < 0) << j;
+                const unsigned any = __ballot_sync(FULL, m != 0);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    if (!(any >> (4 * k) & 0xfu)) continue;
+                    const int from = 4 * k + (lane >> 3);
+                    const uint32_t mk = __shfl_sync(FULL, m, from);
+                    const int32_t pk = __shfl_sync(FULL, p0, from);
+                    if (mk >> (lane & 7) & 1u) atomicAdd(&sup[pk + (lane & 7)], 1u);
                 }
             }
         }
@@ -2398,7 +2415,8 @@ struct LowShared {
 
 __global__ void __launch_bounds__(LOW_THREADS) k_tc_hub_low(
     const int2* __restrict__ rowinfo, const uint2* __restrict__ winrow, const int32_t* __restrict__ col,
-    const int4* __restrict__ low_task, const uint2* __restrict__ in_rec, DevStats* stats, uint32_t* __restrict__ sup) {
+    const int4* __restrict__ low_task, int big_in, const uint32_t* __restrict__ indeg, int32_t hub0,
+    const uint2* __restrict__ in_rec, DevStats* stats, uint32_t* __restrict__ sup) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     LowShared& sh = *reinterpret_cast<LowShared*>(smem_raw);
     const int lane = lane_id(), w = threadIdx.x >> 5;
@@ -2422,8 +2440,9 @@ __global__ void __launch_bounds__(LOW_THREADS) k_tc_hub_low(
         q = nx;
         const int64_t e0 = task.y, e1 = e0 + task.z;
         const int dlow = task.w;
-        if (dlow > HUB_WARP_MAX) continue;  // the list kernel's
         const int2 rv = rowinfo[task.x];
+        if (dlow > HUB_LIST_MIN && (indeg[task.x - hub0] >= (uint32_t)big_in || rv.y > HUB_WARP_MAX))
+            continue;  // the list kernel's
         int lg = 5;
         while ((1 << lg) < HUB_HASH_LOAD * dlow) ++lg;
         const unsigned shift = 32u - (unsigned)lg, mask = (1u << lg) - 1u;
@@ -2829,7 +2848,8 @@ void intersect_impl(const CountBuffers& C, const Strategy& S, cudaEvent_t* ev, c
         if (T.first[1] > 0) {  // something lies below window 1
             if (SUP)
                 k_tc_hub_low<<<L.sms * LOW_BLOCKS, LOW_THREADS, sizeof(LowShared), L.stream>>>(
-                    C.rowinfo, C.winrow, C.col, C.low_task, C.in_rec, C.stats, C.sup);
+                    C.rowinfo, C.winrow, C.col, C.low_task, S.hub_big_in > 0 ? S.hub_big_in : 1, C.hub_cnt,
+                    C.n - C.hub_cap, C.in_rec, C.stats, C.sup);
             else
                 k_tc_hub_win2<<<L.sms * WIN2_BLOCKS, WIN2_THREADS, sizeof(Win2Shared), L.stream>>>(
                     T, C.rowinfo, C.winrow, C.winlow, C.col, C.win, C.win_task, task_cap, C.low_task, probe, S.hub_big_in > 0 ? S.hub_big_in : 1,
