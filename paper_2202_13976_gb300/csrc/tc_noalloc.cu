@@ -451,6 +451,14 @@ extern "C" tc_status tc_count_noalloc(int32_t n, int64_t m, const int32_t* src, 
         S = g_na_ptr[dev];
     }
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+    if (m == 0) {  // no edge: all counts and coefficients are zero
+        if (t_out && n > 0) e = cudaMemsetAsync(t_out, 0, sizeof(uint64_t) * (size_t)n, stream);
+        if (e == cudaSuccess && lcc_out && n > 0) e = cudaMemsetAsync(lcc_out, 0, sizeof(double) * (size_t)n, stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+        if (e != cudaSuccess) return TC_ECUDA;
+        *T_out = 0;
+        return TC_OK;
+    }
     const NaArrays A = na_arrays(S, n, (int32_t)m);
     const size_t word = sizeof(uint32_t) * (size_t)n;
     const auto blocks = [](int64_t work, int64_t per, int64_t most) {

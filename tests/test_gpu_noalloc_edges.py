@@ -58,3 +58,17 @@ def test_noalloc_leaves_the_outputs_when_an_id_is_bad(tc):
         tc.tc_count_noalloc(4, s, s.roll(1), t)
     assert err.value.status == tc.TC_EINVAL
     assert (t == -1).all()
+
+
+@pytest.mark.parametrize("n", [0, 1, 512, 513, 16384])
+@pytest.mark.parametrize("outputs", [0, 1])
+def test_noalloc_without_pairs_launches_nothing(tc, n, outputs):
+    import torch
+    none = torch.empty(0, dtype=torch.int32, device="cuda")
+    t = torch.full((n,), -1, dtype=torch.int64, device="cuda") if outputs else None
+    lcc = torch.full((n,), -1.0, dtype=torch.float64, device="cuda") if outputs else None
+    before = tc.tc_launch_count()
+    assert tc.tc_count_noalloc(n, none, none, t, lcc) == 0
+    assert tc.tc_launch_count() == before
+    if outputs:
+        assert (t == 0).all() and (lcc.view(torch.int64) == 0).all()
