@@ -485,11 +485,13 @@ __global__ void __launch_bounds__(WIN_THREADS) k_win_build(int32_t n, Windows T,
     for (int64_t t0 = (int64_t)blockIdx.x * WIN_THREADS; t0 < c0; t0 += (int64_t)gridDim.x * WIN_THREADS) {
         const int64_t u = t0 + threadIdx.x;
         uint32_t nv = 0, len[WINS + 1] = {};
-        bool hubrow = false;  // a row without a hub has no in-edge records and needs nothing here
+        // a row without a hub has no in-edge records, one of a single entry no suffix: nothing
+        // here is read for them (but for the hubs' own lists)
+        bool hubrow = false;
         if (u < c0 && ((u >= src_lo && u < src_hi) || u >= R)) {  // a shard: its sources and the hubs
             const int2 ri = rowinfo[u];
             const int32_t end = ri.x + ri.y;
-            hubrow = ri.y > 0 && col[end - 1] >= R;
+            hubrow = ri.y > (u < R ? 1 : 0) && col[end - 1] >= R;
             if (hubrow) {
                 int at = ri.y;
                 cut[0][threadIdx.x] = end;
