@@ -393,10 +393,13 @@ __global__ void __launch_bounds__(DG_THREADS, PACKED ? DGH_BLOCKS : DGH_BLOCKS -
             if (i < i1) r = rec[i];
             const uint32_t fuv = (uint32_t)r.w;
             // the group's lanes take positions sb + gl + 8 j, DGH_UNROLL loads in flight
-            for (int p0 = r.y + gl; p0 < r.z; p0 += 8 * DGH_UNROLL) {
+            // (counted from the suffix's start: past the last entries a position may be 2^31 or more)
+            const int64_t at = (int64_t)r.y + gl;
+            const int left = r.z - r.y - gl;
+            for (int p0 = 0; p0 < left; p0 += 8 * DGH_UNROLL) {
                 typename R::X x[DGH_UNROLL];
 #pragma unroll
-                for (int j = 0; j < DGH_UNROLL; ++j) x[j] = p0 + 8 * j < r.z ? rows.at(p0 + 8 * j) : R::none();
+                for (int j = 0; j < DGH_UNROLL; ++j) x[j] = p0 + 8 * j < left ? rows.at(at + p0 + 8 * j) : R::none();
 #pragma unroll
                 for (int j = 0; j < DGH_UNROLL; ++j) {
                     const int32_t w = R::rank(x[j]);

@@ -1961,7 +1961,7 @@ __device__ __forceinline__ uint32_t win_batch(const uint2 rec, int win_no, bool 
                 // two sectors (k_tc_hub for 150 shuffled cliques of 300: each lane its own
                 // entries one by one 1.61 ms, so 0.78)
                 const int32_t cb = __shfl_sync(FULL, cbase, idx[h]), ex = __shfl_sync(FULL, E.excl, idx[h]);
-                const int32_t p0 = cb + 8 * (item + 32 * h - ex);
+                const uint32_t p0 = (uint32_t)cb + 8u * (uint32_t)(item + 32 * h - ex);
                 uint32_t m = 0;
 #pragma unroll
                 for (int j = 0; j < 8; ++j) m |= (uint32_t)(s[j] < 0) << j;
@@ -1971,7 +1971,7 @@ __device__ __forceinline__ uint32_t win_batch(const uint2 rec, int win_no, bool 
                     if (!(any >> (4 * k) & 0xfu)) continue;
                     const int from = 4 * k + (lane >> 3);
                     const uint32_t mk = __shfl_sync(FULL, m, from);
-                    const int32_t pk = __shfl_sync(FULL, p0, from);
+                    const uint32_t pk = __shfl_sync(FULL, p0, from);
                     if (mk >> (lane & 7) & 1u) atomicAdd(&sup[pk + (lane & 7)], 1u);
                 }
             }
@@ -1995,6 +1995,17 @@ __device__ __forceinline__ uint32_t win_batch(const uint2 rec, int win_no, bool 
     }
     __syncwarp();
     return running;
+}
+
+// Positions in col and in the in-edge records are below 2^31; a step or a lane past the last
+// ones is not, so they are compared as 32 unsigned bits.
+__host__ __device__ __forceinline__ constexpr bool before_end(uint32_t at, uint32_t end) { return at < end; }
+static_assert(!before_end((uint32_t)INT_MAX - 1u + HUB_SLICE, (uint32_t)INT_MAX) &&
+                  !before_end((uint32_t)INT_MAX + WINK_THREADS, (uint32_t)INT_MAX),
+              "no position past the end wraps to one before it");
+// The record at `at` of a task's in-edges, {0, 0} past their end.
+__device__ __forceinline__ uint2 record_at(const uint2* __restrict__ in_rec, uint32_t at, uint32_t end) {
+    return before_end(at, end) ? in_rec[at] : make_uint2(0, 0);
 }
 
 // In-edges a warp claims at a time: smaller batches when a slice has fewer than two
@@ -2042,25 +2053,24 @@ __global__ void __launch_bounds__(WINK_THREADS, WINK_BLOCKS) k_tc_hub(
         if (threadIdx.x == 0) next = gridDim.x + atomicAdd(&stats->hub_next, 1u);
         const int4 task = win_task[q];
         const int32_t v = task.x;
-        const int ne = task.w & ((1 << TASK_BITS) - 1), p1 = task.z + (int)((uint32_t)task.w >> TASK_BITS);
-        const int e1 = task.y + ne;
-        for (int p = task.z + (int)threadIdx.x; p < p1; p += WINK_THREADS)
+        const uint32_t ne = (uint32_t)task.w & ((1u << TASK_BITS) - 1u), p1 = (uint32_t)task.z + ((uint32_t)task.w >> TASK_BITS);
+        const uint32_t e1 = (uint32_t)task.y + ne;
+        for (uint32_t p = (uint32_t)task.z + threadIdx.x; before_end(p, p1); p += WINK_THREADS)
             sh.cnt[win_place((uint32_t)(col[p] - T0w))] |= WIN_MARK;
         __syncthreads();
         uint32_t vtot = 0;
-        const int bs = hub_batch_size(ne, WINK_WARPS);
+        const uint32_t bs = (uint32_t)hub_batch_size(ne, WINK_WARPS);
         for (;;) {
             unsigned k = 0;
             if (lane == 0) k = atomicAdd(&sh.bq, 1u);
-            k = __shfl_sync(FULL, k, 0) * (unsigned)bs;
-            if (k >= (unsigned)ne) break;
-            const int e = task.y + (int)k + lane;
-            const uint2 rec = lane < bs && e < e1 ? in_rec[e] : make_uint2(0, 0);
+            k = __shfl_sync(FULL, k, 0) * bs;
+            if (k >= ne) break;
+            const uint2 rec = (uint32_t)lane < bs ? record_at(in_rec, (uint32_t)task.y + k + lane, e1) : make_uint2(0, 0);
             vtot += win_batch<SUP, false>(rec, 1, v >= T0w, rowinfo, winrow, nullptr, win, P, t, sh.at[w], sh.cw[w], sup);
         }
         if (lane == 0) sh.vt[w] = vtot;
         __syncthreads();
-        for (int p = task.z + (int)threadIdx.x; p < p1; p += WINK_THREADS) {
+        for (uint32_t p = (uint32_t)task.z + threadIdx.x; before_end(p, p1); p += WINK_THREADS) {
             const uint32_t x = win_place((uint32_t)(col[p] - T0w));
             const uint32_t c = sh.cnt[x] & ~WIN_MARK;
             sh.cnt[x] = SUP ? 0u : c;
@@ -2131,8 +2141,8 @@ __global__ void __launch_bounds__(WINK_THREADS, WINK_BLOCKS) k_tc_hub_med(
         if (lane == 0) nx = gridDim.x * WINK_WARPS + atomicAdd(&stats->hub_next2, 1u);
         const int4 task = win_task[task_cap - 1 - q];
         const int32_t v = task.x;
-        const int ne = task.w & ((1 << TASK_BITS) - 1), dwin = (int)((uint32_t)task.w >> TASK_BITS);
-        const int e1 = task.y + ne;
+        const int dwin = (int)((uint32_t)task.w >> TASK_BITS);
+        const uint32_t e0 = (uint32_t)task.y, e1 = e0 + ((uint32_t)task.w & ((1u << TASK_BITS) - 1u));
         uint32_t vtot = 0;
         if constexpr (!SUP) {
             const WinMarks P{(uint32_t)__cvta_generic_to_shared(sh.marks), (uint32_t)__cvta_generic_to_shared(sh.cnt),
@@ -2142,10 +2152,10 @@ __global__ void __launch_bounds__(WINK_THREADS, WINK_BLOCKS) k_tc_hub_med(
                 atomicOr(&sh.marks[x >> 1], 1u << (w + 16 * (x & 1)));
             }
             __syncwarp();
-            uint2 rec = task.y + lane < e1 ? in_rec[task.y + lane] : make_uint2(0, 0);
-            for (int bb = task.y; bb < e1; bb += 32) {
+            uint2 rec = record_at(in_rec, e0 + lane, e1);
+            for (uint32_t bb = e0; before_end(bb, e1); bb += 32) {
                 const uint2 cur = rec;  // the next batch's records are loaded ahead
-                rec = bb + 32 + lane < e1 ? in_rec[bb + 32 + lane] : make_uint2(0, 0);
+                rec = record_at(in_rec, bb + 32 + lane, e1);
                 vtot += win_batch<SUP, false>(cur, 1, v >= T0w, rowinfo, winrow, nullptr, win, P, t, sh.at[w], sh.cw[w], sup);
             }
             for (int p = lane; p < dwin; p += 32) {
@@ -2187,8 +2197,8 @@ __global__ void __launch_bounds__(WINK_THREADS, WINK_BLOCKS) k_tc_hub_med(
             __syncwarp();
             const WinBitmap P{(uint32_t)__cvta_generic_to_shared(M.bm), (uint32_t)__cvta_generic_to_shared(M.pre),
                               (uint32_t)__cvta_generic_to_shared(M.cnt)};
-            for (int bb = task.y; bb < e1; bb += 32) {
-                const uint2 rec = bb + lane < e1 ? in_rec[bb + lane] : make_uint2(0, 0);
+            for (uint32_t bb = e0; before_end(bb, e1); bb += 32) {
+                const uint2 rec = record_at(in_rec, bb + lane, e1);
                 win_batch<SUP, false>(rec, 1, v >= T0w, rowinfo, winrow, nullptr, win, P, t, sh.at[w], sh.cw[w], sup);
             }
             for (int p = lane; p < dwin; p += 32) {
@@ -2259,9 +2269,9 @@ struct WinSet {
     static __device__ __forceinline__ uint32_t offset(uint32_t i) { return LOW ? i : 4u * win_place(i); }
     // The entries p0 .. p1 - 1 of col, in window 1 or (LOW) below it.
     template <bool LOW>
-    static __device__ __forceinline__ void insert(uint32_t* slots, const int32_t* __restrict__ col, int32_t first, int p0,
-                                                  int p1) {
-        for (int p = p0 + lane_id(); p < p1; p += 32) {
+    static __device__ __forceinline__ void insert(uint32_t* slots, const int32_t* __restrict__ col, int32_t first,
+                                                  uint32_t p0, uint32_t p1) {
+        for (uint32_t p = p0 + lane_id(); before_end(p, p1); p += 32) {
             const uint32_t o = offset<LOW>((uint32_t)(col[p] - first));
             uint32_t h = home(o);
             while (atomicCAS(&slots[h], SLOT_EMPTY, o << 16) != SLOT_EMPTY) h = after(h);  // entries are distinct
@@ -2269,9 +2279,9 @@ struct WinSet {
         __syncwarp();
     }
     template <bool LOW>
-    static __device__ __forceinline__ void flush(uint32_t* slots, const int32_t* __restrict__ col, int32_t first, int p0,
-                                                 int p1, unsigned long long* __restrict__ t) {
-        for (int p = p0 + lane_id(); p < p1; p += 32) {
+    static __device__ __forceinline__ void flush(uint32_t* slots, const int32_t* __restrict__ col, int32_t first,
+                                                 uint32_t p0, uint32_t p1, unsigned long long* __restrict__ t) {
+        for (uint32_t p = p0 + lane_id(); before_end(p, p1); p += 32) {
             const uint32_t o = offset<LOW>((uint32_t)(col[p] - first));
             uint32_t h = home(o);
             while (slots[h] >> 16 != o) h = after(h);
@@ -2281,7 +2291,7 @@ struct WinSet {
         __syncwarp();
         // Emptied from every entry's home slot on: whoever empties a slot goes on to the
         // next, so each run of taken slots is emptied to its end.
-        for (int p = p0 + lane_id(); p < p1; p += 32)
+        for (uint32_t p = p0 + lane_id(); before_end(p, p1); p += 32)
             for (uint32_t h = home(offset<LOW>((uint32_t)(col[p] - first))); slots[h] != SLOT_EMPTY; h = after(h))
                 slots[h] = SLOT_EMPTY;
         __syncwarp();
@@ -2332,12 +2342,12 @@ __global__ void __launch_bounds__(WIN2_THREADS) k_tc_hub_win2(
     };
     clear(dense ? SLOT_EMPTY : 0u);  // empty sets or bitmaps
     // a task's in-edges in one window; the next batch's records are loaded ahead
-    const auto stream = [&](auto low, const int4& task, int e1, int win_no, bool hub_in_window, const auto& probe) {
+    const auto stream = [&](auto low, const int4& task, uint32_t e1, int win_no, bool hub_in_window, const auto& probe) {
         uint32_t hits = 0;
-        uint2 rec = task.y + lane < e1 ? in_rec[task.y + lane] : make_uint2(0, 0);
-        for (int bb = task.y; bb < e1; bb += 32) {
+        uint2 rec = record_at(in_rec, (uint32_t)task.y + lane, e1);
+        for (uint32_t bb = (uint32_t)task.y; before_end(bb, e1); bb += 32) {
             const uint2 cur = rec;
-            rec = bb + 32 + lane < e1 ? in_rec[bb + 32 + lane] : make_uint2(0, 0);
+            rec = record_at(in_rec, bb + 32 + lane, e1);
             hits += win_batch<false, decltype(low)::value>(cur, win_no, hub_in_window, rowinfo, winrow, winlow, win, probe,
                                                            t, sh.at[w], sh.cw[w], nullptr);
         }
@@ -2355,7 +2365,7 @@ __global__ void __launch_bounds__(WIN2_THREADS) k_tc_hub_win2(
             continue;
         }
         WinSet::insert<false>(bm, col, T.first[1], task.z, p1);
-        const uint32_t hits = stream(std::false_type{}, task, task.y + ne, 1, task.x >= T.first[1], WinSet{bm_addr});
+        const uint32_t hits = stream(std::false_type{}, task, (uint32_t)(task.y + ne), 1, task.x >= T.first[1], WinSet{bm_addr});
         WinSet::flush<false>(bm, col, T.first[1], task.z, p1, t);
         if (lane == 0 && hits) atomicAdd(&t[task.x], (unsigned long long)hits);
     }
@@ -2366,7 +2376,7 @@ __global__ void __launch_bounds__(WIN2_THREADS) k_tc_hub_win2(
         const int4 task = low_task[q];
         q = __shfl_sync(FULL, nx, 0);
         const int32_t v = task.x;
-        const int e1 = task.y + task.z;
+        const uint32_t e1 = (uint32_t)(task.y + task.z);
         const int2 rv = rowinfo[v];
         // in probe mode the list kernel counts the big hubs
         if (probe_mode && (indeg[v - hub0] >= (uint32_t)big_in || rv.y > HUB_WARP_MAX)) continue;
@@ -2385,13 +2395,13 @@ __global__ void __launch_bounds__(WIN2_THREADS) k_tc_hub_win2(
                 continue;
             }
             if (dense) clear(0u);
-            for (int p = p0 + lane; p < p1; p += 32) {
+            for (uint32_t p = p0 + lane; before_end(p, p1); p += 32) {
                 const int x = col[p] - first;
                 atomicOr(&bm[x >> 5], 1u << (x & 31));
             }
             __syncwarp();
             vtot += stream(std::true_type{}, task, e1, win_no, v >= first, WinBits{bm_addr, t + first});
-            for (int p = p0 + lane; p < p1; p += 32) bm[(col[p] - first) >> 5] = 0;
+            for (uint32_t p = p0 + lane; before_end(p, p1); p += 32) bm[(col[p] - first) >> 5] = 0;
             __syncwarp();
             if (dense) clear(SLOT_EMPTY);
             p1 = p0;
