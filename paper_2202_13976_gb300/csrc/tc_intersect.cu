@@ -1060,11 +1060,12 @@ __device__ __forceinline__ unsigned bit_or_none(int d) {
     return r;
 }
 
-// Inclusive warp scan whose adds are predicated by the shuffles themselves.
+// Inclusive warp scan whose adds are predicated by the shuffles themselves.  Volatile: all
+// lanes take part, so no step may be merged with another or sink into a branch.
 __device__ __forceinline__ uint32_t warp_scan_u32(uint32_t x) {
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1)
-        asm("{ .reg .pred p; .reg .u32 y; shfl.sync.up.b32 y|p, %0, %1, 0, 0xffffffff; @p add.u32 %0, %0, y; }"
+        asm volatile("{ .reg .pred p; .reg .u32 y; shfl.sync.up.b32 y|p, %0, %1, 0, 0xffffffff; @p add.u32 %0, %0, y; }"
             : "+r"(x)
             : "r"(o));
     return x;
