@@ -346,7 +346,7 @@ tc_status tc_graph_set_hubs(tc_graph* g, int32_t min_degree, int32_t max_hubs);
  * stream): ms[0] planning (bucket lists and hub in-edge lists), ms[1] small
  * bucket, ms[2] block bucket, ms[3] hub bucket, ms[4] total.  count is the length
  * of ms (up to 5).  Synchronises the stream.  Errors: TC_EINVAL before the first
- * count.
+ * count, and for a graph without vertices, which has no phases.
  */
 tc_status tc_graph_last_timing(const tc_graph* g, float* ms, int count);
 
@@ -354,7 +354,8 @@ tc_status tc_graph_last_timing(const tc_graph* g, float* ms, int count);
  * Timing of the graph's build in milliseconds (CUDA events): ms[0] ingest and
  * checks, ms[1] (degree, id) ranks, ms[2] row counts, ms[3] row fill, ms[4] row
  * sort and deduplication, ms[5] degrees, ms[6] total.  count up to 7.  Errors:
- * TC_EINVAL when the build was not timed (a batch recorded into a CUDA graph).
+ * TC_EINVAL when the build was not timed (a batch recorded into a CUDA graph, a graph
+ * without vertices).
  */
 tc_status tc_graph_build_timing(const tc_graph* g, float* ms, int count);
 

@@ -537,7 +537,7 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
     launch_orient(B, g->L, bev, seg ? nullptr : side_streams(g, &psv));
     if (bev) {
         cudaEventRecord(bev[BP_END], g->stream);
-        g->build_timed = true;
+        g->build_timed = n > 0;  // else no phase has run, and its events may be a former graph's
     }
     free_list(g, &scratch);
     cudaError_t e = cudaGetLastError();
@@ -648,7 +648,7 @@ tc_status run_count(tc_graph* g) {
     TC_CK(cudaGetLastError());
     g->counted = true;
     g->verified = false;
-    g->timed = !g->capture;
+    g->timed = !g->capture && g->n > 0;
     return TC_OK;
 }
 

@@ -122,3 +122,17 @@ def test_a_guard_of_the_count_is_reported(fake, call):
         assert fake.tc_count(g, ctypes.byref(T)) == EINTERNAL
     finally:
         fake.tc_graph_destroy(g)
+
+
+@pytest.mark.parametrize("n", [0, 50])
+def test_timings_are_the_graphs_own(fake, n):
+    """A graph without vertices runs no phases: no timing, whatever the events that it took
+    over from a destroyed graph hold."""
+    ms = (ctypes.c_float * 8)()
+    T = ctypes.c_uint64()
+    for size in (50, n):
+        g = _graph(fake, n=size, m=60 if size else 0)
+        assert fake.tc_count(g, ctypes.byref(T)) == OK
+        for timing in (fake.tc_graph_last_timing, fake.tc_graph_build_timing):
+            assert timing(g, ms, 8) == (OK if size else EINVAL)
+        fake.tc_graph_destroy(g)
