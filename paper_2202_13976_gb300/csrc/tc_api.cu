@@ -47,10 +47,11 @@ DeviceState g_dev[64];
 // What a graph needs of the driver beside memory: the second stream and its events, the
 // events of the build and count phases, and the copy stream and events of host input.
 // Sets are handed from a destroyed graph to the next one of the device: creating them
-// took 20 us per graph, and 500 us with eight threads doing so at once.  A stream still
-// holding a former owner's work only orders the next owner's after it; events are
+// took 20 us per graph, and 500 us with eight threads doing so at once.  A set is handed on
+// once its streams are idle, so that no graph waits for a former owner's work; events are
 // recorded anew.  At most SYNC_KEEP sets stay, until tc_release_cached_graphs.
 struct SyncSet {
+    bool known_idle = false;  // given back by a graph that had waited for all its work: not asked (5 us)
     cudaStream_t side = nullptr, copy = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr, landed = nullptr, allocated = nullptr;
     cudaEvent_t ev[PH_EVENTS] = {};
@@ -68,6 +69,15 @@ struct SyncSet {
             if (e == cudaSuccess) e = cudaEventCreate(&x);
         return e;
     }
+    // Queries are refused while any thread captures in global mode, unless relaxed for the call.
+    bool idle() const {
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        const bool yes = cudaStreamQuery(side) == cudaSuccess && cudaStreamQuery(copy) == cudaSuccess;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (!yes) cudaGetLastError();  // cudaErrorNotReady
+        return yes;
+    }
     void destroy() {
         for (cudaEvent_t x : {fork, join, landed, allocated})
             if (x) cudaEventDestroy(x);
@@ -80,16 +90,19 @@ struct SyncSet {
         *this = SyncSet{};
     }
 };
-constexpr size_t SYNC_KEEP = 64;
+constexpr size_t SYNC_KEEP = 64, SYNC_LOOK = 4;
 std::mutex g_sync_mutex;
 std::vector<SyncSet> g_sync[64];  // per device
 
 cudaError_t take_sync(int dev, SyncSet* out) {
     {
         std::lock_guard<std::mutex> lock(g_sync_mutex);
-        if (!g_sync[dev].empty()) {
-            *out = g_sync[dev].back();
-            g_sync[dev].pop_back();
+        std::vector<SyncSet>& kept = g_sync[dev];
+        // the ones given back first are the likeliest to be idle
+        for (size_t k = 0; k < kept.size() && k < SYNC_LOOK; ++k) {
+            if (!kept[k].known_idle && !kept[k].idle()) continue;
+            *out = kept[k];
+            kept.erase(kept.begin() + (std::ptrdiff_t)k);
             return cudaSuccess;
         }
     }
@@ -215,6 +228,8 @@ struct tc_graph {
     // long rows' sort and the plan's hub part (single graphs only)
     SyncSet sync;
     bool has_sync = false;
+    mutable bool side_busy = false;   // the second stream may hold work
+    bool side_joined = true;          // the graph's stream waits for that work
     bool plan_forked = false;         // the last plan ran its hub part on the second stream
 };
 
@@ -315,6 +330,7 @@ tc_status new_graph(int32_t n, void* stream, tc_graph** out) {
 tc_status read_stats(const tc_graph* g, DevStats* h) {
     TC_CK(cudaMemcpyAsync(h, g->stats, sizeof(DevStats), cudaMemcpyDeviceToHost, g->stream));
     TC_CK(cudaStreamSynchronize(g->stream));
+    if (g->side_joined) g->side_busy = false;
     return TC_OK;
 }
 
@@ -534,6 +550,7 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
     launch_rank(B, deg_bits, g->L);
     if (bev) cudaEventRecord(bev[BP_RANK], g->stream);
     PlanStreams psv{};
+    g->side_busy = true;  // joined by launch_orient
     launch_orient(B, g->L, bev, seg ? nullptr : side_streams(g, &psv));
     if (bev) {
         cudaEventRecord(bev[BP_END], g->stream);
@@ -601,6 +618,7 @@ CountBuffers count_buffers(tc_graph* g) {
 // wherever the hub lists are read outside the count.
 void join_plan(tc_graph* g) {
     if (g->plan_forked) cudaStreamWaitEvent(g->stream, g->sync.join, 0);
+    g->side_joined = true;
 }
 
 // Planning (a4): bucket lists and hub in-edge lists; rerun when hub settings change.
@@ -614,6 +632,8 @@ tc_status run_plan(tc_graph* g) {
     // single graphs build their hub lists on a second stream while the push buckets
     // are counted; batches (which may be recorded into a CUDA graph) keep one stream
     PlanStreams psv{};
+    g->side_busy = true;
+    g->side_joined = false;
     g->plan_forked = launch_plan(count_buffers(g), g->strat, g->L, side_streams(g, &psv));
     TC_CK(cudaGetLastError());
     g->planned = true;
@@ -644,6 +664,7 @@ tc_status run_count(tc_graph* g) {
     if ((st = zero_counts(g)) != TC_OK) return st;
     CountBuffers C = count_buffers(g);
     launch_intersect(C, g->strat, g->capture ? nullptr : g->sync.ev, g->L);
+    g->side_joined = true;  // by C.hub_ready
     launch_sum_t(C, g->L);
     TC_CK(cudaGetLastError());
     g->counted = true;
@@ -656,6 +677,7 @@ void destroy(tc_graph* g) {
     if (!g) return;
     join_plan(g);
     free_list(g, &g->blocks);
+    g->sync.known_idle = !g->side_busy;
     if (g->has_sync) give_sync(g->device, &g->sync);
     delete g;
 }
@@ -1049,7 +1071,8 @@ tc_status tc_edge_support(tc_graph* g, int32_t* u_out, int32_t* v_out, uint32_t*
     if (e == cudaSuccess && (st = run_plan(g)) == TC_OK && (st = zero_counts(g)) == TC_OK) {
         CountBuffers C = count_buffers(g);
         C.sup = sup;
-        launch_intersect(C, g->strat, nullptr, g->L);  // leaves parts of t in t_rank: the next count starts it anew
+        launch_intersect(C, g->strat, nullptr, g->L);
+        g->side_joined = true;  // by C.hub_ready; leaves parts of t in t_rank: the next count starts it anew
         launch_support_out(g->n, g->rank, g->rowlen, g->rowinfo, g->col, sup, id_of, estart, stmp, dev ? u_out : du,
                            dev ? v_out : dv, dev ? support_out : ds, g->L);
         e = cudaGetLastError();

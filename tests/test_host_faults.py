@@ -136,3 +136,58 @@ def test_timings_are_the_graphs_own(fake, n):
         for timing in (fake.tc_graph_last_timing, fake.tc_graph_build_timing):
             assert timing(g, ms, 8) == (OK if size else EINVAL)
         fake.tc_graph_destroy(g)
+
+
+def _count(fake, g):
+    T = ctypes.c_uint64()
+    assert fake.tc_count(g, ctypes.byref(T)) == OK
+
+
+def test_streams_are_handed_on_once_they_are_idle(fake):
+    """A graph that is destroyed with work in flight leaves a busy second stream: the next one
+    takes another, so that its work does not wait for the first graph's."""
+    def side(k):
+        g = _graph(fake)
+        assert fake.lcc_compute(g, ctypes.c_void_p(_ptr(t)), None, DEVICE) == OK  # does not wait
+        fake.tc_graph_destroy(g)
+        return fake.fake_plan_side(k)
+
+    t = np.zeros(50, np.uint64)
+
+    first = side(0)
+    assert first > 0 and side(1) == first
+    fake.fake_busy(first, 1)
+    second = side(2)
+    assert second not in (0, first) and side(3) == second
+    fake.fake_busy(second, 1)
+    third = side(4)
+    assert third not in (0, first, second)
+    fake.fake_busy(first, 0)
+    fake.fake_busy(third, 1)
+    assert side(5) == first
+    fake.tc_release_cached_graphs()
+    assert fake.fake_live_streams() == 0 and fake.fake_live_events() == 0
+
+
+def test_the_sets_kept_are_bounded(fake):
+    streams, t = 0, np.zeros(50, np.uint64)
+    for k in range(80):
+        g = _graph(fake)
+        assert fake.lcc_compute(g, ctypes.c_void_p(_ptr(t)), None, DEVICE) == OK
+        fake.fake_busy(fake.fake_plan_side(k), 1)
+        fake.tc_graph_destroy(g)
+        streams = max(streams, fake.fake_live_streams())
+    assert streams <= 2 * 65
+
+
+@pytest.mark.parametrize("kth", range(1, 20))
+def test_nothing_is_lost_when_an_event_cannot_be_created(fake, kth):
+    s, d = _pairs(60)
+    g = ctypes.c_void_p()
+    fake.fake_fail(b"event", kth)
+    st = fake.tc_graph_create_from_edges(50, 60, _ptr(s), _ptr(d), HOST, None, ctypes.byref(g))
+    assert st in (OK, ECUDA) and bool(g.value) == (st == OK)
+    if st == OK:
+        fake.tc_graph_destroy(g)
+    fake.tc_release_cached_graphs()
+    assert fake.fake_live_streams() == 0 and fake.fake_live_events() == 0 and fake.fake_bytes() == 0
