@@ -52,7 +52,7 @@ DeviceState g_dev[64];
 // recorded anew.  At most SYNC_KEEP sets stay, until tc_release_cached_graphs.
 struct SyncSet {
     bool known_idle = false;  // given back by a graph that had waited for all its work: not asked (5 us)
-    cudaStream_t side = nullptr, copy = nullptr;
+    cudaStream_t side = nullptr, copy = nullptr;  // null: could not be created, the graph's own stream does it
     cudaEvent_t fork = nullptr, join = nullptr, landed = nullptr, allocated = nullptr;
     cudaEvent_t ev[PH_EVENTS] = {};
     cudaEvent_t bev[BP_EVENTS] = {};
@@ -60,7 +60,10 @@ struct SyncSet {
     cudaError_t create() {
         cudaError_t e = cudaSuccess;
         for (cudaStream_t* s : {&side, &copy})
-            if (e == cudaSuccess) e = cudaStreamCreateWithFlags(s, cudaStreamNonBlocking);
+            if (cudaStreamCreateWithFlags(s, cudaStreamNonBlocking) != cudaSuccess) {
+                *s = nullptr;
+                cudaGetLastError();
+            }
         for (cudaEvent_t* x : {&fork, &join, &landed, &allocated})
             if (e == cudaSuccess) e = cudaEventCreateWithFlags(x, cudaEventDisableTiming);
         for (cudaEvent_t& x : ev)
@@ -114,7 +117,7 @@ cudaError_t take_sync(int dev, SyncSet* out) {
 void give_sync(int dev, SyncSet* s) {
     {
         std::lock_guard<std::mutex> lock(g_sync_mutex);
-        if (g_sync[dev].size() < SYNC_KEEP) {
+        if (g_sync[dev].size() < SYNC_KEEP && s->side && s->copy) {
             try {
                 g_sync[dev].push_back(*s);
                 *s = SyncSet{};
@@ -412,7 +415,7 @@ tc_status need_sync(tc_graph* g) {
 
 // The second stream, for single graphs that are not recorded into a CUDA graph.
 const PlanStreams* side_streams(tc_graph* g, PlanStreams* out) {
-    if (g->capture || g->batch_G >= 0 || !g->has_sync) return nullptr;
+    if (g->capture || g->batch_G >= 0 || !g->has_sync || !g->sync.side) return nullptr;
     *out = PlanStreams{g->sync.side, g->sync.fork, g->sync.join};
     return out;
 }
@@ -748,7 +751,7 @@ tc_status tc_graph_create_from_edges(int32_t n, int64_t m, const int32_t* src, c
         return finish_create(g, st, out);
     }
     // the copy stream may only touch ds and dd once their allocation is ordered
-    const HostPairs hp{src, dst, g->sync.copy, g->sync.landed};
+    const HostPairs hp{src, dst, g->sync.copy ? g->sync.copy : g->stream, g->sync.landed};
     cudaError_t e = cudaEventRecord(g->sync.allocated, g->stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(hp.side, g->sync.allocated, 0);
     if (e != cudaSuccess)

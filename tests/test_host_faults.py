@@ -180,6 +180,21 @@ def test_the_sets_kept_are_bounded(fake):
     assert streams <= 2 * 65
 
 
+@pytest.mark.parametrize("kind", [HOST, DEVICE])
+@pytest.mark.parametrize("kth", [1, 2])
+def test_one_stream_is_enough(fake, kind, kth):
+    """Where a second stream cannot be created the work stays on the graph's own."""
+    fake.fake_fail(b"stream", kth)
+    g = _graph(fake, kind=kind)
+    _count(fake, g)
+    assert (fake.fake_plan_side(0) == 0) == (kth == 1)
+    fake.tc_graph_destroy(g)
+    g = _graph(fake, kind=kind)
+    _count(fake, g)
+    assert fake.fake_plan_side(1) != 0
+    fake.tc_graph_destroy(g)
+
+
 @pytest.mark.parametrize("kth", range(1, 20))
 def test_nothing_is_lost_when_an_event_cannot_be_created(fake, kth):
     s, d = _pairs(60)
