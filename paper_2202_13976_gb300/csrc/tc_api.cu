@@ -6,6 +6,7 @@
 // without returning it to the driver and without device-wide synchronisation.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <climits>
 #include <cmath>
@@ -278,6 +279,9 @@ class Slab {
         bytes_ += (count * sizeof(T) + 255) & ~(size_t)255;
         return *this;
     }
+    // Room of at least `bytes` from `from` on (an earlier end), for a second use of the arrays there.
+    void reach(size_t from, size_t bytes) { bytes_ = std::max(bytes_, (from + bytes + 255) & ~(size_t)255); }
+    size_t end() const { return bytes_; }
     tc_status alloc(tc_graph* g, std::vector<void*>* track) {
         char* base = nullptr;
         const tc_status st = dalloc(g, &base, bytes_, track);
@@ -421,7 +425,8 @@ const PlanStreams* side_streams(tc_graph* g, PlanStreams* out) {
 }
 
 tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64_t m, bool checked = true,
-                      const HostPairs* host = nullptr, const SegInfo* seg = nullptr, bool dir_bits = false) {
+                      const HostPairs* host = nullptr, const SegInfo* seg = nullptr, bool dir_bits = false,
+                      bool rows_only = false) {
     const int32_t n = g->n;
     const size_t nn = (size_t)n;
     tc_status st;
@@ -433,20 +438,39 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
     g->core_words = core_words_for(g->core_cap);
     const size_t cc = (size_t)g->core_cap;
     if (!g->capture && (st = need_sync(g)) != TC_OK) return st;
-    Slab kept;
+    // rows may be filled by buckets: room for two slots per pair
+    const bool buckets = seg ? m > 0 : m >= BUCKET_MIN_M;
+    BuildBuffers B{};
+    Slab kept, work;
     kept.add(&g->stats, 1).add(&g->t_rank, nn).add(&g->rank, nn).add(&g->rowstart, nn + 1).add(&g->rowlen, nn).add(&g->rowinfo, nn);
     kept.add(&g->col, (size_t)m).add(&g->deg, nn);
-    for (int32_t*& list : g->small_list) kept.add(&list, nn);
-    kept.add(&g->cta_list, nn);
-    kept.add(&g->hub_cnt, hc + 1).add(&g->hub_start, hc + 1).add(&g->hub_cur64, hc + 1).add(&g->big_list, hc + 1);
-    kept.add(&g->long_list, hc + 1).add(&g->win_task, (size_t)hub_task_cap(g->hub_cap, m));
-    kept.add(&g->low_task, (size_t)hub_task_cap(g->hub_cap, m)).add(&g->winrow, nn).add(&g->winlow, nn);
-    kept.add(&g->win, (size_t)win_vec_cap(n, m)).add(&g->in_rec, (size_t)m).add(&g->rowof, (size_t)m);
-    kept.add((char**)&g->plan_tmp, scan_tmp_bytes((int64_t)hc + 1));
-    kept.add(&g->core_bits, cc * (size_t)g->core_words + 4 * cc);
+    // the zeroed counters first: one memset
+    work.add(&B.dmulti, nn).add(&B.dupin, nn).add(&B.rowcnt, nn + 1).add(&B.bcount, (size_t)BUCKET_MAX + 1);
+    work.add(&B.bcap, (size_t)BUCKET_MAX).add(&B.bstart, (size_t)BUCKET_MAX + 1).add(&B.bfirst, (size_t)BUCKET_MAX + 1);
+    // The arrays of the plan serve the build for its pairs, rank keys and row lists first.  So
+    // the peak beside the input is 92 n + 4 m + max(16 m, 12 m + 16 win_vec_cap) bytes and
+    // arrays of a fixed size, never above 40 m + 100 n.  Rows alone need the build's part only.
+    Slab& plan = rows_only ? work : kept;
+    for (int k = 0; k < 4; ++k) plan.add(&g->small_list[k], (size_t)push_list_cap(n, m, k));
+    if (!rows_only) {
+        kept.add(&g->cta_list, (size_t)push_list_cap(n, m, 4));
+        kept.add(&g->hub_cnt, hc + 1).add(&g->hub_start, hc + 1).add(&g->hub_cur64, hc + 1).add(&g->big_list, hc + 1);
+        kept.add(&g->long_list, hc + 1).add(&g->win_task, (size_t)hub_task_cap(g->hub_cap, m));
+        kept.add(&g->low_task, (size_t)hub_task_cap(g->hub_cap, m)).add(&g->winrow, nn);
+        kept.add((char**)&g->plan_tmp, scan_tmp_bytes((int64_t)hc + 1));
+        kept.add(&g->core_bits, cc * (size_t)g->core_words + 4 * cc);
+    }
+    const size_t keys_at = plan.end();
+    plan.add(&B.keys, 0);
+    if (!rows_only) kept.add(&g->winlow, nn);
+    const size_t keys_alt = (nn + 31) & ~(size_t)31;  // whole sectors
+    plan.reach(keys_at, sizeof(uint64_t) * (keys_alt + nn));
+    const size_t pairs_at = plan.end();
+    plan.add(&B.pairs, 0);
+    if (!rows_only) kept.add(&g->in_rec, (size_t)m).add(&g->rowof, (size_t)m).add(&g->win, (size_t)win_vec_cap(n, m));
+    plan.reach(pairs_at, (buckets ? 2 : 1) * sizeof(int2) * (size_t)m);
     if ((st = kept.alloc(g, &keep)) != TC_OK) return st;
     std::vector<void*> scratch;
-    BuildBuffers B{};
     B.src = src;
     B.dst = dst;
     B.m = m;
@@ -468,21 +492,13 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
     size_t rt = radix_tmp_bytes((int64_t)nn);
     if (rt > tmp_bytes) tmp_bytes = rt;
     char* tmp = nullptr;
-    Slab work;  // the zeroed counters first: one memset
-    work.add(&B.dmulti, nn).add(&B.dupin, nn).add(&B.rowcnt, nn + 1).add(&B.bcount, (size_t)BUCKET_MAX + 1);
-    work.add(&B.keys, nn).add(&B.keys_alt, nn).add(&B.bcap, (size_t)BUCKET_MAX);
-    work.add(&B.bstart, (size_t)BUCKET_MAX + 1).add(&B.bfirst, (size_t)BUCKET_MAX + 1);
     work.add(&tmp, tmp_bytes);
-    // single graphs decide on buckets once the degrees are known; where both kinds fit, which
-    // is not for the very largest n only, the pairs are allocated ahead
-    if (B.bucket_fill || (m >= BUCKET_MIN_M && skewed_buckets_fit(n))) work.add(&B.pairs, 2 * (size_t)m);
     if ((st = work.alloc(g, &scratch)) != TC_OK) return st;
-    const size_t zeroed = (size_t)((char*)B.keys - (char*)B.dmulti);
-    B.seg = reinterpret_cast<uint32_t*>(g->small_list[3]);  // free until the plan
+    const size_t zeroed = (size_t)((char*)B.bcap - (char*)B.dmulti);
+    B.seg = reinterpret_cast<uint32_t*>(g->deg);  // free until the rows are sorted
+    B.keys_alt = B.keys + keys_alt;
     B.tmp = tmp;
-    // the input-order pairs and the sorters' row lists share memory with arrays that the
-    // planner writes after the build is done with them
-    B.oriented = reinterpret_cast<int2*>(g->in_rec);
+    B.oriented = B.pairs;  // one or the other
     B.longlist = g->small_list[0];
     B.midlist = g->small_list[1];
     B.midlist2 = g->small_list[2];
@@ -545,10 +561,6 @@ tc_status build_graph(tc_graph* g, const int32_t* src, const int32_t* dst, int64
         const double mean = n > 0 ? 2.0 * (double)m / (double)n : 0.0;
         B.skewed = (double)h.max_deg > 64.0 * mean;
         B.bucket_fill = m >= BUCKET_MIN_M && (!B.skewed || skewed_buckets_fit(n));
-        if (B.bucket_fill && !B.pairs && (st = dalloc(g, &B.pairs, 2 * (size_t)m, &scratch)) != TC_OK) {
-            free_list(g, &scratch);
-            return st;
-        }
     }
     launch_rank(B, deg_bits, g->L);
     if (bev) cudaEventRecord(bev[BP_RANK], g->stream);
@@ -702,16 +714,12 @@ namespace tcg {
 tc_status build_undirected_rows(int32_t n, int64_t m, const int32_t* src, const int32_t* dst, cudaStream_t stream,
                                 bool dir_bits, tc_graph** g, UndirectedRows* out) {
     *g = nullptr;
-    tc_status st;
-    if (!dir_bits) {
-        st = tc_graph_create_from_edges(n, m, src, dst, TC_MEM_DEVICE, stream, g);
-    } else {
-        if (n < 0 || n > (1 << 29) || m < 0 || m > INT_MAX || (m > 0 && (!src || !dst))) return TC_EINVAL;
-        tc_graph* h = nullptr;
-        if ((st = new_graph(n, stream, &h)) != TC_OK) return st;
-        h->m_in = m;
-        st = finish_create(h, build_graph(h, src, dst, m, true, nullptr, nullptr, true), g);
-    }
+    if (n < 0 || (dir_bits && n > (1 << 29)) || m < 0 || m > INT_MAX || (m > 0 && (!src || !dst))) return TC_EINVAL;
+    tc_graph* built = nullptr;
+    tc_status st = new_graph(n, stream, &built);
+    if (st != TC_OK) return st;
+    built->m_in = m;
+    st = finish_create(built, build_graph(built, src, dst, m, true, nullptr, nullptr, dir_bits, true), g);
     if (st != TC_OK) return st;
     DevStats h;
     if ((st = read_result_stats(*g, &h)) != TC_OK) return st;

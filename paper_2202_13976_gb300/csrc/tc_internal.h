@@ -116,9 +116,9 @@ struct BuildBuffers {
     uint64_t* keys_alt;   // n
     uint32_t* rowcnt;     // n + 1
     uint32_t* seg;        // n: graph of every vertex (batches)
-    int32_t* longlist;    // n
-    int32_t* midlist;     // n: rows of 17..256 entries
-    int32_t* midlist2;    // n: rows of 257..1024 entries
+    int32_t* longlist;    // min(n, m / 1025): rows of more than 1024 entries
+    int32_t* midlist;     // min(n, m / 17): rows of 17..256 entries
+    int32_t* midlist2;    // min(n, m / 257): rows of 257..1024 entries
     uint32_t* dupin;      // n: repeated entries dropped at each target
     uint32_t* bcount;     // BUCKET_MAX + 1: pairs per source bucket; buckets claimed by the fill
     uint32_t* bcap;       // BUCKET_MAX: degrees of each bucket's rows
@@ -218,6 +218,13 @@ inline int64_t hub_task_cap(int64_t hub_cap, int64_t m) { return hub_cap + m / H
 // Largest dense core (tc_core.cu): one core_n x core_n bit matrix.
 constexpr int CORE_MAX = 8192;
 
+// The planner's lists of sources: least d+ of each, and so the most entries.
+constexpr int PUSH_LIST_MIN[5] = {2, 9, 17, 33, 257};
+inline int64_t push_list_cap(int32_t n, int64_t m, int list) {
+    const int64_t by_m = m / PUSH_LIST_MIN[list];
+    return by_m < n ? by_m : n;
+}
+
 struct CountBuffers {
     int32_t n;
     const int64_t* rowstart;
@@ -225,8 +232,8 @@ struct CountBuffers {
     const int2* rowinfo;     // {first index in col, length} per row
     const int32_t* col;
     const int32_t* deg;
-    int32_t* small_list[4];  // n each: d+ <= 8, 16, 32, 256
-    int32_t* cta_list;       // n
+    int32_t* small_list[4];  // push_list_cap each: d+ <= 8, 16, 32, 256
+    int32_t* cta_list;       // push_list_cap
     // hub in-edges (transpose of the oriented edges that point into the hub ranks)
     int32_t hub_cap;         // min(n, HUB_BM_BITS): slots for ranks n - hub_cap .. n-1
     uint32_t* hub_cnt;       // hub_cap + 1

@@ -809,6 +809,9 @@ __global__ void k_hub_lists(int32_t n, int32_t hub_cap, int32_t T0w, const int2*
 // atomic per warp and list serialises on the four list counters.
 constexpr int PLAN_ITEMS = 4;
 constexpr int PLAN_LISTS = 5;  // d+ classes <= 8, <= 16, <= 32, <= SMALL_WIDE_MAX, larger
+static_assert(PUSH_LIST_MIN[0] == 2 && PUSH_LIST_MIN[1] == 9 && PUSH_LIST_MIN[2] == 17 && PUSH_LIST_MIN[3] == 33 &&
+                  PUSH_LIST_MIN[4] == SMALL_WIDE_MAX + 1,
+              "a class's least d+ bounds its list");
 
 // How often the probes of the hub kernels hit, from rows spread over the ranks: is the entry
 // in the middle of a row's upper half in the list of the one in the row's middle, a hub?

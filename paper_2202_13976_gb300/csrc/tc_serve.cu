@@ -56,9 +56,8 @@ double now_s(std::chrono::steady_clock::time_point t0) {
 }  // namespace
 
 uint64_t serve_estimate_bytes(int32_t n, int64_t m) {
-    // peak of one request: its pairs (8 m) and outputs, the graph (CSR, hub in-edges, source
-    // rows and window entries 18 m, per-vertex arrays), the build scratch (pairs 16 m) and
-    // the core
+    // peak of one request: its pairs and outputs (8 m + 16 n), the graph and its build
+    // (40 m + 100 n at most) and the arrays of a fixed size, the core's first
     return (uint64_t)(48 * m + 160 * (int64_t)n) + (16ull << 20);
 }
 

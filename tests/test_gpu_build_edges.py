@@ -71,3 +71,15 @@ def test_bucket_fill_of_large_graphs(tc, n, skewed):
         s[::2] = 0
         s[1:4000:2], d[1:4000:2] = n - 1, n - 2
     assert_matches_oracle(tc, n, s, d, device_io=True)
+
+
+@pytest.mark.parametrize("k", [2, 8, 9, 16, 17, 32, 33, 256, 257, 1025])
+@pytest.mark.parametrize("hubs", [(32, 131072), (1, 0)])
+def test_lists_filled_to_their_bound(tc, k, hubs):
+    """Every source has exactly k entries, so that the planner's list of its class, and the
+    sorters' lists, hold as many rows as the pairs allow."""
+    sources, heavy = 300, k + 40
+    rng = np.random.default_rng(k)
+    s = np.repeat(np.arange(sources), k)
+    d = sources + np.concatenate([rng.permutation(heavy)[:k] for _ in range(sources)])
+    assert_matches_oracle(tc, sources + heavy, s.astype(np.int32), d.astype(np.int32), hubs=hubs, device_io=True)

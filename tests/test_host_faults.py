@@ -206,3 +206,26 @@ def test_nothing_is_lost_when_an_event_cannot_be_created(fake, kth):
         fake.tc_graph_destroy(g)
     fake.tc_release_cached_graphs()
     assert fake.fake_live_streams() == 0 and fake.fake_live_events() == 0 and fake.fake_bytes() == 0
+
+
+MIB = 1 << 20
+
+
+@pytest.mark.parametrize("n,m", [(1 << 20, 16 << 20), (1 << 23, 8 << 23), (1 << 23, 60_000_000), (1 << 22, 1 << 22),
+                                 (100_000_000, 30_000_000), (400_000_000, 1 << 30), (1_500_000_000, (1 << 31) - 1),
+                                 ((1 << 31) - 1, 1000), ((1 << 31) - 1, 500_000_000), (1000, (1 << 31) - 1)])
+@pytest.mark.parametrize("directed", [0, 1])
+def test_memory_of_a_build(fake, n, m, directed):
+    """What a graph can have in pairs and vertices depends on the memory of its build: at most
+    40 bytes a pair beside the input and 100 a vertex, and the arrays of a fixed size."""
+    one = ctypes.c_void_p(64)  # never read here
+    fake.fake_max_deg(100)
+    if directed:
+        assert fake.fake_undirected_rows(n, m, one, one, 0) == OK
+    else:
+        g = ctypes.c_void_p()
+        assert fake.tc_graph_create_from_edges(n, m, one, one, DEVICE, None, ctypes.byref(g)) == OK
+        # and what stays: the arrays of the count
+        assert fake.fake_bytes() <= 32 * m + 130 * n + 64 * MIB
+        fake.tc_graph_destroy(g)
+    assert fake.fake_peak() <= 40 * m + 100 * n + 64 * MIB
