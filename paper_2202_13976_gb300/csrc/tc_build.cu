@@ -927,8 +927,6 @@ __global__ void __launch_bounds__(SEG_WARPS * 32, MAXK <= 8 ? 4 : 2) k_segsort_w
                 kept = warp_sort_row<4>(row, len, dupin, dup, lane);
             else
                 kept = warp_sort_row<8>(row, len, dupin, dup, lane);
-        } else if (MAXK <= 16) {
-            kept = warp_sort_row<16>(row, len, dupin, dup, lane);
         } else {
             if (len <= 512)
                 kept = warp_sort_row<16>(row, len, dupin, dup, lane);

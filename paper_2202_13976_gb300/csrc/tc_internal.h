@@ -28,7 +28,7 @@ struct DevStats {
     unsigned int ingest_blocks;    // build: blocks that have counted their pairs
     // from here on, zero when a plan starts
     unsigned int small_count[4];   // planner: vertices per small-list class (d+ <= 8, 16, 32, 256)
-    unsigned int cta_count;        // planner: vertices with d+ > 32
+    unsigned int cta_count;        // planner: vertices with d+ > 256
     unsigned int hub_count;        // vertices staged as hubs (ranks n - hub_count .. n-1)
     unsigned int hub_candidates;   // vertices whose degree reaches the hub threshold
     unsigned int hub_blocks;       // planner: blocks that have counted their candidates

@@ -263,33 +263,9 @@ __device__ void build_bitmap(uint32_t* bm, uint16_t* pre, uint32_t* slice, const
 // A = Lu[a0, du) (shared, sorted), B = N+(v) (global, sorted).  A match at position
 // p of Lu adds one to cnt[p].
 
-__device__ uint32_t lane_merge(const int32_t* Lu, int a0, int du, const int32_t* __restrict__ B, int b,
-                               uint32_t* cnt) {
-    if (a0 >= du || b == 0) return 0;
-    uint32_t c = 0;
-    int i = a0, k = 0;
-    int32_t x = Lu[i], y = B[0];
-    for (;;) {
-        if (x == y) {
-            atomicAdd(&cnt[i], 1u);
-            ++c;
-            if (++i >= du || ++k >= b) break;
-            x = Lu[i];
-            y = B[k];
-        } else if (x < y) {
-            if (++i >= du) break;
-            x = Lu[i];
-        } else {
-            if (++k >= b) break;
-            y = B[k];
-        }
-    }
-    return c;
-}
-
 // Merge with B read eight entries at a time (independent loads), A in shared memory.
 __device__ uint32_t lane_merge_batched(const int32_t* Lu, int a0, int du, const int32_t* __restrict__ B, int b,
-                                       uint32_t* cnt, uint32_t* __restrict__ supB) {
+                                       uint32_t* cnt) {
     uint32_t c = 0;
     int i = a0;
     const int32_t mx = Lu[du - 1];
@@ -302,7 +278,6 @@ __device__ uint32_t lane_merge_batched(const int32_t* Lu, int a0, int du, const 
             while (i < du && Lu[i] < y[q]) ++i;
             if (i < du && Lu[i] == y[q]) {
                 atomicAdd(&cnt[i], 1u);
-                if (supB) atomicAdd(&supB[k0 + q], 1u);
                 ++c;
                 ++i;
             }
@@ -314,7 +289,7 @@ __device__ uint32_t lane_merge_batched(const int32_t* Lu, int a0, int du, const 
 
 // keys of A looked up in B
 __device__ uint32_t lane_search(const int32_t* Lu, int a0, int du, const int32_t* __restrict__ B, int b,
-                                uint32_t* cnt, uint32_t* __restrict__ supB) {
+                                uint32_t* cnt) {
     uint32_t c = 0;
     int lo = 0;
     for (int i = a0; i < du && lo < b; ++i) {
@@ -323,7 +298,6 @@ __device__ uint32_t lane_search(const int32_t* Lu, int a0, int du, const int32_t
         lo = p;
         if (p < b && B[p] == x) {
             atomicAdd(&cnt[i], 1u);
-            if (supB) atomicAdd(&supB[p], 1u);
             ++c;
         }
     }
@@ -332,7 +306,7 @@ __device__ uint32_t lane_search(const int32_t* Lu, int a0, int du, const int32_t
 
 // keys of B looked up in A
 __device__ uint32_t lane_search_rev(const int32_t* Lu, int a0, int du, const int32_t* __restrict__ B, int b,
-                                    uint32_t* cnt, uint32_t* __restrict__ supB) {
+                                    uint32_t* cnt) {
     uint32_t c = 0;
     int lo = a0;
     const int32_t mx = Lu[du - 1];
@@ -343,7 +317,6 @@ __device__ uint32_t lane_search_rev(const int32_t* Lu, int a0, int du, const int
         lo = p;
         if (p < du && Lu[p] == y) {
             atomicAdd(&cnt[p], 1u);
-            if (supB) atomicAdd(&supB[k], 1u);
             ++c;
         }
     }
@@ -897,16 +870,14 @@ __global__ void __launch_bounds__(THREADS) k_plan(int32_t n, int samplers, const
 
 // ---- small bucket: groups of G lanes, one lane per edge -----------------------
 
-template <int G, bool SUP>
+template <int G>
 __global__ void __launch_bounds__(SMALL_WARPS * 32, SMALL_BLOCKS) k_tc_small(int32_t n, const int64_t* __restrict__ rowstart,
                                                                const int32_t* __restrict__ rowlen,
                                                                const int2* __restrict__ rowinfo,
                                                                const int32_t* __restrict__ col,
                                                                const int32_t* __restrict__ list, int cls,
                                                                unsigned long long* __restrict__ t, DevStats* stats,
-                                                               int strategy, float factor,
-                                                               uint32_t* __restrict__ sup_arg) {
-    uint32_t* const sup = SUP ? sup_arg : nullptr;  // per-edge support (tc_edge_support) or none
+                                                               int strategy, float factor) {
     constexpr int GPW = 32 / G;
     __shared__ int32_t sLu[SMALL_WARPS * 32];
     __shared__ uint32_t sCnt[SMALL_WARPS * 32];
@@ -938,15 +909,14 @@ __global__ void __launch_bounds__(SMALL_WARPS * 32, SMALL_BLOCKS) k_tc_small(int
             const int dv = ri.y;
             if (dv > 0) {
                 const int32_t* B = col + ri.x;
-                uint32_t* supB = sup ? sup + ri.x : nullptr;
                 const int a = du - g - 1;
                 int method = strategy;
                 if (method == TC_STRAT_AUTO) method = small_auto(a, dv, factor);
                 if (method == TC_STRAT_MERGE)
-                    c = lane_merge_batched(Lu, g + 1, du, B, dv, cnt, supB);
+                    c = lane_merge_batched(Lu, g + 1, du, B, dv, cnt);
                 else
-                    c = a <= dv ? lane_search(Lu, g + 1, du, B, dv, cnt, supB)
-                                : lane_search_rev(Lu, g + 1, du, B, dv, cnt, supB);
+                    c = a <= dv ? lane_search(Lu, g + 1, du, B, dv, cnt)
+                                : lane_search_rev(Lu, g + 1, du, B, dv, cnt);
                 if (c) atomicAdd(&cnt[g], c);
             }
         }
@@ -954,10 +924,7 @@ __global__ void __launch_bounds__(SMALL_WARPS * 32, SMALL_BLOCKS) k_tc_small(int
         for (int o = G / 2; o > 0; o >>= 1) c += __shfl_down_sync(gmask, c, o, G);
         __syncwarp(gmask);
         const uint32_t cv = cnt[g];
-        if (g < du && cv) {
-            atomicAdd(&t[Lu[g]], (unsigned long long)cv);
-            if (sup) atomicAdd(&sup[base + g], cv);  // edge (u, Lu[g]): as v of its edge and as w of others
-        }
+        if (g < du && cv) atomicAdd(&t[Lu[g]], (unsigned long long)cv);
         if (g == 0 && c) atomicAdd(&t[u], (unsigned long long)c);
         __syncwarp(gmask);
         u = un;
@@ -975,14 +942,11 @@ constexpr int SMALL_WIDE_G = 16;
 constexpr int SMALL_WIDE_BLOCKS = 6;  // blocks per SM
 constexpr int SMALL_WIDE_GROUPS = SMALL_WARPS * 32 / SMALL_WIDE_G;  // per block
 
-template <bool SUP>
 __global__ void __launch_bounds__(SMALL_WARPS * 32) k_tc_small_wide(int32_t n, const int2* __restrict__ rowinfo,
                                                                    const int32_t* __restrict__ col,
                                                                    const int32_t* __restrict__ list,
                                                                    unsigned long long* __restrict__ t,
-                                                                   DevStats* stats, int strategy, float factor,
-                                                                   uint32_t* __restrict__ sup_arg) {
-    uint32_t* const sup = SUP ? sup_arg : nullptr;
+                                                                   DevStats* stats, int strategy, float factor) {
     extern __shared__ __align__(16) unsigned char wide_sh[];
     constexpr int G = SMALL_WIDE_G;
     const int lane = lane_id(), w = threadIdx.x >> 5;
@@ -1011,14 +975,13 @@ __global__ void __launch_bounds__(SMALL_WARPS * 32) k_tc_small_wide(int32_t n, c
             const int dv = ri.y;
             if (dv == 0) continue;
             const int32_t* B = col + ri.x;
-            uint32_t* supB = sup ? sup + ri.x : nullptr;
             const int a = du - j - 1;
             int method = strategy;
             if (method == TC_STRAT_AUTO) method = small_auto(a, dv, factor);
             const uint32_t cj = method == TC_STRAT_MERGE
-                                    ? lane_merge_batched(Lu, j + 1, du, B, dv, cnt, supB)
-                                    : (a <= dv ? lane_search(Lu, j + 1, du, B, dv, cnt, supB)
-                                               : lane_search_rev(Lu, j + 1, du, B, dv, cnt, supB));
+                                    ? lane_merge_batched(Lu, j + 1, du, B, dv, cnt)
+                                    : (a <= dv ? lane_search(Lu, j + 1, du, B, dv, cnt)
+                                               : lane_search_rev(Lu, j + 1, du, B, dv, cnt));
             if (cj) atomicAdd(&cnt[j], cj);
             c += cj;
         }
@@ -1027,17 +990,14 @@ __global__ void __launch_bounds__(SMALL_WARPS * 32) k_tc_small_wide(int32_t n, c
         __syncwarp(gmask);
         for (int p = g; p < du; p += G) {
             const uint32_t cv = cnt[p];
-            if (cv) {
-                atomicAdd(&t[Lu[p]], (unsigned long long)cv);
-                if (sup) atomicAdd(&sup[ru.x + p], cv);
-            }
+            if (cv) atomicAdd(&t[Lu[p]], (unsigned long long)cv);
         }
         if (g == 0 && c) atomicAdd(&t[u], (unsigned long long)c);
         __syncwarp(gmask);
     }
 }
 
-// ---- block bucket: |N+(u)| > 32, non-hub targets ------------------------------
+// ---- block bucket: |N+(u)| > 256, non-hub targets ------------------------------
 
 // Open-addressing hash set of a staged list in shared memory (Fibonacci hashing, linear
 // probing, empty slots hold -1).  The table has at least twice as many slots as
@@ -1629,7 +1589,7 @@ __global__ void __launch_bounds__(CTA_THREADS) k_tc_cta(int32_t n, const int64_t
 //   k_tc_hub_med  window 1, the other hubs: a warp per hub
 //   k_tc_hub_win2 the windows below: a warp per slice
 //   k_tc_hub_low  the same for per-edge support, over a hash set of 32-bit ids
-//   k_tc_hub_list per-edge support of big hubs with a long list below window 1; in probe
+//   k_tc_hub_list per-edge support of big hubs with many entries below window 1; in probe
 //                 mode all big hubs
 // For R-MAT scale 20 / 23 they take 1.03 / 4.7 ms together; 32-bit ids against one bitmap
 // or hash set per hub took 1.28 / 5.94 ms.
@@ -1655,12 +1615,12 @@ struct ListProbe {
 };
 
 // One batch of up to 32 in-edges [k0, min(k0 + 32, e1)) of hub v, processed by one warp
-// over 32-bit ids (k_tc_hub_list): the whole suffixes (WHOLE), or their entries below
+// over 32-bit ids (k_tc_hub_list): the whole suffixes, or (SUP) their entries below
 // window 1.  Suffixes of HUB_LONG or more entries are read by lane groups (the read
 // stops above max N+(v)); shorter ones are laid end to end and read 32 entries at a
 // time.  Matches add to cnt[p] (or t[x] when cnt is null) and to the
 // per-in-edge total, which goes to t[u].  Returns the batch total (all lanes).
-template <bool SUP, bool WHOLE, class Probe>
+template <bool SUP, class Probe>
 __device__ uint32_t hub_batch(int64_t k0, int64_t e1, const uint2* __restrict__ in_rec,
                               const int2* __restrict__ rowinfo, const uint2* __restrict__ winrow,
                               const int32_t* __restrict__ col, int32_t maxv, const Probe& probe, uint32_t* cnt,
@@ -1676,7 +1636,7 @@ __device__ uint32_t hub_batch(int64_t k0, int64_t e1, const uint2* __restrict__ 
     if (a > 0) {
         const int2 ri = rowinfo[uu];
         b0 = ri.x + ri.y - a;
-        if (!WHOLE) a -= (int)winrow[uu].y;
+        if (SUP) a -= (int)winrow[uu].y;
     }
     uint32_t total_c = 0;
     const bool islong = a >= HUB_LONG;
@@ -2560,17 +2520,17 @@ struct HubListShared {
     unsigned bq;  // next batch of the current hub
 };
 
-// One block per hub: big hubs whose list below the window is too long for one warp (the
-// suffixes' entries below the window against that part of N+(v), staged as a bitmap
-// with prefix counts); in probe mode every big hub, the whole suffixes against the
-// sorted list N+(v).
+// One block per hub.  Per-edge support (SUP): big hubs with more than HUB_LIST_MIN entries
+// below the window, the suffixes' entries there against that part of N+(v), staged as a
+// bitmap with prefix counts.  Else probe mode: every big hub, the whole suffixes against
+// the sorted list N+(v).
 template <bool SUP>
 __global__ void __launch_bounds__(HUB_THREADS) k_tc_hub_list(
     int32_t n, int32_t hub_cap, const int2* __restrict__ rowinfo, const uint2* __restrict__ winrow,
     const int32_t* __restrict__ col, const int64_t* __restrict__ hub_start, const int32_t* __restrict__ list,
-    const uint2* __restrict__ in_rec, unsigned long long* __restrict__ t, DevStats* stats, int probe_mode,
-    uint32_t* __restrict__ sup_arg) {
+    const uint2* __restrict__ in_rec, unsigned long long* __restrict__ t, DevStats* stats, uint32_t* __restrict__ sup_arg) {
     uint32_t* const sup = SUP ? sup_arg : nullptr;
+    constexpr bool probe_mode = !SUP;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     HubListShared& sh = *reinterpret_cast<HubListShared*>(smem_raw);
     const int lane = lane_id(), w = threadIdx.x >> 5;
@@ -2613,10 +2573,10 @@ __global__ void __launch_bounds__(HUB_THREADS) k_tc_hub_list(
             const int64_t bb = e0 + (int64_t)__shfl_sync(FULL, k, 0) * bs;
             if (bb >= e1) break;
             const int64_t be = min(bb + bs, e1);
-            if (!probe_mode)
-                vtot += hub_batch<SUP, false>(bb, be, in_rec, rowinfo, winrow, col, maxv, PB, cnt, t, sh.cw[w], sup, base);
+            if constexpr (SUP)
+                vtot += hub_batch<true>(bb, be, in_rec, rowinfo, winrow, col, maxv, PB, cnt, t, sh.cw[w], sup, base);
             else
-                vtot += hub_batch<SUP, true>(bb, be, in_rec, rowinfo, winrow, col, maxv, PL, cnt, t, sh.cw[w], sup, base);
+                vtot += hub_batch<false>(bb, be, in_rec, rowinfo, winrow, col, maxv, PL, cnt, t, sh.cw[w], sup, base);
         }
         if (lane == 0) sh.vt[w] = vtot;
         __syncthreads();
@@ -2770,8 +2730,7 @@ cudaError_t intersect_init_attributes() {
     cudaError_t e = cudaSuccess;
     if ((e = cudaFuncSetAttribute(k_tc_cta<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CtaShared))) ||
         (e = cudaFuncSetAttribute(k_tc_cta<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CtaShared))) ||
-        (e = cudaFuncSetAttribute(k_tc_small_wide<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, wide)) ||
-        (e = cudaFuncSetAttribute(k_tc_small_wide<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, wide)) ||
+        (e = cudaFuncSetAttribute(k_tc_small_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, wide)) ||
         (e = cudaFuncSetAttribute(k_tc_hub<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(HubShared))) ||
         (e = cudaFuncSetAttribute(k_tc_hub<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(HubShared))) ||
         (e = cudaFuncSetAttribute(k_tc_hub_med<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2796,7 +2755,7 @@ void intersect_impl(const CountBuffers& C, const Strategy& S, cudaEvent_t* ev, c
     const int ss = S.strat[TC_BUCKET_SMALL];
     const float sf = S.factor[TC_BUCKET_SMALL];
     const int64_t top = C.dplus_bound;  // classes of longer sources are empty: left out
-    if (ss == TC_STRAT_HASH) {
+    if (SUP || ss == TC_STRAT_HASH) {  // the support always hashes
         k_tc_small_sets<8, SUP><<<L.sms * SETS_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
             C.n, C.rowinfo, C.col, C.small_list[0], 0, C.t_rank, C.stats, C.sup);
         count_launch();
@@ -2816,23 +2775,23 @@ void intersect_impl(const CountBuffers& C, const Strategy& S, cudaEvent_t* ev, c
             count_launch();
         }
     } else {
-        k_tc_small<8, SUP><<<L.sms * SMALL_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
-            C.n, C.rowstart, C.rowlen, C.rowinfo, C.col, C.small_list[0], 0, C.t_rank, C.stats, ss, sf, C.sup);
+        k_tc_small<8><<<L.sms * SMALL_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
+            C.n, C.rowstart, C.rowlen, C.rowinfo, C.col, C.small_list[0], 0, C.t_rank, C.stats, ss, sf);
         count_launch();
         if (top > 8) {
-            k_tc_small<16, SUP><<<L.sms * SMALL_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
-                C.n, C.rowstart, C.rowlen, C.rowinfo, C.col, C.small_list[1], 1, C.t_rank, C.stats, ss, sf, C.sup);
+            k_tc_small<16><<<L.sms * SMALL_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
+                C.n, C.rowstart, C.rowlen, C.rowinfo, C.col, C.small_list[1], 1, C.t_rank, C.stats, ss, sf);
             count_launch();
         }
         if (top > 16) {
-            k_tc_small<32, SUP><<<L.sms * SMALL_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
-                C.n, C.rowstart, C.rowlen, C.rowinfo, C.col, C.small_list[2], 2, C.t_rank, C.stats, ss, sf, C.sup);
+            k_tc_small<32><<<L.sms * SMALL_BLOCKS, SMALL_WARPS * 32, 0, L.stream>>>(
+                C.n, C.rowstart, C.rowlen, C.rowinfo, C.col, C.small_list[2], 2, C.t_rank, C.stats, ss, sf);
             count_launch();
         }
         if (top > 32) {
-            k_tc_small_wide<SUP><<<L.sms * SMALL_WIDE_BLOCKS, SMALL_WARPS * 32,
+            k_tc_small_wide<<<L.sms * SMALL_WIDE_BLOCKS, SMALL_WARPS * 32,
                               2 * SMALL_WIDE_GROUPS * SMALL_WIDE_MAX * sizeof(int32_t), L.stream>>>(
-                C.n, C.rowinfo, C.col, C.small_list[3], C.t_rank, C.stats, ss, sf, C.sup);
+                C.n, C.rowinfo, C.col, C.small_list[3], C.t_rank, C.stats, ss, sf);
             count_launch();
         }
     }
@@ -2872,10 +2831,10 @@ void intersect_impl(const CountBuffers& C, const Strategy& S, cudaEvent_t* ev, c
                     C.hub_cnt, C.n - C.hub_cap, C.in_rec, C.t_rank, C.stats);
             count_launch();
         }
-        if (probe || (SUP && T.first[1] > 0)) {
+        if (SUP ? T.first[1] > 0 : probe) {
             k_tc_hub_list<SUP><<<L.sms * HUB_BLOCKS, HUB_THREADS, sizeof(HubListShared), L.stream>>>(
-                C.n, C.hub_cap, C.rowinfo, C.winrow, C.col, C.hub_start, probe ? C.big_list : C.long_list, C.in_rec,
-                C.t_rank, C.stats, probe ? 1 : 0, C.sup);
+                C.n, C.hub_cap, C.rowinfo, C.winrow, C.col, C.hub_start, SUP ? C.long_list : C.big_list, C.in_rec,
+                C.t_rank, C.stats, C.sup);
             count_launch();
         }
     }
