@@ -191,90 +191,23 @@ __global__ void k_rank_invert(const uint64_t* __restrict__ sorted, int32_t n, in
 }
 
 // The ranks of a small graph by one block, in place of keys, a radix sort and an
-// inversion (8 launches or more, 20 us of GPU time; this one takes 8): a stable counting
-// sort on the degree, cut at RANK_BINS - 1.  Warp w takes a contiguous piece of the ids, so
-// a bin's ids are in order by (warp, round, lane).  The last bin's vertices, at most
-// 2 m / (RANK_BINS - 1) of them, are then ranked among each other directly.
+// inversion (8 launches or more, 20 us of GPU time; this one takes 8).  The last bin holds at
+// most 2 m / (RANK_BINS - 1) vertices.
 constexpr int RANK_ONE_N = 16384;
 constexpr int RANK_BINS = 1024;
 constexpr int RANK_TAIL = 1024;
 constexpr int64_t RANK_ONE_M = (int64_t)RANK_TAIL * (RANK_BINS - 1) / 2;  // pairs whose degrees fill the last bin
-constexpr int RANK_WARPS = RANK_BINS / 32;
-constexpr int RANK_HIST_BYTES = RANK_WARPS * RANK_BINS * (int)sizeof(uint16_t);
+constexpr int RANK_HIST_BYTES = RANK_BINS / 32 * RANK_BINS * (int)sizeof(uint16_t);
 
 __global__ void __launch_bounds__(RANK_BINS) k_rank_one(int32_t n, uint32_t* __restrict__ dmulti,
                                                         uint32_t* __restrict__ by_rank, int32_t* __restrict__ rank,
                                                         DevStats* stats) {
-    extern __shared__ uint16_t rank_hist[];  // [warp][bin]: counts, then the next rank
-    __shared__ uint32_t tdeg[RANK_TAIL];
-    __shared__ int32_t tid_of[RANK_TAIL];
-    __shared__ int warp_tot[RANK_WARPS];
-    __shared__ int tail0;
-    const int lane = lane_id(), w = threadIdx.x >> 5;
-    uint16_t* const mine = rank_hist + w * RANK_BINS;
-    for (int b = lane; b < RANK_BINS; b += 32) mine[b] = 0;
-    __syncwarp();
-    const int chunk = ((n + RANK_WARPS - 1) / RANK_WARPS + 31) & ~31;
-    const int i0 = min(w * chunk, n), i1 = min(i0 + chunk, n);
-    for (int b = i0; b < i1; b += 32) {
-        const int id = b + lane;
-        const int key = id < i1 ? (int)min(dmulti[id], (uint32_t)RANK_BINS - 1) : RANK_BINS + lane;
-        const unsigned peers = __match_any_sync(FULL, key);
-        if (id < i1 && lane == __ffs(peers) - 1) mine[key] = (uint16_t)(mine[key] + __popc(peers));
-        __syncwarp();
-    }
-    __syncthreads();
-    int cnt = 0;  // thread b: the bin's vertices, then its first rank
-    for (int k = 0; k < RANK_WARPS; ++k) cnt += rank_hist[k * RANK_BINS + threadIdx.x];
-    const int inc = warp_inclusive_scan(cnt);
-    if (lane == 31) warp_tot[w] = inc;
-    __syncthreads();
-    if (w == 0) {
-        const int v = warp_tot[lane];
-        warp_tot[lane] = warp_inclusive_scan(v) - v;
-    }
-    __syncthreads();
-    int base = warp_tot[w] + inc - cnt;
-    if (threadIdx.x == RANK_BINS - 1) tail0 = base;
-    for (int k = 0; k < RANK_WARPS; ++k) {
-        const int c = rank_hist[k * RANK_BINS + threadIdx.x];
-        rank_hist[k * RANK_BINS + threadIdx.x] = (uint16_t)base;
-        base += c;
-    }
-    __syncthreads();
-    const int t0 = tail0;
-    for (int b = i0; b < i1; b += 32) {
-        const int id = b + lane;
-        const uint32_t d = id < i1 ? dmulti[id] : 0u;
-        const int key = id < i1 ? (int)min(d, (uint32_t)RANK_BINS - 1) : RANK_BINS + lane;
-        const unsigned peers = __match_any_sync(FULL, key);
-        const int at = id < i1 ? mine[key] : 0;
-        __syncwarp();
-        if (id < i1) {
-            const int r = at + __popc(peers & lanemask_lt());
-            if (key < RANK_BINS - 1) {
-                rank[id] = r;
-                by_rank[r] = d;
-            } else if (r - t0 < RANK_TAIL) {  // always true: RANK_ONE_M
-                tdeg[r - t0] = d;
-                tid_of[r - t0] = id;
-            } else {
-                atomicOr(&stats->err, ERR_OVERFLOW);
-            }
-            if (lane == __ffs(peers) - 1) mine[key] = (uint16_t)(at + __popc(peers));
-        }
-        __syncwarp();
-    }
-    __syncthreads();
-    const int k = min(n - t0, RANK_TAIL);
-    if ((int)threadIdx.x < k) {
-        const uint32_t d = tdeg[threadIdx.x];
-        int r = t0;
-        for (int j = 0; j < k; ++j) r += tdeg[j] < d || (tdeg[j] == d && j < (int)threadIdx.x);
-        rank[tid_of[threadIdx.x]] = r;
+    extern __shared__ uint16_t rank_hist[];
+    const bool all = block_degree_ranks<RANK_BINS, RANK_TAIL>(n, dmulti, rank_hist, [&](int id, int r, uint32_t d) {
+        rank[id] = r;
         by_rank[r] = d;
-    }
-    __syncthreads();
+    });
+    if (!all && threadIdx.x == 0) atomicOr(&stats->err, ERR_OVERFLOW);  // never: RANK_ONE_M
     for (int r = threadIdx.x; r < n; r += RANK_BINS) dmulti[r] = by_rank[r];  // rewritten in rank space
 }
 

@@ -120,72 +120,15 @@ __device__ void na_degrees(const NaArrays& A, const int32_t* __restrict__ src, c
         if (na_sh[v]) atomicAdd(&A.dmulti[v], na_sh[v]);
 }
 
-// Ranks in (degree, id) order by one block: a stable counting sort on the degree, cut at
-// NA_BINS - 1.  Warp w takes a contiguous piece of the ids, so a bin's ids are in order by
-// (warp, round, lane).  The last bin's few vertices (2 m / (NA_BINS - 1) at most) are then
-// ranked among each other directly.
+// Ranks in (degree, id) order by one block; the last bin holds at most 2 m / (NA_BINS - 1)
+// vertices.
 constexpr int NA_BINS = 1024;
 constexpr int NA_TAIL = 2 * (int)NA_MAX_M / (NA_BINS - 1) + 1;
 static_assert(NA_BINS == NA_THREADS, "one bin per thread");
 
-__device__ void na_rank(const NaArrays& A, uint16_t* na_hist) {  // [warp][bin]: counts, then the next rank
-    __shared__ uint32_t tdeg[NA_TAIL];
-    __shared__ int32_t tid_of[NA_TAIL];
-    __shared__ int warp_tot[NA_WARPS], total, tail0;
-    const int lane = lane_id(), w = threadIdx.x >> 5;
-    uint16_t* const mine = na_hist + w * NA_BINS;
-    for (int b = lane; b < NA_BINS; b += 32) mine[b] = 0;
-    __syncwarp();
-    const int chunk = ((A.n + NA_WARPS - 1) / NA_WARPS + 31) & ~31;
-    const int i0 = min(w * chunk, A.n), i1 = min(i0 + chunk, A.n);
-    for (int b = i0; b < i1; b += 32) {
-        const int id = b + lane;
-        const int key = id < i1 ? (int)min(A.dmulti[id], (uint32_t)NA_BINS - 1) : NA_BINS + lane;
-        const unsigned peers = __match_any_sync(FULL, key);
-        if (id < i1 && lane == __ffs(peers) - 1) mine[key] = (uint16_t)(mine[key] + __popc(peers));
-        __syncwarp();
-    }
-    __syncthreads();
-    int run = 0;
-    for (int k = 0; k < NA_WARPS; ++k) run += na_hist[k * NA_BINS + threadIdx.x];
-    int base = block_scan_excl(run, warp_tot, &total);
-    if (threadIdx.x == NA_BINS - 1) tail0 = base;
-    for (int k = 0; k < NA_WARPS; ++k) {
-        const int c = na_hist[k * NA_BINS + threadIdx.x];
-        na_hist[k * NA_BINS + threadIdx.x] = (uint16_t)base;
-        base += c;
-    }
-    __syncthreads();
-    const int t0 = tail0;
-    for (int b = i0; b < i1; b += 32) {
-        const int id = b + lane;
-        const uint32_t d = id < i1 ? A.dmulti[id] : 0u;
-        const int key = id < i1 ? (int)min(d, (uint32_t)NA_BINS - 1) : NA_BINS + lane;
-        const unsigned peers = __match_any_sync(FULL, key);
-        const int at = id < i1 ? mine[key] : 0;
-        __syncwarp();
-        if (id < i1) {
-            const int r = at + __popc(peers & lanemask_lt());
-            if (key < NA_BINS - 1) {
-                A.rank[id] = r;
-            } else if (r - t0 < NA_TAIL) {  // always true
-                tdeg[r - t0] = d;
-                tid_of[r - t0] = id;
-            }
-            if (lane == __ffs(peers) - 1) mine[key] = (uint16_t)(at + __popc(peers));
-        }
-        __syncwarp();
-    }
-    __syncthreads();
-    const int k = min(A.n - t0, NA_TAIL);
-    if ((int)threadIdx.x < k) {
-        int r = 0;
-        for (int j = 0; j < k; ++j)
-            r += tdeg[j] < tdeg[threadIdx.x] || (tdeg[j] == tdeg[threadIdx.x] && j < (int)threadIdx.x);
-        A.rank[tid_of[threadIdx.x]] = t0 + r;
-    }
+__device__ void na_rank(const NaArrays& A, uint16_t* na_hist) {
+    block_degree_ranks<NA_BINS, NA_TAIL>(A.n, A.dmulti, na_hist, [&](int id, int r, uint32_t) { A.rank[id] = r; });
 }
-static_assert(NA_TAIL <= NA_THREADS, "one thread per vertex of the last bin");
 
 // Oriented pairs, each with its slot in its row.
 __device__ void na_count(const NaArrays& A, const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int blk,
