@@ -37,7 +37,7 @@ struct DevStats {
     unsigned int hub_tasks;        // window tasks of big hubs (slices of their in-edges)
     unsigned int hub_med;          // window tasks of the other hubs
     unsigned int hub_low;          // below-window tasks
-    unsigned int hub_long;         // big hubs with a long list below the window
+    unsigned int hub_long;         // big hubs with many entries below the window (per-edge support)
     unsigned int win_vecs;         // planner: 16-byte vectors of window entries written
     unsigned int samples;          // planner: hub probes sampled
     unsigned int sample_hits;      // planner: those of them that hit
@@ -240,7 +240,7 @@ struct CountBuffers {
     int64_t* hub_start;      // hub_cap + 1
     unsigned long long* hub_cur64;  // hub_cap + 1: next free slot of every hub's segment (planner)
     int32_t* big_list;       // hub_cap: big hubs, nearly highest rank first
-    int32_t* long_list;      // hub_cap: the big hubs with a long list below the window
+    int32_t* long_list;      // hub_cap: the big hubs with many entries below the window (per-edge support)
     int4* win_task;          // hub_task_cap: window tasks, big hubs from the front, the others from the back
     int4* low_task;          // hub_task_cap: tasks below window 1
     uint2* in_rec;           // m: in-edge {u, entries of N+(u) after the hub}

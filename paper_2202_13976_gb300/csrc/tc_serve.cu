@@ -118,7 +118,8 @@ void run_one(cudaMemPool_t pool, int sms, cudaStream_t stream, const tc_request&
             fail(st);
             break;
         }
-        // everything is queued before the first wait, which tc_count makes
+        // count, outputs and checksums are queued together; the checksums' copy waits for them,
+        // then tc_count and tc_graph_info read the statistics
         if ((st = lcc_compute(g, reinterpret_cast<uint64_t*>(t), lcc, TC_MEM_DEVICE)) != TC_OK) {
             fail(st);
             break;

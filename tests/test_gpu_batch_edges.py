@@ -31,8 +31,9 @@ def test_an_id_of_the_next_graph_is_refused(tc, at):
     n, off, s, d = _pack([_er(30, 255, 1), EMPTY, _er(30, 257, 2), _er(30, 288, 3)])
     s[at] = 30
     with tc.Graph.batch(n, off, torch.from_numpy(s).cuda(), torch.from_numpy(d).cuda()) as g:
-        with pytest.raises(Exception):
+        with pytest.raises(tc.TCError) as err:
             g.batch_count()
+        assert err.value.status == tc.TC_EINVAL
 
 
 @pytest.mark.parametrize("order", [0, 1])
