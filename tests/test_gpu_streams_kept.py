@@ -49,12 +49,30 @@ def test_threads_reuse_the_sets_of_destroyed_graphs(tc):
         tc.tc_release_cached_graphs()
 
 
+def test_graph_destroyed_with_work_in_flight(tc):
+    """The same graph in turn on one stream; each is destroyed before its outputs are done."""
+    import torch
+    n = 1 << 16
+    s, d = graphgen.rmat(16, 16 * n, seed=8)
+    ref = oracle.triangles(n, s, d)
+    src, dst = torch.from_numpy(s).cuda(), torch.from_numpy(d).cuda()
+    outs = []
+    for _ in range(6):
+        t = torch.empty(n, dtype=torch.int64, device="cuda")
+        with tc.Graph.from_edges(n, src, dst) as g:
+            g.lcc(t, torch.empty(n, dtype=torch.float64, device="cuda"))
+        outs.append(t)
+    torch.cuda.synchronize()
+    for t in outs:
+        np.testing.assert_array_equal(t.cpu().numpy().view(np.uint64), ref["t"])
+
+
 def _lcc_without_waiting(tc, g, t, lcc):
     """lcc_compute itself: the binding's lcc() reads the graph's size, which waits."""
     assert tc.lib().lcc_compute(g.handle, t.data_ptr(), lcc.data_ptr(), tc.TC_MEM_DEVICE) == tc.TC_OK
 
 
-def test_graphs_destroyed_with_work_in_flight(tc):
+def test_graphs_on_two_streams_destroyed_with_work_in_flight(tc):
     """Different graphs on two streams in turn; each is destroyed while its count runs, so the
     next one may find its streams and events busy, its memory free."""
     import torch
